@@ -246,6 +246,7 @@ static PathConsts path_consts(const Physics& ph) {
   PathConsts c;
   c.f = path_k_of<float>(ph);
   c.d = path_k_of<double>(ph);
+  c.x = xconsts(ph.gamma, ph.eps);
   return c;
 }
 

@@ -20,6 +20,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "xfix.cuh"
+
 namespace gbcfd {
 
 constexpr int HALO = 2;
@@ -85,6 +87,7 @@ template <typename T> struct PathK {
 struct PathConsts {
   PathK<float> f;
   PathK<double> d;
+  XConsts x;  // FP64 path: the Roe flux's constants as 64-bit block-floating values
 };
 
 // ---- one block as the stage kernel sees it (device-resident descriptor table) --------------

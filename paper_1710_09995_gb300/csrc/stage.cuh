@@ -308,6 +308,82 @@ template <typename T> __device__ __forceinline__ const PathK<T>& path_k(const Gr
 template <> __device__ __forceinline__ const PathK<float>& path_k<float>(const GroupParams& P) { return P.pk.f; }
 template <> __device__ __forceinline__ const PathK<double>& path_k<double>(const GroupParams& P) { return P.pk.d; }
 
+// The end of stages 1 and 3, called by all threads of every CTA: the CTA's sums of R^2 (nacc) and
+// largest rate go to its partial slot; the last CTA to finish (atomic counter) reduces, per block,
+// the slots of the CTAs that worked on it (in CTA order: deterministic), and for stage 3 takes the
+// group's time step from the largest rate.
+template <int STAGE, int NWARP>
+__device__ __forceinline__ void stage_reduce(const GroupParams& P, double* red, int* slast, const double (&nacc)[5],
+                                             double rate) {
+  constexpr int NT = 32 * NWARP;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double part[6] = {nacc[0], nacc[1], nacc[2], nacc[3], nacc[4], rate};
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+    for (int m = 0; m < 5; ++m) part[m] += __shfl_xor_sync(0xffffffffu, part[m], off);
+    part[5] = fmax(part[5], __shfl_xor_sync(0xffffffffu, part[5], off));
+  }
+  __syncthreads();
+  if (lane == 0)
+    for (int m = 0; m < 6; ++m) red[warp * NPART + m] = part[m];
+  __syncthreads();
+  if (tid == 0) {
+    double sum[6] = {0, 0, 0, 0, 0, 0};
+    for (int w = 0; w < NWARP; ++w) {
+      for (int m = 0; m < 5; ++m) sum[m] += red[w * NPART + m];
+      sum[5] = fmax(sum[5], red[w * NPART + 5]);
+    }
+    for (int m = 0; m < 6; ++m) P.partial[(size_t)blockIdx.x * NPART + m] = sum[m];
+    __threadfence();
+    const unsigned prev = atomicAdd(&P.gctrl->counter, 1u);
+    *slast = (prev == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!*slast) return;
+  __threadfence();
+  // every warp of the last CTA folds blocks warp, warp + NWARP, ... (a group may hold many
+  // blocks: one warp walking all of them serially left the SMs idle behind it)
+  double wmax = 0.0;
+  for (int b = warp; b < P.nblocks; b += NWARP) {
+    const BlockDesc* Db = P.table + b;
+    double s[6] = {0, 0, 0, 0, 0, 0};
+    for (int c = lane; c < Db->ctas; c += 32) {
+      const double* src = P.partial + (size_t)(Db->cta0 + c) * NPART;
+      for (int m = 0; m < 5; ++m) s[m] += __ldcg(src + m);
+      s[5] = fmax(s[5], __ldcg(src + 5));
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+      for (int m = 0; m < 5; ++m) s[m] += __shfl_xor_sync(0xffffffffu, s[m], off);
+      s[5] = fmax(s[5], __shfl_xor_sync(0xffffffffu, s[5], off));
+    }
+    wmax = fmax(wmax, s[5]);
+    if (lane == 0) {
+      const double n = (double)Db->g.nx * Db->g.ny * Db->g.nz;
+      if (STAGE == 1)
+        for (int m = 0; m < 5; ++m) Db->ctrl->norms[m] = sqrt(s[m] / n);
+      if (STAGE == 3) Db->ctrl->rate = s[5];
+    }
+  }
+  if constexpr (STAGE == 3) {
+    if (lane == 0) red[warp] = wmax;
+    __syncthreads();
+    double gmax = 0.0;
+    for (int w = 0; w < NWARP; ++w) gmax = fmax(gmax, red[w]);
+    const double dtn = P.ph.cfl / gmax;
+    for (int b = tid; b < P.nblocks; b += NT) P.table[b].ctrl->dt = dtn;
+    if (tid == 0) {
+      P.gctrl->rate = gmax;
+      P.gctrl->dt = dtn;
+    }
+  }
+  if (tid == 0) {
+    P.gctrl->counter = 0u;
+  }
+}
+
 // ---- the kernel ------------------------------------------------------------------------------
 // One launch advances one Runge-Kutta stage of a group of blocks (a single block is a group of
 // one).  STAGE 0: residual only (one block, R to P.rout); 1..3: the stages of Eqs. 4-6.
@@ -350,6 +426,7 @@ __global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) 
   K.mu = VISC ? (CURVI ? PK.mu : PK.mu + PK.mu) : T(0);
   K.kappa = VISC ? (CURVI ? PK.kappa : T(4) * PK.kappa) : T(0);
   K.lim = ph.limiter;
+  if constexpr (!MIXED) static_cast<XConsts&>(K.x) = P.pk.x;
   const T gm1 = PK.gm1;
   const RateK<T> RK = {PK.gam, PK.vf};
   const T cflT = PK.cfl;
@@ -394,38 +471,6 @@ __global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) 
   const long long u_end = (long long)(lcta + 1) * W / nctas;
   constexpr unsigned QBYTES = 5u * MS * sizeof(T);
   constexpr unsigned DBYTES = 5u * MS * sizeof(float);
-
-  // this CTA's sums -> partial slot blockIdx.x; all threads call it together
-  auto flush = [&]() {
-    if constexpr (STAGE == 1 || STAGE == 3) {
-      double part[6];
-#pragma unroll
-      for (int m = 0; m < 5; ++m) {
-        part[m] = nacc[m];
-        nacc[m] = 0.0;
-      }
-      part[5] = double(rate_max);
-      rate_max = T(0);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int m = 0; m < 5; ++m) part[m] += __shfl_xor_sync(0xffffffffu, part[m], off);
-        part[5] = fmax(part[5], __shfl_xor_sync(0xffffffffu, part[5], off));
-      }
-      __syncthreads();
-      if (lane == 0)
-        for (int m = 0; m < 6; ++m) red[warp * NPART + m] = part[m];
-      __syncthreads();
-      if (tid == 0) {
-        double sum[6] = {0, 0, 0, 0, 0, 0};
-        for (int w = 0; w < NWARP; ++w) {
-          for (int m = 0; m < 5; ++m) sum[m] += red[w * NPART + m];
-          sum[5] = fmax(sum[5], red[w * NPART + 5]);
-        }
-        for (int m = 0; m < 6; ++m) P.partial[(size_t)blockIdx.x * NPART + m] = sum[m];
-      }
-    }
-  };
 
   // ring slot of plane kp (kp >= -2)
   auto rslot = [](int kp) { return kp & 3; };
@@ -782,59 +827,7 @@ __global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) 
   }
   if (bad) atomicOr(&D->ctrl->flag, FLAG_NONPHYSICAL);
 
-  if constexpr (STAGE == 1 || STAGE == 3) {
-    flush();
-    // the last CTA to finish reduces, per block, the slots of the CTAs that worked on it (in CTA
-    // order: deterministic), and for stage 3 takes the group's time step from the largest rate
-    if (tid == 0) {
-      __threadfence();
-      const unsigned prev = atomicAdd(&P.gctrl->counter, 1u);
-      *slast = (prev == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!*slast) return;
-    __threadfence();
-    // every warp of the last CTA folds blocks warp, warp + NWARP, ... (a group may hold many
-    // blocks: one warp walking all of them serially left the SMs idle behind it)
-    double wmax = 0.0;
-    for (int b = warp; b < P.nblocks; b += NWARP) {
-      const BlockDesc* Db = P.table + b;
-      double s[6] = {0, 0, 0, 0, 0, 0};
-      for (int c = lane; c < Db->ctas; c += 32) {
-        const double* src = P.partial + (size_t)(Db->cta0 + c) * NPART;
-        for (int m = 0; m < 5; ++m) s[m] += __ldcg(src + m);
-        s[5] = fmax(s[5], __ldcg(src + 5));
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int m = 0; m < 5; ++m) s[m] += __shfl_xor_sync(0xffffffffu, s[m], off);
-        s[5] = fmax(s[5], __shfl_xor_sync(0xffffffffu, s[5], off));
-      }
-      wmax = fmax(wmax, s[5]);
-      if (lane == 0) {
-        const double n = (double)Db->g.nx * Db->g.ny * Db->g.nz;
-        if (STAGE == 1)
-          for (int m = 0; m < 5; ++m) Db->ctrl->norms[m] = sqrt(s[m] / n);
-        if (STAGE == 3) Db->ctrl->rate = s[5];
-      }
-    }
-    if constexpr (STAGE == 3) {
-      if (lane == 0) red[warp] = wmax;
-      __syncthreads();
-      double gmax = 0.0;
-      for (int w = 0; w < NWARP; ++w) gmax = fmax(gmax, red[w]);
-      const double dtn = ph.cfl / gmax;
-      for (int b = tid; b < P.nblocks; b += NT) P.table[b].ctrl->dt = dtn;
-      if (tid == 0) {
-        P.gctrl->rate = gmax;
-        P.gctrl->dt = dtn;
-      }
-    }
-    if (tid == 0) {
-      P.gctrl->counter = 0u;
-    }
-  }
+  if constexpr (STAGE == 1 || STAGE == 3) stage_reduce<STAGE, NWARP>(P, red, slast, nacc, double(rate_max));
 }
 
 }  // namespace gbcfd

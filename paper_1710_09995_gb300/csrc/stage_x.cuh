@@ -1,0 +1,485 @@
+// stage_x.cuh -- the fused Runge-Kutta stage of the FP64 path on Cartesian blocks, with the faces in
+// 64-bit block-floating arithmetic (xfix.cuh).
+//
+// Same method, tiles, TMA staging, group table and reductions as stage_kernel (stage.cuh); what
+// differs is where the work runs.  This part's FP64 pipe issues one operation per 64 integer ones,
+// and the faces' reconstruction and fluxes were ~95% of the FP64 operations of a cell.  Here the
+// staged planes are converted once per cell to primitives in the ring as a 60-bit signed integer
+// and an exponent each, and the faces (MUSCL, Roe, viscous flux) run on the integer pipes.
+//
+// Faces are work items of a warp: the tile's z-, y- and x-rows (32 faces each) and one item of the
+// TY faces on the tile's upper x side, 3 TY + 2 items per plane dealt round-robin to the warps.  The
+// three directions go through the same instructions (index offsets and the frame's permutation
+// are data): a face is about 2000 instructions, and a copy per direction (six call sites in the
+// first version) streamed the code through the instruction caches on every plane.
+#pragma once
+#include "stage.cuh"
+
+namespace gbcfd {
+
+template <bool VISC, int TYV, int NWV>
+struct XPlan {
+  static constexpr int TY = TYV, BY = box_rows(TYV), NW = NWV;
+  static constexpr int NV = VISC ? 6 : 5;  // rho u v w p [theta]
+  static constexpr int BOX = BY * BX;
+  static constexpr size_t QSLOT = (sizeof(double) * 5 * BOX + 127) / 128 * 128;
+  static constexpr size_t stq = 0;                                          // staged conserved planes
+  static constexpr size_t ringm = stq + NSTAGE * QSLOT;                     // primitives: 60-bit integers
+  static constexpr size_t ringe = ringm + sizeof(long long) * NRING * NV * BOX;  // and their exponents (biased)
+  static constexpr size_t fx = (ringe + sizeof(short) * NRING * NV * BOX + 15) / 16 * 16;
+  static constexpr size_t fy = fx + sizeof(double) * 5 * TY * (TX + 1);
+  static constexpr size_t fz = fy + sizeof(double) * 5 * (TY + 1) * TX;     // two planes of z-faces
+  static constexpr size_t red = fz + sizeof(double) * 2 * 5 * TY * TX;
+  static constexpr size_t visc = red + sizeof(double) * NW * NPART;         // viscous coefficients (XVisc)
+  static constexpr size_t bar = visc + 5 * 3 * sizeof(XVal);
+  static constexpr size_t misc = bar + 8 * NSTAGE;
+  static constexpr size_t push = (misc + 16 + 15) / 16 * 16;
+  static constexpr size_t bytes = (push + 27 * sizeof(PushDst) + 127) / 128 * 128;
+};
+
+// viscous coefficients of the three directions: 2 mu / h and the tangential 2 mu / (4 h), with the
+// factors 4/3 and 2/3 of the normal stress, and 4 kappa / h
+struct XVisc {
+  XVal a[3], a43[3], b[3], b23[3], k[3];
+};
+
+// a ring value from a double: 60 bits, value = m 2^(e - 1021 - 61); subnormals read as zero
+__device__ __forceinline__ void xring_store(double a, long long* m, short* e) {
+  const unsigned long long b = xbits(a);
+  const int hi = (int)(b >> 32);
+  const int ex = (int)(((unsigned)hi >> 20) & 0x7ffu);
+  const unsigned long long mag = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b;
+  const long long s = hi >> 31;
+  *m = ex ? ((long long)(mag << 7) ^ s) - s : 0ll;
+  *e = (short)ex;
+}
+constexpr int XRING_BIAS = 1021;
+
+// half the minmod slope's double: 0 when a and b differ in sign, else the one of smaller magnitude
+__device__ __forceinline__ long long xminmod(long long a, long long b) {
+  const long long r = ((a < b) != (a < 0)) ? a : b;
+  return (a ^ b) < 0 ? 0ll : r;
+}
+
+// one warp item's index data: cells c[0..3] along the normal (c[1] = L, c[2] = R) as indices into
+// variable 0 of the ring; variable offsets of the normal and tangential velocities; tangential
+// neighbours (added to c[1], c[2])
+struct XItem {
+  int c[4];
+  int vn, v1, v2;
+  int t1p, t1m, t2p, t2m;
+};
+
+// twice the flux (F - Fv) through the lane's face
+template <bool VISC, int MS>
+__device__ __forceinline__ void xface(const long long* __restrict__ rm, const short* __restrict__ re, const XItem& I,
+                                      int d, const XVisc* __restrict__ X, const XConsts& K, int lim, XFlux& F) {
+  long long dn[3];  // R - L of the velocities (viscous)
+  long long us[3];
+  int eu[3];
+  // MUSCL in the class of the stencil's largest exponent; states doubled (class e - 1) with minmod
+  auto states = [&](int off, int q) -> XPair {
+    int e[4];
+    long long m[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      m[c] = rm[I.c[c] + off];
+      e[c] = re[I.c[c] + off];
+    }
+    const int E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3]));
+#pragma unroll
+    for (int c = 0; c < 4; ++c) m[c] = xshr(m[c], E - e[c]);  // [60]
+    const long long d01 = m[1] - m[0], d12 = m[2] - m[1], d23 = m[3] - m[2];
+    if (VISC && q >= 0) {
+      dn[q] = d12;
+      us[q] = m[1] + m[2];
+      eu[q] = E - XRING_BIAS;
+    }
+    if (lim) return {m[1] + ((d01 + d12) >> 2), m[2] - ((d12 + d23) >> 2), E - XRING_BIAS};
+    return {2 * m[1] + xminmod(d01, d12), 2 * m[2] - xminmod(d12, d23), E - XRING_BIAS - 1};
+  };
+  const XPair r = states(0, -1), u = states(I.vn, 0), v = states(I.v1, 1), w = states(I.v2, 2), p = states(4 * MS, -1);
+  xroe(r, u, v, w, p, K, F);
+  if constexpr (VISC) {
+    // sum over the two cells of the central differences of a variable along a tangent, [62]
+    auto tang = [&](int off, int tp, int tm, int& E) -> long long {
+      int e[4];
+      long long m[4];
+      const int ix[4] = {I.c[1] + tp, I.c[1] + tm, I.c[2] + tp, I.c[2] + tm};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        m[c] = rm[ix[c] + off];
+        e[c] = re[ix[c] + off];
+      }
+      E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3]));
+#pragma unroll
+      for (int c = 0; c < 4; ++c) m[c] = xshr(m[c], E - e[c]);
+      E -= XRING_BIAS;
+      return (m[0] - m[1]) + (m[2] - m[3]);
+    };
+    const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
+    // tau_nn = (4/3) 2 mu dun/dn - (2/3) 2 mu (dut1/dt1 + dut2/dt2), tau_nt = 2 mu (dut/dn + dun/dt)
+    XVal tn, t1, t2, th;
+    {
+      int e1, e2;
+      const long long g1 = tang(I.v1, I.t1p, I.t1m, e1), g2 = tang(I.v2, I.t2p, I.t2m, e2);
+      const int f0 = X->a43[d].e + eu[0] + 1, f1 = X->b23[d1].e + e1 + 1, f2 = X->b23[d2].e + e2 + 1;
+      tn.e = xmax(f0, xmax(f1, f2)) + 2;
+      tn.m = xshr(xmul<2>(X->a43[d].m, dn[0]), tn.e - f0) - xshr(xmul<2>(X->b23[d1].m, g1), tn.e - f1) -
+             xshr(xmul<2>(X->b23[d2].m, g2), tn.e - f2);
+    }
+    {
+      int e1;
+      const long long g1 = tang(I.vn, I.t1p, I.t1m, e1);
+      const int f0 = X->a[d].e + eu[1] + 1, f1 = X->b[d1].e + e1 + 1;
+      t1.e = xmax(f0, f1) + 1;
+      t1.m = xshr(xmul<2>(X->a[d].m, dn[1]), t1.e - f0) + xshr(xmul<2>(X->b[d1].m, g1), t1.e - f1);
+    }
+    {
+      int e2;
+      const long long g2 = tang(I.vn, I.t2p, I.t2m, e2);
+      const int f0 = X->a[d].e + eu[2] + 1, f2 = X->b[d2].e + e2 + 1;
+      t2.e = xmax(f0, f2) + 1;
+      t2.m = xshr(xmul<2>(X->a[d].m, dn[2]), t2.e - f0) + xshr(xmul<2>(X->b[d2].m, g2), t2.e - f2);
+    }
+    {
+      const int el = re[I.c[1] + 5 * MS], er = re[I.c[2] + 5 * MS], E = xmax(el, er);
+      th.m = xmul<2>(X->k[d].m, xshr(rm[I.c[2] + 5 * MS], E - er) - xshr(rm[I.c[1] + 5 * MS], E - el));
+      th.e = X->k[d].e + E - XRING_BIAS + 1;
+    }
+    auto sub = [&](int q, const XVal& t) {
+      const int E = xmax(F.e[q], t.e) + 1;
+      F.m[q] = xshr(F.m[q], E - F.e[q]) - xshr(t.m, E - t.e);
+      F.e[q] = E;
+    };
+    sub(1, tn);
+    sub(2, t1);
+    sub(3, t2);
+    const int f0 = eu[0] + tn.e + 1, f1 = eu[1] + t1.e + 1, f2 = eu[2] + t2.e + 1;
+    const int E = xmax(xmax(f0, f1), xmax(f2, th.e)) + 2;
+    const long long g = xshr(xmul<2>(us[0], tn.m), E - f0) + xshr(xmul<2>(us[1], t1.m), E - f1) +
+                        xshr(xmul<2>(us[2], t2.m), E - f2) + xshr(th.m, E - th.e);
+    sub(4, {g, E - 1});
+  }
+}
+
+// registers: NW warps in one CTA per SM (65536 / (32 NW) per thread)
+template <bool VISC, int STAGE, int TYV, int NWV, bool PUSH>
+__global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P) {
+  using PL = XPlan<VISC, TYV, NWV>;
+  constexpr int TY = TYV, BY = PL::BY, NW = NWV, NT = 32 * NWV, NV = PL::NV, MS = BY * BX, SL = NV * MS;
+  constexpr int NITEM = 3 * TY + 2;
+  using Fm = VM<double>;
+
+  extern __shared__ __align__(128) unsigned char smem[];
+  long long* rm = reinterpret_cast<long long*>(smem + PL::ringm);
+  short* re = reinterpret_cast<short*>(smem + PL::ringe);
+  double* fx = reinterpret_cast<double*>(smem + PL::fx);
+  double* fy = reinterpret_cast<double*>(smem + PL::fy);
+  double* fz = reinterpret_cast<double*>(smem + PL::fz);
+  double* red = reinterpret_cast<double*>(smem + PL::red);
+  XVisc* xv = reinterpret_cast<XVisc*>(smem + PL::visc);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + PL::bar);
+  int* sabort = reinterpret_cast<int*>(smem + PL::misc);
+  int* slast = sabort + 1;
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const Physics& ph = P.ph;
+  const double gm1 = P.pk.d.gm1;
+
+  // the block of this CTA and the CTA's contiguous share of its tile-planes
+  int bsel;
+  {
+    int lo = 0, hi = P.nblocks - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (P.table[mid].cta0 <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+    }
+    bsel = lo;
+  }
+  const BlockDesc* D = P.table + bsel;
+  const double hx = D->ihx, hy = D->ihy, hz = D->ihz;
+  PushDst* pushdst = reinterpret_cast<PushDst*>(smem + PL::push);
+  if (tid == 0) {
+    for (int s = 0; s < NSTAGE; ++s) mbar_init(&bar[s], 1);
+    fence_barrier_init();
+    *sabort = 0;
+  }
+  if constexpr (VISC) {
+    if (tid < 3) {
+      const double h = tid == 0 ? hx : (tid == 1 ? hy : hz), m2 = P.pk.d.mu + P.pk.d.mu;
+      xv->a[tid] = xdec_pos<62>(m2 * h);
+      xv->a43[tid] = xdec_pos<62>((4.0 / 3.0) * m2 * h);
+      xv->b[tid] = xdec_pos<62>(m2 * (0.25 * h));
+      xv->b23[tid] = xdec_pos<62>((2.0 / 3.0) * m2 * (0.25 * h));
+      xv->k[tid] = xdec_pos<62>(4.0 * P.pk.d.kappa * h);
+    }
+  }
+  if constexpr (PUSH && (STAGE == 1 || STAGE == 2)) {
+    if (tid < 27) push_table<double, STAGE>(P.table, bsel, tid, pushdst);
+  }
+  __syncthreads();
+
+  const double dt = (STAGE == 0) ? 0.0 : P.gctrl->dt;
+  unsigned phase_bits = 0;  // parity of each staging slot (uniform across the CTA)
+  unsigned pending = 0;     // slots with a copy in flight (meaningful in thread 0)
+  bool bad = false;         // non-physical value met by this thread
+  double nacc[5] = {0, 0, 0, 0, 0};
+  double rate_max = 0.0;
+
+  const int lcta = (int)blockIdx.x - D->cta0, nctas = D->ctas;
+  const long long W = D->units;
+  const long long u_begin = (long long)lcta * W / nctas;
+  const long long u_end = (long long)(lcta + 1) * W / nctas;
+  constexpr unsigned QBYTES = 5u * MS * sizeof(double);
+  const Geometry g = D->g;
+  // arrays of this stage
+  constexpr int in = STAGE == 0 ? 0 : STAGE - 1;
+  const CUtensorMap* tmq = &D->tq[in];
+  const double *qs = D->q[in], *qn = D->q[0];
+  double* qout = D->q[STAGE % 3];
+  const double hx2 = 0.5 * hx, hy2 = 0.5 * hy, hz2 = 0.5 * hz, hs2 = hx * hx + hy * hy + hz * hz;
+
+  for (long long u = u_begin; u < u_end;) {
+    const int nz = g.nz;
+    const long long tile = u / nz;
+    const int k0 = (int)(u - tile * nz);
+    const int k1 = (int)min((long long)nz, (long long)k0 + (u_end - u));
+    u += k1 - k0;
+    const int tix = (int)(tile % D->ntx), tiy = (int)(tile / D->ntx);
+    const int x0 = tix * TX, y0 = tiy * TY;  // storage coordinates of the box origin
+    const int last_plane = k1 + 1;
+
+    auto request = [&](int kp) {  // thread 0 only
+      const int s = (kp + 2) & (NSTAGE - 1);
+      fence_proxy_async();
+      mbar_expect_tx(&bar[s], QBYTES);
+      tma_load_4d(smem + PL::stq + s * PL::QSLOT, tmq, &bar[s], x0, y0, kp + HALO, 0);
+      pending |= 1u << s;
+    };
+    // wait for plane kp, convert it into ring slot kp & 3, then refill the staging slot
+    auto consume = [&](int kp) -> bool {
+      const int s = (kp + 2) & (NSTAGE - 1);
+      const bool ok = mbar_wait_bounded(&bar[s], (phase_bits >> s) & 1u);
+      if (!ok) atomicOr(sabort, 1);
+      phase_bits ^= 1u << s;
+      const double* sq = reinterpret_cast<const double*>(smem + PL::stq + s * PL::QSLOT);
+      long long* m = rm + (kp & 3) * SL;
+      short* e = re + (kp & 3) * SL;
+      for (int c = tid; c < MS; c += NT) {
+        const int cy = c / BX, cx = c - cy * BX;
+        double q[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) q[v] = sq[v * MS + c];
+        const bool valid = (x0 - HALO + cx < g.nx + HALO) && (y0 - HALO + cy < g.ny + HALO);
+        const double ir = Fm::rcp(q[0]);
+        const double uu = q[1] * ir, vv = q[2] * ir, ww = q[3] * ir;
+        const double p = gm1 * (q[4] - 0.5 * q[0] * (uu * uu + vv * vv + ww * ww));
+        // positive and finite, on the bit patterns
+        const long long br = __double_as_longlong(q[0]), bp = __double_as_longlong(p);
+        const bool phys = br > 0 && bp > 0 && br < 0x7ff0000000000000ll && bp < 0x7ff0000000000000ll;
+        if (valid && !phys) bad = true;
+        const bool fill = !valid || !phys;
+        xring_store(fill ? 1.0 : q[0], m + c, e + c);
+        xring_store(fill ? 0.0 : uu, m + MS + c, e + MS + c);
+        xring_store(fill ? 0.0 : vv, m + 2 * MS + c, e + 2 * MS + c);
+        xring_store(fill ? 0.0 : ww, m + 3 * MS + c, e + 3 * MS + c);
+        xring_store(fill ? 1.0 : p, m + 4 * MS + c, e + 4 * MS + c);
+        if (VISC) xring_store(fill ? 1.0 : p * ir, m + 5 * MS + c, e + 5 * MS + c);
+      }
+      __syncthreads();
+      if (tid == 0) {
+        pending &= ~(1u << s);
+        if (kp + NSTAGE <= last_plane && *sabort == 0) request(kp + NSTAGE);
+      }
+      return *sabort == 0;
+    };
+
+    if (tid == 0) {
+      tensormap_acquire(tmq);
+      request(k0 - 2);
+      request(k0 - 1);
+    }
+    bool ok = true;
+    for (int kp = k0 - 2; kp <= k0 && ok; ++kp) ok = consume(kp);
+    if (!ok) break;
+
+    // plane k0 - 1 only gives the lower z-faces of plane k0
+    for (int k = k0 - 1; k < k1; ++k) {
+      if (!consume(k + 2)) { ok = false; break; }
+      const int sm = ((k - 1) & 3) * SL, sk = (k & 3) * SL, sp = ((k + 1) & 3) * SL, s2 = ((k + 2) & 3) * SL;
+      double* fzk = fz + (k & 1) * (5 * TY * TX);
+      const int nitem = k < k0 ? TY : NITEM;
+#pragma unroll 1
+      for (int it = warp; it < nitem; it += NW) {
+        const int d = it < TY ? 2 : (it < 2 * TY + 1 ? 1 : 0);
+        int row = it < TY ? it : (it < 2 * TY + 1 ? it - TY : it - (2 * TY + 1));
+        int col = lane;
+        // rows of a ragged tile past the block's edge: y-rows up to the block's upper face
+        if (y0 + row > g.ny - (d == 1 ? 0 : 1) && row < TY) continue;
+        if (d == 1 && row == TY && y0 + TY > g.ny) continue;
+        if (d == 0 && row == TY) {  // the upper x-faces of the tile
+          if (x0 + TX > g.nx || lane >= TY || y0 + lane >= g.ny) continue;
+          row = lane;
+          col = TX;
+        }
+        const int b = sk + (row + HALO) * BX + col + HALO;
+        XItem I;
+        I.vn = (1 + d) * MS;
+        I.v1 = (d == 2 ? 1 : 2 + d) * MS;
+        I.v2 = (d == 0 ? 3 : d) * MS;
+        if (d == 2) {
+          I.c[0] = b - sk + sm; I.c[1] = b; I.c[2] = b - sk + sp; I.c[3] = b - sk + s2;
+          I.t1p = 1; I.t1m = -1; I.t2p = BX; I.t2m = -BX;
+        } else {
+          const int st = d == 0 ? 1 : BX;
+          I.c[0] = b - 2 * st; I.c[1] = b - st; I.c[2] = b; I.c[3] = b + st;
+          const int zp = sp - sk, zm = sm - sk;
+          I.t1p = d == 0 ? BX : zp; I.t1m = d == 0 ? -BX : zm;
+          I.t2p = d == 0 ? zp : 1; I.t2m = d == 0 ? zm : -1;
+        }
+        XFlux F;
+        xface<VISC, MS>(rm, re, I, d, xv, P.pk.x, ph.limiter, F);
+        double* f = d == 2 ? fzk + row * TX + col : (d == 1 ? fy + row * TX + col : fx + row * (TX + 1) + col);
+        const int fs = d == 2 ? TY * TX : (d == 1 ? (TY + 1) * TX : TY * (TX + 1));
+        f[0] = xflux(F, 0, 0);
+        f[(1 + d) * fs] = xflux(F, 1, 0);
+        f[(d == 2 ? 1 : 2 + d) * fs] = xflux(F, 2, 0);
+        f[(d == 0 ? 3 : d) * fs] = xflux(F, 3, 0);
+        f[4 * fs] = xflux(F, 4, 0);
+      }
+      __syncthreads();
+      if (k < k0) continue;
+      const double* fzl = fz + ((k - 1) & 1) * (5 * TY * TX);
+#pragma unroll 1
+      for (int row = warp; row < TY; row += NW) {
+        const int ci = x0 + lane, cj = y0 + row;
+        if (ci >= g.nx || cj >= g.ny) continue;
+        const long long o = gidx(g, ci, cj, k);
+        double dtc = dt;
+        if constexpr (STAGE >= 1 && !VISC)  // local time steps: inviscid blocks only
+          if (ph.local_dt) dtc = __ldg(static_cast<const double*>(D->dtl) + o);
+        double qs_[5], qn_[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          if constexpr (STAGE >= 1) qs_[v] = __ldg(qs + v * g.field + o);
+          if constexpr (STAGE >= 2) qn_[v] = __ldg(qn + v * g.field + o);
+        }
+        double R[5], out[5];
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+          const double ddx = fx[(m * TY + row) * (TX + 1) + lane + 1] - fx[(m * TY + row) * (TX + 1) + lane];
+          const double ddy = fy[(m * (TY + 1) + row + 1) * TX + lane] - fy[(m * (TY + 1) + row) * TX + lane];
+          const double ddz = fzk[(m * TY + row) * TX + lane] - fzl[(m * TY + row) * TX + lane];
+          R[m] = (ddx * hx2 + ddy * hy2) + ddz * hz2;  // doubled fluxes
+        }
+        if constexpr (STAGE == 0) {
+          const long long oc = ((long long)k * g.ny + cj) * g.nx + ci;
+          const long long n = (long long)g.nx * g.ny * g.nz;
+#pragma unroll
+          for (int m = 0; m < 5; ++m) P.rout[m * n + oc] = R[m];
+        } else {
+#pragma unroll
+          for (int m = 0; m < 5; ++m) {
+            const double adv = qs_[m] - dtc * R[m];
+            if constexpr (STAGE == 1) out[m] = adv;
+            else if constexpr (STAGE == 2) out[m] = 0.75 * qn_[m] + 0.25 * adv;
+            else out[m] = fma(2.0 / 3.0, adv, (1.0 / 3.0) * qn_[m]);  // an FP64 division costs ~7 FMAs here
+            qout[m * g.field + o] = out[m];
+          }
+          if constexpr (PUSH && (STAGE == 1 || STAGE == 2))
+            if (ci < HALO || cj < HALO || k < HALO || ci >= g.nx - HALO || cj >= g.ny - HALO || k >= g.nz - HALO)
+              push_halo<double>(pushdst, g.nx, g.ny, g.nz, ci, cj, k, out[0], out[1], out[2], out[3], out[4]);
+          if constexpr (STAGE == 1) {
+#pragma unroll
+            for (int m = 0; m < 5; ++m) nacc[m] = fma(R[m], R[m], nacc[m]);
+          }
+          if constexpr (STAGE == 3) {
+            const double ir = Fm::rcp(out[0]);
+            const double uu = out[1] * ir, vv = out[2] * ir, ww = out[3] * ir;
+            const double pp = gm1 * (out[4] - 0.5 * out[0] * (uu * uu + vv * vv + ww * ww));
+            if (!(out[0] > 0.0 && pp > 0.0)) bad = true;
+            const RateK<double> RK = {P.pk.d.gam, P.pk.d.vf};
+            const double rate = cell_rate<double>(out[0], uu, vv, ww, pp, RK, ph.viscous, hx, hy, hz, hs2);
+            rate_max = fmax(rate_max, rate);
+            if constexpr (!VISC)
+              if (ph.local_dt) static_cast<double*>(D->dtl)[o] = ph.cfl * Fm::rcp(rate);
+          }
+        }
+      }
+    }
+    if (!ok) break;
+  }
+
+  // abort path: drain copies still in flight (bounded), flag the timeout
+  if (*sabort) {
+    if (tid == 0) {
+      for (int s = 0; s < NSTAGE; ++s)
+        if (pending & (1u << s)) mbar_wait_bounded(&bar[s], (phase_bits >> s) & 1u);
+      atomicOr(&D->ctrl->flag, FLAG_TIMEOUT);
+    }
+  }
+  if (bad) atomicOr(&D->ctrl->flag, FLAG_NONPHYSICAL);
+
+  if constexpr (STAGE == 1 || STAGE == 3) stage_reduce<STAGE, NW>(P, red, slast, nacc, rate_max);
+}
+
+// ---- launch helpers --------------------------------------------------------------------------
+// warps per tile height: 3 TY + 2 items a plane
+constexpr int xwarps(int ty) { return ty == 8 ? 13 : 12; }
+
+template <bool VISC, int STAGE, int TYV, bool PUSH = false>
+cudaError_t xstage_attr() {
+  constexpr int NW = xwarps(TYV);
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((done.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
+  e = cudaFuncSetAttribute(xstage_kernel<VISC, STAGE, TYV, NW, PUSH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)XPlan<VISC, TYV, NW>::bytes);
+  if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_acq_rel);
+  return e;
+}
+template <bool VISC, int STAGE, int TYV, bool PUSH = false>
+cudaError_t xstage_go(const GroupParams& P, int grid, cudaStream_t s) {
+  constexpr int NW = xwarps(TYV);
+  cudaError_t e = xstage_attr<VISC, STAGE, TYV, PUSH>();
+  if (e != cudaSuccess) return e;
+  xstage_kernel<VISC, STAGE, TYV, NW, PUSH><<<grid, 32 * NW, XPlan<VISC, TYV, NW>::bytes, s>>>(P);
+  return cudaGetLastError();
+}
+template <bool VISC, int TYV>
+cudaError_t xstage_prepare() {
+  cudaError_t e = xstage_attr<VISC, 0, TYV>();
+  if (e == cudaSuccess) e = xstage_attr<VISC, 1, TYV>();
+  if (e == cudaSuccess) e = xstage_attr<VISC, 2, TYV>();
+  if (e == cudaSuccess) e = xstage_attr<VISC, 3, TYV>();
+  return e;
+}
+template <bool VISC, int TYV>
+cudaError_t xstage_dispatch(int stage, const GroupParams& P, int grid, cudaStream_t s) {
+  switch (stage) {
+    case 0: return xstage_go<VISC, 0, TYV>(P, grid, s);
+    case 1: return xstage_go<VISC, 1, TYV>(P, grid, s);
+    case 2: return xstage_go<VISC, 2, TYV>(P, grid, s);
+    case 3: return xstage_go<VISC, 3, TYV>(P, grid, s);
+  }
+  return cudaErrorInvalidValue;
+}
+template <int TYV>
+cudaError_t xstage_dispatch_push(int stage, const GroupParams& P, int grid, cudaStream_t s) {
+  switch (stage) {
+    case 1: return xstage_go<false, 1, TYV, true>(P, grid, s);
+    case 2: return xstage_go<false, 2, TYV, true>(P, grid, s);
+  }
+  return cudaErrorInvalidValue;
+}
+template <int TYV>
+cudaError_t xstage_prepare_push() {
+  cudaError_t e = xstage_attr<false, 1, TYV, true>();
+  if (e == cudaSuccess) e = xstage_attr<false, 2, TYV, true>();
+  return e;
+}
+
+}  // namespace gbcfd

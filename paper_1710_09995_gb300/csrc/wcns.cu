@@ -1016,6 +1016,7 @@ void fill_coef(const Args& a, Coef<T>& c) {
   c.K.mu = T(a.mu);
   c.K.kappa = T(kappa);
   c.K.lim = 0;
+  if constexpr (sizeof(T) == 8) static_cast<XConsts&>(c.K.x) = xconsts(a.gamma, a.eps);
 }
 
 Args make_args(gbcfd_wcns w) {
