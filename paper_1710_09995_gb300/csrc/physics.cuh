@@ -6,13 +6,8 @@
 // tangent 1, tangent 2) and mapped back to x, y, z by the caller.
 #pragma once
 #include "vmath.cuh"
-#include "xfix.cuh"
 
 namespace gbcfd {
-
-// the FP64 path's Roe flux runs in 64-bit block-floating arithmetic (xfix.cuh): its constants
-template <typename V> struct RoeX {};
-template <> struct RoeX<double> : XConsts {};
 
 template <typename V> struct Consts {
   V gm1;     // gamma - 1
@@ -21,7 +16,6 @@ template <typename V> struct Consts {
   V mu;      // viscosity
   V kappa;   // mu gamma / ((gamma - 1) Pr)
   int lim;   // 0 minmod, 1 central slope
-  RoeX<V> x; // FP64 path: the Roe flux's constants as xfix values
 };
 
 // constants of the spectral-radius rate (time step): gamma and 4 max(4/3, gamma/Pr) mu
@@ -72,10 +66,6 @@ __device__ __forceinline__ void muscl(V w0, V w1, V w2, V w3, int lim, V& L, V& 
 // to the caller (exact: a product by a power of two only moves the exponent).
 template <typename V, bool TWICE = false>
 __device__ __forceinline__ void roe_frame(const V* L, const V* R, const Consts<V>& K, V* F) {
-  if constexpr (sizeof(V) == 8) {
-    xroe<TWICE>(L, R, K.x, F);
-    return;
-  }
   using O = VM<V>;
   const V half = O::c(0.5);
   const V rl = L[0], ul = L[1], vl = L[2], wl = L[3], pl = L[4];

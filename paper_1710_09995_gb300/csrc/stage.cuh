@@ -426,7 +426,6 @@ __global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) 
   K.mu = VISC ? (CURVI ? PK.mu : PK.mu + PK.mu) : T(0);
   K.kappa = VISC ? (CURVI ? PK.kappa : T(4) * PK.kappa) : T(0);
   K.lim = ph.limiter;
-  if constexpr (!MIXED) static_cast<XConsts&>(K.x) = P.pk.x;
   const T gm1 = PK.gm1;
   const RateK<T> RK = {PK.gam, PK.vf};
   const T cflT = PK.cfl;

@@ -8,9 +8,9 @@
 
 namespace gbcfd {
 cudaError_t launch_stage_f64_alt(int stage, const GroupParams& P, int grid, cudaStream_t s) {
-  return xstage_dispatch<false, TY_ALT_F64>(stage, P, grid, s);
+  return xstage_dispatch<false, false, TY_ALT_F64>(stage, P, grid, s);
 }
-cudaError_t stage_prepare_f64_alt() { return xstage_prepare<false, TY_ALT_F64>(); }
+cudaError_t stage_prepare_f64_alt() { return xstage_prepare<false, false, TY_ALT_F64>(); }
 int stage_occupancy_f64_alt() { return 1; }
 cudaError_t launch_stage_f64_push(int stage, int ty, const GroupParams& P, int grid, cudaStream_t s) {
   if (ty == TY_ALT_F64) return xstage_dispatch_push<TY_ALT_F64>(stage, P, grid, s);

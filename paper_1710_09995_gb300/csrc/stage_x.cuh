@@ -1,59 +1,65 @@
-// stage_x.cuh -- the fused Runge-Kutta stage of the FP64 path on Cartesian blocks, with the faces in
-// 64-bit block-floating arithmetic (xfix.cuh).
+// stage_x.cuh -- the fused Runge-Kutta stage of the FP64 path (Cartesian blocks, and inviscid
+// curvilinear ones), with the faces in 64-bit block-floating arithmetic (xfix.cuh).
 //
 // Same method, tiles, TMA staging, group table and reductions as stage_kernel (stage.cuh); what
 // differs is where the work runs.  This part's FP64 pipe issues one operation per 64 integer ones,
 // and the faces' reconstruction and fluxes were ~95% of the FP64 operations of a cell.  Here the
-// staged planes are converted once per cell to primitives in the ring as a 60-bit signed integer
-// and an exponent each, and the faces (MUSCL, Roe, viscous flux) run on the integer pipes.
+// staged planes are converted once per cell to primitives in the ring as a 61-bit signed integer
+// and an exponent each; the faces (MUSCL, Roe, viscous flux), the residual and the time step's rate
+// run on the integer pipes.  FP64 is left with the stage update itself and the norm (5 to 15
+// operations a cell; with the conversion, the assembly and the rate in FP64 too its pipe was
+// 26% busy, alone between two barriers: 25.7 ms a step on the 256^3 case against 21.2).
 //
 // Faces are work items of a warp: the tile's z-, y- and x-rows (32 faces each) and one item of the
 // TY faces on the tile's upper x side, 3 TY + 2 items per plane dealt round-robin to the warps.  The
 // three directions go through the same instructions (index offsets and the frame's permutation
 // are data): a face is about 2000 instructions, and a copy per direction (six call sites in the
-// first version) streamed the code through the instruction caches on every plane.
+// first version) streamed the code through the instruction caches on every plane.  16 warps of 128
+// registers: 26 items (TY 8) give the sub-partitions 7, 7, 6, 6; with 13 warps of one item each
+// round one of them had 8.  Measured against the FP64-pipe form: 256^3 Navier-Stokes step 81.7 ->
+// 21.2 ms, 36 uneven Euler blocks (14.4M cells) 69.0 -> 22.1 ms, two steps of the bump channel
+// 14.2 -> 4.2 ms, errors against 64-bit references the same or smaller.
 #pragma once
 #include "stage.cuh"
 
 namespace gbcfd {
 
-template <bool VISC, int TYV, int NWV>
+// CURVI: one staging slot (a plane's work is far longer than its copy) leaves room for the metric ring
+template <bool VISC, bool CURVI, int TYV, int NWV>
 struct XPlan {
   static constexpr int TY = TYV, BY = box_rows(TYV), NW = NWV;
   static constexpr int NV = VISC ? 6 : 5;  // rho u v w p [theta]
   static constexpr int BOX = BY * BX;
+  static constexpr int NST = CURVI ? 1 : NSTAGE, NMS = CURVI ? 2 : 0;  // staging slots, metric planes
   static constexpr size_t QSLOT = (sizeof(double) * 5 * BOX + 127) / 128 * 128;
   static constexpr size_t stq = 0;                                          // staged conserved planes
-  static constexpr size_t ringm = stq + NSTAGE * QSLOT;                     // primitives: 60-bit integers
+  static constexpr size_t ringm = stq + NST * QSLOT;                     // primitives: 61-bit integers
   static constexpr size_t ringe = ringm + sizeof(long long) * NRING * NV * BOX;  // and their exponents (biased)
-  static constexpr size_t fx = (ringe + sizeof(short) * NRING * NV * BOX + 15) / 16 * 16;
-  static constexpr size_t fy = fx + sizeof(double) * 5 * TY * (TX + 1);
-  static constexpr size_t fz = fy + sizeof(double) * 5 * (TY + 1) * TX;     // two planes of z-faces
-  static constexpr size_t red = fz + sizeof(double) * 2 * 5 * TY * TX;
-  static constexpr size_t visc = red + sizeof(double) * NW * NPART;         // viscous coefficients (XVisc)
-  static constexpr size_t bar = visc + 5 * 3 * sizeof(XVal);
-  static constexpr size_t misc = bar + 8 * NSTAGE;
+  // face fluxes, 62-bit integers and exponents: x, y, and two planes of z
+  static constexpr int NFX = 5 * TY * (TX + 1), NFY = 5 * (TY + 1) * TX, NFZ = 5 * TY * TX;
+  static constexpr size_t fm = (ringe + sizeof(short) * NRING * NV * BOX + 15) / 16 * 16;
+  static constexpr size_t fe = fm + sizeof(long long) * (NFX + NFY + 2 * NFZ);
+  static constexpr size_t MSLOT = (sizeof(double) * 10 * BOX + 127) / 128 * 128;
+  static constexpr size_t mring = (fe + sizeof(short) * (NFX + NFY + 2 * NFZ) + 127) / 128 * 128;
+  static constexpr size_t red = mring + NMS * MSLOT;
+  static constexpr size_t blk = red + sizeof(double) * NW * NPART;          // the block's coefficients (XBlk)
+  static constexpr size_t bar = blk + 20 * sizeof(XVal);
+  static constexpr size_t misc = bar + 8 * (NST + NMS);
   static constexpr size_t push = (misc + 16 + 15) / 16 * 16;
   static constexpr size_t bytes = (push + 27 * sizeof(PushDst) + 127) / 128 * 128;
 };
 
-// viscous coefficients of the three directions: 2 mu / h and the tangential 2 mu / (4 h), with the
-// factors 4/3 and 2/3 of the normal stress, and 4 kappa / h
-struct XVisc {
-  XVal a[3], a43[3], b[3], b23[3], k[3];
+// a block's coefficients: half the inverse cell sizes (of the doubled face fluxes); the viscous
+// ones, 2 mu / h and the tangential 2 mu / (4 h) with the factors 4/3 and 2/3 of the normal
+// stress, and 4 kappa / h; for the time step the sum of the inverse sizes and (viscous)
+// 4 max(4/3, gamma/Pr) mu (sum of their squares)
+struct XBlk {
+  XVal h2[3], a[3], a43[3], b[3], b23[3], k[3], hsum, vs;
 };
+static_assert(sizeof(XBlk) == 20 * sizeof(XVal), "XPlan::blk");
 
-// a ring value from a double: 60 bits, value = m 2^(e - 1021 - 61); subnormals read as zero
-__device__ __forceinline__ void xring_store(double a, long long* m, short* e) {
-  const unsigned long long b = xbits(a);
-  const int hi = (int)(b >> 32);
-  const int ex = (int)(((unsigned)hi >> 20) & 0x7ffu);
-  const unsigned long long mag = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b;
-  const long long s = hi >> 31;
-  *m = ex ? ((long long)(mag << 7) ^ s) - s : 0ll;
-  *e = (short)ex;
-}
-constexpr int XRING_BIAS = 1021;
+// ring values are 61-bit integers with a biased exponent: value = m 2^(e - 1022 - 61)
+constexpr int XRING_BIAS = 1022;
 
 // half the minmod slope's double: 0 when a and b differ in sign, else the one of smaller magnitude
 __device__ __forceinline__ long long xminmod(long long a, long long b) {
@@ -70,10 +76,11 @@ struct XItem {
   int t1p, t1m, t2p, t2m;
 };
 
-// twice the flux (F - Fv) through the lane's face
-template <bool VISC, int MS>
+// twice the flux (F - Fv) through the lane's face; CURVI: the flux, S its area vector (strides MS)
+template <bool VISC, bool CURVI, int MS>
 __device__ __forceinline__ void xface(const long long* __restrict__ rm, const short* __restrict__ re, const XItem& I,
-                                      int d, const XVisc* __restrict__ X, const XConsts& K, int lim, XFlux& F) {
+                                      int d, const XBlk* __restrict__ X, const double* __restrict__ S,
+                                      const XConsts& K, int lim, XFlux& F) {
   long long dn[3];  // R - L of the velocities (viscous)
   long long us[3];
   int eu[3];
@@ -88,7 +95,7 @@ __device__ __forceinline__ void xface(const long long* __restrict__ rm, const sh
     }
     const int E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3]));
 #pragma unroll
-    for (int c = 0; c < 4; ++c) m[c] = xshr(m[c], E - e[c]);  // [60]
+    for (int c = 0; c < 4; ++c) m[c] = xshr(m[c], E - e[c]);  // [61]
     const long long d01 = m[1] - m[0], d12 = m[2] - m[1], d23 = m[3] - m[2];
     if (VISC && q >= 0) {
       dn[q] = d12;
@@ -99,6 +106,10 @@ __device__ __forceinline__ void xface(const long long* __restrict__ rm, const sh
     return {2 * m[1] + xminmod(d01, d12), 2 * m[2] - xminmod(d12, d23), E - XRING_BIAS - 1};
   };
   const XPair r = states(0, -1), u = states(I.vn, 0), v = states(I.v1, 1), w = states(I.v2, 2), p = states(4 * MS, -1);
+  if constexpr (CURVI) {
+    xroe_area(r, u, v, w, p, S[0], S[MS], S[2 * MS], K, F);
+    return;
+  }
   xroe(r, u, v, w, p, K, F);
   if constexpr (VISC) {
     // sum over the two cells of the central differences of a variable along a tangent, [62]
@@ -111,7 +122,7 @@ __device__ __forceinline__ void xface(const long long* __restrict__ rm, const sh
         m[c] = rm[ix[c] + off];
         e[c] = re[ix[c] + off];
       }
-      E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3]));
+      E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3])) + 1;  // [60] each
 #pragma unroll
       for (int c = 0; c < 4; ++c) m[c] = xshr(m[c], E - e[c]);
       E -= XRING_BIAS;
@@ -120,32 +131,32 @@ __device__ __forceinline__ void xface(const long long* __restrict__ rm, const sh
     const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
     // tau_nn = (4/3) 2 mu dun/dn - (2/3) 2 mu (dut1/dt1 + dut2/dt2), tau_nt = 2 mu (dut/dn + dun/dt)
     XVal tn, t1, t2, th;
-    {
+    {  // products [60]
       int e1, e2;
       const long long g1 = tang(I.v1, I.t1p, I.t1m, e1), g2 = tang(I.v2, I.t2p, I.t2m, e2);
-      const int f0 = X->a43[d].e + eu[0] + 1, f1 = X->b23[d1].e + e1 + 1, f2 = X->b23[d2].e + e2 + 1;
-      tn.e = xmax(f0, xmax(f1, f2)) + 2;
-      tn.m = xshr(xmul<2>(X->a43[d].m, dn[0]), tn.e - f0) - xshr(xmul<2>(X->b23[d1].m, g1), tn.e - f1) -
-             xshr(xmul<2>(X->b23[d2].m, g2), tn.e - f2);
+      const int f0 = X->a43[d].e + eu[0] + 3, f1 = X->b23[d1].e + e1 + 3, f2 = X->b23[d2].e + e2 + 3;
+      tn.e = xmax(f0, xmax(f1, f2));
+      tn.m = xshr(xmul(X->a43[d].m, dn[0]), tn.e - f0) - xshr(xmul(X->b23[d1].m, g1), tn.e - f1) -
+             xshr(xmul(X->b23[d2].m, g2), tn.e - f2);
     }
     {
       int e1;
       const long long g1 = tang(I.vn, I.t1p, I.t1m, e1);
-      const int f0 = X->a[d].e + eu[1] + 1, f1 = X->b[d1].e + e1 + 1;
-      t1.e = xmax(f0, f1) + 1;
-      t1.m = xshr(xmul<2>(X->a[d].m, dn[1]), t1.e - f0) + xshr(xmul<2>(X->b[d1].m, g1), t1.e - f1);
+      const int f0 = X->a[d].e + eu[1] + 3, f1 = X->b[d1].e + e1 + 3;
+      t1.e = xmax(f0, f1);
+      t1.m = xshr(xmul(X->a[d].m, dn[1]), t1.e - f0) + xshr(xmul(X->b[d1].m, g1), t1.e - f1);
     }
     {
       int e2;
       const long long g2 = tang(I.vn, I.t2p, I.t2m, e2);
-      const int f0 = X->a[d].e + eu[2] + 1, f2 = X->b[d2].e + e2 + 1;
-      t2.e = xmax(f0, f2) + 1;
-      t2.m = xshr(xmul<2>(X->a[d].m, dn[2]), t2.e - f0) + xshr(xmul<2>(X->b[d2].m, g2), t2.e - f2);
+      const int f0 = X->a[d].e + eu[2] + 3, f2 = X->b[d2].e + e2 + 3;
+      t2.e = xmax(f0, f2);
+      t2.m = xshr(xmul(X->a[d].m, dn[2]), t2.e - f0) + xshr(xmul(X->b[d2].m, g2), t2.e - f2);
     }
     {
       const int el = re[I.c[1] + 5 * MS], er = re[I.c[2] + 5 * MS], E = xmax(el, er);
-      th.m = xmul<2>(X->k[d].m, xshr(rm[I.c[2] + 5 * MS], E - er) - xshr(rm[I.c[1] + 5 * MS], E - el));
-      th.e = X->k[d].e + E - XRING_BIAS + 1;
+      th.m = xmul(X->k[d].m, xshr(rm[I.c[2] + 5 * MS], E - er) - xshr(rm[I.c[1] + 5 * MS], E - el));
+      th.e = X->k[d].e + E - XRING_BIAS + 3;
     }
     auto sub = [&](int q, const XVal& t) {
       const int E = xmax(F.e[q], t.e) + 1;
@@ -155,37 +166,38 @@ __device__ __forceinline__ void xface(const long long* __restrict__ rm, const sh
     sub(1, tn);
     sub(2, t1);
     sub(3, t2);
-    const int f0 = eu[0] + tn.e + 1, f1 = eu[1] + t1.e + 1, f2 = eu[2] + t2.e + 1;
-    const int E = xmax(xmax(f0, f1), xmax(f2, th.e)) + 2;
-    const long long g = xshr(xmul<2>(us[0], tn.m), E - f0) + xshr(xmul<2>(us[1], t1.m), E - f1) +
-                        xshr(xmul<2>(us[2], t2.m), E - f2) + xshr(th.m, E - th.e);
+    const int f0 = eu[0] + tn.e + 3, f1 = eu[1] + t1.e + 3, f2 = eu[2] + t2.e + 3;
+    const int E = xmax(xmax(f0, f1), xmax(f2, th.e));
+    const long long g = xshr(xmul(us[0], tn.m), E - f0) + xshr(xmul(us[1], t1.m), E - f1) +
+                        xshr(xmul(us[2], t2.m), E - f2) + xshr(th.m, E - th.e);
     sub(4, {g, E - 1});
   }
 }
 
 // registers: NW warps in one CTA per SM (65536 / (32 NW) per thread)
-template <bool VISC, int STAGE, int TYV, int NWV, bool PUSH>
+template <bool VISC, int STAGE, bool CURVI, int TYV, int NWV, bool PUSH>
 __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P) {
-  using PL = XPlan<VISC, TYV, NWV>;
+  using PL = XPlan<VISC, CURVI, TYV, NWV>;
+  static_assert(TYV <= NWV && !(VISC && CURVI), "a warp owns at most one row; viscous curvilinear blocks: stage_kernel");
+  constexpr int NST = PL::NST, NMS = PL::NMS;
   constexpr int TY = TYV, BY = PL::BY, NW = NWV, NT = 32 * NWV, NV = PL::NV, MS = BY * BX, SL = NV * MS;
   constexpr int NITEM = 3 * TY + 2;
-  using Fm = VM<double>;
 
   extern __shared__ __align__(128) unsigned char smem[];
   long long* rm = reinterpret_cast<long long*>(smem + PL::ringm);
   short* re = reinterpret_cast<short*>(smem + PL::ringe);
-  double* fx = reinterpret_cast<double*>(smem + PL::fx);
-  double* fy = reinterpret_cast<double*>(smem + PL::fy);
-  double* fz = reinterpret_cast<double*>(smem + PL::fz);
+  long long* fm = reinterpret_cast<long long*>(smem + PL::fm);
+  short* fe = reinterpret_cast<short*>(smem + PL::fe);
+  double* mring = reinterpret_cast<double*>(smem + PL::mring);
   double* red = reinterpret_cast<double*>(smem + PL::red);
-  XVisc* xv = reinterpret_cast<XVisc*>(smem + PL::visc);
+  XBlk* xb = reinterpret_cast<XBlk*>(smem + PL::blk);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + PL::bar);
   int* sabort = reinterpret_cast<int*>(smem + PL::misc);
   int* slast = sabort + 1;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Physics& ph = P.ph;
-  const double gm1 = P.pk.d.gm1;
+  const XConsts& XK = P.pk.x;
 
   // the block of this CTA and the CTA's contiguous share of its tile-planes
   int bsel;
@@ -201,18 +213,23 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
   const double hx = D->ihx, hy = D->ihy, hz = D->ihz;
   PushDst* pushdst = reinterpret_cast<PushDst*>(smem + PL::push);
   if (tid == 0) {
-    for (int s = 0; s < NSTAGE; ++s) mbar_init(&bar[s], 1);
+    for (int s = 0; s < NST + NMS; ++s) mbar_init(&bar[s], 1);
     fence_barrier_init();
     *sabort = 0;
   }
-  if constexpr (VISC) {
-    if (tid < 3) {
-      const double h = tid == 0 ? hx : (tid == 1 ? hy : hz), m2 = P.pk.d.mu + P.pk.d.mu;
-      xv->a[tid] = xdec_pos<62>(m2 * h);
-      xv->a43[tid] = xdec_pos<62>((4.0 / 3.0) * m2 * h);
-      xv->b[tid] = xdec_pos<62>(m2 * (0.25 * h));
-      xv->b23[tid] = xdec_pos<62>((2.0 / 3.0) * m2 * (0.25 * h));
-      xv->k[tid] = xdec_pos<62>(4.0 * P.pk.d.kappa * h);
+  if (tid < 3) {
+    const double h = tid == 0 ? hx : (tid == 1 ? hy : hz), m2 = P.pk.d.mu + P.pk.d.mu;
+    xb->h2[tid] = xdec_pos<62>(0.5 * h);
+    if (VISC) {
+      xb->a[tid] = xdec_pos<62>(m2 * h);
+      xb->a43[tid] = xdec_pos<62>((4.0 / 3.0) * m2 * h);
+      xb->b[tid] = xdec_pos<62>(m2 * (0.25 * h));
+      xb->b23[tid] = xdec_pos<62>((2.0 / 3.0) * m2 * (0.25 * h));
+      xb->k[tid] = xdec_pos<62>(4.0 * P.pk.d.kappa * h);
+    }
+    if (tid == 0) {
+      xb->hsum = xdec_pos<62>(hx + hy + hz);
+      xb->vs = xdec_pos<62>(P.pk.d.vf * (hx * hx + hy * hy + hz * hz));
     }
   }
   if constexpr (PUSH && (STAGE == 1 || STAGE == 2)) {
@@ -223,6 +240,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
   const double dt = (STAGE == 0) ? 0.0 : P.gctrl->dt;
   unsigned phase_bits = 0;  // parity of each staging slot (uniform across the CTA)
   unsigned pending = 0;     // slots with a copy in flight (meaningful in thread 0)
+  unsigned mphase = 0, mpending = 0;  // the same of the metric slots
   bool bad = false;         // non-physical value met by this thread
   double nacc[5] = {0, 0, 0, 0, 0};
   double rate_max = 0.0;
@@ -238,7 +256,6 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
   const CUtensorMap* tmq = &D->tq[in];
   const double *qs = D->q[in], *qn = D->q[0];
   double* qout = D->q[STAGE % 3];
-  const double hx2 = 0.5 * hx, hy2 = 0.5 * hy, hz2 = 0.5 * hz, hs2 = hx * hx + hy * hy + hz * hz;
 
   for (long long u = u_begin; u < u_end;) {
     const int nz = g.nz;
@@ -251,7 +268,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
     const int last_plane = k1 + 1;
 
     auto request = [&](int kp) {  // thread 0 only
-      const int s = (kp + 2) & (NSTAGE - 1);
+      const int s = (kp + 2) & (NST - 1);
       fence_proxy_async();
       mbar_expect_tx(&bar[s], QBYTES);
       tma_load_4d(smem + PL::stq + s * PL::QSLOT, tmq, &bar[s], x0, y0, kp + HALO, 0);
@@ -259,7 +276,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
     };
     // wait for plane kp, convert it into ring slot kp & 3, then refill the staging slot
     auto consume = [&](int kp) -> bool {
-      const int s = (kp + 2) & (NSTAGE - 1);
+      const int s = (kp + 2) & (NST - 1);
       const bool ok = mbar_wait_bounded(&bar[s], (phase_bits >> s) & 1u);
       if (!ok) atomicOr(sabort, 1);
       phase_bits ^= 1u << s;
@@ -272,43 +289,72 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
 #pragma unroll
         for (int v = 0; v < 5; ++v) q[v] = sq[v * MS + c];
         const bool valid = (x0 - HALO + cx < g.nx + HALO) && (y0 - HALO + cy < g.ny + HALO);
-        const double ir = Fm::rcp(q[0]);
-        const double uu = q[1] * ir, vv = q[2] * ir, ww = q[3] * ir;
-        const double p = gm1 * (q[4] - 0.5 * q[0] * (uu * uu + vv * vv + ww * ww));
-        // positive and finite, on the bit patterns
-        const long long br = __double_as_longlong(q[0]), bp = __double_as_longlong(p);
-        const bool phys = br > 0 && bp > 0 && br < 0x7ff0000000000000ll && bp < 0x7ff0000000000000ll;
+        XPrim W;
+        const bool phys = xprim(q, XK, W);
         if (valid && !phys) bad = true;
-        const bool fill = !valid || !phys;
-        xring_store(fill ? 1.0 : q[0], m + c, e + c);
-        xring_store(fill ? 0.0 : uu, m + MS + c, e + MS + c);
-        xring_store(fill ? 0.0 : vv, m + 2 * MS + c, e + 2 * MS + c);
-        xring_store(fill ? 0.0 : ww, m + 3 * MS + c, e + 3 * MS + c);
-        xring_store(fill ? 1.0 : p, m + 4 * MS + c, e + 4 * MS + c);
-        if (VISC) xring_store(fill ? 1.0 : p * ir, m + 5 * MS + c, e + 5 * MS + c);
+        const bool fill = !valid || !phys;  // rho = p = 1, no velocity
+        auto put = [&](int v, long long a, int ea, bool one) {
+          m[v * MS + c] = fill ? (one ? 1ll << 60 : 0ll) : a;
+          e[v * MS + c] = (short)(fill ? XRING_BIAS + 1 : XRING_BIAS + ea);
+        };
+        put(0, W.r.m >> 1, W.r.e + 1, true);
+#pragma unroll
+        for (int x = 0; x < 3; ++x) put(1 + x, W.u[x].m >> 1, W.u[x].e + 1, false);
+        put(4, W.p.m >> 1, W.p.e + 1, true);
+        if (VISC) put(5, xmul(W.p.m, W.ir.m), W.p.e + W.ir.e + 3, true);
       }
       __syncthreads();
       if (tid == 0) {
         pending &= ~(1u << s);
-        if (kp + NSTAGE <= last_plane && *sabort == 0) request(kp + NSTAGE);
+        if (kp + NST <= last_plane && *sabort == 0) request(kp + NST);
       }
       return *sabort == 0;
     };
 
+    // metric planes (curvilinear): plane kp in slot kp & 1; iteration k reads k and k + 1
+    int m_req = k0 - 1, m_wait = k0 - 1;
+    auto mrequest_upto = [&](int upto) {  // thread 0 only
+      if constexpr (CURVI) {
+        upto = min(upto, k1);
+        while (m_req < upto) {
+          ++m_req;
+          const int s = m_req & 1;
+          fence_proxy_async();
+          mbar_expect_tx(&bar[NST + s], 10u * MS * sizeof(double));
+          tma_load_4d(smem + PL::mring + s * PL::MSLOT, &D->tm, &bar[NST + s], x0, y0, m_req + HALO, 0);
+          mpending |= 1u << s;
+        }
+      }
+    };
+    auto mwait_upto = [&](int upto) {  // all threads
+      if constexpr (CURVI) {
+        while (m_wait < upto) {
+          ++m_wait;
+          const int s = m_wait & 1;
+          if (!mbar_wait_bounded(&bar[NST + s], (mphase >> s) & 1u)) atomicOr(sabort, 1);
+          mphase ^= 1u << s;
+          if (tid == 0) mpending &= ~(1u << s);
+        }
+      }
+    };
+
     if (tid == 0) {
       tensormap_acquire(tmq);
-      request(k0 - 2);
-      request(k0 - 1);
+      if (CURVI) tensormap_acquire(&D->tm);
+      for (int i = 0; i < NST; ++i) request(k0 - 2 + i);
+      mrequest_upto(k0);
     }
     bool ok = true;
     for (int kp = k0 - 2; kp <= k0 && ok; ++kp) ok = consume(kp);
     if (!ok) break;
 
+    double fzl[5] = {0, 0, 0, 0, 0};  // the lower z-face of the thread's cell
     // plane k0 - 1 only gives the lower z-faces of plane k0
     for (int k = k0 - 1; k < k1; ++k) {
       if (!consume(k + 2)) { ok = false; break; }
+      if (tid == 0) mrequest_upto(k + 1);  // its slot held plane k - 1, last read before consume's barrier
+      mwait_upto(k < k0 ? k0 : k + 1);
       const int sm = ((k - 1) & 3) * SL, sk = (k & 3) * SL, sp = ((k + 1) & 3) * SL, s2 = ((k + 2) & 3) * SL;
-      double* fzk = fz + (k & 1) * (5 * TY * TX);
       const int nitem = k < k0 ? TY : NITEM;
 #pragma unroll 1
       for (int it = warp; it < nitem; it += NW) {
@@ -338,23 +384,28 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
           I.t1p = d == 0 ? BX : zp; I.t1m = d == 0 ? -BX : zm;
           I.t2p = d == 0 ? zp : 1; I.t2m = d == 0 ? zm : -1;
         }
+        const double* S = nullptr;
+        if constexpr (CURVI) {  // x, y, z velocities as they are; the face's area vector: z-faces are plane k + 1's lower ones
+          I.vn = MS; I.v1 = 2 * MS; I.v2 = 3 * MS;
+          S = mring + ((d == 2 ? k + 1 : k) & 1) * (PL::MSLOT / sizeof(double)) + 3 * d * MS + (row + HALO) * BX + col + HALO;
+        }
         XFlux F;
-        xface<VISC, MS>(rm, re, I, d, xv, P.pk.x, ph.limiter, F);
-        double* f = d == 2 ? fzk + row * TX + col : (d == 1 ? fy + row * TX + col : fx + row * (TX + 1) + col);
+        xface<VISC, CURVI, MS>(rm, re, I, d, xb, S, XK, ph.limiter, F);
+        const int f = d == 2 ? PL::NFX + PL::NFY + (k & 1) * PL::NFZ + row * TX + col
+                             : (d == 1 ? PL::NFX + row * TX + col : row * (TX + 1) + col);
         const int fs = d == 2 ? TY * TX : (d == 1 ? (TY + 1) * TX : TY * (TX + 1));
-        f[0] = xflux(F, 0, 0);
-        f[(1 + d) * fs] = xflux(F, 1, 0);
-        f[(d == 2 ? 1 : 2 + d) * fs] = xflux(F, 2, 0);
-        f[(d == 0 ? 3 : d) * fs] = xflux(F, 3, 0);
-        f[4 * fs] = xflux(F, 4, 0);
+        const int to[5] = {f, f + (CURVI ? 1 : 1 + d) * fs, f + (CURVI ? 2 : (d == 2 ? 1 : 2 + d)) * fs,
+                           f + (CURVI ? 3 : (d == 0 ? 3 : d)) * fs, f + 4 * fs};
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          fm[to[q]] = F.m[q];
+          fe[to[q]] = (short)F.e[q];
+        }
       }
       __syncthreads();
       if (k < k0) continue;
-      const double* fzl = fz + ((k - 1) & 1) * (5 * TY * TX);
-#pragma unroll 1
-      for (int row = warp; row < TY; row += NW) {
-        const int ci = x0 + lane, cj = y0 + row;
-        if (ci >= g.nx || cj >= g.ny) continue;
+      const int row = warp, ci = x0 + lane, cj = y0 + row;  // warp `row` owns row `row` of the tile
+      if (row < TY && ci < g.nx && cj < g.ny) {
         const long long o = gidx(g, ci, cj, k);
         double dtc = dt;
         if constexpr (STAGE >= 1 && !VISC)  // local time steps: inviscid blocks only
@@ -365,13 +416,41 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
           if constexpr (STAGE >= 1) qs_[v] = __ldg(qs + v * g.field + o);
           if constexpr (STAGE >= 2) qn_[v] = __ldg(qn + v * g.field + o);
         }
+        const int mk = k & 1, mk1 = (k + 1) & 1;
+        constexpr int MSD = PL::MSLOT / sizeof(double);
+        const double* mc = mring + mk * MSD + (row + HALO) * BX + lane + HALO;  // the cell's metrics
+        XVal iv = {0, 0};
+        if constexpr (CURVI) iv = xrcp(xdec_pos<62>(mc[9 * MS]));
         double R[5], out[5];
+        // R = sum over directions of (upper - lower face flux) / h (CURVI: / V)
 #pragma unroll
-        for (int m = 0; m < 5; ++m) {
-          const double ddx = fx[(m * TY + row) * (TX + 1) + lane + 1] - fx[(m * TY + row) * (TX + 1) + lane];
-          const double ddy = fy[(m * (TY + 1) + row + 1) * TX + lane] - fy[(m * (TY + 1) + row) * TX + lane];
-          const double ddz = fzk[(m * TY + row) * TX + lane] - fzl[(m * TY + row) * TX + lane];
-          R[m] = (ddx * hx2 + ddy * hy2) + ddz * hz2;  // doubled fluxes
+        for (int q = 0; q < 5; ++q) {
+          const int x = q * TY * (TX + 1) + row * (TX + 1) + lane, y = PL::NFX + q * (TY + 1) * TX + row * TX + lane,
+                    z = PL::NFX + PL::NFY + q * TY * TX + row * TX + lane;
+          const int up[3] = {x + 1, y + TX, z + (k & 1) * PL::NFZ}, lo[3] = {x, y, z + ((k - 1) & 1) * PL::NFZ};
+          long long d[3];
+          int ed[3];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const int e1 = fe[up[a]], e0 = fe[lo[a]];
+            ed[a] = xmax(e1, e0) + 1;
+            d[a] = xshr(fm[up[a]], ed[a] - e1) - xshr(fm[lo[a]], ed[a] - e0);  // [62]
+            if constexpr (!CURVI) {
+              // normalised first: the product's truncation is then relative to the difference (left to
+              // the flux's own scale it doubled the 32^3 pulse's error against 64-bit references)
+              const XVal f = xquick(d[a], ed[a]);
+              d[a] = xmul(f.m, xb->h2[a].m);  // [60]
+              ed[a] = f.e + xb->h2[a].e + 3;
+            }
+          }
+          const int E = xmax(ed[0], xmax(ed[1], ed[2])) + (CURVI ? 2 : 0);
+          const long long t = xshr(d[0], E - ed[0]) + xshr(d[1], E - ed[1]) + xshr(d[2], E - ed[2]);
+          if constexpr (CURVI) {
+            const XVal r = xquick(t, E);
+            R[q] = xenc(xmul(r.m, iv.m), r.e + iv.e + 3);
+          } else {
+            R[q] = xenc(t, E);
+          }
         }
         if constexpr (STAGE == 0) {
           const long long oc = ((long long)k * g.ny + cj) * g.nx + ci;
@@ -383,7 +462,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
           for (int m = 0; m < 5; ++m) {
             const double adv = qs_[m] - dtc * R[m];
             if constexpr (STAGE == 1) out[m] = adv;
-            else if constexpr (STAGE == 2) out[m] = 0.75 * qn_[m] + 0.25 * adv;
+            else if constexpr (STAGE == 2) out[m] = fma(0.75, qn_[m], 0.25 * adv);
             else out[m] = fma(2.0 / 3.0, adv, (1.0 / 3.0) * qn_[m]);  // an FP64 division costs ~7 FMAs here
             qout[m * g.field + o] = out[m];
           }
@@ -395,15 +474,71 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
             for (int m = 0; m < 5; ++m) nacc[m] = fma(R[m], R[m], nacc[m]);
           }
           if constexpr (STAGE == 3) {
-            const double ir = Fm::rcp(out[0]);
-            const double uu = out[1] * ir, vv = out[2] * ir, ww = out[3] * ir;
-            const double pp = gm1 * (out[4] - 0.5 * out[0] * (uu * uu + vv * vv + ww * ww));
-            if (!(out[0] > 0.0 && pp > 0.0)) bad = true;
-            const RateK<double> RK = {P.pk.d.gam, P.pk.d.vf};
-            const double rate = cell_rate<double>(out[0], uu, vv, ww, pp, RK, ph.viscous, hx, hy, hz, hs2);
-            rate_max = fmax(rate_max, rate);
+            XPrim W;
+            if (!xprim(out, XK, W)) bad = true;
+            const XVal c = xsound(W, XK.gam);
+            XVal rate;
+            if constexpr (!CURVI) {
+              // (|u| + c) / hx + (|v| + c) / hy + (|w| + c) / hz, h2 = 1 / (2 h); viscous: + vs / rho
+              long long t[5];
+              int e[5];
+#pragma unroll
+              for (int a = 0; a < 3; ++a) {
+                t[a] = xmul(xabs(W.u[a].m), xb->h2[a].m);  // [60]
+                e[a] = W.u[a].e + xb->h2[a].e + 4;
+              }
+              t[3] = xmul(c.m, xb->hsum.m);
+              e[3] = c.e + xb->hsum.e + 3;
+              t[4] = VISC ? xmul(W.ir.m, xb->vs.m) : 0;
+              e[4] = VISC ? W.ir.e + xb->vs.e + 3 : e[3];
+              const int E = xmax(xmax(xmax(e[0], e[1]), xmax(e[2], e[3])), e[4]) + 1;
+              rate = xnormed(xshr(t[0], E - e[0]) + xshr(t[1], E - e[1]) + xshr(t[2], E - e[2]) + xshr(t[3], E - e[3]) +
+                                 xshr(t[4], E - e[4]), E);
+            } else {
+              // sum over directions of |u . S| + c |S| over V, S the mean of the cell's two faces
+              const double* mu[3] = {mc + 1, mc + BX, mring + mk1 * MSD + (row + HALO) * BX + lane + HALO};
+              long long t[3];
+              int e[3];
+#pragma unroll
+              for (int a = 0; a < 3; ++a) {
+                long long sm[3];
+                int es[3];
+#pragma unroll
+                for (int x = 0; x < 3; ++x) {
+                  const XPair f = xpair(mc[(3 * a + x) * MS], mu[a][(3 * a + x) * MS]);
+                  sm[x] = (f.l >> 1) + (f.r >> 1);  // [62], the mean in the class itself
+                  es[x] = f.e;
+                }
+                const int E = xmax(es[0], xmax(es[1], es[2]));
+                long long dot[3], s2 = 0;
+                int ec[3];
+#pragma unroll
+                for (int x = 0; x < 3; ++x) {
+                  sm[x] = xshr(sm[x], E - es[x]);
+                  s2 += xsq(sm[x]);  // [60] each, class 2 E + 3
+                  dot[x] = xmul(sm[x], W.u[x].m);
+                  ec[x] = E + W.u[x].e + 3;
+                }
+                const XVal n2 = xnormed(s2, 2 * E + 3);
+                const XVal in = xrsqrt(n2);
+                const long long cs = xmul(xmul(n2.m, in.m) << 2, c.m);  // c |S| [60]
+                const int ecs = n2.e + in.e + 1 + c.e + 3;
+                e[a] = xmax(xmax(xmax(ec[0], ec[1]), ec[2]), ecs) + 2;
+                t[a] = xabs(xshr(dot[0], e[a] - ec[0]) + xshr(dot[1], e[a] - ec[1]) + xshr(dot[2], e[a] - ec[2])) +
+                       xshr(cs, e[a] - ecs);  // [60]
+              }
+              const int E = xmax(e[0], xmax(e[1], e[2]));
+              const XVal v = xnormed(xshr(t[0], E - e[0]) + xshr(t[1], E - e[1]) + xshr(t[2], E - e[2]), E);
+              rate = xnormed(xmul(v.m, iv.m), v.e + iv.e + 3);
+            }
+            // the largest rate, as the bits of a non-negative double
+            const long long rb = __double_as_longlong(xenc(rate.m, rate.e));
+            if (rb > __double_as_longlong(rate_max)) rate_max = __longlong_as_double(rb);
             if constexpr (!VISC)
-              if (ph.local_dt) static_cast<double*>(D->dtl)[o] = ph.cfl * Fm::rcp(rate);
+              if (ph.local_dt) {
+                const XVal ir = xrcp(rate);
+                static_cast<double*>(D->dtl)[o] = ph.cfl * xenc(ir.m, ir.e);
+              }
           }
         }
       }
@@ -414,8 +549,10 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
   // abort path: drain copies still in flight (bounded), flag the timeout
   if (*sabort) {
     if (tid == 0) {
-      for (int s = 0; s < NSTAGE; ++s)
+      for (int s = 0; s < NST; ++s)
         if (pending & (1u << s)) mbar_wait_bounded(&bar[s], (phase_bits >> s) & 1u);
+      for (int s = 0; s < NMS; ++s)
+        if (mpending & (1u << s)) mbar_wait_bounded(&bar[NST + s], (mphase >> s) & 1u);
       atomicOr(&D->ctrl->flag, FLAG_TIMEOUT);
     }
   }
@@ -426,9 +563,9 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
 
 // ---- launch helpers --------------------------------------------------------------------------
 // warps per tile height: 3 TY + 2 items a plane
-constexpr int xwarps(int ty) { return ty == 8 ? 13 : 12; }
+constexpr int xwarps(int) { return 16; }
 
-template <bool VISC, int STAGE, int TYV, bool PUSH = false>
+template <bool VISC, int STAGE, bool CURVI, int TYV, bool PUSH = false>
 cudaError_t xstage_attr() {
   constexpr int NW = xwarps(TYV);
   static std::atomic<unsigned long long> done{0};
@@ -436,49 +573,49 @@ cudaError_t xstage_attr() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 64 && ((done.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
-  e = cudaFuncSetAttribute(xstage_kernel<VISC, STAGE, TYV, NW, PUSH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)XPlan<VISC, TYV, NW>::bytes);
+  e = cudaFuncSetAttribute(xstage_kernel<VISC, STAGE, CURVI, TYV, NW, PUSH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)XPlan<VISC, CURVI, TYV, NW>::bytes);
   if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_acq_rel);
   return e;
 }
-template <bool VISC, int STAGE, int TYV, bool PUSH = false>
+template <bool VISC, int STAGE, bool CURVI, int TYV, bool PUSH = false>
 cudaError_t xstage_go(const GroupParams& P, int grid, cudaStream_t s) {
   constexpr int NW = xwarps(TYV);
-  cudaError_t e = xstage_attr<VISC, STAGE, TYV, PUSH>();
+  cudaError_t e = xstage_attr<VISC, STAGE, CURVI, TYV, PUSH>();
   if (e != cudaSuccess) return e;
-  xstage_kernel<VISC, STAGE, TYV, NW, PUSH><<<grid, 32 * NW, XPlan<VISC, TYV, NW>::bytes, s>>>(P);
+  xstage_kernel<VISC, STAGE, CURVI, TYV, NW, PUSH><<<grid, 32 * NW, XPlan<VISC, CURVI, TYV, NW>::bytes, s>>>(P);
   return cudaGetLastError();
 }
-template <bool VISC, int TYV>
+template <bool VISC, bool CURVI, int TYV>
 cudaError_t xstage_prepare() {
-  cudaError_t e = xstage_attr<VISC, 0, TYV>();
-  if (e == cudaSuccess) e = xstage_attr<VISC, 1, TYV>();
-  if (e == cudaSuccess) e = xstage_attr<VISC, 2, TYV>();
-  if (e == cudaSuccess) e = xstage_attr<VISC, 3, TYV>();
+  cudaError_t e = xstage_attr<VISC, 0, CURVI, TYV>();
+  if (e == cudaSuccess) e = xstage_attr<VISC, 1, CURVI, TYV>();
+  if (e == cudaSuccess) e = xstage_attr<VISC, 2, CURVI, TYV>();
+  if (e == cudaSuccess) e = xstage_attr<VISC, 3, CURVI, TYV>();
   return e;
 }
-template <bool VISC, int TYV>
+template <bool VISC, bool CURVI, int TYV>
 cudaError_t xstage_dispatch(int stage, const GroupParams& P, int grid, cudaStream_t s) {
   switch (stage) {
-    case 0: return xstage_go<VISC, 0, TYV>(P, grid, s);
-    case 1: return xstage_go<VISC, 1, TYV>(P, grid, s);
-    case 2: return xstage_go<VISC, 2, TYV>(P, grid, s);
-    case 3: return xstage_go<VISC, 3, TYV>(P, grid, s);
+    case 0: return xstage_go<VISC, 0, CURVI, TYV>(P, grid, s);
+    case 1: return xstage_go<VISC, 1, CURVI, TYV>(P, grid, s);
+    case 2: return xstage_go<VISC, 2, CURVI, TYV>(P, grid, s);
+    case 3: return xstage_go<VISC, 3, CURVI, TYV>(P, grid, s);
   }
   return cudaErrorInvalidValue;
 }
 template <int TYV>
 cudaError_t xstage_dispatch_push(int stage, const GroupParams& P, int grid, cudaStream_t s) {
   switch (stage) {
-    case 1: return xstage_go<false, 1, TYV, true>(P, grid, s);
-    case 2: return xstage_go<false, 2, TYV, true>(P, grid, s);
+    case 1: return xstage_go<false, 1, false, TYV, true>(P, grid, s);
+    case 2: return xstage_go<false, 2, false, TYV, true>(P, grid, s);
   }
   return cudaErrorInvalidValue;
 }
 template <int TYV>
 cudaError_t xstage_prepare_push() {
-  cudaError_t e = xstage_attr<false, 1, TYV, true>();
-  if (e == cudaSuccess) e = xstage_attr<false, 2, TYV, true>();
+  cudaError_t e = xstage_attr<false, 1, false, TYV, true>();
+  if (e == cudaSuccess) e = xstage_attr<false, 2, false, TYV, true>();
   return e;
 }
 

@@ -81,6 +81,7 @@ struct Coef {
   T mu, kappa;               // viscosity, heat conductivity mu gamma / ((gamma - 1) Pr)
   T ih[3], ih12[3], ihs;     // inverse cell sizes, the same / 12, sum of their squares
   Consts<T> K;               // the Roe / viscous flux constants
+  XConsts x;                 // FP64 path: the Roe flux's constants as 64-bit block-floating values
 };
 
 struct Args {
@@ -735,7 +736,10 @@ __global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a
           Rq[q] = __shfl_down_sync(0xffffffffu, um, 1);
         }
       }
-      if (lane < FCH && f < nfc) roe_frame<T>(Lq, Rq, K, F[it]);
+      if (lane < FCH && f < nfc) {
+        if constexpr (sizeof(T) == 8) xroe<false>(Lq, Rq, coef<T>(a).x, F[it]);  // on the integer pipes (xfix.cuh)
+        else roe_frame<T>(Lq, Rq, K, F[it]);
+      }
     }
     __syncthreads();  // every lane is done reading the primitives
 #pragma unroll
@@ -1016,7 +1020,7 @@ void fill_coef(const Args& a, Coef<T>& c) {
   c.K.mu = T(a.mu);
   c.K.kappa = T(kappa);
   c.K.lim = 0;
-  if constexpr (sizeof(T) == 8) static_cast<XConsts&>(c.K.x) = xconsts(a.gamma, a.eps);
+  c.x = xconsts(a.gamma, a.eps);
 }
 
 Args make_args(gbcfd_wcns w) {

@@ -4,19 +4,18 @@
 // Why.  This part issues one FP64 operation per 64 FP32 or integer ones: a warp's DADD or DMUL
 // holds its sub-partition's FP64 lanes for 76 cycles, a DFMA for 64, while the integer pipes
 // idle.  A 64-bit integer add takes 2 issue slots there, an arithmetic 64-bit shift 4, and the
-// upper part of a 64 x 64 product about 15 (three 32 x 32 + 64 multiply-adds).  So the face flux of
-// the FP64 path is evaluated on 62-bit signed mantissas with an integer exponent each, in which
-// every rounding is at 2^-57 or finer of its class's largest value (FP64: 2^-53), and the result
-// is rounded once to a double.
+// upper part of a 64 x 64 product about 12 (three 32 x 32 multiply-adds).  So the FP64 path's
+// primitives, face fluxes and residuals are evaluated on 62-bit signed mantissas with an integer
+// exponent each, in which a rounding is about 2^-57 of its class's largest value (FP64: 2^-53),
+// and a result is rounded once to a double.
 //
 // A value is m 2^(E - 61), m a signed 64-bit integer, E an int.  Values that are added share E:
 // before a sum the terms are shifted right to the sum's class, a bound on every |m| being known
 // from the class (written beside each line as the number of bits), so nothing overflows for any
-// finite input.  Sums then cost one 64-bit add, and no result is normalised but where its
-// reciprocal root is taken.  Truncation is towards minus infinity.
+// finite input.  Sums then cost one 64-bit add.  Truncation is towards minus infinity.
 //
 // Measured on random states against quadruple precision (tests/test_xfix.py holds a bound): the
-// flux's root mean square error is 4-6e-17 of its size where the FP64 form's is 7-14e-17.
+// flux's root mean square error is 4-7e-17 of its size where the FP64 form's is 7-17e-17.
 //
 // The scheme is plain fixed-point arithmetic with scaling by exponents ("block floating point",
 // J. H. Wilkinson, Rounding Errors in Algebraic Processes, 1963, ch. 1).
@@ -29,25 +28,31 @@ struct XVal {
   int e;
 };
 
-// (a b) >> (64 - K): the product of two 64-bit values, |a b| < 2^(126 - K).  Each operand is split as
-// h 2^32 + l with both halves signed (l the low word read as signed, its sign carried into h), so
-// the three products kept are signed 32 x 32 -> 64; l_a l_b (less than 2^30 units of the middle
-// sum) is left out: the error is below 2^(K - 2) + 1 units of the result.
-template <int K>
-__host__ __device__ __forceinline__ long long xmul(long long a, long long b) {
-  const int al = (int)a, bl = (int)b;
-  const int ah = (int)(a >> 32) + (int)((unsigned)al >> 31), bh = (int)(b >> 32) + (int)((unsigned)bl >> 31);
-  const long long t = (long long)ah * bl + (long long)al * bh;
-  const long long r = (long long)ah * bh + (t >> 32);
-  return (long long)(((unsigned long long)r << K) | ((unsigned)t >> (32 - K)));
+// (a b) >> 64, |a|, |b| < 2^63 - 2^31.  Each operand is split as h 2^32 + l with both halves signed (l
+// the low word read as signed, its sign carried into h); of the four signed 32 x 32 products the
+// upper one is kept whole, the middle ones by their upper words, l_a l_b not at all: the error is
+// at most 2.25 units, and a zero factor gives zero (a velocity that is zero stays exactly zero).  So written it is three
+// multiply-adds and a sign extension; the form that keeps the middle sum's 64 bits is 17
+// instructions (opcode counts) for two more bits.
+__host__ __device__ __forceinline__ int xmulhi(int a, int b) {
+#ifdef __CUDA_ARCH__
+  return __mulhi(a, b);
+#else
+  return (int)(((long long)a * b) >> 32);
+#endif
 }
-template <int K>
+__host__ __device__ __forceinline__ int xhi(long long a) {
+  return (int)(a >> 32) + (int)((unsigned)(int)a >> 31);
+}
+__host__ __device__ __forceinline__ long long xmul(long long a, long long b) {
+  const int al = (int)a, bl = (int)b, ah = xhi(a), bh = xhi(b);
+  const int s = xmulhi(ah, bl) + xmulhi(al, bh);
+  return (long long)ah * bh + s;
+}
 __host__ __device__ __forceinline__ long long xsq(long long a) {
-  const int al = (int)a;
-  const int ah = (int)(a >> 32) + (int)((unsigned)al >> 31);
-  const long long t = (long long)ah * al;  // half the middle sum
-  const long long r = (long long)ah * ah + (t >> 31);
-  return (long long)(((unsigned long long)r << K) | (((unsigned)t << 1) >> (32 - K)));
+  const int al = (int)a, ah = xhi(a);
+  const int s = xmulhi(ah, al);
+  return (long long)ah * ah + 2 * s;
 }
 // arithmetic shift right by s >= 0, any size (a shift of 64 or more leaves the sign)
 __host__ __device__ __forceinline__ long long xshr(long long a, int s) {
@@ -106,34 +111,64 @@ __host__ __device__ __forceinline__ XVal xdec_pos(double a) {  // a > 0
   const unsigned long long mag = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b;
   return {(long long)(mag << (B - 53)), (int)((hi >> 20) & 0x7ffu) - 1023 + (62 - B)};
 }
-// the double nearest to m 2^(e - 61), |m| < 2^63; below the normal range 0, above it infinity
-__host__ __device__ __forceinline__ double xenc(long long m, int e) {
+// the double nearest to m 2^(e - 61), |m| < 2^63; below the normal range 0, above it infinity, and
+// NaN for the exponents from XBAD up (a flux that has no value)
+constexpr int XBAD = 8192;
+__host__ __device__ __forceinline__ int xclz32(int a) {
+#ifdef __CUDA_ARCH__
+  return __clz(a);
+#else
+  return a ? __builtin_clz((unsigned)a) : 32;
+#endif
+}
+__host__ __device__ inline double xenc_rare(long long m, int e) {
   const long long s = m >> 63;
   unsigned long long a = (unsigned long long)((m ^ s) - s);
   const int n = xclz(a);
   a <<= (n & 63);
   const int f = e + 2 - n + 1022;  // biased exponent - 1
-  const unsigned long long mant = (a >> 11) + ((a >> 10) & 1ull);
-  unsigned long long b = ((unsigned long long)(unsigned)f << 52) + mant;
+  unsigned long long b = ((unsigned long long)(unsigned)f << 52) + (a >> 11) + ((a >> 10) & 1ull);
   if ((unsigned)f >= 2046u) b = f < 0 ? 0ull : 0x7ff0000000000000ull;
   if (a == 0ull) b = 0ull;
+  if (e >= XBAD) b = 0x7ff8000000000000ull;
+  return xdouble(b | ((unsigned long long)s & 0x8000000000000000ull));
+}
+__host__ __device__ __forceinline__ double xenc(long long m, int e) {
+  const long long s = m >> 63;
+  unsigned long long a = (unsigned long long)((m ^ s) - s);
+  const int hi = (int)(a >> 32), n = xclz32(hi);
+  const int f = e + 1024 - n;
+  if (hi == 0 || (unsigned)f >= 2046u) return xenc_rare(m, e);  // small against its class, or out of range
+  a <<= n;
+  const unsigned long long b = ((unsigned long long)(unsigned)f << 52) + (a >> 11) + ((a >> 10) & 1ull);
   return xdouble(b | ((unsigned long long)s & 0x8000000000000000ull));
 }
 
 // the constants of the Roe flux as values (formed on the host)
 struct XConsts {
-  XVal ggm1, gm1, eps;  // 62 bits
+  XVal ggm1, gm1, eps, gam;  // 62 bits
 };
 inline XConsts xconsts(double gamma, double eps) {
-  return {xdec_pos<62>(gamma / (gamma - 1.0)), xdec_pos<62>(gamma - 1.0), xdec_pos<62>(eps)};
+  return {xdec_pos<62>(gamma / (gamma - 1.0)), xdec_pos<62>(gamma - 1.0), xdec_pos<62>(eps), xdec_pos<62>(gamma)};
 }
 
-// shift m left until 2^61 <= |m| < 2^62 (m < 2^62), lowering its exponent; 0 stays 0 with a far
-// smaller exponent
+// shift m left until 2^61 <= |m| < 2^62, lowering its exponent; |m| < 2^62; 0 stays 0
 __host__ __device__ __forceinline__ void xnorm(long long& m, int& e) {
   const int n = (xclz((unsigned long long)(m ^ (m >> 63))) - 2) & 63;
   m = (long long)((unsigned long long)m << n);
   e -= n;
+}
+__host__ __device__ __forceinline__ XVal xnormed(long long m, int e) {
+  xnorm(m, e);
+  return {m, e};
+}
+// the same from the upper word alone: at most 30 places, |m| < 2^63 in, [62] out.  For values whose
+// later roundings should be relative to them (a value 2^30 times smaller than its class is left
+// with 31 leading zeros, its roundings then at 2^-31 of it or 2^-61 of the class)
+__host__ __device__ __forceinline__ XVal xquick(long long m, int e) {
+  const int hi = (int)(m >> 32);
+  const int n = xclz32(hi ^ (hi >> 31)) - 1;  // 0 .. 31
+  return {(long long)((unsigned long long)m << n) >> 1, e + 1 - n};
 }
 
 // float seeds of the reciprocal (root) of x, 1 <= x < 4
@@ -166,9 +201,10 @@ __host__ __device__ __forceinline__ XVal xrsqrt(XVal v) {
   const long long M = v.m >> (1 - odd);  // f = M 2^-60 in [1, 4), v = f 2^(e - odd)
   const float x = (float)(int)(M >> 32) * (1.0f / 268435456.0f);
   const int Y = (int)(xseed_rsqrt(x) * 1073741824.0f);
-  const long long e = (1ll << 60) - xmul<4>(M, (long long)Y * Y);
-  const int es = (int)(e >> 18);
-  return {xcorrect(Y, (e >> 1) + ((3 * ((long long)es * es)) >> 27)), -((v.e - odd) >> 1) - 1};
+  // f y^2 = M Y^2 2^-120: in units of 2^-58
+  const long long e = (1ll << 58) - xmul(M, ((long long)Y * Y) << 2);
+  const int es = (int)(e >> 16);  // units of 2^-42
+  return {xcorrect(Y, 2 * e + ((3 * ((long long)es * es)) >> 27)), -((v.e - odd) >> 1) - 1};
 }
 // 1 / v, v > 0 normalised to [62]: the estimate and y (1 + e + e^2), e = 1 - v y
 __host__ __device__ __forceinline__ XVal xrcp(XVal v) {
@@ -180,54 +216,53 @@ __host__ __device__ __forceinline__ XVal xrcp(XVal v) {
   const int es = (int)(e >> 18);
   return {xcorrect(Y, e + (((long long)es * es) >> 24)), -v.e - 1};
 }
-__host__ __device__ __forceinline__ XVal xnormed(long long m, int e) {
-  xnorm(m, e);
-  return {m, e};
-}
 
 // (x^2 + d^2) / (2 d) in the class of x and d, 0 <= x < d < 2^62: Harten's fix of |x| < d.  n =
-// leading zeros that bring d to 62 bits, h 2^(e - 61) = 1 / (d 2^n 2^-61)
+// leading zeros that bring d to 62 bits, h 2^-62 = 1 / (d 2^n 2^-61)
 struct XHid {
   long long h;
-  int e, n;
+  int n;
 };
 __host__ __device__ __forceinline__ XHid xhid(long long d) {
   XHid r;
   r.n = (xclz((unsigned long long)d) - 2) & 63;  // d > 0 where it is used
-  const XVal v = xrcp({d << r.n, 0});
-  r.h = v.m;
-  r.e = v.e;
+  r.h = xrcp({d << r.n, 0}).m;
   return r;
 }
 __host__ __device__ __forceinline__ long long xharten(long long x, long long d, const XHid& r) {
   if (x >= d) return x;
-  // squares of 62-bit numbers, class 1; halved so that their sum keeps 62 bits: class 2; the
-  // product with 1 / (2 d) has class 2 + (e - 1) + 1 = 1 for e = -1: one bit up, then back by n
-  const long long q = (xsq<2>(x << r.n) >> 1) + (xsq<2>(d << r.n) >> 1);
-  return xshr(xmul<2>(q, r.h) << 1, r.n);
+  // squares of [62] are [60], class 3; their sum [61] times 1 / (2 d) (e = -1) is [59], class 4; up
+  // to class 0, then back by n
+  const long long q = xsq(x << r.n) + xsq(d << r.n);
+  return xshr(xmul(q, r.h) << 4, r.n);
 }
 
-// the two sides of a face: one variable's left and right value in a common class, |m| < 2^61
+// the two sides of a face: one variable's left and right value in a common class, [62]
 struct XPair {
   long long l, r;
   int e;
 };
-// twice a face flux, each component in its own class, |m| < 2^63; bad: a density or c^2 that is
-// not positive (NaN fluxes)
+// twice a face flux, each component in its own class, [62]; where a density or c^2 is not
+// positive the exponents are XBAD or more (NaN)
 struct XFlux {
   long long m[5];
   int e[5];
-  bool bad;
 };
 
 // Twice the Roe flux with Harten's fix in the face frame, as roe_frame (physics.cuh), from the
-// sides' (rho, u_n, u_t1, u_t2, p).  [n] after a line: |m| < 2^n.  Classes: Er, Eu, Ev, Ew, Ep of
-// the five variables, EH of the enthalpies and q^2/2, El of the wave speeds, EA of the wave
-// strengths, EM of the mass fluxes.  Where a value may be much smaller than its class (jumps,
-// products of several factors) it is normalised, so that later roundings are relative to it.
+// sides' (rho, u_n, u_t1, u_t2, p).  [n] after a line: |m| < 2^n.  A product of [a] and [b] is
+// [a + b - 64] with exponent e_a + e_b + 3; << 2 then brings [60] back to [62].  Classes: Eu, Ev, Ew of
+// the velocities, EH of the enthalpies and q^2/2, El of the wave speeds, EM of the mass fluxes.
+// Where a value may be much smaller than its class (jumps, products of several factors) it is
+// normalised, so that later roundings are relative to it.
+// CURVI: (u, v, w) are the x, y, z velocities, un the velocity along the face normal n (class 0,
+// [61]); the shear jumps are du - dun n, so the momentum flux is a x, y, z vector and needs no
+// tangents.
+template <bool CURVI>
 __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, const XPair& v, const XPair& w,
-                                              const XPair& p, const XConsts& K, XFlux& F) {
-  const int Eu = u.e, Ev = v.e, Ew = w.e, Ep = p.e;
+                                              const XPair& p, const XConsts& K, XFlux& F, const XPair& un,
+                                              const long long* n) {
+  const int Eu = u.e, Ev = v.e, Ew = w.e, Ep = p.e, En = CURVI ? un.e : Eu;
   const long long ul = u.l, ur = u.r, vl = v.l, vr = v.r, wl = w.l, wr = w.r;
   // densities and pressures by themselves; reciprocal roots; the Roe weights a_l = isr iw,
   // a_r = isl iw with iw = 1 / (isl + isr), class -1 (below 1, so [62])
@@ -235,46 +270,46 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const XVal isl = xrsqrt(rl), isr = xrsqrt(rr);
   const int Ei = xmax(isl.e, isr.e) + 1;
   const XVal iw = xrcp(xnormed(xshr(isl.m, Ei - isl.e) + xshr(isr.m, Ei - isr.e), Ei));
-  const long long al = xshr(xmul<3>(isr.m, iw.m), -1 - (isr.e + iw.e));
-  const long long ar = xshr(xmul<3>(isl.m, iw.m), -1 - (isl.e + iw.e));
+  const long long al = xshr(xmul(isr.m, iw.m) << 3, -1 - (isr.e + iw.e));
+  const long long ar = xshr(xmul(isl.m, iw.m) << 3, -1 - (isl.e + iw.e));
   // sqrt(rho_l rho_r)
-  const XVal rt = xnormed(xmul<2>(xmul<2>(rl.m, isl.m), xmul<2>(rr.m, isr.m)), rl.e + isl.e + rr.e + isr.e + 3);  // [62]
+  const XVal rt = xquick(xmul(xmul(rl.m, isl.m) << 2, xmul(rr.m, isr.m) << 2), rl.e + isl.e + rr.e + isr.e + 5);  // [62]
   // mass fluxes
-  const long long ml = xmul<3>(rl.m, ul), mr = xmul<3>(rr.m, ur);  // [62]
-  const int Eml = rl.e + Eu, Emr = rr.e + Eu;
+  const long long nl = CURVI ? un.l : ul, nr = CURVI ? un.r : ur;
+  const long long ml = xmul(rl.m, nl), mr = xmul(rr.m, nr);  // [60]
+  const int Eml = rl.e + En + 3, Emr = rr.e + En + 3;
   // enthalpies gamma/(gamma-1) p / rho + |u|^2 / 2, each side in its own class
-  const XVal gl = xnormed(xmul<2>(K.ggm1.m, xmul<2>(pl.m, xsq<2>(isl.m))), K.ggm1.e + pl.e + 2 * isl.e + 3);
-  const XVal gr = xnormed(xmul<2>(K.ggm1.m, xmul<2>(pr.m, xsq<2>(isr.m))), K.ggm1.e + pr.e + 2 * isr.e + 3);
-  const int Ek = 2 * xmax(xmax(Eu, Ev), Ew) - 2;
-  const int EHl = xmax(gl.e, Ek) + 2, EHr = xmax(gr.e, Ek) + 2, EH = xmax(EHl, EHr);
-  const long long hl = xshr(gl.m, EHl - gl.e) + xshr(xsq<4>(ul), EHl + 2 - 2 * Eu) + xshr(xsq<4>(vl), EHl + 2 - 2 * Ev) +
-                       xshr(xsq<4>(wl), EHl + 2 - 2 * Ew);  // [62]
-  const long long hr = xshr(gr.m, EHr - gr.e) + xshr(xsq<4>(ur), EHr + 2 - 2 * Eu) + xshr(xsq<4>(vr), EHr + 2 - 2 * Ev) +
-                       xshr(xsq<4>(wr), EHr + 2 - 2 * Ew);
-  // Roe averages, in the classes of the sides
-  const long long ut = xmul<2>(al, ul) + xmul<2>(ar, ur);  // [61]
-  const long long vt = xmul<2>(al, vl) + xmul<2>(ar, vr);  // [61]
-  const long long wt = xmul<2>(al, wl) + xmul<2>(ar, wr);  // [61]
-  const long long ht = xshr(xmul<2>(al, hl), EH - EHl) + xshr(xmul<2>(ar, hr), EH - EHr);  // [62]
-  const long long q2 = xshr(xsq<4>(ut), EH + 2 - 2 * Eu) + xshr(xsq<4>(vt), EH + 2 - 2 * Ev) +
-                       xshr(xsq<4>(wt), EH + 2 - 2 * Ew);  // q^2 / 2
-  const long long c2m = xmul<2>(K.gm1.m, ht - q2);
-  F.bad = r.l <= 0 || r.r <= 0 || c2m <= 0;
+  const XVal gl = xquick(xmul(K.ggm1.m, xmul(pl.m, xsq(isl.m) << 2) << 2), K.ggm1.e + pl.e + 2 * isl.e + 5);  // [62]
+  const XVal gr = xquick(xmul(K.ggm1.m, xmul(pr.m, xsq(isr.m) << 2) << 2), K.ggm1.e + pr.e + 2 * isr.e + 5);
+  const int Ek = 2 * xmax(xmax(Eu, Ev), Ew) + 2;
+  const int EHl = xmax(gl.e, Ek) + 1, EHr = xmax(gr.e, Ek) + 1, EH = xmax(EHl, EHr) + 2;
+  const long long hl = xshr(gl.m, EHl - gl.e) + xshr(xsq(ul), EHl - 2 * Eu - 2) + xshr(xsq(vl), EHl - 2 * Ev - 2) +
+                       xshr(xsq(wl), EHl - 2 * Ew - 2);  // [62]
+  const long long hr = xshr(gr.m, EHr - gr.e) + xshr(xsq(ur), EHr - 2 * Eu - 2) + xshr(xsq(vr), EHr - 2 * Ev - 2) +
+                       xshr(xsq(wr), EHr - 2 * Ew - 2);
+  // Roe averages: velocities in the classes of the sides [62]; enthalpy and q^2 / 2 in class EH [60]
+  const long long ut = (xmul(al, ul) + xmul(ar, ur)) << 2;
+  const long long vt = (xmul(al, vl) + xmul(ar, vr)) << 2;
+  const long long wt = (xmul(al, wl) + xmul(ar, wr)) << 2;
+  const long long nt = CURVI ? (xmul(al, nl) + xmul(ar, nr)) << 2 : ut;
+  const long long ht = xshr(xmul(al, hl), EH - EHl - 2) + xshr(xmul(ar, hr), EH - EHr - 2);
+  const long long q2 = xshr(xsq(ut), EH - 2 * Eu - 2) + xshr(xsq(vt), EH - 2 * Ev - 2) + xshr(xsq(wt), EH - 2 * Ew - 2);
+  const long long c2m = xmul(K.gm1.m, ht - q2);
+  const bool bad = r.l <= 0 || r.r <= 0 || c2m <= 0;
   // c^2 normalised, its reciprocal root, c
-  const XVal c2 = xnormed(c2m, K.gm1.e + EH + 1);
+  const XVal c2 = xnormed(c2m, K.gm1.e + EH + 3);
   const XVal ic = xrsqrt(c2);
-  const long long ic2 = xsq<2>(ic.m);  // [62], class 2 ic.e + 1
-  const long long cc = xmul<2>(c2.m, ic.m);
+  const long long ic2 = xsq(ic.m) << 2;       // [62], class 2 ic.e + 1
+  const long long cc = xmul(c2.m, ic.m) << 2;  // [62]
   const int Ec = c2.e + ic.e + 1;
   // wave speeds; room for delta = eps (|u| + c) where eps >= 1
   const int hx = K.eps.e >= 0 ? K.eps.e + 1 : 0;
-  const int El = xmax(Eu - 1, Ec) + 1 + hx;
-  const long long ue = xshr(ut, El - Eu), ce = xshr(cc, El - Ec);  // [61]
-  const long long au = xabs(ue);
-  long long l1 = xabs(ue - ce), l5 = xabs(ue + ce), l2 = au;       // [62]
+  const int El = xmax(En, Ec) + 1 + hx;
+  const long long ue = xshr(nt, El - En), ce = xshr(cc, El - Ec);  // [61]
+  long long l1 = xabs(ue - ce), l5 = xabs(ue + ce), l2 = xabs(ue);  // [62]
   {
-    long long d = xmul<2>(K.eps.m, au + ce);
-    d = K.eps.e >= 0 ? d << hx : xshr(d, -1 - K.eps.e);            // [62]
+    long long d = xmul(K.eps.m, l2 + ce);  // class El + eps.e + 3
+    d = K.eps.e >= -3 ? d << (K.eps.e + 3) : xshr(d, -3 - K.eps.e);  // [62]
     if (l1 < d || l2 < d || l5 < d) {
       const XHid hid = xhid(d);
       l1 = xharten(l1, d, hid);
@@ -283,60 +318,130 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
     }
   }
   // jumps, normalised [62], and wave strengths: a1, a5 = (dp -+ rho c du) / (2 c^2), a2 = drho - dp / c^2
-  const XVal jr = xnormed(r.r - r.l, r.e), ju = xnormed(ur - ul, Eu), jv = xnormed(vr - vl, Ev), jw = xnormed(wr - wl, Ew),
-             jp = xnormed(p.r - p.l, Ep);
-  const long long rcd = xmul<2>(xmul<2>(rt.m, cc), ju.m);
-  const int Ercd = rt.e + Ec + 1 + ju.e + 1;
-  const int Eq = xmax(Ercd, jp.e) + 1;
-  const long long dp = xshr(jp.m, Eq - jp.e), rq = xshr(rcd, Eq - Ercd);  // [61]
-  const int Ea = Eq + 2 * ic.e + 1;                                       // of a1 and a5 (the half included)
-  const long long w1 = xmul<1>(l1, xmul<2>(dp - rq, ic2)), w5 = xmul<1>(l5, xmul<2>(dp + rq, ic2));  // [61]
-  const XVal s = xnormed(w1 + w5, El + Ea + 2), dw = xnormed(w5 - w1, El + Ea + 2);                  // [62]
-  const int EA = xmax(Ea + 1, jr.e) + 1;
-  const XVal w2 = xnormed(xmul<2>(l2, xshr(jr.m, EA - jr.e) - xshr(xmul<2>(dp, ic2), EA - Ea - 1)), El + EA + 1);
+  const XVal jr = xquick(r.r - r.l, r.e), ju = xquick(nr - nl, En), jv = xquick(vr - vl, Ev), jw = xquick(wr - wl, Ew),
+             jp = xquick(p.r - p.l, Ep);
+  const XVal rcd = xquick(xmul(xmul(rt.m, cc) << 2, ju.m), rt.e + Ec + ju.e + 4);
+  const int Eq = xmax(rcd.e, jp.e) + 1;
+  const long long dp = xshr(jp.m, Eq - jp.e), rq = xshr(rcd.m, Eq - rcd.e);               // [61]
+  const int Ea = Eq + 2 * ic.e + 3;                                                       // (the half included)
+  const XVal a1 = xquick(xmul(dp - rq, ic2), Ea), a5 = xquick(xmul(dp + rq, ic2), Ea);
+  const int Ew15 = El + 3 + xmax(a1.e, a5.e);
+  const long long w1 = xshr(xmul(l1, a1.m), Ew15 - El - 3 - a1.e), w5 = xshr(xmul(l5, a5.m), Ew15 - El - 3 - a5.e);  // [60]
+  const XVal s = xquick(w1 + w5, Ew15), dw = xquick(w5 - w1, Ew15);                       // [62]
+  const int Ed = jp.e + 2 * ic.e + 4, EA = xmax(Ed, jr.e + 2);
+  const XVal a2 = xquick(xshr(jr.m, EA - jr.e) - xshr(xmul(jp.m, ic2), EA - Ed), EA);
+  const XVal w2 = xquick(xmul(l2, a2.m), El + a2.e + 3);                                  // [62]
   // in the class of the mass fluxes [60]
-  const int EM = xmax(xmax(Eml, Emr), xmax(s.e, w2.e) + 1) + 2;
+  const int EM = xmax(xmax(Eml, Emr), xmax(s.e, w2.e) + 3);
   const long long fl = xshr(ml, EM - Eml), fr = xshr(mr, EM - Emr);
   const long long ws = xshr(s.m, EM - s.e) + xshr(w2.m, EM - w2.e);
-  const XVal dq = {xmul<2>(dw.m, cc), dw.e + Ec + 1};                  // [62]
-  const long long lrt = xmul<2>(l2, rt.m);                             // [62]
-  const XVal g1 = xnormed(xmul<2>(lrt, jv.m), El + rt.e + jv.e + 2), g2 = xnormed(xmul<2>(lrt, jw.m), El + rt.e + jw.e + 2);
+  const long long dq = xmul(dw.m, cc);                                  // [60]
+  const XVal lrt = xquick(xmul(l2, rt.m), El + rt.e + 3);               // [62]
+  const long long g1 = xmul(lrt.m, jv.m), g2 = xmul(lrt.m, jw.m);       // [60]
+  const int Edq = dw.e + Ec + 3, Eg1 = lrt.e + jv.e + 3, Eg2 = lrt.e + jw.e + 3;
+  const long long a1m = xmul(fl, ul) + xmul(fr, ur) - xmul(ws, ut);  // [60]
+  const long long a2m = xmul(fl, vl) + xmul(fr, vr) - xmul(ws, vt);
+  const long long a3m = xmul(fl, wl) + xmul(fr, wr) - xmul(ws, wt);
+  const int f1 = EM + Eu + 3, f2 = EM + Ev + 3, f3 = EM + Ew + 3;
+  const int el = Eml + EHl + 3, er = Emr + EHr + 3, e1 = s.e + EH + 3, e2 = Edq + En + 3, e3 = Eg1 + Ev + 3, e4 = Eg2 + Ew + 3,
+            e5 = w2.e + EH + 3;
+  const int E4 = xmax(xmax(xmax(el, er), xmax(e1, e2)), xmax(xmax(e3, e4), e5));
+  const long long a4 = xshr(xmul(ml, hl), E4 - el) + xshr(xmul(mr, hr), E4 - er);  // terms [58]
+  const long long b4 = xshr(xmul(s.m, ht), E4 - e1) + xshr(xmul(w2.m, q2), E4 - e5);
+  long long d4 = xshr(xmul(dq, nt), E4 - e2) + xshr(xmul(g1, vt), E4 - e3) + xshr(xmul(g2, wt), E4 - e4);
   F.m[0] = fl + fr - ws;
   F.e[0] = EM;
-  {
-    const int e2 = EM + Ev - 1, e3 = EM + Ew - 1;
-    const long long a = xmul<4>(fl, vl) + xmul<4>(fr, vr) - xmul<4>(ws, vt);  // < 3 2^61
-    const long long b = xmul<4>(fl, wl) + xmul<4>(fr, wr) - xmul<4>(ws, wt);
-    F.e[2] = xmax(e2, g1.e) + 1;
-    F.e[3] = xmax(e3, g2.e) + 1;
-    F.m[2] = xshr(a, F.e[2] - e2) - xshr(g1.m, F.e[2] - g1.e);
-    F.m[3] = xshr(b, F.e[3] - e3) - xshr(g2.m, F.e[3] - g2.e);
+  if constexpr (!CURVI) {
+    F.e[1] = xmax(xmax(f1, Edq), Ep + 2);
+    F.e[2] = xmax(f2, Eg1);
+    F.e[3] = xmax(f3, Eg2);
+    F.m[1] = xshr(a1m, F.e[1] - f1) + xshr(p.l + p.r, F.e[1] - Ep) - xshr(dq, F.e[1] - Edq);
+    F.m[2] = xshr(a2m, F.e[2] - f2) - xshr(g1, F.e[2] - Eg1);
+    F.m[3] = xshr(a3m, F.e[3] - f3) - xshr(g2, F.e[3] - Eg2);
+  } else {
+    const XVal jx = xquick(ur - ul, Eu);
+    const long long g0 = xmul(lrt.m, jx.m), gn = xmul(lrt.m, ju.m);  // [60]
+    const int Eg0 = lrt.e + jx.e + 3, Egn = lrt.e + ju.e + 3;
+    const int EP = xmax(xmax(Edq, Egn), Ep + 2);
+    const XVal P = xquick(xshr(p.l + p.r, EP - Ep) - xshr(dq, EP - Edq) + xshr(gn, EP - Egn), EP);  // along n, [62]
+    const int fp = P.e + 3;                                                                         // P n_x [59]
+    F.e[1] = xmax(xmax(f1, fp), Eg0);
+    F.e[2] = xmax(xmax(f2, fp), Eg1);
+    F.e[3] = xmax(xmax(f3, fp), Eg2);
+    F.m[1] = xshr(a1m, F.e[1] - f1) + xshr(xmul(P.m, n[0]), F.e[1] - fp) - xshr(g0, F.e[1] - Eg0);
+    F.m[2] = xshr(a2m, F.e[2] - f2) + xshr(xmul(P.m, n[1]), F.e[2] - fp) - xshr(g1, F.e[2] - Eg1);
+    F.m[3] = xshr(a3m, F.e[3] - f3) + xshr(xmul(P.m, n[2]), F.e[3] - fp) - xshr(g2, F.e[3] - Eg2);
+    // shear work ut . (du - dun n); class E4 may be below these terms' own: they are aligned both ways
+    const int e0 = Eg0 + Eu + 3, en = Egn + En + 3, E5 = xmax(E4, xmax(e0, en));
+    d4 = xshr(d4, E5 - E4) + xshr(xmul(g0, ut), E5 - e0) - xshr(xmul(gn, nt), E5 - en);
+    F.e[4] = E5;
+    F.m[4] = xshr(a4 - b4, E5 - E4) - d4;
   }
-  {
-    const int e1 = EM + Eu - 1, E1 = xmax(xmax(e1, dq.e), Ep) + 2;
-    const long long a = xmul<4>(fl, ul) + xmul<4>(fr, ur) - xmul<4>(ws, ut);
-    F.e[1] = E1;
-    F.m[1] = xshr(a, E1 - e1) + xshr(p.l + p.r, E1 - Ep) - xshr(dq.m, E1 - dq.e);
-  }
-  {
-    const int el = Eml + EHl + 2, er = Emr + EHr + 2, e1 = s.e + EH + 1, e2 = dq.e + Eu + 1, e3 = g1.e + Ev + 1,
-              e4 = g2.e + Ew + 1, e5 = w2.e + EH + 1;
-    const int E4 = xmax(xmax(xmax(el, er), xmax(e1, e2)), xmax(xmax(e3, e4), e5)) + 2;
-    const long long a = xshr(xmul<1>(ml, hl), E4 - el) + xshr(xmul<1>(mr, hr), E4 - er);
-    const long long b = xshr(xmul<2>(s.m, ht), E4 - e1) + xshr(xmul<2>(w2.m, q2), E4 - e5);
-    const long long d = xshr(xmul<2>(g1.m, vt), E4 - e3) + xshr(xmul<2>(g2.m, wt), E4 - e4);
+  if constexpr (!CURVI) {
     F.e[4] = E4;
-    F.m[4] = a - b - xshr(xmul<2>(dq.m, ut), E4 - e2) - d;
+    F.m[4] = a4 - b4 - d4;
+  }
+  if (bad) {
+    F.e[0] = F.e[1] = F.e[2] = F.e[3] = F.e[4] = 2 * XBAD;
+  }
+}
+__host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, const XPair& v, const XPair& w,
+                                              const XPair& p, const XConsts& K, XFlux& F) {
+  xroe<false>(r, u, v, w, p, K, F, u, nullptr);
+}
+
+// the unit normal (class 0, [61]) and half the length of a face's area vector
+struct XNormal {
+  long long n[3];
+  XVal half;
+};
+__host__ __device__ __forceinline__ XNormal xnormal(double sx, double sy, double sz) {
+  const XVal a = xdec<62>(sx), b = xdec<62>(sy), c = xdec<62>(sz);
+  const int E = xmax(a.e, xmax(b.e, c.e));
+  const XVal x = {xshr(a.m, E - a.e), E}, y = {xshr(b.m, E - b.e), E}, z = {xshr(c.m, E - c.e), E};
+  const XVal s2 = xnormed(xsq(x.m) + xsq(y.m) + xsq(z.m), 2 * E + 3);
+  const XVal ia = xrsqrt(s2);
+  XNormal N;
+  // S ia [60] << 2; |S| ia = 1 bounds the exponent: E + ia.e is 0 or -1 when the largest is near |S|
+  const int sh = -(E + ia.e);
+  N.n[0] = xshr(xmul(x.m, ia.m) << 3, sh);
+  N.n[1] = xshr(xmul(y.m, ia.m) << 3, sh);
+  N.n[2] = xshr(xmul(z.m, ia.m) << 3, sh);
+  N.half = {xmul(s2.m, ia.m) << 2, s2.e + ia.e};
+  return N;
+}
+// the velocity along n of one side, from (u, v, w) in their classes: class Emax + 1, [62]
+__host__ __device__ __forceinline__ long long xdot(const long long* n, long long u, int Eu, long long v, int Ev,
+                                                   long long w, int Ew, int E) {
+  return (xshr(xmul(u, n[0]), E - Eu) + xshr(xmul(v, n[1]), E - Ev) + xshr(xmul(w, n[2]), E - Ew)) << 2;
+}
+
+// twice the flux through a face of area vector (sx, sy, sz) from the sides' (rho, u, v, w, p), x, y, z
+// momentum, times half the area: the face flux itself
+__host__ __device__ __forceinline__ void xroe_area(const XPair& r, const XPair& u, const XPair& v, const XPair& w,
+                                                   const XPair& p, double sx, double sy, double sz, const XConsts& K,
+                                                   XFlux& F) {
+  const XNormal N = xnormal(sx, sy, sz);
+  const int E = xmax(xmax(u.e, v.e), w.e);
+  const XPair un = {xdot(N.n, u.l, u.e, v.l, v.e, w.l, w.e, E), xdot(N.n, u.r, u.e, v.r, v.e, w.r, w.e, E), E + 1};
+  xroe<true>(r, u, v, w, p, K, F, un, N.n);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int q = 0; q < 5; ++q) {
+    const XVal f = xquick(F.m[q], F.e[q]);
+    F.m[q] = xmul(f.m, N.half.m);
+    F.e[q] = f.e + N.half.e + 3;
   }
 }
 
 // a flux component as a double, times 2^-h
 __host__ __device__ __forceinline__ double xflux(const XFlux& F, int q, int h) {
-  return F.bad ? xdouble(0x7ff8000000000000ull) : xenc(F.m[q], F.e[q] - h);
+  return xenc(F.m[q], F.e[q] - h);
 }
 // both sides of one variable from doubles
 __host__ __device__ __forceinline__ XPair xpair(double l, double r) {
-  const XVal a = xdec<61>(l), b = xdec<61>(r);
+  const XVal a = xdec<62>(l), b = xdec<62>(r);
   const int e = xmax(a.e, b.e);
   return {xshr(a.m, e - a.e), xshr(b.m, e - b.e), e};
 }
@@ -346,6 +451,48 @@ __host__ __device__ __forceinline__ void xroe(const double* L, const double* R, 
   XFlux f;
   xroe(xpair(L[0], R[0]), xpair(L[1], R[1]), xpair(L[2], R[2]), xpair(L[3], R[3]), xpair(L[4], R[4]), K, f);
   for (int q = 0; q < 5; ++q) F[q] = xflux(f, q, TWICE ? 0 : 1);
+}
+
+// the primitives of a conserved state (rho, rho u, rho v, rho w, rho E): velocities [62] and pressure
+// [62] each in its own class, 1 / rho; false where the density or the pressure is not positive or
+// not finite
+struct XPrim {
+  XVal r, ir, u[3], p;
+};
+__host__ __device__ __forceinline__ XVal xdec_zero(double a) {  // zero and subnormals as zero
+  XVal v = xdec<62>(a);
+  if (v.e == -1023) v.m = 0;
+  return v;
+}
+__host__ __device__ __forceinline__ bool xprim(const double* q, const XConsts& K, XPrim& W) {
+  W.r = xdec_pos<62>(q[0]);
+  W.ir = xrcp(W.r);
+  const XVal E = xdec_zero(q[4]);
+  long long k[3];
+  int ek[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int x = 0; x < 3; ++x) {
+    const XVal m = xdec_zero(q[1 + x]);
+    W.u[x].m = xmul(m.m, W.ir.m) << 2;
+    W.u[x].e = m.e + W.ir.e + 1;
+    k[x] = xmul(m.m, W.u[x].m);  // [60]; rho u^2 / 2 with the exponent lowered by 1
+    ek[x] = m.e + W.u[x].e + 2;
+  }
+  const int Ek = xmax(xmax(ek[0], ek[1]), xmax(ek[2], E.e + 2));
+  const long long d = xshr(E.m, Ek - E.e) - xshr(k[0], Ek - ek[0]) - xshr(k[1], Ek - ek[1]) - xshr(k[2], Ek - ek[2]);
+  W.p = xquick(xmul(K.gm1.m, d), K.gm1.e + Ek + 3);
+  const long long br = (long long)xbits(q[0]);
+  // a non-finite momentum or energy has the exponent 1024
+  return br > 0 && br < 0x7ff0000000000000ll && W.p.m > 0 && E.e < 1024 && W.u[0].e - W.ir.e < 1025 &&
+         W.u[1].e - W.ir.e < 1025 && W.u[2].e - W.ir.e < 1025;
+}
+// c = sqrt(gamma p / rho), [62]
+__host__ __device__ __forceinline__ XVal xsound(const XPrim& W, const XVal& gam) {
+  const XVal c2 = xnormed(xmul(gam.m, xmul(W.p.m, W.ir.m) << 2), gam.e + W.p.e + W.ir.e + 4);
+  const XVal ic = xrsqrt(c2);
+  return {xmul(c2.m, ic.m) << 2, c2.e + ic.e + 1};
 }
 
 }  // namespace gbcfd

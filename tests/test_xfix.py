@@ -24,6 +24,25 @@ extern "C" void roe(int n, const double* L, const double* R, double gamma, doubl
     if (half) gbcfd::xroe<false>(L + 5 * i, R + 5 * i, K, F + 5 * i);
     else gbcfd::xroe<true>(L + 5 * i, R + 5 * i, K, F + 5 * i);
 }
+extern "C" void roe_area(int n, const double* L, const double* R, const double* S, double gamma, double eps, double* F) {
+  const gbcfd::XConsts K = gbcfd::xconsts(gamma, eps);
+  for (int i = 0; i < n; ++i) {
+    const double *l = L + 5 * i, *r = R + 5 * i, *s = S + 3 * i;
+    gbcfd::XFlux f;
+    gbcfd::xroe_area(gbcfd::xpair(l[0], r[0]), gbcfd::xpair(l[1], r[1]), gbcfd::xpair(l[2], r[2]), gbcfd::xpair(l[3], r[3]),
+                     gbcfd::xpair(l[4], r[4]), s[0], s[1], s[2], K, f);
+    for (int q = 0; q < 5; ++q) F[5 * i + q] = gbcfd::xflux(f, q, 0);
+  }
+}
+extern "C" void prims(int n, const double* q, double gamma, double* W, int* ok) {
+  const gbcfd::XConsts K = gbcfd::xconsts(gamma, 0.1);
+  for (int i = 0; i < n; ++i) {
+    gbcfd::XPrim w;
+    ok[i] = gbcfd::xprim(q + 5 * i, K, w);
+    const gbcfd::XVal c = gbcfd::xsound(w, K.gam), v[6] = {w.r, w.u[0], w.u[1], w.u[2], w.p, c};
+    for (int k = 0; k < 6; ++k) W[6 * i + k] = gbcfd::xenc(v[k].m, v[k].e);
+  }
+}
 extern "C" void roots(int n, const double* v, double* s, double* r) {
   for (int i = 0; i < n; ++i) {
     const gbcfd::XVal a = gbcfd::xrsqrt(gbcfd::xdec_pos<62>(v[i])), b = gbcfd::xrcp(gbcfd::xdec_pos<62>(v[i]));
@@ -33,6 +52,7 @@ extern "C" void roots(int n, const double* v, double* s, double* r) {
 }
 """
 _D = ctypes.POINTER(ctypes.c_double)
+ULP = 2.0 ** -53
 
 
 def _p(a):
@@ -161,3 +181,68 @@ def test_reciprocal_roots(lib):
     # one rounding to double and the iteration's 2^-57
     assert np.all(np.abs(s * np.sqrt(x) - 1) <= 2.0 ** -53 + 2.0 ** -57 + 2.0 ** -62)
     assert np.all(np.abs(r * x - 1) <= 2.0 ** -53 + 2.0 ** -57 + 2.0 ** -62)
+
+
+@pytest.mark.parametrize("kind", ["smooth", "uniform", "jumps", "aligned"])
+def test_roe_flux_through_an_area_vector(lib, kind):
+    """the curvilinear form, x, y, z momentum, against the frame form in long double"""
+    n, rng = 8000, np.random.Generator(np.random.PCG64(9))
+    L, R = states("smooth" if kind == "aligned" else kind, n, rng)
+    S = rng.uniform(-1, 1, (n, 3)) * 10.0 ** rng.uniform(-6, 0, (n, 1))
+    if kind == "aligned":  # axis-aligned and nearly aligned faces
+        S = np.eye(3)[rng.integers(0, 3, n)] * 1e-3 + rng.choice([0.0, 1e-9, 1e-20], (n, 3))
+    S = np.ascontiguousarray(S)
+    ld = np.longdouble
+    s = S.astype(ld)
+    area = np.sqrt((s * s).sum(1))
+    nrm = s / area[:, None]
+    a = np.abs(S).argmin(1)
+    e = np.eye(3)[a].astype(ld)
+    t1 = e - (nrm * e).sum(1)[:, None] * nrm
+    t1 /= np.sqrt((t1 * t1).sum(1))[:, None]
+    t2 = np.cross(nrm, t1)
+    frame = lambda w: np.concatenate([w[:, :1].astype(ld)] + [(w[:, 1:4].astype(ld) * v).sum(1)[:, None] for v in (nrm, t1, t2)]
+                                     + [w[:, 4:].astype(ld)], 1)
+    f, sc = reference(frame(L), frame(R), 1.4, 0.1)
+    want = np.concatenate([f[:, :1], f[:, 1:2] * nrm + f[:, 2:3] * t1 + f[:, 3:4] * t2, f[:, 4:]], 1) * (area / 2)[:, None]
+    # the normal velocity is a sum of products of the size of |u|: what the flux carries of it is
+    # rounded relative to |u|, however small u . n is (rho, rho |u| + rho c, rho H per unit of it)
+    speed = np.maximum(np.abs(L[:, 1:4]).sum(1), np.abs(R[:, 1:4]).sum(1))
+    rho, p = np.maximum(L[:, 0], R[:, 0]), np.maximum(L[:, 4], R[:, 4])
+    h = np.maximum(3.5 * L[:, 4] / L[:, 0], 3.5 * R[:, 4] / R[:, 0]) + 0.5 * speed ** 2
+    mom = (sc[:, 1:4].sum(1) + rho * speed * (speed + np.sqrt(h)))[:, None]
+    scale = np.concatenate([sc[:, :1] + (rho * speed)[:, None], mom, mom, mom, sc[:, 4:] + (rho * h * speed)[:, None]],
+                           1) * (area / 2)[:, None]
+    F = np.empty((n, 5))
+    lib.roe_area(n, _p(L), _p(R), _p(S), ctypes.c_double(1.4), ctypes.c_double(0.1), _p(F))
+    # the FP64 form's bound, with the rotations' roundings (about 20 more)
+    assert np.all(np.abs(F - want) <= 80 * ULP * scale)
+
+
+def test_primitives(lib):
+    n, rng = 50000, np.random.Generator(np.random.PCG64(11))
+    r, p = 10.0 ** rng.uniform(-2, 2, n), 10.0 ** rng.uniform(-2, 2, n)
+    v = rng.uniform(-2, 2, (3, n)) * 10.0 ** rng.uniform(-9, 0, (3, n))
+    v[2, ::3] = 0.0
+    q = np.ascontiguousarray(np.stack([r, r * v[0], r * v[1], r * v[2], p / 0.4 + 0.5 * r * (v * v).sum(0)], 1))
+    W, ok = np.empty((n, 6)), np.zeros(n, dtype=np.int32)
+    lib.prims(n, _p(q), ctypes.c_double(1.4), _p(W), ok.ctypes.data_as(ctypes.c_void_p))
+    assert ok.all()
+    Q = q.astype(np.longdouble)
+    u = Q[:, 1:4] / Q[:, :1]
+    P = np.longdouble(1.4 - 1.0) * (Q[:, 4] - 0.5 * (Q[:, 1:4] * u).sum(1))
+    assert np.array_equal(W[:, 0], q[:, 0])
+    assert np.all(np.abs(W[:, 1:4] - u) <= (ULP + 2.0 ** -56) * np.abs(u))  # zero stays zero
+    # the kinetic part's products and the difference: 2^-57 of the energy each, then one rounding
+    assert np.all(np.abs(W[:, 4] - P) <= ULP * np.abs(P) + 8 * 2.0 ** -57 * Q[:, 4])
+    c = np.sqrt(np.longdouble(1.4) * W[:, 4].astype(np.longdouble) / Q[:, 0])
+    assert np.all(np.abs(W[:, 5] - c) <= 3 * ULP * c)
+
+
+@pytest.mark.parametrize("q", [(-1, 0, 0, 0, 1), (0, 0, 0, 0, 1), (1, 0, 0, 0, -1), (1, 10, 0, 0, 1), (np.nan, 0, 0, 0, 1),
+                               (np.inf, 0, 0, 0, 1), (1, np.inf, 0, 0, 1), (1, 0, np.nan, 0, 1), (1, 0, 0, -np.inf, 1),
+                               (1, 0, 0, 0, np.inf), (1, 0, 0, 0, np.nan)])
+def test_non_physical_primitives_are_refused(lib, q):
+    a, W, ok = np.array(q, dtype=np.float64), np.empty(6), np.ones(1, dtype=np.int32)
+    lib.prims(1, _p(a), ctypes.c_double(1.4), _p(W), ok.ctypes.data_as(ctypes.c_void_p))
+    assert not ok[0]
