@@ -292,3 +292,25 @@ def test_try_smooth_keeps_or_restores(gb, precision, nsteps):
     assert kept == (r1 < r0)
     gb.step([blk], 2)
     assert np.all(np.isfinite(blk.residual_norm()))
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (1, 1, 3, 31), (1, 2, 4, 32), (2, 1, 5, 33), (3, 2, 9, 65)])
+@pytest.mark.parametrize("zper", [True, False])
+def test_train_gradient_at_the_edges_of_the_32_by_4_tiles(gb, shape, zper):
+    """one tile, less than one, and one cell more in x and y, several batches (some CTAs without a
+    tile): every tensor's gradient against the oracle's, relative L2 <= 1e-2 (the bound of the other
+    gradient tests: the bf16 roundings of the activations' gradients)"""
+    B, Z, Y, X = shape
+    p, x, t = random_params(31), rng(32).standard_normal((B, 10, Z, Y, X)), rng(33).standard_normal((B, 5, Z, Y, X))
+    xg = to_gpu_features(x)
+    th = np.zeros((B, Z, Y, X, 8), dtype=np.float32)
+    th[..., :5] = np.transpose(t, (0, 2, 3, 4, 1))
+    tg = torch.from_numpy(th.reshape(-1, 8)).cuda()
+    a = gb.Accel(X, Y, Z, B, zperiodic=zper)
+    a.set_params(p)
+    loss = a.train_step(xg, tg, 1e-3)
+    grad = a.train_state()[0].astype(np.float64)
+    want_loss, want = batch_loss_and_grad(p, from_gpu(xg, B, Z, Y, X, C=10), t, zper)
+    assert abs(loss - want_loss) <= 1e-3 * want_loss
+    for name, sl in tensor_slices():
+        assert np.linalg.norm(grad[sl] - want[sl]) <= 1e-2 * np.linalg.norm(want[sl]), name
