@@ -5,17 +5,24 @@
 //
 // A tile is 128 consecutive cells along x (one y, z, batch); GEMM view M = 128 cells,
 // N = output channels (16 or 32), K = 27 taps x CIP input channels, issued as 27 x CIP/16 MMAs
-// of K = 16.  Persistent CTAs of 128 threads; shared memory holds all weights and two input
-// boxes of 3 x 3 rows of 130 cells (rows padded to 136), as 8 x 16-byte core matrices:
-//   box    element (row r, cell c, channel k) at ((k / 8) NBOX + 136 r + c) 8 + k % 8
+// of K = 16.  A CTA takes a contiguous range of tiles with y fastest, so that consecutive tiles
+// share six of their nine input rows: shared memory holds the weights and a ring of five y-rows
+// (of the three z-planes each) of 130 cells, as 8 x 16-byte core matrices:
+//   row    element (slot s, plane z, cell c, channel k) at (((3 s + z) CIP/8 + k / 8) RP + c) 8 + k % 8
 //   weight element (tap t, out o, in k) at ((t CIP/8 + k / 8) N + o) 8 + k % 8
-// so for tap t the A matrix of the tile starts at box cell (dz 3 + dy) 136 + dx (rows = cells,
-// 8 consecutive rows one 128-byte core matrix, SBO 128 B, LBO = NBOX x 16 B along K) and the B
-// matrix at weight group t CIP/8 (SBO 128 B, LBO = N x 16 B).  The boxes are filled by TMA.
+// so for tap t the A matrix of the tile starts at cell dx of plane dz of the slot of row y + dy - 1
+// (rows = cells, 8 consecutive rows one 128-byte core matrix, SBO 128 B, LBO = RP x 16 B along K)
+// and the B matrix at weight group t CIP/8 (SBO 128 B, LBO = N x 16 B).
+//
+// Warps: four per 16 output channels read the accumulators back (thread = TMEM lane = cell) and
+// apply the epilogue, four load rows by cp.async (two groups of two warps, alternate rows), one
+// thread of the last issues the MMAs, its descriptors a constant away from the three rows'
+// (unrolled: formed per tap they were 1100 instructions of a single thread a tile).  They meet only at mbarriers: a row landed, a tile's MMAs done (tcgen05.commit), an
+// accumulator read back.  The first version copied a tile's nine rows anew by TMA, with the
+// channel groups as 16-byte inner boxes: 36 copies of 130 such pieces a tile held it at 12 us
+// (every unit below 30% busy); now a tile loads three rows, in pieces the threads copy whole cells
+// at a time.  192 x 96 x 64 cells, three layers: 1.86 -> 0.53 ms.
 #include <atomic>
-
-#include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include "internal.cuh"
 #include "learn.cuh"
@@ -25,9 +32,9 @@ namespace learn {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int TC_M = 128, TC_BX = TC_M + 2, TC_RP = 136, TC_NBOX = TC_RP * 3 * 3, TC_THREADS = 128;
-// a box row (130 cells) is padded to TC_RP = 136 cells so that every row of every channel group
-// starts on a 128-byte boundary (the TMA destination alignment)
+constexpr int TC_M = 128, TC_BX = TC_M + 2, TC_NR = 5, TC_LOADERS = 64;
+// cells a channel group's row is padded to: the four (two) groups of a cell fall into different banks
+template <int CIP> struct TcPitch { static constexpr int value = CIP == 32 ? 138 : 140; };
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return static_cast<unsigned>(__cvta_generic_to_shared(p));
@@ -70,253 +77,231 @@ __device__ __forceinline__ bool mbar_wait_limited(unsigned bar, unsigned parity)
   }
 }
 
-// tile -> (x0, y, z, b)
-__device__ __forceinline__ void tc_tile(long long tile, const ConvArgs& A, int& x0, int& y, int& z, int& b) {
-  const int tx = (A.X + TC_M - 1) / TC_M;
-  x0 = (int)(tile % tx) * TC_M;
-  tile /= tx;
-  y = (int)(tile % A.Y);
-  tile /= A.Y;
-  z = (int)(tile % A.Z);
-  b = (int)(tile / A.Z);
+__device__ __forceinline__ void mbar_arrive1(unsigned bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 
-// the input box of a tile by TMA: for each of the 3 x 3 (y, z) rows and each 8-channel group one
-// 130 x 16-byte copy of the activation tensor viewed as [Z B][Y][X][CIP/8][8], box (8, 1, 130,
-// 1, 1) at x0 - 1; the copy unit fills x and y outside the volume with zeros.  Rows outside the
-// volume in a non-periodic z are zeroed by the threads (a z - 1 row would otherwise belong to
-// the previous batch).  Thread 0 issues the copies; returns the bytes the barrier expects.
-template <int CIP>
-__device__ __forceinline__ void tc_load_box(const ConvArgs& A, const CUtensorMap* map, long long tile, unsigned box,
-                                            unsigned bar, int tid) {
-  int x0, y, z, b;
-  tc_tile(tile, A, x0, y, z, b);
-  if (tid == 0) {
-    unsigned bytes = 0;
-    for (int r = 0; r < 9; ++r) {
-      int zz = z + r / 3 - 1;
-      if (A.zper) zz = (zz + A.Z) % A.Z;
-      if (zz >= 0 && zz < A.Z) bytes += (CIP / 8) * TC_BX * 16u;
-    }
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-    for (int r = 0; r < 9; ++r) {
-      const int by = r % 3, bz = r / 3;
-      int zz = z + bz - 1;
-      if (A.zper) zz = (zz + A.Z) % A.Z;
-      if (zz < 0 || zz >= A.Z) continue;
-      for (int kg = 0; kg < CIP / 8; ++kg) {
-        const unsigned dst = box + (unsigned)((kg * TC_NBOX + r * TC_RP) * 16);
-        asm volatile(
-            "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, "
-            "%6}], [%7];\n" ::"r"(dst),
-            "l"(reinterpret_cast<unsigned long long>(map)), "r"(0), "r"(kg), "r"(x0 - 1), "r"(y + by - 1),
-            "r"(b * A.Z + zz), "r"(bar)
-            : "memory");
-      }
-    }
+// a CTA's range of tiles, walked in columns (x tile, z, b) of consecutive y
+struct TcWalk {
+  long long t, end;   // next tile, end of the range
+  int x0, z, b, ya, n;  // the current column piece: rows ya .. ya + n - 1
+  __device__ __forceinline__ bool next(const ConvArgs& A) {
+    if (t >= end) return false;
+    const int tx = (A.X + TC_M - 1) / TC_M;
+    const long long col = t / A.Y;
+    ya = (int)(t - col * A.Y);
+    n = (int)min((long long)(A.Y - ya), end - t);
+    x0 = (int)(col % tx) * TC_M;
+    z = (int)((col / tx) % A.Z);
+    b = (int)(col / tx / A.Z);
+    t += n;
+    return true;
   }
-  if (!A.zper) {  // zero rows outside the volume in z
-    for (int r = 0; r < 9; r += 3) {
-      const int zz = z + r / 3 - 1;
-      if (zz >= 0 && zz < A.Z) continue;
-      for (int i = tid; i < 3 * (CIP / 8) * TC_RP; i += TC_THREADS) {
-        const int kg = i / (3 * TC_RP), rest = i % (3 * TC_RP);
-        bf16* p = reinterpret_cast<bf16*>(__cvta_shared_to_generic(box)) + ((size_t)kg * TC_NBOX + r * TC_RP + rest) * 8;
-        *reinterpret_cast<uint4*>(p) = make_uint4(0u, 0u, 0u, 0u);
-      }
-    }
-  }
-}
+};
 
-// the 27 x CIP/16 MMAs of one tile into the accumulator at tmem (one thread), then a commit
+// the 27 x CIP/16 MMAs of one tile into the accumulator at tmem (one thread), then a commit;
+// row[dy] = the descriptor of cell 0, plane 0 of the slot of row y + dy - 1, wdesc the weights'
 template <int CIP, int N>
-__device__ __forceinline__ void tc_issue(unsigned box0, unsigned w0, unsigned tmem, unsigned bar) {
-  constexpr unsigned idesc = instr_desc(N);
+__device__ __forceinline__ void tc_issue(const unsigned long long (&row)[3], unsigned long long wdesc, unsigned tmem,
+                                         unsigned bar) {
+  constexpr unsigned idesc = instr_desc(N), RP = TcPitch<CIP>::value;
+#pragma unroll
   for (int t = 0; t < NTAP; ++t) {
     const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
-    const unsigned cell0 = (unsigned)((dz * 3 + dy) * TC_RP + dx);
 #pragma unroll
-    for (int kk = 0; kk < CIP / 16; ++kk) {
-      const unsigned a = box0 + ((unsigned)(2 * kk) * TC_NBOX + cell0) * 16u;
-      const unsigned bw = w0 + ((unsigned)(t * (CIP / 8) + 2 * kk) * N) * 16u;
-      tc_mma(tmem, smem_desc(a, TC_NBOX * 16u, 128u), smem_desc(bw, N * 16u, 128u), idesc, (t | kk) != 0);
-    }
+    for (int kk = 0; kk < CIP / 16; ++kk)  // descriptor addresses count 16 bytes: one cell of a channel group
+      tc_mma(tmem, row[dy] + (unsigned)((dz * (CIP / 8) + 2 * kk) * RP + dx),
+             wdesc + (unsigned)((t * (CIP / 8) + 2 * kk) * N), idesc, (t | kk) != 0);
   }
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
 }
 
-// persistent: CTA c takes tiles c, c + G, c + 2G, ...; the weights are staged once; two input
-// boxes (loaded by TMA) and two tensor-memory accumulators let the copies of tile k+2 and the
-// MMAs of tile k+1 run during the epilogue of tile k
-template <int CIP, int N, int COP, int MODE>
-__global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const ConvArgs A, const __grid_constant__ CUtensorMap map,
-                                                             const bf16* __restrict__ wtc, int* __restrict__ flag,
-                                                             long long ntiles) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  bf16* boxes = reinterpret_cast<bf16*>(smem);                      // 2 x TC_NBOX x CIP (128-byte rows)
-  bf16* wsm = boxes + 2 * TC_NBOX * CIP;                            // 27 x CIP x N
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(wsm + NTAP * CIP * N);  // full[2], done[2]
-  unsigned* tslot = reinterpret_cast<unsigned*>(bar + 4);
-  int* sabort = reinterpret_cast<int*>(tslot + 1);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  constexpr int COLS = 2 * (N < 32 ? 32 : N);
-  constexpr unsigned BOXB = TC_NBOX * CIP * 2;
+// NC output channels c0 .. c0 + NC - 1 of one cell: bias, SiLU (and the pre-activation kept for
+// training), the linear output, or the product with SiLU' of the saved pre-activation
+template <int COP, int NC, int MODE>
+__device__ __forceinline__ void tc_epilogue(const ConvArgs& A, const float* bias, const float (&acc)[16], long long cell,
+                                            int c0) {
+  const long long at = cell * COP + c0;
+  if constexpr (MODE == FWD_LINEAR) {
+    float* out = static_cast<float*>(A.out) + at;
+#pragma unroll
+    for (int c = 0; c < NC; c += 4)
+      *reinterpret_cast<float4*>(out + c) = make_float4(acc[c] + bias[c0 + c], acc[c + 1] + bias[c0 + c + 1],
+                                                        acc[c + 2] + bias[c0 + c + 2], acc[c + 3] + bias[c0 + c + 3]);
+  } else {
+    __align__(16) bf16 o[NC];
+#pragma unroll
+    for (int c = 0; c < NC; c += 4) {
+      if constexpr (MODE == FWD_SILU) {
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          v[q] = acc[c + q] + bias[c0 + c + q];
+          o[c + q] = __float2bfloat16(v[q] / (1.0f + __expf(-v[q])));
+        }
+        if (A.zsave) *reinterpret_cast<float4*>(A.zsave + at + c) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+        const float4 z4 = *reinterpret_cast<const float4*>(A.zprev + at + c);
+        const float zp[4] = {z4.x, z4.y, z4.z, z4.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float sg = 1.0f / (1.0f + __expf(-zp[q]));
+          o[c + q] = __float2bfloat16(acc[c + q] * (sg * (1.0f + zp[q] * (1.0f - sg))));
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NC / 8; ++q)
+      reinterpret_cast<uint4*>(static_cast<bf16*>(A.out) + at)[q] = reinterpret_cast<const uint4*>(o)[q];
+  }
+}
 
-  if (warp == 0) {
+// Steps (tiles) s = 0, 1, ... and rows g = 0, 1, ... of a CTA are counted over its columns; a column
+// piece of n tiles has n + 2 rows, step i of it reads rows i, i + 1, i + 2.  Row g lives in slot g % 5
+// (full[g % 5], phase g / 5); step s's accumulator is s % 2, its completion done[s % 4], phase s / 4;
+// epi[s % 2] says the accumulator was read back.  A row may be loaded once the last step that read
+// the row five before it is done: within a piece that is step i - 5 (of row i), which trails the
+// steps that can have been issued by at most two, so four done barriers never wrap past a waiter.
+// Every wait is bounded (2 s); a role that gives up flags the timeout and leaves, the others follow.
+template <int N> struct TcWarps {  // epilogue warps, then four loaders, then the issuer
+  static constexpr int epi = 4 * (N / 16), threads = 32 * (epi + 5);
+};
+template <int CIP, int N, int COP, int MODE>
+__global__ void __launch_bounds__(TcWarps<N>::threads, CIP == 16 ? 2 : 1) conv_tc_kernel(const ConvArgs A, const bf16* __restrict__ wtc,
+                                                             int* __restrict__ flag, long long ntiles) {
+  constexpr int CG = CIP / 8, RP = TcPitch<CIP>::value, EPI = TcWarps<N>::epi, TC_THREADS = TcWarps<N>::threads;
+  constexpr unsigned SLOTB = 3u * CG * RP * 16u;
+  extern __shared__ __align__(128) unsigned char smem[];
+  bf16* wsm = reinterpret_cast<bf16*>(smem + TC_NR * SLOTB);         // 27 x CIP x N
+  float* bias = reinterpret_cast<float*>(wsm + NTAP * CIP * N);      // COP (FWD)
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(bias + 32);  // full[5], done[4], epi[2]
+  unsigned* tslot = reinterpret_cast<unsigned*>(bar + 11);
+  const int tid = threadIdx.x, warp = tid >> 5;
+  constexpr unsigned COLW = N < 32 ? 32 : N, COLS = 2 * COLW;
+
+  if (warp == EPI + 4) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)),
                  "r"(COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
+  const unsigned rows0 = smem_u32(smem), w0 = smem_u32(wsm), full0 = smem_u32(bar), done0 = full0 + 5 * 8, epi0 = done0 + 4 * 8;
   if (tid == 0) {
-    for (int j = 0; j < 4; ++j) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar + j)));
+    for (int j = 0; j < 11; ++j)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(full0 + 8u * j),
+                   "r"(j < 5 ? TC_LOADERS : (j < 9 ? 1 : EPI * 32)));
     asm volatile("fence.mbarrier_init.release.cluster;\n");
-    *sabort = 0;
   }
-  for (int i = tid; i < NTAP * N * (CIP / 8); i += TC_THREADS) {  // global [27][N][CIP] -> core matrices
-    const int t = i / (N * (CIP / 8)), r = i % (N * (CIP / 8)), o = r / (CIP / 8), kg = r % (CIP / 8);
+  for (int i = tid; i < NTAP * N * CG; i += TC_THREADS) {  // global [27][N][CIP] -> core matrices
+    const int t = i / (N * CG), r = i % (N * CG), o = r / CG, kg = r % CG;
     const uint4 v = *reinterpret_cast<const uint4*>(wtc + ((size_t)t * N + o) * CIP + kg * 8);
-    *reinterpret_cast<uint4*>(wsm + (((size_t)t * (CIP / 8) + kg) * N + o) * 8) = v;
+    *reinterpret_cast<uint4*>(wsm + (((size_t)t * CG + kg) * N + o) * 8) = v;
   }
-  __syncthreads();  // barriers initialised
-  const unsigned boxa = smem_u32(boxes), w0 = smem_u32(wsm), full0 = smem_u32(bar), done0 = smem_u32(bar + 2);
-  const long long first = blockIdx.x, stride = gridDim.x;
-  tc_load_box<CIP>(A, &map, first, boxa, full0, tid);
-  if (first + stride < ntiles) tc_load_box<CIP>(A, &map, first + stride, boxa + BOXB, full0 + 8u, tid);
+  if (MODE != BWD_DSILU && tid < COP) bias[tid] = A.bias[tid];
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const unsigned tmem0 = *tslot, colw = (unsigned)(N < 32 ? 32 : N);
-  unsigned fphase = 0, dphase = 0;  // parities of the next completion of full[j] / done[j]
-  unsigned inflight = 0;            // thread 0: copy groups (bits 0-1) and MMA groups (bits 2-3) not yet waited for
-  if (tid == 0) {
-    inflight = (first + stride < ntiles) ? 3u : 1u;
-    const bool ok = mbar_wait_limited(full0, 0u);
-    fphase ^= 1u;
-    inflight &= ~1u;
-    if (ok) {
-      tc_issue<CIP, N>(boxa, w0, tmem0, done0);
-      inflight |= 4u;
-    } else {
-      atomicOr(flag, FLAG_TIMEOUT);
-      *sabort = 1;
+  const unsigned tmem0 = *tslot;
+  TcWalk walk;
+  walk.t = (long long)blockIdx.x * ntiles / gridDim.x;
+  walk.end = (long long)(blockIdx.x + 1) * ntiles / gridDim.x;
+  bool ok = true;
+
+  if (warp >= EPI && warp < EPI + 4) {
+    // ---- loaders: group 0 the even rows, group 1 the odd ones ----
+    const int group = (warp - EPI) >> 1, lt = tid - 32 * EPI - group * TC_LOADERS;
+    const int kg = lt % CG, c0 = lt / CG;  // a thread's channel group and first cell; then every TC_LOADERS / CG cells
+    int g0 = 0, s0 = 0;
+    while (ok && walk.next(A)) {
+      const int cells = min(TC_BX, A.X - walk.x0 + 2);  // from x0 - 1 to the tile's or the volume's edge + 1
+      for (int r = 0; r < walk.n + 2; ++r) {
+        const int g = g0 + r;
+        if ((g & 1) != group) continue;
+        const int need = r >= TC_NR ? s0 + r - TC_NR : s0 - 1;  // the last step that read this slot
+        if (need >= 0 && !(ok = mbar_wait_limited(done0 + 8u * (need & 3), (need >> 2) & 1))) break;
+        const int y = walk.ya - 1 + r;
+        const unsigned dst0 = rows0 + (unsigned)(g % TC_NR) * SLOTB;
+        const bool iny = y >= 0 && y < A.Y;
+#pragma unroll
+        for (int pz = 0; pz < 3; ++pz) {
+          int zz = walk.z + pz - 1;
+          if (A.zper) zz = zz < 0 ? zz + A.Z : (zz >= A.Z ? zz - A.Z : zz);
+          const bool inp = iny && zz >= 0 && zz < A.Z;
+          const bf16* src = A.in + (inp ? ((((long long)walk.b * A.Z + zz) * A.Y + y) * A.X + walk.x0 - 1) * CIP + kg * 8 : 0);
+          const unsigned dst = dst0 + (unsigned)((pz * CG + kg) * RP) * 16u;
+#pragma unroll 3
+          for (int c = c0; c < cells; c += TC_LOADERS / CG) {
+            const int x = walk.x0 - 1 + c;
+            const bool in = inp && x >= 0 && x < A.X;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst + c * 16u),
+                         "l"(in ? src + (long long)c * CIP : A.in), "r"(in ? 16 : 0)
+                         : "memory");
+          }
+        }
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the tensor cores read it next
+        mbar_arrive1(full0 + 8u * (g % TC_NR));
+      }
+      g0 += walk.n + 2;
+      s0 += walk.n;
     }
-  }
-  __syncthreads();
-  int k = 0;
-  for (long long tile = first; tile < ntiles && !*sabort; tile += stride, ++k) {
-    const int cur = k & 1, nxt = cur ^ 1;
-    // MMA(k) done: box[cur] and tensor memory [cur] hold tile k's results
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_limited(done0 + 8u * cur, (dphase >> cur) & 1u));
-    if (!ok) {
-      if (tid == 0) atomicOr(flag, FLAG_TIMEOUT);
-      atomicOr(sabort, 1);
-      __syncthreads();
-      break;
+  } else if (tid == 32 * (EPI + 4)) {
+    // ---- MMA issue ----
+    const unsigned long long rdesc = smem_desc(rows0, RP * 16u, 128u), wdesc = smem_desc(w0, N * 16u, 128u);
+    int g0 = 0, s = 0;
+    while (ok && walk.next(A)) {
+      for (int r = 0; r < walk.n + 2 && ok; ++r) {
+        const int g = g0 + r;
+        ok = mbar_wait_limited(full0 + 8u * (g % TC_NR), (g / TC_NR) & 1);
+        if (!ok || r < 2) continue;
+        if (s >= 2 && !(ok = mbar_wait_limited(epi0 + 8u * (s & 1), ((s >> 1) - 1) & 1))) break;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        const unsigned long long row[3] = {rdesc + (unsigned)((g - 2) % TC_NR) * (SLOTB / 16u),
+                                           rdesc + (unsigned)((g - 1) % TC_NR) * (SLOTB / 16u),
+                                           rdesc + (unsigned)(g % TC_NR) * (SLOTB / 16u)};
+        tc_issue<CIP, N>(row, wdesc, tmem0 + (s & 1) * COLW, done0 + 8u * (s & 3));
+        ++s;
+      }
+      g0 += walk.n + 2;
     }
-    dphase ^= 1u << cur;
-    if (tid == 0) inflight &= ~(4u << cur);
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (tile + 2 * stride < ntiles) {  // copies of tile k+2 into the box tile k used
-      tc_load_box<CIP>(A, &map, tile + 2 * stride, boxa + cur * BOXB, full0 + 8u * cur, tid);
-      if (tid == 0) inflight |= 1u << cur;
-    }
-    if (tid == 0 && tile + stride < ntiles) {  // MMA(k+1) once its box has landed
-      const bool okf = mbar_wait_limited(full0 + 8u * nxt, (fphase >> nxt) & 1u);
-      fphase ^= 1u << nxt;
-      inflight &= ~(1u << nxt);
-      if (okf) {
-        tc_issue<CIP, N>(boxa + nxt * BOXB, w0, tmem0 + nxt * colw, done0 + 8u * nxt);
-        inflight |= 4u << nxt;
-      } else {
-        atomicOr(flag, FLAG_TIMEOUT);
-        *sabort = 1;
+    if (s > 0) mbar_wait_limited(done0 + 8u * ((s - 1) & 3), ((s - 1) >> 2) & 1);  // nothing in flight when it leaves
+  } else if (warp < EPI) {
+    // ---- epilogue: warps w and w + 4 the lanes of quarter w, 16 columns each ----
+    const int lane_cell = tid & 127, c0 = (warp >> 2) * 16;
+    int s = 0;
+    while (ok && walk.next(A)) {
+      for (int i = 0; i < walk.n; ++i, ++s) {
+        ok = __all_sync(0xffffffffu, mbar_wait_limited(done0 + 8u * (s & 3), (s >> 2) & 1));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        float acc[16];
+        const unsigned taddr = tmem0 + (s & 1) * COLW + (unsigned)c0 + ((unsigned)((warp & 3) * 32) << 16);
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+            : "=f"(acc[0]), "=f"(acc[1]), "=f"(acc[2]), "=f"(acc[3]), "=f"(acc[4]), "=f"(acc[5]), "=f"(acc[6]),
+              "=f"(acc[7]), "=f"(acc[8]), "=f"(acc[9]), "=f"(acc[10]), "=f"(acc[11]), "=f"(acc[12]), "=f"(acc[13]),
+              "=f"(acc[14]), "=f"(acc[15])
+            : "r"(taddr));
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        mbar_arrive1(epi0 + 8u * (s & 1));  // in registers: the accumulator may be overwritten
+        const int gx = walk.x0 + lane_cell;
+        if (gx < A.X)
+          tc_epilogue<COP, (COP < 16 ? COP : 16), MODE>(
+              A, bias, acc, (((long long)walk.b * A.Z + walk.z) * A.Y + walk.ya + i) * A.X + gx, c0);
       }
     }
-    int x0, y, z, b;
-    tc_tile(tile, A, x0, y, z, b);
-    float acc[32];
-    const unsigned taddr = tmem0 + cur * colw + ((unsigned)(warp * 32) << 16);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-        : "=f"(acc[0]), "=f"(acc[1]), "=f"(acc[2]), "=f"(acc[3]), "=f"(acc[4]), "=f"(acc[5]), "=f"(acc[6]),
-          "=f"(acc[7]), "=f"(acc[8]), "=f"(acc[9]), "=f"(acc[10]), "=f"(acc[11]), "=f"(acc[12]), "=f"(acc[13]),
-          "=f"(acc[14]), "=f"(acc[15]), "=f"(acc[16]), "=f"(acc[17]), "=f"(acc[18]), "=f"(acc[19]),
-          "=f"(acc[20]), "=f"(acc[21]), "=f"(acc[22]), "=f"(acc[23]), "=f"(acc[24]), "=f"(acc[25]),
-          "=f"(acc[26]), "=f"(acc[27]), "=f"(acc[28]), "=f"(acc[29]), "=f"(acc[30]), "=f"(acc[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-    const int gx = x0 + tid;
-    if (gx < A.X) {
-      const long long cell = (((long long)b * A.Z + z) * A.Y + y) * A.X + gx;
-      if constexpr (MODE == FWD_SILU) {
-        __align__(16) bf16 o[COP];
-#pragma unroll
-        for (int c = 0; c < COP; ++c) {
-          const float v = acc[c] + A.bias[c];
-          if (A.zsave) A.zsave[cell * COP + c] = v;
-          o[c] = __float2bfloat16(v / (1.0f + __expf(-v)));
-        }
-#pragma unroll
-        for (int q = 0; q < COP / 8; ++q)
-          reinterpret_cast<uint4*>(static_cast<bf16*>(A.out) + cell * COP)[q] = reinterpret_cast<const uint4*>(o)[q];
-      } else if constexpr (MODE == FWD_LINEAR) {
-        float* out = static_cast<float*>(A.out) + cell * COP;
-#pragma unroll
-        for (int c = 0; c < COP; ++c) out[c] = acc[c] + A.bias[c];
-      } else {
-        __align__(16) bf16 o[COP];
-#pragma unroll
-        for (int c = 0; c < COP; ++c) {
-          const float zp = A.zprev[cell * COP + c];
-          const float sg = 1.0f / (1.0f + __expf(-zp));
-          o[c] = __float2bfloat16(acc[c] * (sg * (1.0f + zp * (1.0f - sg))));
-        }
-#pragma unroll
-        for (int q = 0; q < COP / 8; ++q)
-          reinterpret_cast<uint4*>(static_cast<bf16*>(A.out) + cell * COP)[q] = reinterpret_cast<const uint4*>(o)[q];
-      }
-    }
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // zeroed rows of box[cur]
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();  // tensor memory [cur] read by everyone; zero rows written
   }
-  // after an abort: give copies and MMAs still in flight a bounded wait before freeing anything
-  if (tid == 0)
-    for (int j = 0; j < 2; ++j) {
-      if (inflight & (1u << j)) mbar_wait_limited(full0 + 8u * j, (fphase >> j) & 1u);
-      if (inflight & (4u << j)) mbar_wait_limited(done0 + 8u * j, (dphase >> j) & 1u);
-    }
+  if (!ok) atomicOr(flag, FLAG_TIMEOUT);
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem0), "r"(COLS));
-}
-
-// the TMA map of an activation tensor [Z B][Y][X][CIP] as 5 dimensions (8, CIP/8, X, Y, Z B)
-static cudaError_t tc_map(CUtensorMap* m, const void* base, int CIP, const ConvArgs& a) {
-  static PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
-  if (!enc) {
-    cudaDriverEntryPointQueryResult q;
-    void* f = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      return cudaErrorNotSupported;
-    enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-  }
-  cuuint64_t dims[5] = {8, (cuuint64_t)(CIP / 8), (cuuint64_t)a.X, (cuuint64_t)a.Y, (cuuint64_t)a.Z * a.B};
-  cuuint64_t strides[4] = {16, (cuuint64_t)CIP * 2, (cuuint64_t)a.X * CIP * 2, (cuuint64_t)a.Y * a.X * CIP * 2};
-  cuuint32_t box[5] = {8, 1, (cuuint32_t)TC_BX, 1, 1};
-  cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+  __syncwarp();
+  if (warp == EPI + 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem0), "r"(COLS));
 }
 
 template <int CIP, int N, int COP, int MODE>
 static cudaError_t conv_tc_go(const ConvArgs& a, const bf16* wtc, int* flag, cudaStream_t s) {
-  const size_t bytes = (size_t)(2 * TC_NBOX * CIP + NTAP * CIP * N) * sizeof(bf16) + 64;
+  const size_t bytes = (size_t)TC_NR * 3 * (CIP / 8) * TcPitch<CIP>::value * 16 + (size_t)NTAP * CIP * N * sizeof(bf16) + 32 * sizeof(float) + 128;
   static std::atomic<unsigned long long> done{0};  // per-device bit; host threads may race here
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -328,18 +313,15 @@ static cudaError_t conv_tc_go(const ConvArgs& a, const bf16* wtc, int* flag, cud
     if (dev < 64) done.fetch_or(1ull << dev, std::memory_order_acq_rel);
   }
   if (((uintptr_t)a.in & 15u) != 0) return cudaErrorMisalignedAddress;
-  CUtensorMap map;
-  e = tc_map(&map, a.in, CIP, a);
-  if (e != cudaSuccess) return e;
   int nsm = 0, occ = 0;
   e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, conv_tc_kernel<CIP, N, COP, MODE>, TC_THREADS, bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, conv_tc_kernel<CIP, N, COP, MODE>, TcWarps<N>::threads, bytes);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)((a.X + TC_M - 1) / TC_M) * a.Y * a.Z * a.B;
   long long grid = (long long)nsm * (occ > 0 ? occ : 1);
   if (grid > tiles) grid = tiles;
-  conv_tc_kernel<CIP, N, COP, MODE><<<(unsigned)grid, TC_THREADS, bytes, s>>>(a, map, wtc, flag, tiles);
+  conv_tc_kernel<CIP, N, COP, MODE><<<(unsigned)grid, TcWarps<N>::threads, bytes, s>>>(a, wtc, flag, tiles);
   return cudaGetLastError();
 }
 

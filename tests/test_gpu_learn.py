@@ -314,3 +314,19 @@ def test_train_gradient_at_the_edges_of_the_32_by_4_tiles(gb, shape, zper):
     assert abs(loss - want_loss) <= 1e-3 * want_loss
     for name, sl in tensor_slices():
         assert np.linalg.norm(grad[sl] - want[sl]) <= 1e-2 * np.linalg.norm(want[sl]), name
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (1, 3, 2, 127), (2, 2, 5, 128), (1, 2, 7, 129), (1, 1, 300, 20), (3, 4, 3, 260)])
+@pytest.mark.parametrize("zper", [True, False])
+def test_forward_at_the_edges_of_the_row_ring(gb, shape, zper):
+    """columns of one to hundreds of rows (pieces shorter than the ring, pieces that wrap it), x tiles
+    of one cell less and more than 128, several volumes: relative L2 <= 2e-3 (the forward bound)"""
+    B, Z, Y, X = shape
+    p, x = random_params(41), rng(42).standard_normal((B, 10, Z, Y, X))
+    xg = to_gpu_features(x)
+    a = gb.Accel(X, Y, Z, B, zperiodic=zper)
+    a.set_params(p)
+    y = from_gpu(a.forward(xg), B, Z, Y, X)
+    xb = from_gpu(xg, B, Z, Y, X, C=10)
+    want = np.stack([L.forward(p, xb[b], zper)[0] for b in range(B)])
+    assert np.linalg.norm(y - want) <= 2e-3 * np.linalg.norm(want)
