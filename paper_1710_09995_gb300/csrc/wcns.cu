@@ -521,15 +521,7 @@ __device__ __forceinline__ void edges(V u0, V u1, V u2, V u3, V u4, bool linear,
   const V nA = O::c(1.0 / 16.0) * bc, nB = O::c(10.0 / 16.0) * ac, nC = O::c(5.0 / 16.0) * ab;
   const V kA = O::c(5.0 / 16.0) * bc, kC = O::c(1.0 / 16.0) * ab;
   const V dp = nA + nB + nC, dm = kA + nB + kC;
-  V rp, rm;
-  if constexpr (sizeof(V) == 8) {  // one FP64 division for both (dp, dm >= ~1e-25: no underflow)
-    const V r = O::rcp(dp * dm);
-    rp = dm * r;
-    rm = dp * r;
-  } else {
-    rp = O::rcp(dp);
-    rm = O::rcp(dm);
-  }
+  const V rp = O::rcp(dp), rm = O::rcp(dm);
   up = u2 + O::fma(nA, pA, O::fma(nB, pB, nC * pC)) * rp;
   um = u2 + O::fma(kA, mA, O::fma(nB, mB, kC * mC)) * rm;
 }
@@ -579,27 +571,66 @@ template <> struct Fr<0> { static constexpr int N = 1, T1 = 2, T2 = 3; };
 template <> struct Fr<1> { static constexpr int N = 2, T1 = 3, T2 = 1; };
 template <> struct Fr<2> { static constexpr int N = 3, T1 = 1, T2 = 2; };
 
-template <typename T>
-struct Smem {
+struct Smem {  // the mixed path's direction passes (FP64: XSmem)
+  using T = float;
   static constexpr int WS = 5 * (LMAX + 10) * NLP;   // staged primitives [5][L+10][NLP], then
                                                      // the edge fluxes [5][L+5][NLP] over them;
                                                      // two buffers (the next tile lands in one)
-  static constexpr int RS = sizeof(T) == 4 ? 5 * LMAX * NLP : 0;  // the running residual of the tile's
-                                                                   // cells (mixed path only)
+  static constexpr int RS = 5 * LMAX * NLP;          // the running residual of the tile's cells
   static constexpr size_t rs = (2 * sizeof(T) * WS + 15) / 16 * 16;
   static constexpr size_t red = (rs + sizeof(T) * RS + 15) / 16 * 16;  // norm partials (double)
   static constexpr size_t bytes = red + sizeof(double) * (NTW / 32) * 5;
 };
 
-
+// the residual norm at the end of stage 1's z pass, called by all threads: per-thread sums of R^2 (sq)
+// to the CTA's partial slot; the last CTA folds the slots in a fixed order
+__device__ __forceinline__ void norm_fold(const Args& a, double (&sq)[5], double* red, int* last) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // residual norm of R(Q^n): per-CTA sums of squares, the last CTA folds them in CTA order
+#pragma unroll
+  for (int q = 0; q < 5; ++q)
+    for (int off = 16; off > 0; off >>= 1) sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], off);
+  __syncthreads();
+  if (lane == 0)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) red[warp * 5 + q] = sq[q];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 5; ++q) {
+      double s = 0.0;
+      for (int w = 0; w < NTW / 32; ++w) s += red[w * 5 + q];
+      a.partial[(size_t)blockIdx.x * NPART + q] = s;
+    }
+    __threadfence();
+    *last = (atomicAdd(&a.ctrl->counter, 1u) == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!*last || threadIdx.x >= 32) return;
+  __threadfence();
+  // the last CTA's first warp folds the per-CTA sums: lane-strided in CTA order, then a fixed
+  // shuffle tree (the same order every run: deterministic)
+  double tot[5] = {0, 0, 0, 0, 0};
+  for (unsigned c = threadIdx.x; c < gridDim.x; c += 32)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) tot[q] += __ldcg(a.partial + (size_t)c * NPART + q);
+#pragma unroll
+  for (int q = 0; q < 5; ++q)
+    for (int off = 16; off > 0; off >>= 1) tot[q] += __shfl_xor_sync(0xffffffffu, tot[q], off);
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 5; ++q) a.ctrl->norms[q] = sqrt(tot[q] / (double)a.n);
+    a.ctrl->counter = 0u;
+  }
+}
 
 // MODE: 0 x pass (R =), 1 y pass (R +=), 2 z pass (stage update or residual output)
-template <typename T, int D, int MODE>
-__global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a) {
+// The mixed path's kernel; the FP64 path's is xdir_kernel (wcns_x.cuh)
+template <int D, int MODE>
+__global__ void __launch_bounds__(NTW, 3) dir_kernel(Args a) {
+  using T = float;
   using O = VM<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* const Wbuf = reinterpret_cast<T*>(smem_raw);
-  double* red = reinterpret_cast<double*>(smem_raw + Smem<T>::red);
+  double* red = reinterpret_cast<double*>(smem_raw + Smem::red);
   __shared__ int last;
   const Box& b = a.b;
   const int nd = D == 0 ? b.nx : (D == 1 ? b.ny : b.nz);   // along the lines
@@ -670,7 +701,7 @@ __global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a
   };
   // the y and z passes add to the residual R of the earlier passes: the tile's R lands in shared
   // memory (as its own commit group) while the edge fluxes are computed
-  T* const Rs = reinterpret_cast<T*>(smem_raw + Smem<T>::rs);
+  T* const Rs = reinterpret_cast<T*>(smem_raw + Smem::rs);
   auto issue_r = [&](const TileInfo& t) {
     for (int q = 0; q < 5; ++q)
       for (int e = threadIdx.x; e < t.Ls * NL; e += NTW) {
@@ -687,15 +718,15 @@ __global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a
   for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
     const TileInfo t = decode(tile);
     const int s0 = t.s0, Ls = t.Ls, a0 = t.a0;
-    T* const Ws = Wbuf + buf * Smem<T>::WS;
+    T* const Ws = Wbuf + buf * Smem::WS;
     T* const Fs = Ws;  // the edge fluxes replace the primitives once every lane holds its fluxes
     const int nfc = Ls + 5;
     cp_async_wait_all();
     __syncthreads();  // the tile has landed; the previous tile's cells are done with the other buffer
-    constexpr bool RSTAGE = MODE != 0 && sizeof(T) == 4;  // FP64: shared memory is kept for occupancy
+    constexpr bool RSTAGE = MODE != 0;
     if (RSTAGE) issue_r(t);
     const bool more = tile + gridDim.x < tiles;
-    if (more) issue_stage(decode(tile + gridDim.x), Wbuf + (buf ^ 1) * Smem<T>::WS);
+    if (more) issue_stage(decode(tile + gridDim.x), Wbuf + (buf ^ 1) * Smem::WS);
     // 2. edge fluxes: edge f lies between staged cells f + 2 and f + 3, so cell c (staged c + 5)
     //    has edges c .. c + 5 around it.  Item (line, chunk): lane t takes staged cell
     //    m = 31 chunk + t + 2, evaluates its two edge states, and edge f = m - 2 pairs its
@@ -708,7 +739,7 @@ __global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a
       if (a0 + l >= na || FCH * ch >= nfc) continue;  // warp-uniform
       const int m = min(f + 2, nfc + 2);              // centres 2 .. nfc + 2 (stencil <= nst - 1)
       T Lq[5], Rq[5];
-      if constexpr (sizeof(T) == 4) {  // mixed: frame variables (0, 1) and (2, 3) as packed pairs
+      {  // frame variables (0, 1) and (2, 3) as packed pairs
 #pragma unroll
         for (int q = 0; q < 4; q += 2) {
           const T* w0 = Ws + (idx[q] * (LMAX + 10) + m - 2) * NLP + l;
@@ -726,20 +757,8 @@ __global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a
         edges<T>(w[0], w[NLP], w[2 * NLP], w[3 * NLP], w[4 * NLP], linear, up, um);
         Lq[4] = up;
         Rq[4] = __shfl_down_sync(0xffffffffu, um, 1);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const T* w = Ws + (idx[q] * (LMAX + 10) + m - 2) * NLP + l;
-          T up, um;
-          edges<T>(w[0], w[NLP], w[2 * NLP], w[3 * NLP], w[4 * NLP], linear, up, um);
-          Lq[q] = up;
-          Rq[q] = __shfl_down_sync(0xffffffffu, um, 1);
-        }
       }
-      if (lane < FCH && f < nfc) {
-        if constexpr (sizeof(T) == 8) xroe<false>(Lq, Rq, coef<T>(a).x, F[it]);  // on the integer pipes (xfix.cuh)
-        else roe_frame<T>(Lq, Rq, K, F[it]);
-      }
+      if (lane < FCH && f < nfc) roe_frame<T>(Lq, Rq, K, F[it]);
     }
     __syncthreads();  // every lane is done reading the primitives
 #pragma unroll
@@ -788,23 +807,7 @@ __global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a
         for (int q = 0; q < 5; ++q) R[q * a.n + cc] = add[q];
       } else if (MODE == 1) {
 #pragma unroll
-        for (int q = 0; q < 5; ++q) R[q * a.n + cc] = (RSTAGE ? Rs[(q * LMAX + c) * NLP + l] : R[q * a.n + cc]) + add[q];
-      } else if (sizeof(T) == 8) {  // FP64: Eqs. 4-6 as written
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const double tot = double(R[q * a.n + cc]) + double(add[q]);
-          if (a.stage == 0) {
-            a.rout[q * a.n + cc] = tot;
-            continue;
-          }
-          if (a.stage == 1) sq[q] += tot * tot;
-          const double adv = a.qs[q * a.n + cc] - dt * tot;
-          double out;
-          if (a.stage == 1) out = adv;
-          else if (a.stage == 2) out = 0.75 * a.qn[q * a.n + cc] + 0.25 * adv;
-          else out = a.qn[q * a.n + cc] / 3.0 + 2.0 / 3.0 * adv;
-          a.qout[q * a.n + cc] = out;
-        }
+        for (int q = 0; q < 5; ++q) R[q * a.n + cc] = Rs[(q * LMAX + c) * NLP + l] + add[q];
       } else {  // mixed: f32 increments, FP64 only for Q^{n+1} = Q^n + 2/3 (D2 - dt R)
         const float dtf = float(dt);
 #pragma unroll
@@ -827,51 +830,28 @@ __global__ void __launch_bounds__(NTW, sizeof(T) == 4 ? 3 : 2) dir_kernel(Args a
       }
     }
   }
-  if (MODE != 2 || a.stage != 1) return;
-  // residual norm of R(Q^n): per-CTA sums of squares, the last CTA folds them in CTA order
-#pragma unroll
-  for (int q = 0; q < 5; ++q)
-    for (int off = 16; off > 0; off >>= 1) sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], off);
-  __syncthreads();
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < 5; ++q) red[warp * 5 + q] = sq[q];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < 5; ++q) {
-      double s = 0.0;
-      for (int w = 0; w < NTW / 32; ++w) s += red[w * 5 + q];
-      a.partial[(size_t)blockIdx.x * NPART + q] = s;
-    }
-    __threadfence();
-    last = (atomicAdd(&a.ctrl->counter, 1u) == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!last || threadIdx.x >= 32) return;
-  __threadfence();
-  // the last CTA's first warp folds the per-CTA sums: lane-strided in CTA order, then a fixed
-  // shuffle tree (the same order every run: deterministic)
-  double tot[5] = {0, 0, 0, 0, 0};
-  for (unsigned c = threadIdx.x; c < gridDim.x; c += 32)
-#pragma unroll
-    for (int q = 0; q < 5; ++q) tot[q] += __ldcg(a.partial + (size_t)c * NPART + q);
-#pragma unroll
-  for (int q = 0; q < 5; ++q)
-    for (int off = 16; off > 0; off >>= 1) tot[q] += __shfl_xor_sync(0xffffffffu, tot[q], off);
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < 5; ++q) a.ctrl->norms[q] = sqrt(tot[q] / (double)a.n);
-    a.ctrl->counter = 0u;
-  }
+  if (MODE == 2 && a.stage == 1) norm_fold(a, sq, red, &last);
 }
+
+}  // namespace wcns
+}  // namespace gbcfd
+
+#include "wcns_x.cuh"  // the FP64 path's direction passes
+
+namespace gbcfd {
+namespace wcns {
 
 template <typename T>
 static cudaError_t set_smem() {
-  const int bytes = (int)Smem<T>::bytes;
   cudaError_t e;
-#define GB_SET(D, M)                                                                                    \
-  e = cudaFuncSetAttribute(dir_kernel<T, D, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); \
+#define GB_SET(K, B)                                                                          \
+  e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(B)); \
   if (e != cudaSuccess) return e;
-  GB_SET(0, 0) GB_SET(1, 1) GB_SET(2, 2)
+  if constexpr (sizeof(T) == 8) {
+    GB_SET((xdir_kernel<0, 0>), XSmem::bytes) GB_SET((xdir_kernel<1, 1>), XSmem::bytes) GB_SET((xdir_kernel<2, 2>), XSmem::bytes)
+  } else {
+    GB_SET((dir_kernel<0, 0>), Smem::bytes) GB_SET((dir_kernel<1, 1>), Smem::bytes) GB_SET((dir_kernel<2, 2>), Smem::bytes)
+  }
 #undef GB_SET
   e = cudaFuncSetAttribute(viscres_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RSmem<T>::bytes);
   if (e != cudaSuccess) return e;
@@ -888,7 +868,8 @@ static int viscres_occupancy() {
 template <typename T>
 static int dir_occupancy() {
   int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dir_kernel<T, 0, 0>, NTW, Smem<T>::bytes);
+  if constexpr (sizeof(T) == 8) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, xdir_kernel<0, 0>, NTW, XSmem::bytes);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dir_kernel<0, 0>, NTW, Smem::bytes);
   return std::max(1, occ);
 }
 
@@ -1060,13 +1041,20 @@ cudaError_t launch_rest(gbcfd_wcns w, const Args& a, const cudaEvent_t* ev, cuda
   };
   if (a.viscous) viscres_kernel<T><<<w->nsm * w->rocc, NTW, RSmem<T>::bytes, s>>>(a);
   mark(2);
-  const size_t sm = Smem<T>::bytes;
   const int g = w->dir_grid;
-  dir_kernel<T, 0, 0><<<g, NTW, sm, s>>>(a);
-  mark(3);
-  dir_kernel<T, 1, 1><<<g, NTW, sm, s>>>(a);
-  mark(4);
-  dir_kernel<T, 2, 2><<<g, NTW, sm, s>>>(a);
+  if constexpr (sizeof(T) == 8) {
+    xdir_kernel<0, 0><<<g, NTW, XSmem::bytes, s>>>(a);
+    mark(3);
+    xdir_kernel<1, 1><<<g, NTW, XSmem::bytes, s>>>(a);
+    mark(4);
+    xdir_kernel<2, 2><<<g, NTW, XSmem::bytes, s>>>(a);
+  } else {
+    dir_kernel<0, 0><<<g, NTW, Smem::bytes, s>>>(a);
+    mark(3);
+    dir_kernel<1, 1><<<g, NTW, Smem::bytes, s>>>(a);
+    mark(4);
+    dir_kernel<2, 2><<<g, NTW, Smem::bytes, s>>>(a);
+  }
   mark(5);
   return cudaGetLastError();
 }

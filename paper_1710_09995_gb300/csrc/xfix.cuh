@@ -445,14 +445,6 @@ __host__ __device__ __forceinline__ XPair xpair(double l, double r) {
   const int e = xmax(a.e, b.e);
   return {xshr(a.m, e - a.e), xshr(b.m, e - b.e), e};
 }
-// roe_frame's interface: L, R = (rho, u_n, u_t1, u_t2, p), F twice the flux or (TWICE false) the flux
-template <bool TWICE = true>
-__host__ __device__ __forceinline__ void xroe(const double* L, const double* R, const XConsts& K, double* F) {
-  XFlux f;
-  xroe(xpair(L[0], R[0]), xpair(L[1], R[1]), xpair(L[2], R[2]), xpair(L[3], R[3]), xpair(L[4], R[4]), K, f);
-  for (int q = 0; q < 5; ++q) F[q] = xflux(f, q, TWICE ? 0 : 1);
-}
-
 // the primitives of a conserved state (rho, rho u, rho v, rho w, rho E): velocities [62] and pressure
 // [62] each in its own class, 1 / rho; false where the density or the pressure is not positive or
 // not finite
@@ -493,6 +485,101 @@ __host__ __device__ __forceinline__ XVal xsound(const XPrim& W, const XVal& gam)
   const XVal c2 = xnormed(xmul(gam.m, xmul(W.p.m, W.ir.m) << 2), gam.e + W.p.e + W.ir.e + 4);
   const XVal ic = xrsqrt(c2);
   return {xmul(c2.m, ic.m) << 2, c2.e + ic.e + 1};
+}
+
+// ---- WCNS-E-5 lines ----------------------------------------------------------------------------
+#ifdef __CUDACC__
+#define XNOINLINE __noinline__  // called per variable: inlined five times it was half the kernel's code
+#else
+#define XNOINLINE inline
+#endif
+constexpr int XW_BIAS = 1018;       // staged value = m 2^(e - 1018 - 61), |m| < 2^57
+constexpr int XW_BAD = 2 * XBAD;    // exponent of a staged value that is not finite
+
+// a double as a staged value (zero and subnormals as zero, a value that is not finite by its exponent)
+__host__ __device__ __forceinline__ void xline_value(double v, long long* m, short* e) {
+  const unsigned long long bits = xbits(v);
+  const int hi = (int)(bits >> 32), ex = (int)(((unsigned)hi >> 20) & 0x7ffu);
+  const unsigned long long mag = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)bits;
+  const long long sg = hi >> 31;
+  *m = ex ? ((long long)(mag << 4) ^ sg) - sg : 0ll;
+  *e = (short)(ex == 0x7ff ? XW_BAD : ex);
+}
+// a face's sides normalised together: the products of xroe are then rounded relative to the larger (edge
+// values have up to four spare bits: their squares lost eight, three times the FP64 form's error in
+// the energy residual)
+__host__ __device__ __forceinline__ XPair xpair_norm(long long l, long long r, int e) {
+  const int n = xclz32((int)((l ^ (l >> 63)) >> 32) | (int)((r ^ (r >> 63)) >> 32)) - 2;  // 0 .. 30
+  return {l << n, r << n, e - n};
+}
+// both edge values of a cell: u_{i+1/2} from the left, u_{i-1/2} from the right, class e, [62]
+struct XEdge {
+  long long up, um;
+  int e;
+};
+// the weighted interpolation of WCNS-E-5 (edges() in wcns.cu) from the five staged values at wm, we.
+// With d_j the first differences of u_{i-2} .. u_{i+2}: eight times the candidates' distances from u_i
+// are small integer combinations of them, twice the first derivatives too.  Each stencil's
+// smoothness is formed from its own normalised differences, and the weights are compared in the
+// class of the largest: one 2^61 times smaller has no part in the value.
+template <int STRIDE>
+__host__ __device__ XNOINLINE XEdge xedges(const long long* __restrict__ wm, const short* __restrict__ we, bool linear,
+                                             XVal eps) {
+  long long u[5];
+  int e[5];
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    u[c] = wm[c * STRIDE];
+    e[c] = we[c * STRIDE];
+  }
+  int E = xmax(xmax(xmax(e[0], e[1]), xmax(e[2], e[3])), e[4]);
+#pragma unroll
+  for (int c = 0; c < 5; ++c) u[c] = xshr(u[c], E - e[c]);  // [57]
+  E -= XW_BIAS;
+  const long long d0 = u[1] - u[0], d1 = u[2] - u[1], d2 = u[3] - u[2], d3 = u[4] - u[3];  // [58]
+  auto x3 = [](long long a) { return (a << 1) + a; };
+  auto x5 = [](long long a) { return (a << 2) + a; };
+  auto x7 = [](long long a) { return (a << 3) - a; };
+  auto x10 = [](long long a) { return (a << 3) + (a << 1); };
+  // 8 (candidate - u_i) at i + 1/2 and i - 1/2 [62]
+  long long pA = x7(d1) - x3(d0), pB = x3(d2) + d1, pC = x5(d2) - d3;
+  long long qA = d0 - x5(d1), qB = -(x3(d1) + d2), qC = x3(d3) - x7(d2);
+  XEdge o;
+  o.e = E - 3;
+  if (linear) {
+    o.up = (u[2] << 3) + ((pA >> 4) + x10(pB >> 4) + x5(pC >> 4));
+    o.um = (u[2] << 3) + (x5(qA >> 4) + x10(qB >> 4) + (qC >> 4));
+    return o;
+  }
+  // (1e-6 + g^2 + s^2)^2 of a stencil from 2 g and 2 s [60], normalised [62]
+  auto weight = [&](long long g, long long s) -> XVal {
+    const int n = xclz32((int)((g ^ (g >> 63)) >> 32) | (int)((s ^ (s >> 63)) >> 32)) - 2;  // 2 .. 30
+    const long long q = xsq(g << n) + xsq(s << n);                                          // 4 (g^2 + s^2) [61]
+    const int eb = 2 * (E - n) + 1, ed = xmax(eb, eps.e + 1);
+    const XVal d = xquick(xshr(q, ed - eb) + xshr(eps.m, ed - eps.e), ed);
+    return {xsq(d.m) << 2, 2 * d.e + 1};
+  };
+  const XVal A = weight(x3(d1) - d0, (d1 - d0) << 1), B = weight(d1 + d2, (d2 - d1) << 1),
+             C = weight(x3(d2) - d3, (d3 - d2) << 1);
+  const int ea = B.e + C.e, eb = A.e + C.e, ec = A.e + B.e, Em = xmax(ea, xmax(eb, ec)) + 2;
+  const long long a = xshr(xmul(B.m, C.m), Em - ea), b = x10(xshr(xmul(A.m, C.m), Em - eb)), c = xshr(xmul(A.m, B.m), Em - ec);
+  const int En = Em + 3;
+  const long long a5 = x5(a), c5 = x5(c);  // a, c [58]; b, a5, c5 [62]
+  const XVal rp = xrcp(xnormed(a + b + c5, En)), rm = xrcp(xnormed(a5 + b + c, En));
+  // the candidates' distances, normalised together
+  const long long any = (pA ^ (pA >> 63)) | (pB ^ (pB >> 63)) | (pC ^ (pC >> 63)) | (qA ^ (qA >> 63)) | (qB ^ (qB >> 63)) |
+                        (qC ^ (qC >> 63));
+  const int n = xclz32((int)(any >> 32)) - 2;
+  const int et = En + E - 3 - n + 3;
+  auto value = [&](long long t, const XVal& r) -> long long {  // u_i + t r in class E - 3
+    const XVal f = xquick(t, et);
+    const long long v = xmul(f.m, r.m);
+    const int sh = E - 3 - (f.e + r.e + 3);  // at least -4: the distance is at most 10/8 of the values' span
+    return (u[2] << 3) + (sh >= 0 ? xshr(v, sh) : v << -sh);
+  };
+  o.up = value(xmul(a, pA << n) + xmul(b, pB << n) + xmul(c5, pC << n), rp);
+  o.um = value(xmul(a5, qA << n) + xmul(b, qB << n) + xmul(c, qC << n), rm);
+  return o;
 }
 
 }  // namespace gbcfd

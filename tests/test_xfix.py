@@ -18,11 +18,27 @@ HARNESS = r"""
 #define __device__
 #define __forceinline__ inline
 #include "xfix.cuh"
+extern "C" void edges(int n, const double* u, int linear, double* out) {
+  const gbcfd::XVal eps = gbcfd::xdec_pos<62>(1e-6);
+  for (int i = 0; i < n; ++i) {
+    long long m[5];
+    short e[5];
+    for (int c = 0; c < 5; ++c) gbcfd::xline_value(u[5 * i + c], m + c, e + c);
+    const gbcfd::XEdge g = gbcfd::xedges<1>(m, e, linear != 0, eps);
+    out[2 * i] = gbcfd::xenc(g.up, g.e);
+    out[2 * i + 1] = gbcfd::xenc(g.um, g.e);
+  }
+}
+// the frame flux from doubles, twice or (half) once
+static void frame(const double* l, const double* r, const gbcfd::XConsts& K, int half, double* F) {
+  gbcfd::XFlux f;
+  gbcfd::xroe(gbcfd::xpair(l[0], r[0]), gbcfd::xpair(l[1], r[1]), gbcfd::xpair(l[2], r[2]), gbcfd::xpair(l[3], r[3]),
+              gbcfd::xpair(l[4], r[4]), K, f);
+  for (int q = 0; q < 5; ++q) F[q] = gbcfd::xflux(f, q, half);
+}
 extern "C" void roe(int n, const double* L, const double* R, double gamma, double eps, int half, double* F) {
   const gbcfd::XConsts K = gbcfd::xconsts(gamma, eps);
-  for (int i = 0; i < n; ++i)
-    if (half) gbcfd::xroe<false>(L + 5 * i, R + 5 * i, K, F + 5 * i);
-    else gbcfd::xroe<true>(L + 5 * i, R + 5 * i, K, F + 5 * i);
+  for (int i = 0; i < n; ++i) frame(L + 5 * i, R + 5 * i, K, half, F + 5 * i);
 }
 extern "C" void roe_area(int n, const double* L, const double* R, const double* S, double gamma, double eps, double* F) {
   const gbcfd::XConsts K = gbcfd::xconsts(gamma, eps);
@@ -246,3 +262,46 @@ def test_non_physical_primitives_are_refused(lib, q):
     a, W, ok = np.array(q, dtype=np.float64), np.empty(6), np.ones(1, dtype=np.int32)
     lib.prims(1, _p(a), ctypes.c_double(1.4), _p(W), ok.ctypes.data_as(ctypes.c_void_p))
     assert not ok[0]
+
+
+@pytest.mark.parametrize("kind", ["smooth", "rough", "step", "flat", "tiny", "offset", "zero", "mixed sizes"])
+@pytest.mark.parametrize("linear", [0, 1])
+def test_weighted_interpolation(lib, kind, linear):
+    """both edge values of the WCNS-E-5 interpolation against the definition in long double.  The FP64
+    form rounds the candidates and the sum relative to the stencil's largest value; its weights'
+    roundings (about 20) act on the candidates' distances."""
+    n, rng = 20000, np.random.Generator(np.random.PCG64(21))
+    x = np.arange(5) * 0.1
+    u = {"smooth": lambda: np.sin(x + rng.uniform(0, 6.3, (n, 1))) + 2.0,
+         "rough": lambda: rng.uniform(-1, 1, (n, 5)),
+         "step": lambda: np.where(np.arange(5) < rng.integers(0, 6, (n, 1)), 1.0, 0.125) + 1e-4 * rng.uniform(-1, 1, (n, 5)),
+         "flat": lambda: np.repeat(rng.uniform(-1, 1, (n, 1)), 5, 1),
+         "tiny": lambda: 1e-200 * rng.uniform(-1, 1, (n, 5)),
+         "offset": lambda: 1e5 + rng.uniform(-1, 1, (n, 5)),
+         "zero": lambda: np.zeros((n, 5)),
+         "mixed sizes": lambda: rng.uniform(-1, 1, (n, 5)) * 10.0 ** rng.uniform(-8, 2, (n, 5))}[kind]()
+    u = np.ascontiguousarray(u)
+    out = np.empty((n, 2))
+    lib.edges(n, _p(u), linear, _p(out))
+    w = u.astype(np.longdouble).T
+
+    def edge(a):
+        g = [(a[0] - 4 * a[1] + 3 * a[2]) / 2, (a[3] - a[1]) / 2, (-3 * a[2] + 4 * a[3] - a[4]) / 2]
+        s = [a[0] - 2 * a[1] + a[2], a[1] - 2 * a[2] + a[3], a[2] - 2 * a[3] + a[4]]
+        al = [c if linear else c / (np.longdouble(1e-6) + gk * gk + sk * sk) ** 2
+              for c, gk, sk in zip((np.longdouble(1), 10, 5), g, s)]
+        return a[2] + sum(k * (gk / 2 + sk / 8) for k, gk, sk in zip(al, g, s)) / sum(al)
+
+    want = np.stack([edge(w), edge(w[::-1])], 1)
+    big, span = np.abs(u).max(1, keepdims=True), (u.max(1) - u.min(1))[:, None]
+    assert np.all(np.abs(out - want) <= 4 * ULP * big + 20 * ULP * span)
+    if kind in ("flat", "zero"):
+        assert np.array_equal(out, u[:, 2:3].repeat(2, 1))
+
+
+def test_staged_values_that_are_not_finite_stay_so(lib):
+    u = np.ones((3, 5))
+    u[0, 0], u[1, 2], u[2, 4] = np.nan, np.inf, -np.inf
+    out = np.empty((3, 2))
+    lib.edges(3, _p(u), 0, _p(out))
+    assert not np.isfinite(out).any()
