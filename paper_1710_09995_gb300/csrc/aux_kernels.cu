@@ -142,59 +142,149 @@ cudaError_t launch_gather(const Geometry& g, const double* src, double* dst, cud
 // rate = sum over directions of (|u_d| + c) / h_d (+ 4 max(4/3, gamma/Pr) mu / rho / h_d^2 when
 // viscous); the CFL step is cfl / max(rate).  From the padded f64 state, in the path's flux
 // precision T (the mixed path's time step is an f32 evaluation, like its fluxes).
-template <typename T>
-__global__ void init_rate_kernel(Geometry g, Physics ph, const double* __restrict__ q, DevCtrl* ctrl,
-                                 double* partial, T* dtl) {
-  __shared__ double wmax[32];
+// A warp per row of cells.  FP64 blocks evaluate it on the integer pipes (xfix.cuh).  The maxima are
+// compared as bit patterns and the CTAs' folded by a warp of the last CTA: one thread walking all
+// partial rows took most of the 60 us this pass cost a 32^3 block.
+constexpr int RATE_THREADS = 256;
+__device__ __forceinline__ void rate_fold(long long best, DevCtrl* ctrl, double* partial, double cfl) {
+  __shared__ long long wmax[RATE_THREADS / 32];
   __shared__ int last;
-  const long long n = (long long)g.nx * g.ny * g.nz;
-  double best = 0.0;
-  const T f = T(fmax(4.0 / 3.0, ph.gamma / ph.Pr));
-  const T s2 = T(ph.ihx * ph.ihx + ph.ihy * ph.ihy + ph.ihz * ph.ihz);
-  const T gam = T(ph.gamma), gm1 = T(ph.gamma - 1.0), mu4 = T(4.0 * ph.mu);
-  const T ihx = T(ph.ihx), ihy = T(ph.ihy), ihz = T(ph.ihz);
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(c % g.nx);
-    const long long r = c / g.nx;
-    const int j = (int)(r % g.ny), k = (int)(r / g.ny);
-    const long long o = gidx(g, i, j, k);
-    const T rho = T(q[o]), ir = T(1) / rho;
-    const T u = T(q[g.field + o]) * ir, v = T(q[2 * g.field + o]) * ir, w = T(q[3 * g.field + o]) * ir;
-    const T p = gm1 * (T(q[4 * g.field + o]) - T(0.5) * rho * (u * u + v * v + w * w));
-    const T a = sqrt(gam * p * ir);
-    T rate = (fabs(u) + a) * ihx + (fabs(v) + a) * ihy + (fabs(w) + a) * ihz;
-    if (ph.viscous) rate += f * mu4 * ir * s2;
-    if (dtl) dtl[sizeof(T) == 8 ? o : gidxf(g, i, j, k)] = T(ph.cfl) / rate;
-    if (!(rho > T(0) && p > T(0))) atomicOr(&ctrl->flag, FLAG_NONPHYSICAL);
-    best = fmax(best, double(rate));
-  }
-  for (int off = 16; off > 0; off >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, off));
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = best;
+  const int lane = threadIdx.x & 31;
+  best = warp_max_bits(best);
+  if (lane == 0) wmax[threadIdx.x >> 5] = best;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wmax[w]);
-    partial[(size_t)blockIdx.x * NPART + 5] = m;
-    __threadfence();
-    last = (atomicAdd(&ctrl->counter, 1u) == gridDim.x - 1);
+  if (threadIdx.x < 32) {
+    const long long m = warp_max_bits(lane < RATE_THREADS / 32 ? wmax[lane] : 0ll);
+    if (lane == 0) {
+      partial[(size_t)blockIdx.x * NPART + 5] = __longlong_as_double(m);
+      __threadfence();
+      last = (atomicAdd(&ctrl->counter, 1u) == gridDim.x - 1);
+    }
   }
   __syncthreads();
-  if (!last || threadIdx.x != 0) return;
+  if (!last || threadIdx.x >= 32) return;
   __threadfence();
-  double m = 0.0;
-  for (unsigned b = 0; b < gridDim.x; ++b) m = fmax(m, __ldcg(partial + (size_t)b * NPART + 5));
-  ctrl->rate = m;
-  ctrl->dt = ph.cfl / m;
-  ctrl->counter = 0u;
+  long long m = 0;
+#pragma unroll 4
+  for (unsigned b = lane; b < gridDim.x; b += 32) {
+    const long long v = __double_as_longlong(__ldcg(partial + (size_t)b * NPART + 5));
+    m = v > m ? v : m;
+  }
+  m = warp_max_bits(m);
+  if (lane == 0) {
+    const double r = __longlong_as_double(m);
+    ctrl->rate = r;
+    ctrl->dt = cfl / r;
+    ctrl->counter = 0u;
+  }
+}
+
+// the mixed path's constants, formed on the host
+struct RateConsts {
+  float gam, gm1, f, mu4, fmu4, ihx, ihy, ihz, s2, cfl;
+};
+static RateConsts rate_consts(const Physics& ph) {
+  const double f = std::max(4.0 / 3.0, ph.gamma / ph.Pr);
+  return {float(ph.gamma), float(ph.gamma - 1.0), float(f), float(4.0 * ph.mu), float(4.0 * f * ph.mu), float(ph.ihx),
+          float(ph.ihy), float(ph.ihz), float(ph.ihx * ph.ihx + ph.ihy * ph.ihy + ph.ihz * ph.ihz), float(ph.cfl)};
+}
+
+__global__ void __launch_bounds__(RATE_THREADS) init_rate_kernel(Geometry g, int viscous, RateConsts C, double cfl,
+                                                                  const double* __restrict__ q, DevCtrl* ctrl,
+                                                                  double* partial, float* dtl) {
+  float best = 0.f;
+  bool bad = false;
+  const int rows = g.ny * g.nz, lane = threadIdx.x & 31;
+  for (int row = blockIdx.x * (RATE_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += gridDim.x * (RATE_THREADS / 32)) {
+    const int j = row % g.ny, k = row / g.ny;
+    for (int i = lane; i < g.nx; i += 32) {
+      const long long o = gidx(g, i, j, k);
+      const float rho = float(q[o]), ir = 1.f / rho;
+      const float u = float(q[g.field + o]) * ir, v = float(q[2 * g.field + o]) * ir, w = float(q[3 * g.field + o]) * ir;
+      const float p = C.gm1 * (float(q[4 * g.field + o]) - 0.5f * rho * (u * u + v * v + w * w));
+      const float a = sqrtf(C.gam * p * ir);
+      float rate = (fabsf(u) + a) * C.ihx + (fabsf(v) + a) * C.ihy + (fabsf(w) + a) * C.ihz;
+      if (viscous) rate += C.f * C.mu4 * ir * C.s2;
+      if (dtl) dtl[gidxf(g, i, j, k)] = C.cfl / rate;
+      if (!(rho > 0.f && p > 0.f)) bad = true;
+      best = rate > best ? rate : best;
+    }
+  }
+  if (bad) atomicOr(&ctrl->flag, FLAG_NONPHYSICAL);
+  rate_fold(__double_as_longlong(double(best)), ctrl, partial, cfl);
+}
+
+// FP64: M = null on uniform grids, else the metric fields
+template <bool VISC, bool CURVI>
+__global__ void __launch_bounds__(RATE_THREADS) init_rate_x_kernel(Geometry g, Physics ph, XConsts K,
+                                                                    const double* __restrict__ q,
+                                                                    const double* __restrict__ M, DevCtrl* ctrl,
+                                                                    double* partial, double* dtl) {
+  __shared__ XVal h2[3], hsum, vs;  // vs: 4 max(4/3, gamma/Pr) mu (uniform: times the sum of 1 / h^2)
+  if (threadIdx.x < 3) h2[threadIdx.x] = xdec_pos<62>(0.5 * (threadIdx.x == 0 ? ph.ihx : (threadIdx.x == 1 ? ph.ihy : ph.ihz)));
+  if (threadIdx.x == 32) {
+    hsum = xdec_pos<62>(ph.ihx + ph.ihy + ph.ihz);
+    const double f = 4.0 * fmax(4.0 / 3.0, ph.gamma / ph.Pr) * ph.mu;
+    vs = xdec_pos<62>(CURVI ? f : f * (ph.ihx * ph.ihx + ph.ihy * ph.ihy + ph.ihz * ph.ihz));
+  }
+  __syncthreads();
+  long long best = 0;
+  bool bad = false;
+  const int rows = g.ny * g.nz, lane = threadIdx.x & 31;
+  for (int row = blockIdx.x * (RATE_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += gridDim.x * (RATE_THREADS / 32)) {
+    const int j = row % g.ny, k = row / g.ny;
+    for (int i = lane; i < g.nx; i += 32) {
+      const long long o = gidx(g, i, j, k);
+      const double Q[5] = {q[o], q[g.field + o], q[2 * g.field + o], q[3 * g.field + o], q[4 * g.field + o]};
+      XPrim W;
+      const bool phys = xprim(Q, K, W);
+      if (!phys) bad = true;
+      const XVal c = xsound(W, K.gam);
+      XVal rate;
+      if constexpr (!CURVI) {
+        rate = xrate<VISC>(W, c, h2, hsum, vs);
+      } else {
+        const XVal iv = xrcp(xdec_pos<62>(M[9 * g.field + o]));
+        XVal f = {0, 0};
+        if (VISC) f = {xmul(xmul(vs.m, W.ir.m) << 2, iv.m) << 2, vs.e + W.ir.e + iv.e + 2};
+        const long long up[3] = {1, g.px, g.plane};
+        XVal r[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          double lo[3], hi[3];
+#pragma unroll
+          for (int x = 0; x < 3; ++x) {
+            lo[x] = M[(3 * d + x) * g.field + o];
+            hi[x] = M[(3 * d + x) * g.field + o + up[d]];
+          }
+          r[d] = xradius<VISC>(W, c, lo, hi, f);
+        }
+        const XVal v = xsum3(r[0], r[1], r[2]);
+        rate = xnormed(xmul(v.m, iv.m), v.e + iv.e + 3);
+      }
+      if (dtl) {
+        const XVal ir = xrcp(rate);
+        dtl[o] = ph.cfl * xenc(ir.m, ir.e);
+      }
+      const long long rb = __double_as_longlong(xenc(rate.m, rate.e));
+      if (phys && rb > best) best = rb;
+    }
+  }
+  if (bad) atomicOr(&ctrl->flag, FLAG_NONPHYSICAL);
+  rate_fold(best, ctrl, partial, ph.cfl);
 }
 
 cudaError_t launch_init_rate(const Geometry& g, const Physics& ph, const double* q, DevCtrl* ctrl,
                              double* partial, int grid, int mixed, void* dtl, cudaStream_t s) {
   if (mixed)
-    init_rate_kernel<float><<<grid, 256, 0, s>>>(g, ph, q, ctrl, partial, static_cast<float*>(dtl));
+    init_rate_kernel<<<grid, RATE_THREADS, 0, s>>>(g, ph.viscous, rate_consts(ph), ph.cfl, q, ctrl, partial,
+                                                   static_cast<float*>(dtl));
+  else if (ph.viscous)
+    init_rate_x_kernel<true, false><<<grid, RATE_THREADS, 0, s>>>(g, ph, xconsts(ph.gamma, ph.eps), q, nullptr, ctrl,
+                                                                  partial, static_cast<double*>(dtl));
   else
-    init_rate_kernel<double><<<grid, 256, 0, s>>>(g, ph, q, ctrl, partial, static_cast<double*>(dtl));
+    init_rate_x_kernel<false, false><<<grid, RATE_THREADS, 0, s>>>(g, ph, xconsts(ph.gamma, ph.eps), q, nullptr, ctrl,
+                                                                   partial, static_cast<double*>(dtl));
   return cudaGetLastError();
 }
 
@@ -314,70 +404,59 @@ cudaError_t launch_metrics(const Geometry& g, const double* nodes, void* M, int 
 
 // spectral-radius rate on a curvilinear grid: sum over directions of |u.Sb| + c |Sb| (+ 4 max(4/3,
 // gamma/Pr) mu/rho |Sb|^2 / V), divided by V, with Sb the mean of a cell's two faces in a direction
-template <typename T>
-__global__ void init_rate_curvi_kernel(Geometry g, Physics ph, const double* __restrict__ q,
-                                       const T* __restrict__ M, DevCtrl* ctrl, double* partial, T* dtl) {
-  __shared__ double wmax[32];
-  __shared__ int last;
-  const long long n = (long long)g.nx * g.ny * g.nz;
-  const long long fm = sizeof(T) == 8 ? g.field : g.fieldf;
-  const double f = fmax(4.0 / 3.0, ph.gamma / ph.Pr);
-  double best = 0.0;
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(c % g.nx);
-    const long long r = c / g.nx;
-    const int j = (int)(r % g.ny), k = (int)(r / g.ny);
-    const long long o = gidx(g, i, j, k);
-    const long long om = sizeof(T) == 8 ? o : gidxf(g, i, j, k);
-    const long long up[3] = {1, sizeof(T) == 8 ? g.px : g.pxf, sizeof(T) == 8 ? g.plane : g.planef};
-    const T rho = T(q[o]), ir = T(1) / rho;
-    const T u = T(q[g.field + o]) * ir, v = T(q[2 * g.field + o]) * ir, w = T(q[3 * g.field + o]) * ir;
-    const T p = T(ph.gamma - 1.0) * (T(q[4 * g.field + o]) - T(0.5) * rho * (u * u + v * v + w * w));
-    const T a = sqrt(T(ph.gamma) * p * ir);
-    const T vol = M[9 * fm + om], iv = T(1) / vol;
-    T rate = T(0);
-    for (int d = 0; d < 3; ++d) {
-      T sb[3];
-      for (int x = 0; x < 3; ++x) sb[x] = T(0.5) * (M[(3 * d + x) * fm + om] + M[(3 * d + x) * fm + om + up[d]]);
-      const T s2 = sb[0] * sb[0] + sb[1] * sb[1] + sb[2] * sb[2];
-      T lam = fabs(u * sb[0] + v * sb[1] + w * sb[2]) + a * sqrt(s2);
-      if (ph.viscous) lam += T(4.0 * f * ph.mu) * ir * s2 * iv;
-      rate += lam;
+__global__ void __launch_bounds__(RATE_THREADS) init_rate_curvi_kernel(Geometry g, int viscous, RateConsts C, double cfl,
+                                                                        const double* __restrict__ q,
+                                                                        const float* __restrict__ M, DevCtrl* ctrl,
+                                                                        double* partial, float* dtl) {
+  const long long fm = g.fieldf;
+  float best = 0.f;
+  bool bad = false;
+  const int rows = g.ny * g.nz, lane = threadIdx.x & 31;
+  for (int row = blockIdx.x * (RATE_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += gridDim.x * (RATE_THREADS / 32)) {
+    const int j = row % g.ny, k = row / g.ny;
+    for (int i = lane; i < g.nx; i += 32) {
+      const long long o = gidx(g, i, j, k), om = gidxf(g, i, j, k);
+      const long long up[3] = {1, g.pxf, g.planef};
+      const float rho = float(q[o]), ir = 1.f / rho;
+      const float u = float(q[g.field + o]) * ir, v = float(q[2 * g.field + o]) * ir, w = float(q[3 * g.field + o]) * ir;
+      const float p = C.gm1 * (float(q[4 * g.field + o]) - 0.5f * rho * (u * u + v * v + w * w));
+      const float a = sqrtf(C.gam * p * ir);
+      const float vol = M[9 * fm + om], iv = 1.f / vol;
+      float rate = 0.f;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        float sb[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) sb[x] = 0.5f * (M[(3 * d + x) * fm + om] + M[(3 * d + x) * fm + om + up[d]]);
+        const float s2 = sb[0] * sb[0] + sb[1] * sb[1] + sb[2] * sb[2];
+        float lam = fabsf(u * sb[0] + v * sb[1] + w * sb[2]) + a * sqrtf(s2);
+        if (viscous) lam += C.fmu4 * ir * s2 * iv;
+        rate += lam;
+      }
+      rate *= iv;
+      if (dtl) dtl[om] = C.cfl / rate;
+      if (!(rho > 0.f && p > 0.f)) bad = true;
+      best = rate > best ? rate : best;
     }
-    rate *= iv;
-    if (dtl) dtl[om] = T(ph.cfl) / rate;
-    if (!(rho > T(0) && p > T(0))) atomicOr(&ctrl->flag, FLAG_NONPHYSICAL);
-    best = fmax(best, double(rate));
   }
-  for (int off = 16; off > 0; off >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, off));
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = best;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wmax[w]);
-    partial[(size_t)blockIdx.x * NPART + 5] = m;
-    __threadfence();
-    last = (atomicAdd(&ctrl->counter, 1u) == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  __threadfence();
-  double m = 0.0;
-  for (unsigned b = 0; b < gridDim.x; ++b) m = fmax(m, __ldcg(partial + (size_t)b * NPART + 5));
-  ctrl->rate = m;
-  ctrl->dt = ph.cfl / m;
-  ctrl->counter = 0u;
+  if (bad) atomicOr(&ctrl->flag, FLAG_NONPHYSICAL);
+  rate_fold(__double_as_longlong(double(best)), ctrl, partial, cfl);
 }
 
 cudaError_t launch_init_rate_curvi(const Geometry& g, const Physics& ph, const double* q, const void* M,
                                    DevCtrl* ctrl, double* partial, int grid, int mixed, void* dtl, cudaStream_t s) {
   if (mixed)
-    init_rate_curvi_kernel<float><<<grid, 256, 0, s>>>(g, ph, q, static_cast<const float*>(M), ctrl, partial,
-                                                       static_cast<float*>(dtl));
+    init_rate_curvi_kernel<<<grid, RATE_THREADS, 0, s>>>(g, ph.viscous, rate_consts(ph), ph.cfl, q,
+                                                         static_cast<const float*>(M), ctrl, partial,
+                                                         static_cast<float*>(dtl));
+  else if (ph.viscous)
+    init_rate_x_kernel<true, true><<<grid, RATE_THREADS, 0, s>>>(g, ph, xconsts(ph.gamma, ph.eps), q,
+                                                                 static_cast<const double*>(M), ctrl, partial,
+                                                                 static_cast<double*>(dtl));
   else
-    init_rate_curvi_kernel<double><<<grid, 256, 0, s>>>(g, ph, q, static_cast<const double*>(M), ctrl, partial,
-                                                        static_cast<double*>(dtl));
+    init_rate_x_kernel<false, true><<<grid, RATE_THREADS, 0, s>>>(g, ph, xconsts(ph.gamma, ph.eps), q,
+                                                                  static_cast<const double*>(M), ctrl, partial,
+                                                                  static_cast<double*>(dtl));
   return cudaGetLastError();
 }
 

@@ -308,33 +308,60 @@ template <typename T> __device__ __forceinline__ const PathK<T>& path_k(const Gr
 template <> __device__ __forceinline__ const PathK<float>& path_k<float>(const GroupParams& P) { return P.pk.f; }
 template <> __device__ __forceinline__ const PathK<double>& path_k<double>(const GroupParams& P) { return P.pk.d; }
 
-// The end of stages 1 and 3, called by all threads of every CTA: the CTA's sums of R^2 (nacc) and
-// largest rate go to its partial slot; the last CTA to finish (atomic counter) reduces, per block,
-// the slots of the CTAs that worked on it (in CTA order: deterministic), and for stage 3 takes the
-// group's time step from the largest rate.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// The end of stages 1 and 3, called by all threads of every CTA: the CTA's sums of R^2 (nacc, stage 1)
+// or largest rate (stage 3) go to its partial slot; the last CTA to finish (atomic counter)
+// reduces, per block, the slots of the CTAs that worked on it (a fixed order: deterministic), and
+// for stage 3 takes the group's time step from the largest rate.
+//
+// This is the tail of every such launch, and FP64 here is latency: a dependent FP64 operation takes
+// ~80 cycles and a warp's add holds the pipe for 76.  So the threads' sums are added by one warp per
+// variable from shared memory (NWARP adds and five shuffles, not 30 shuffled adds in every warp), the
+// slots by one warp per block and variable with its own root (not one lane's five divisions and
+// roots in a row), and maxima compare bit patterns on the integer pipe.  The tail it replaced took
+// 18 us of a launch (45 us per stage on a 32^3 block).  scratch: 5 x 32 NWARP doubles of shared memory.
 template <int STAGE, int NWARP>
-__device__ __forceinline__ void stage_reduce(const GroupParams& P, double* red, int* slast, const double (&nacc)[5],
-                                             double rate) {
+__device__ __forceinline__ void stage_reduce(const GroupParams& P, double* scratch, double* red, int* slast,
+                                             const double (&nacc)[5], double rate) {
   constexpr int NT = 32 * NWARP;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double part[6] = {nacc[0], nacc[1], nacc[2], nacc[3], nacc[4], rate};
+  long long* redb = reinterpret_cast<long long*>(red);
+  double* mine = P.partial + (size_t)blockIdx.x * NPART;
+  __syncthreads();  // everyone is done with the shared memory reused here
+  if constexpr (STAGE == 1) {
+    static_assert(NWARP >= 5, "a warp per variable");
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
+    for (int m = 0; m < 5; ++m) scratch[m * NT + tid] = nacc[m];
+    __syncthreads();
+    if (warp < 5) {
+      double s = 0.0;
 #pragma unroll
-    for (int m = 0; m < 5; ++m) part[m] += __shfl_xor_sync(0xffffffffu, part[m], off);
-    part[5] = fmax(part[5], __shfl_xor_sync(0xffffffffu, part[5], off));
+      for (int i = 0; i < NWARP; ++i) s += scratch[warp * NT + i * 32 + lane];
+      s = warp_sum(s);
+      if (lane == 0) {
+        mine[warp] = s;
+        __threadfence();
+      }
+    }
+  } else {
+    const long long b = warp_max_bits(__double_as_longlong(rate));
+    if (lane == 0) redb[warp] = b;
+    __syncthreads();
+    if (warp == 0) {
+      const long long m = warp_max_bits(lane < NWARP ? redb[lane] : 0ll);
+      if (lane == 0) {
+        mine[5] = __longlong_as_double(m);
+        __threadfence();
+      }
+    }
   }
   __syncthreads();
-  if (lane == 0)
-    for (int m = 0; m < 6; ++m) red[warp * NPART + m] = part[m];
-  __syncthreads();
   if (tid == 0) {
-    double sum[6] = {0, 0, 0, 0, 0, 0};
-    for (int w = 0; w < NWARP; ++w) {
-      for (int m = 0; m < 5; ++m) sum[m] += red[w * NPART + m];
-      sum[5] = fmax(sum[5], red[w * NPART + 5]);
-    }
-    for (int m = 0; m < 6; ++m) P.partial[(size_t)blockIdx.x * NPART + m] = sum[m];
     __threadfence();
     const unsigned prev = atomicAdd(&P.gctrl->counter, 1u);
     *slast = (prev == gridDim.x - 1);
@@ -342,46 +369,44 @@ __device__ __forceinline__ void stage_reduce(const GroupParams& P, double* red, 
   __syncthreads();
   if (!*slast) return;
   __threadfence();
-  // every warp of the last CTA folds blocks warp, warp + NWARP, ... (a group may hold many
-  // blocks: one warp walking all of them serially left the SMs idle behind it)
-  double wmax = 0.0;
-  for (int b = warp; b < P.nblocks; b += NWARP) {
-    const BlockDesc* Db = P.table + b;
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int c = lane; c < Db->ctas; c += 32) {
-      const double* src = P.partial + (size_t)(Db->cta0 + c) * NPART;
-      for (int m = 0; m < 5; ++m) s[m] += __ldcg(src + m);
-      s[5] = fmax(s[5], __ldcg(src + 5));
+  if constexpr (STAGE == 1) {
+    for (int it = warp; it < 5 * P.nblocks; it += NWARP) {  // a warp per block and variable
+      const BlockDesc* Db = P.table + it / 5;
+      const int m = it % 5;
+      const double* src = P.partial + (size_t)Db->cta0 * NPART + m;
+      double s = 0.0;
+#pragma unroll 4
+      for (int c = lane; c < Db->ctas; c += 32) s += __ldcg(src + (size_t)c * NPART);
+      s = warp_sum(s);
+      if (lane == 0) Db->ctrl->norms[m] = sqrt(s / ((double)Db->g.nx * Db->g.ny * Db->g.nz));
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-      for (int m = 0; m < 5; ++m) s[m] += __shfl_xor_sync(0xffffffffu, s[m], off);
-      s[5] = fmax(s[5], __shfl_xor_sync(0xffffffffu, s[5], off));
+  } else {
+    long long wmax = 0;
+    for (int b = warp; b < P.nblocks; b += NWARP) {
+      const BlockDesc* Db = P.table + b;
+      const double* src = P.partial + (size_t)Db->cta0 * NPART + 5;
+      long long s = 0;
+#pragma unroll 4
+      for (int c = lane; c < Db->ctas; c += 32) {
+        const long long v = __double_as_longlong(__ldcg(src + (size_t)c * NPART));
+        s = v > s ? v : s;
+      }
+      s = warp_max_bits(s);
+      if (lane == 0) Db->ctrl->rate = __longlong_as_double(s);
+      wmax = s > wmax ? s : wmax;
     }
-    wmax = fmax(wmax, s[5]);
-    if (lane == 0) {
-      const double n = (double)Db->g.nx * Db->g.ny * Db->g.nz;
-      if (STAGE == 1)
-        for (int m = 0; m < 5; ++m) Db->ctrl->norms[m] = sqrt(s[m] / n);
-      if (STAGE == 3) Db->ctrl->rate = s[5];
-    }
-  }
-  if constexpr (STAGE == 3) {
-    if (lane == 0) red[warp] = wmax;
+    if (lane == 0) redb[warp] = wmax;
     __syncthreads();
-    double gmax = 0.0;
-    for (int w = 0; w < NWARP; ++w) gmax = fmax(gmax, red[w]);
-    const double dtn = P.ph.cfl / gmax;
+    long long g = 0;
+    for (int w = 0; w < NWARP; ++w) g = redb[w] > g ? redb[w] : g;
+    const double gmax = __longlong_as_double(g), dtn = P.ph.cfl / gmax;
     for (int b = tid; b < P.nblocks; b += NT) P.table[b].ctrl->dt = dtn;
     if (tid == 0) {
       P.gctrl->rate = gmax;
       P.gctrl->dt = dtn;
     }
   }
-  if (tid == 0) {
-    P.gctrl->counter = 0u;
-  }
+  if (tid == 0) P.gctrl->counter = 0u;
 }
 
 // ---- the kernel ------------------------------------------------------------------------------
@@ -826,7 +851,7 @@ __global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) 
   }
   if (bad) atomicOr(&D->ctrl->flag, FLAG_NONPHYSICAL);
 
-  if constexpr (STAGE == 1 || STAGE == 3) stage_reduce<STAGE, NWARP>(P, red, slast, nacc, double(rate_max));
+  if constexpr (STAGE == 1 || STAGE == 3) stage_reduce<STAGE, NWARP>(P, reinterpret_cast<double*>(smem + PL::ring), red, slast, nacc, double(rate_max));
 }
 
 }  // namespace gbcfd

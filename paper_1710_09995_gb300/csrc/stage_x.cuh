@@ -475,65 +475,27 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
           }
           if constexpr (STAGE == 3) {
             XPrim W;
-            if (!xprim(out, XK, W)) bad = true;
+            const bool phys = xprim(out, XK, W);
+            if (!phys) bad = true;
             const XVal c = xsound(W, XK.gam);
             XVal rate;
             if constexpr (!CURVI) {
-              // (|u| + c) / hx + (|v| + c) / hy + (|w| + c) / hz, h2 = 1 / (2 h); viscous: + vs / rho
-              long long t[5];
-              int e[5];
-#pragma unroll
-              for (int a = 0; a < 3; ++a) {
-                t[a] = xmul(xabs(W.u[a].m), xb->h2[a].m);  // [60]
-                e[a] = W.u[a].e + xb->h2[a].e + 4;
-              }
-              t[3] = xmul(c.m, xb->hsum.m);
-              e[3] = c.e + xb->hsum.e + 3;
-              t[4] = VISC ? xmul(W.ir.m, xb->vs.m) : 0;
-              e[4] = VISC ? W.ir.e + xb->vs.e + 3 : e[3];
-              const int E = xmax(xmax(xmax(e[0], e[1]), xmax(e[2], e[3])), e[4]) + 1;
-              rate = xnormed(xshr(t[0], E - e[0]) + xshr(t[1], E - e[1]) + xshr(t[2], E - e[2]) + xshr(t[3], E - e[3]) +
-                                 xshr(t[4], E - e[4]), E);
-            } else {
-              // sum over directions of |u . S| + c |S| over V, S the mean of the cell's two faces
+              rate = xrate<VISC>(W, c, xb->h2, xb->hsum, xb->vs);
+            } else {  // sum over directions of |u . S| + c |S|, over V
               const double* mu[3] = {mc + 1, mc + BX, mring + mk1 * MSD + (row + HALO) * BX + lane + HALO};
-              long long t[3];
-              int e[3];
+              XVal r[3];
 #pragma unroll
               for (int a = 0; a < 3; ++a) {
-                long long sm[3];
-                int es[3];
-#pragma unroll
-                for (int x = 0; x < 3; ++x) {
-                  const XPair f = xpair(mc[(3 * a + x) * MS], mu[a][(3 * a + x) * MS]);
-                  sm[x] = (f.l >> 1) + (f.r >> 1);  // [62], the mean in the class itself
-                  es[x] = f.e;
-                }
-                const int E = xmax(es[0], xmax(es[1], es[2]));
-                long long dot[3], s2 = 0;
-                int ec[3];
-#pragma unroll
-                for (int x = 0; x < 3; ++x) {
-                  sm[x] = xshr(sm[x], E - es[x]);
-                  s2 += xsq(sm[x]);  // [60] each, class 2 E + 3
-                  dot[x] = xmul(sm[x], W.u[x].m);
-                  ec[x] = E + W.u[x].e + 3;
-                }
-                const XVal n2 = xnormed(s2, 2 * E + 3);
-                const XVal in = xrsqrt(n2);
-                const long long cs = xmul(xmul(n2.m, in.m) << 2, c.m);  // c |S| [60]
-                const int ecs = n2.e + in.e + 1 + c.e + 3;
-                e[a] = xmax(xmax(xmax(ec[0], ec[1]), ec[2]), ecs) + 2;
-                t[a] = xabs(xshr(dot[0], e[a] - ec[0]) + xshr(dot[1], e[a] - ec[1]) + xshr(dot[2], e[a] - ec[2])) +
-                       xshr(cs, e[a] - ecs);  // [60]
+                const double lo[3] = {mc[3 * a * MS], mc[(3 * a + 1) * MS], mc[(3 * a + 2) * MS]};
+                const double up[3] = {mu[a][3 * a * MS], mu[a][(3 * a + 1) * MS], mu[a][(3 * a + 2) * MS]};
+                r[a] = xradius<false>(W, c, lo, up, iv);
               }
-              const int E = xmax(e[0], xmax(e[1], e[2]));
-              const XVal v = xnormed(xshr(t[0], E - e[0]) + xshr(t[1], E - e[1]) + xshr(t[2], E - e[2]), E);
+              const XVal v = xsum3(r[0], r[1], r[2]);
               rate = xnormed(xmul(v.m, iv.m), v.e + iv.e + 3);
             }
             // the largest rate, as the bits of a non-negative double
             const long long rb = __double_as_longlong(xenc(rate.m, rate.e));
-            if (rb > __double_as_longlong(rate_max)) rate_max = __longlong_as_double(rb);
+            if (phys && rb > __double_as_longlong(rate_max)) rate_max = __longlong_as_double(rb);
             if constexpr (!VISC)
               if (ph.local_dt) {
                 const XVal ir = xrcp(rate);
@@ -558,7 +520,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
   }
   if (bad) atomicOr(&D->ctrl->flag, FLAG_NONPHYSICAL);
 
-  if constexpr (STAGE == 1 || STAGE == 3) stage_reduce<STAGE, NW>(P, red, slast, nacc, rate_max);
+  if constexpr (STAGE == 1 || STAGE == 3) stage_reduce<STAGE, NW>(P, reinterpret_cast<double*>(smem + PL::ringm), red, slast, nacc, rate_max);
 }
 
 // ---- launch helpers --------------------------------------------------------------------------

@@ -487,6 +487,70 @@ __host__ __device__ __forceinline__ XVal xsound(const XPrim& W, const XVal& gam)
   return {xmul(c2.m, ic.m) << 2, c2.e + ic.e + 1};
 }
 
+// the spectral-radius rate of a cell, normalised: uniform grids, (|u| + c) / hx + (|v| + c) / hy +
+// (|w| + c) / hz (+ vs / rho, viscous), from h2 = 1 / (2 h), hsum = the sum of 1 / h
+template <bool VISC>
+__host__ __device__ __forceinline__ XVal xrate(const XPrim& W, const XVal& c, const XVal* h2, const XVal& hsum,
+                                               const XVal& vs) {
+  long long t[5];
+  int e[5];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int a = 0; a < 3; ++a) {
+    t[a] = xmul(xabs(W.u[a].m), h2[a].m);  // [60]
+    e[a] = W.u[a].e + h2[a].e + 4;
+  }
+  t[3] = xmul(c.m, hsum.m);
+  e[3] = c.e + hsum.e + 3;
+  t[4] = VISC ? xmul(W.ir.m, vs.m) : 0;
+  e[4] = VISC ? W.ir.e + vs.e + 3 : e[3];
+  const int E = xmax(xmax(xmax(e[0], e[1]), xmax(e[2], e[3])), e[4]) + 1;
+  return xnormed(xshr(t[0], E - e[0]) + xshr(t[1], E - e[1]) + xshr(t[2], E - e[2]) + xshr(t[3], E - e[3]) +
+                     xshr(t[4], E - e[4]), E);
+}
+// curvilinear grids: one direction's part, |u . S| + c |S| (+ f |S|^2, viscous: f = 4 max(4/3, gamma/Pr)
+// mu / (rho V)), S the mean of the cell's lower and upper face vectors; [61] or less
+template <bool VISC>
+__host__ __device__ __forceinline__ XVal xradius(const XPrim& W, const XVal& c, const double* lo, const double* up,
+                                                 const XVal& f) {
+  long long s[3];
+  int es[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int x = 0; x < 3; ++x) {
+    const XPair p = xpair(lo[x], up[x]);
+    s[x] = (p.l >> 1) + (p.r >> 1);  // [62], the mean in the class itself
+    es[x] = p.e;
+  }
+  const int E = xmax(es[0], xmax(es[1], es[2]));
+  long long dot[3], s2 = 0;
+  int ec[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int x = 0; x < 3; ++x) {
+    s[x] = xshr(s[x], E - es[x]);
+    s2 += xsq(s[x]);  // [60] each, class 2 E + 3
+    dot[x] = xmul(s[x], W.u[x].m);
+    ec[x] = E + W.u[x].e + 3;
+  }
+  const XVal n2 = xnormed(s2, 2 * E + 3);
+  const XVal in = xrsqrt(n2);
+  const long long cs = xmul(xmul(n2.m, in.m) << 2, c.m);  // c |S| [60]
+  const int ecs = n2.e + in.e + 1 + c.e + 3;
+  const long long fs = VISC ? xmul(f.m, n2.m) : 0;
+  const int efs = VISC ? f.e + n2.e + 3 : ecs;
+  const int e = xmax(xmax(xmax(ec[0], ec[1]), xmax(ec[2], ecs)), efs) + 2;
+  return {xabs(xshr(dot[0], e - ec[0]) + xshr(dot[1], e - ec[1]) + xshr(dot[2], e - ec[2])) + xshr(cs, e - ecs) +
+              xshr(fs, e - efs), e};
+}
+__host__ __device__ __forceinline__ XVal xsum3(const XVal& a, const XVal& b, const XVal& c) {  // [60] each
+  const int E = xmax(a.e, xmax(b.e, c.e)) + 1;
+  return xnormed(xshr(a.m, E - a.e) + xshr(b.m, E - b.e) + xshr(c.m, E - c.e), E);
+}
+
 // ---- WCNS-E-5 lines ----------------------------------------------------------------------------
 #ifdef __CUDACC__
 #define XNOINLINE __noinline__  // called per variable: inlined five times it was half the kernel's code
