@@ -100,8 +100,8 @@ struct Plan {
   static constexpr size_t ring = std_ + NSTAGE * DSLOT;
   static constexpr size_t fx = ring + sizeof(T) * NRING * RSLOT;
   static constexpr size_t fy = fx + sizeof(T) * 5 * TY * (TX + 1);
-  // curvilinear: a ring of metric planes (10 fields, k and k+1 in use, the next one landing)
-  static constexpr int NMS = CURVI ? (sizeof(T) == 4 ? 3 : 2) : 0;
+  // curvilinear (FP64 viscous blocks only): a ring of metric planes (10 fields, k and k+1)
+  static constexpr int NMS = CURVI ? 2 : 0;
   static constexpr size_t MSLOT = (sizeof(T) * 10 * BOX + 127) / 128 * 128;
   static constexpr size_t mring = (fy + sizeof(T) * 5 * (TY + 1) * TX + 127) / 128 * 128;
   static constexpr size_t red = (mring + NMS * MSLOT + 15) / 16 * 16;
@@ -414,14 +414,14 @@ __device__ __forceinline__ void stage_reduce(const GroupParams& P, double* scrat
 // one).  STAGE 0: residual only (one block, R to P.rout); 1..3: the stages of Eqs. 4-6.
 // registers: the register file is split over the SM's four sub-partitions (16K each) and warps
 // are spread round-robin, so two 9-warp CTAs (5 warps on one sub-partition) allow 96 registers
-// per thread on the mixed path, four 5-warp CTAs (TYV = 4) 102, one CTA of 9 or 12 warps (3 per
-// sub-partition) 168 on the FP64 and curvilinear paths
+// per thread on the mixed path, four 5-warp CTAs (TYV = 4) 102, one CTA of 9 warps 168 on the FP64 path
 // PUSH: stages 1 and 2 of a group with the halo exchange folded in (GroupParams::push); a separate
 // instantiation, so kernels without it carry none of its code
 template <typename T, bool VISC, int STAGE, bool CURVI, int TYV, bool PUSH = false>
-__global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) ? (TYV <= 4 ? 4 : 2) : 1)
+__global__ void __launch_bounds__(tile_threads(TYV), sizeof(T) == 4 ? (TYV <= 4 ? 4 : 2) : 1)
     stage_kernel(const GroupParams P) {
   constexpr bool MIXED = sizeof(T) == 4;
+  static_assert(MIXED ? !CURVI : CURVI && VISC, "FP64 Cartesian and inviscid blocks: stage_x.cuh; mixed curvilinear: stage_c.cuh");
   constexpr bool LOADD = MIXED && (STAGE == 2 || STAGE == 3);
   using PL = Plan<T, VISC, CURVI, TYV>;
   constexpr int TY = TYV, BY = PL::BY, NWARP = PL::NWARP, NT = tile_threads(TYV);
@@ -753,26 +753,16 @@ __global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) 
             else out[m] = fma(2.0 / 3.0, adv, (1.0 / 3.0) * qn_[m]);  // an FP64 division costs ~7 FMAs here
             qout[m * g.field + o] = out[m];
           }
-          if constexpr (PUSH && (STAGE == 1 || STAGE == 2))
-            if (ci < HALO || cj < HALO || k < HALO || ci >= g.nx - HALO || cj >= g.ny - HALO || k >= g.nz - HALO)
-              push_halo<double>(pushdst, g.nx, g.ny, g.nz, ci, cj, k, out[0], out[1], out[2], out[3], out[4]);
           if constexpr (STAGE == 3) {
             const double ir = VM<double>::rcp(out[0]);
             const double uu = out[1] * ir, vv = out[2] * ir, ww = out[3] * ir;
             const double pp = double(gm1) * (out[4] - 0.5 * out[0] * (uu * uu + vv * vv + ww * ww));
             if (!(out[0] > 0.0 && pp > 0.0)) bad = true;
-            double rate;
-            if constexpr (CURVI) {
-              T sb[9];
-              cell_face_means<T, BY>(mring, mk, mk1, ocy, ocx, sb);
-              rate = cell_rate_curvi<double>(out[0], uu, vv, ww, pp, sb, mring[mb<BY>(mk, ocy, ocx) + 9 * MS], RK,
-                                             ph.viscous);
-            } else {
-              rate = cell_rate<double>(out[0], uu, vv, ww, pp, RK, ph.viscous, hx, hy, hz, hs2);
-            }
+            T sb[9];
+            cell_face_means<T, BY>(mring, mk, mk1, ocy, ocx, sb);
+            const double rate = cell_rate_curvi<double>(out[0], uu, vv, ww, pp, sb, mring[mb<BY>(mk, ocy, ocx) + 9 * MS],
+                                                        RK, ph.viscous);
             rate_max = fmax(rate_max, T(rate));
-            if constexpr (!VISC)
-              if (ph.local_dt) static_cast<double*>(D->dtl)[o] = ph.cfl * VM<double>::rcp(rate);
           }
         } else {
           float inc[5];
@@ -804,15 +794,7 @@ __global__ void __launch_bounds__(tile_threads(TYV), (sizeof(T) == 4 && !CURVI) 
             const float uu = qf[1] * ir, vv = qf[2] * ir, ww = qf[3] * ir;
             const float pp = gm1 * (qf[4] - 0.5f * qf[0] * (uu * uu + vv * vv + ww * ww));
             if (!(qf[0] > 0.0f && pp > 0.0f)) bad = true;
-            float rate;
-            if constexpr (CURVI) {
-              T sb[9];
-              cell_face_means<T, BY>(mring, mk, mk1, ocy, ocx, sb);
-              rate = cell_rate_curvi<float>(qf[0], uu, vv, ww, pp, sb, mring[mb<BY>(mk, ocy, ocx) + 9 * MS], RK,
-                                            ph.viscous);
-            } else {
-              rate = cell_rate<float>(qf[0], uu, vv, ww, pp, RK, ph.viscous, hx, hy, hz, hs2);
-            }
+            const float rate = cell_rate<float>(qf[0], uu, vv, ww, pp, RK, ph.viscous, hx, hy, hz, hs2);
             rate_max = fmax(rate_max, T(rate));
             if constexpr (!VISC)
               if (ph.local_dt) static_cast<float*>(D->dtl)[of] = cflT / rate;

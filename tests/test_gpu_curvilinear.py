@@ -66,6 +66,25 @@ def test_steps_warped_mixed(gb):
     assert err[0] <= 1e-6 and max(err) <= 1e-5, err
 
 
+@pytest.mark.parametrize("viscous", [False, True])
+@pytest.mark.parametrize("n", [(32, 8, 4), (33, 9, 5), (31, 7, 9), (95, 25, 6)])
+def test_mixed_tile_edges(gb, n, viscous):
+    """A full tile, one cell over and one short in each direction, and several ragged tiles: residual,
+    state, residual norm and time step.  FP32 faces differ from the oracle's by some 1e-6 of the terms
+    that cancel in a residual (1e-4 of it, as in test_residual_warped); three steps leave dt times
+    that in the state, and a rate has about 20 FP32 roundings."""
+    c = warped_case(*n, viscous, seed=11)
+    M = oracle.metrics(c.nodes)
+    blk = gb.block_for_case(c, precision=gb.MIXED)
+    R = blk.compute_residual().cpu().numpy()
+    assert max(per_var(R, oracle.residual(oparams(c), oracle.pad(c.state), M))) <= 1e-4
+    ref, dts, norms = oracle.step(oparams(c), oracle.pad(c.state), M, 3)
+    gb.step([blk], 3)
+    assert max(per_var(blk.get_state().cpu().numpy(), oracle.interior(ref))) <= 1e-5
+    assert np.allclose(blk.residual_norm(), norms[-1], rtol=1e-4, atol=1e-7 * np.max(norms[-1]))
+    assert abs(blk.get_dt() - oracle.dt(oparams(c), ref, M)) <= 1e-5 * dts[0]
+
+
 @pytest.mark.parametrize("precision", [0, 1])
 def test_freestream_preserved_warped(gb, precision):
     c = warped_case(36, 17, 10, True, amp=0.0)
