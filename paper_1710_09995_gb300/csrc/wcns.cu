@@ -15,7 +15,7 @@
 //                interior cells in one pass: tiles marching in z form the gradient tensor (D4 of
 //                u, v, w, theta) once per cell of the tile's union box from a TMA-fed ring of
 //                planes, keep the three viscous-flux families of Eq. 1 in shared rings and write
-//                only Rv.
+//                only Rv (FP64: xviscres_kernel, wcns_x.cuh).
 //   dir_kernel<D> for D = x, y, z: a tile of 16 lines x L cells along D.  The tile's primitives
 //                (L + 10 cells per line) land in shared memory by cp.async one tile ahead; a lane
 //                per cell evaluates both edge values of its cell (the two share the stencils'
@@ -185,6 +185,15 @@ __device__ __forceinline__ void prim_body(const Args& a, int with_rate, const WT
   const T ih0 = C.ih[0], ih1 = C.ih[1], ih2 = C.ih[2], ihs = C.ihs;
   T best = T(0);
   bool bad = false;
+  __shared__ XVal h2[3], hsum, vs;  // FP64: 1 / (2 h), the sum of 1 / h, the viscous rate's factor of 1 / rho
+  if constexpr (sizeof(T) == 8) {
+    if (threadIdx.x < 3) h2[threadIdx.x] = xdec_pos<62>(0.5 * C.ih[threadIdx.x]);
+    if (threadIdx.x == 32) {
+      hsum = xdec_pos<62>(ih0 + ih1 + ih2);
+      vs = xdec_pos<62>(vf * ihs);
+    }
+    __syncthreads();
+  }
   for (int row = blockIdx.x; row < wy * wz; row += gridDim.x) {  // rows (j, k) of the padded box
     const int jj = row % wy, kk = row / wy;
     const int j = jj - H, k = kk - H;
@@ -217,6 +226,25 @@ __device__ __forceinline__ void prim_body(const Args& a, int with_rate, const WT
       } else {
         si = wrap(i, b.nx);
         load_conserved<T>(a, ((long long)sk * b.ny + sj) * b.nx + si, U);
+      }
+      if constexpr (sizeof(T) == 8) {
+        // on the integer pipes (the FP64 form held the FP64 pipe 82% of the time: 117 us at 96^3, now 70); a state
+        // that has no positive density and pressure goes on to the plain form
+        XPrim P;
+        if (xprim(U, C.x, P)) {
+          dst[ii] = U[0];
+#pragma unroll
+          for (int x = 0; x < 3; ++x) dst[(1 + x) * b.field + ii] = xenc(P.u[x].m, P.u[x].e);
+          dst[4 * b.field + ii] = xenc(P.p.m, P.p.e);
+          dst[5 * b.field + ii] = xenc(xmul(P.p.m, P.ir.m), P.p.e + P.ir.e + 3);
+          if (with_rate && inner_row && i == si) {
+            const XVal c = xsound(P, C.x.gam);
+            const XVal rate = a.viscous ? xrate<true>(P, c, h2, hsum, vs) : xrate<false>(P, c, h2, hsum, vs);
+            const long long r = __double_as_longlong(xenc(rate.m, rate.e)), o = __double_as_longlong(best);
+            best = __longlong_as_double(r > o ? r : o);
+          }
+          continue;
+        }
       }
       const T rho = U[0], ir = T(1) / rho;
       const T u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
@@ -320,7 +348,6 @@ constexpr int RX = 32, RY = 8;                 // tile
 constexpr int GX = RX + 4, GY = RY + 4;        // union box of gradient cells (36 x 12)
 constexpr int WX = 44, WY = RY + 8;            // primitive box (44 x 16): cells x0-5 .., y0-4 ..
 constexpr int WRING = 6, ZRING = 5;            // 5 planes in use + 1 landing; z-fluxes k-2 .. k+2
-template <typename T>
 struct RSmem {
   static constexpr int WF = WY * WX;                 // one field's plane box
   static constexpr int WP = 4 * WF;                  // u, v, w, theta
@@ -328,10 +355,10 @@ struct RSmem {
   static constexpr int GYP = 4 * GY * RX;            // y-fluxes: 4 x 12 rows x 32
   static constexpr int HZP = 4 * RY * RX;            // z-fluxes: 4 x 8 x 32
   static constexpr size_t w = 0;
-  static constexpr size_t fx = w + sizeof(T) * WRING * WP;
-  static constexpr size_t gy = fx + sizeof(T) * FXP;
-  static constexpr size_t hz = gy + sizeof(T) * GYP;
-  static constexpr size_t bar = (hz + sizeof(T) * ZRING * HZP + 15) / 16 * 16;
+  static constexpr size_t fx = w + sizeof(float) * WRING * WP;
+  static constexpr size_t gy = fx + sizeof(float) * FXP;
+  static constexpr size_t hz = gy + sizeof(float) * GYP;
+  static constexpr size_t bar = (hz + sizeof(float) * ZRING * HZP + 15) / 16 * 16;
   static constexpr size_t bytes = bar + 8 * WRING + 16;
 };
 
@@ -342,14 +369,14 @@ __device__ __forceinline__ void tma_abort(uint64_t* bar, unsigned pending, unsig
   atomicOr(&ctrl->flag, FLAG_TIMEOUT);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(NTW) viscres_kernel(const __grid_constant__ Args a) {
+  using T = float;  // (FP64: xviscres_kernel, wcns_x.cuh)
   extern __shared__ __align__(128) unsigned char rsm[];
-  T* wr = reinterpret_cast<T*>(rsm + RSmem<T>::w);
-  T* fxr = reinterpret_cast<T*>(rsm + RSmem<T>::fx);
-  T* gyr = reinterpret_cast<T*>(rsm + RSmem<T>::gy);
-  T* hzr = reinterpret_cast<T*>(rsm + RSmem<T>::hz);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(rsm + RSmem<T>::bar);
+  T* wr = reinterpret_cast<T*>(rsm + RSmem::w);
+  T* fxr = reinterpret_cast<T*>(rsm + RSmem::fx);
+  T* gyr = reinterpret_cast<T*>(rsm + RSmem::gy);
+  T* hzr = reinterpret_cast<T*>(rsm + RSmem::hz);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(rsm + RSmem::bar);
   int* sabort = reinterpret_cast<int*>(bar + WRING);
   const Box& b = a.b;
   T* Rv = static_cast<T*>(a.Rv);
@@ -379,12 +406,12 @@ __global__ void __launch_bounds__(NTW) viscres_kernel(const __grid_constant__ Ar
     const int tx = (int)(tile % ntx), x0 = tx * RX, y0 = (int)(tile / ntx) * RY;
     auto issue = [&](int kp) {  // thread 0: u, v, w, theta of plane kp (fields 1, 2, 3, 5)
       const int q = ws(kp);
-      T* dst = wr + q * RSmem<T>::WP;
+      T* dst = wr + q * RSmem::WP;
       fence_proxy_async();
-      mbar_expect_tx(&bar[q], (unsigned)(sizeof(T) * RSmem<T>::WP));
+      mbar_expect_tx(&bar[q], (unsigned)(sizeof(T) * RSmem::WP));
       const int fld[4] = {1, 2, 3, 5};
       for (int f = 0; f < 4; ++f)  // storage column x0 is cell x0 - 5; storage row y0 + 1 is cell y0 - 4
-        tma_load_4d(dst + f * RSmem<T>::WF, &a.mwv, &bar[q], x0, y0 + 1, kp + H, fld[f]);
+        tma_load_4d(dst + f * RSmem::WF, &a.mwv, &bar[q], x0, y0 + 1, kp + H, fld[f]);
       pending |= 1u << q;
     };
     auto wait = [&](int kp) {  // all threads; a copy that never landed stays pending
@@ -408,8 +435,8 @@ __global__ void __launch_bounds__(NTW) viscres_kernel(const __grid_constant__ Ar
       if (*sabort) break;
       const T* pl[5];
 #pragma unroll
-      for (int m = 0; m < 5; ++m) pl[m] = wr + ws(p - 2 + m) * RSmem<T>::WP;
-      T* hzp = hzr + zs(p) * RSmem<T>::HZP;
+      for (int m = 0; m < 5; ++m) pl[m] = wr + ws(p - 2 + m) * RSmem::WP;
+      T* hzp = hzr + zs(p) * RSmem::HZP;
       // the union box: a warp per 32-cell row (rows 0..7, then 8..11), and warps 4, 5 of the second
       // pass take the 4 extra columns of all 12 rows (a row stride of 44 spreads them over distinct
       // banks); walking the 36-wide box row-major would split warps over two rows and conflict
@@ -431,11 +458,11 @@ __global__ void __launch_bounds__(NTW) viscres_kernel(const __grid_constant__ Ar
         T gr[4][3], vel[3];
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
-          const T* p0 = pl[2] + f * RSmem<T>::WF;
+          const T* p0 = pl[2] + f * RSmem::WF;
           if (f < 3) vel[f] = p0[c];
           gr[f][0] = ((p0[c - 2] - p0[c + 2]) + T(8) * (p0[c + 1] - p0[c - 1])) * ih0;
           gr[f][1] = ((p0[c - 2 * WX] - p0[c + 2 * WX]) + T(8) * (p0[c + WX] - p0[c - WX])) * ih1;
-          const int o = f * RSmem<T>::WF + c;
+          const int o = f * RSmem::WF + c;
           gr[f][2] = ((pl[0][o] - pl[4][o]) + T(8) * (pl[3][o] - pl[1][o])) * ih2;
         }
         const T div = gr[0][0] + gr[1][1] + gr[2][2];
@@ -477,8 +504,8 @@ __global__ void __launch_bounds__(NTW) viscres_kernel(const __grid_constant__ Ar
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int o = (q * RY + warp) * RX + lane;
-          const T dz = (hzr[zs(k - 2) * RSmem<T>::HZP + o] - hzr[zs(k + 2) * RSmem<T>::HZP + o]) +
-                       T(8) * (hzr[zs(k + 1) * RSmem<T>::HZP + o] - hzr[zs(k - 1) * RSmem<T>::HZP + o]);
+          const T dz = (hzr[zs(k - 2) * RSmem::HZP + o] - hzr[zs(k + 2) * RSmem::HZP + o]) +
+                       T(8) * (hzr[zs(k + 1) * RSmem::HZP + o] - hzr[zs(k - 1) * RSmem::HZP + o]);
           Rv[q * a.n + cc] = -(rv2[q] + dz * ih2);
         }
       }
@@ -853,15 +880,15 @@ static cudaError_t set_smem() {
     GB_SET((dir_kernel<0, 0>), Smem::bytes) GB_SET((dir_kernel<1, 1>), Smem::bytes) GB_SET((dir_kernel<2, 2>), Smem::bytes)
   }
 #undef GB_SET
-  e = cudaFuncSetAttribute(viscres_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RSmem<T>::bytes);
-  if (e != cudaSuccess) return e;
-  return cudaSuccess;
+  if constexpr (sizeof(T) == 8)
+    return cudaFuncSetAttribute(xviscres_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XRSmem::bytes);
+  else
+    return cudaFuncSetAttribute(viscres_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RSmem::bytes);
 }
 
-template <typename T>
 static int viscres_occupancy() {
   int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, viscres_kernel<T>, NTW, RSmem<T>::bytes);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, viscres_kernel, NTW, RSmem::bytes);
   return std::max(1, occ);
 }
 
@@ -1039,7 +1066,10 @@ cudaError_t launch_rest(gbcfd_wcns w, const Args& a, const cudaEvent_t* ev, cuda
   auto mark = [&](int m) {
     if (ev) cudaEventRecord(ev[m], s);
   };
-  if (a.viscous) viscres_kernel<T><<<w->nsm * w->rocc, NTW, RSmem<T>::bytes, s>>>(a);
+  if (a.viscous) {
+    if constexpr (sizeof(T) == 8) xviscres_kernel<<<w->nsm, XVT, XRSmem::bytes, s>>>(a);
+    else viscres_kernel<<<w->nsm * w->rocc, NTW, RSmem::bytes, s>>>(a);
+  }
   mark(2);
   const int g = w->dir_grid;
   if constexpr (sizeof(T) == 8) {
@@ -1256,7 +1286,7 @@ extern "C" int gbcfd_wcns_create(int nx, int ny, int nz, const gbcfd_params* par
     }
   }
   w->occ = mixed ? dir_occupancy<float>() : dir_occupancy<double>();
-  w->rocc = mixed ? viscres_occupancy<float>() : viscres_occupancy<double>();
+  w->rocc = mixed ? viscres_occupancy() : 1;
   w->dir_grid = std::min(w->rows, nsm * w->occ);
   e = cudaMemset(w->ctrl, 0, sizeof(DevCtrl));
   if (e != cudaSuccess) {

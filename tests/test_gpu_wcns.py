@@ -64,6 +64,27 @@ def test_residual_fp64_small_and_ragged(gb, shape):
     assert np.abs(R - ref).max() <= 1e-12 * max(np.abs(ref).max(), 1.0)
 
 
+@pytest.mark.parametrize("stretch", [(1, 1, 1), (1, 64, 1 / 64), (1e-3, 1, 1)])
+@pytest.mark.parametrize("shape", [(32, 8, 6), (33, 9, 5), (31, 7, 7)])
+def test_viscous_residual_stretched(gb, stretch, shape):
+    """The viscous part alone (residuals with and without viscosity) at the edges of its tiles and on
+    stretched meshes, where gradients of different directions meet in one stress: both sides round each
+    edge flux and each stress some 50 times at 1.1e-16 of it, the difference cancels nothing but the
+    inviscid part, and mu makes the two parts alike in size."""
+    c = ragged(True, seed=13, nx=shape[0], ny=shape[1], nz=shape[2], amp=0.1)
+    c.spacing = tuple(h * f for h, f in zip(c.spacing, stretch))
+    c.mu = 1e-2 * min(c.spacing)
+    p = oparams(c)
+    blk = gb.wcns_block_for_case(c, precision=gb.FP64)
+    R = blk.compute_residual().cpu().numpy()
+    ref = oracle.wcns_residual(p, c.state, c.spacing)
+    c.viscous = False
+    inv = oracle.wcns_residual(oparams(c), c.state, c.spacing)
+    visc = np.linalg.norm((ref - inv)[1:].ravel())
+    assert visc > 0
+    assert np.linalg.norm((R - ref).ravel()) <= 1e-13 * (visc + np.linalg.norm(inv.ravel()))
+
+
 @pytest.mark.parametrize("viscous", [False, True])
 def test_residual_mixed(gb, viscous):
     """FP32 edge states and fluxes: the differences of Eq. 2 carry ~1e-7 |F| / h of rounding."""
