@@ -8,7 +8,7 @@
 // and an exponent each; the faces (MUSCL, Roe, viscous flux), the residual and the time step's rate
 // run on the integer pipes.  FP64 is left with the stage update itself and the norm (5 to 15
 // operations a cell; with the conversion, the assembly and the rate in FP64 too its pipe was
-// 26% busy, alone between two barriers: 25.7 ms a step on the 256^3 case against 21.2).
+// 26% busy, alone between two barriers: 25.7 ms a step on the 256^3 case against 21.2 then).
 //
 // Faces are work items of a warp: the tile's z-, y- and x-rows (32 faces each) and one item of the
 // TY faces on the tile's upper x side, 3 TY + 2 items per plane dealt round-robin to the warps.  The
@@ -16,9 +16,13 @@
 // are data): a face is about 2000 instructions, and a copy per direction (six call sites in the
 // first version) streamed the code through the instruction caches on every plane.  16 warps of 128
 // registers: 26 items (TY 8) give the sub-partitions 7, 7, 6, 6; with 13 warps of one item each
-// round one of them had 8.  Measured against the FP64-pipe form: 256^3 Navier-Stokes step 81.7 ->
-// 21.2 ms, 36 uneven Euler blocks (14.4M cells) 69.0 -> 22.1 ms, two steps of the bump channel
-// 14.2 -> 4.2 ms, errors against 64-bit references the same or smaller.
+// round one of them had 8.  On Cartesian blocks at TY 8 the flux buffers of two planes fit (PIPE): the warps
+// that have one face item update the rows of the plane before in the same turn, where 8 warps updated
+// between two barriers while 8 waited (36 uneven Euler blocks 19.6 -> 18.4 ms, 256^3 Navier-Stokes 20.4 -> 19.6).
+// Bound by the integer pipes: ALU 60% busy, issue slots 58-61%, the rest multiply-add latency at 4 warps a
+// scheduler.  Measured against the FP64-pipe form: 256^3 Navier-Stokes step 81.7 -> 19.6 ms, 36 uneven Euler
+// blocks (14.4M cells) 69.0 -> 18.4 ms, two steps of the bump channel 14.2 -> 3.9 ms, errors against 64-bit
+// references the same or smaller.
 #pragma once
 #include "stage.cuh"
 
@@ -30,23 +34,28 @@ struct XPlan {
   static constexpr int TY = TYV, BY = box_rows(TYV), NW = NWV;
   static constexpr int NV = VISC ? 6 : 5;  // rho u v w p [theta]
   static constexpr int BOX = BY * BX;
-  static constexpr int NST = CURVI ? 1 : NSTAGE, NMS = CURVI ? 2 : 0;  // staging slots, metric planes
+  // PIPE: the update of a plane runs beside the faces of the next one (more flux buffers); where they fit
+  static constexpr bool PIPE = !CURVI && TYV == TY_DEFAULT;
+  static constexpr int NST = CURVI || (PIPE && VISC) ? 1 : NSTAGE, NMS = CURVI ? 2 : 0;  // staging slots, metric planes
   static constexpr size_t QSLOT = (sizeof(double) * 5 * BOX + 127) / 128 * 128;
   static constexpr size_t stq = 0;                                          // staged conserved planes
   static constexpr size_t ringm = stq + NST * QSLOT;                     // primitives: 61-bit integers
   static constexpr size_t ringe = ringm + sizeof(long long) * NRING * NV * BOX;  // and their exponents (biased)
-  // face fluxes, 62-bit integers and exponents: x, y, and two planes of z
+  // face fluxes, 62-bit integers and exponents: one or two planes of x and y, two or three of z
   static constexpr int NFX = 5 * TY * (TX + 1), NFY = 5 * (TY + 1) * TX, NFZ = 5 * TY * TX;
+  static constexpr int NBX = PIPE ? 2 : 1, NBZ = PIPE ? 3 : 2;
+  static constexpr int FY0 = NBX * NFX, FZ0 = FY0 + NBX * NFY, NF = FZ0 + NBZ * NFZ;
   static constexpr size_t fm = (ringe + sizeof(short) * NRING * NV * BOX + 15) / 16 * 16;
-  static constexpr size_t fe = fm + sizeof(long long) * (NFX + NFY + 2 * NFZ);
+  static constexpr size_t fe = fm + sizeof(long long) * NF;
   static constexpr size_t MSLOT = (sizeof(double) * 10 * BOX + 127) / 128 * 128;
-  static constexpr size_t mring = (fe + sizeof(short) * (NFX + NFY + 2 * NFZ) + 127) / 128 * 128;
+  static constexpr size_t mring = (fe + sizeof(short) * NF + 127) / 128 * 128;
   static constexpr size_t red = mring + NMS * MSLOT;
   static constexpr size_t blk = red + sizeof(double) * NW * NPART;          // the block's coefficients (XBlk)
   static constexpr size_t bar = blk + 20 * sizeof(XVal);
   static constexpr size_t misc = bar + 8 * (NST + NMS);
   static constexpr size_t push = (misc + 16 + 15) / 16 * 16;
   static constexpr size_t bytes = (push + 27 * sizeof(PushDst) + 127) / 128 * 128;
+  static_assert(bytes <= 232448, "227 KB of shared memory per CTA");
 };
 
 // a block's coefficients: half the inverse cell sizes (of the doubled face fluxes); the viscous
@@ -182,6 +191,9 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
   constexpr int NST = PL::NST, NMS = PL::NMS;
   constexpr int TY = TYV, BY = PL::BY, NW = NWV, NT = 32 * NWV, NV = PL::NV, MS = BY * BX, SL = NV * MS;
   constexpr int NITEM = 3 * TY + 2;
+  constexpr bool PIPE = PL::PIPE;
+  constexpr int W1 = PIPE ? NITEM - NW : 0, WU = NW - W1;  // PIPE: warps W1 .. have one item, and update
+  static_assert(!PIPE || (W1 > 0 && WU > 0), "two items a warp at most");
 
   extern __shared__ __align__(128) unsigned char smem[];
   long long* rm = reinterpret_cast<long long*>(smem + PL::ringm);
@@ -348,14 +360,122 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
     for (int kp = k0 - 2; kp <= k0 && ok; ++kp) ok = consume(kp);
     if (!ok) break;
 
-    double fzl[5] = {0, 0, 0, 0, 0};  // the lower z-face of the thread's cell
-    // plane k0 - 1 only gives the lower z-faces of plane k0
-    for (int k = k0 - 1; k < k1; ++k) {
-      if (!consume(k + 2)) { ok = false; break; }
+    auto zslot = [](int k) { return PL::FZ0 + (k + 1) % PL::NBZ * PL::NFZ; };  // of the upper z-faces of plane k >= -1
+    auto xslot = [](int k) { return PL::NBX == 2 ? k & 1 : 0; };
+    // the update of the tile's row `row` of plane k, a cell a lane
+    auto update = [&](int k, int row) {
+      const int ci = x0 + lane, cj = y0 + row;
+      if (ci >= g.nx || cj >= g.ny) return;
+      const long long o = gidx(g, ci, cj, k);
+      double dtc = dt;
+      if constexpr (STAGE >= 1 && !VISC)  // local time steps: inviscid blocks only
+        if (ph.local_dt) dtc = __ldg(static_cast<const double*>(D->dtl) + o);
+      double qs_[5], qn_[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        if constexpr (STAGE >= 1) qs_[v] = __ldg(qs + v * g.field + o);
+        if constexpr (STAGE >= 2) qn_[v] = __ldg(qn + v * g.field + o);
+      }
+      const int mk = k & 1, mk1 = (k + 1) & 1;
+      constexpr int MSD = PL::MSLOT / sizeof(double);
+      const double* mc = mring + mk * MSD + (row + HALO) * BX + lane + HALO;  // the cell's metrics
+      XVal iv = {0, 0};
+      if constexpr (CURVI) iv = xrcp(xdec_pos<62>(mc[9 * MS]));
+      double R[5], out[5];
+      // R = sum over directions of (upper - lower face flux) / h (CURVI: / V)
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        const int x = xslot(k) * PL::NFX + q * TY * (TX + 1) + row * (TX + 1) + lane,
+                  y = PL::FY0 + xslot(k) * PL::NFY + q * (TY + 1) * TX + row * TX + lane, z = q * TY * TX + row * TX + lane;
+        const int up[3] = {x + 1, y + TX, z + zslot(k)}, lo[3] = {x, y, z + zslot(k - 1)};
+        long long d[3];
+        int ed[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int e1 = fe[up[a]], e0 = fe[lo[a]];
+          ed[a] = xmax(e1, e0) + 1;
+          d[a] = xshr(fm[up[a]], ed[a] - e1) - xshr(fm[lo[a]], ed[a] - e0);  // [62]
+          if constexpr (!CURVI) {
+            // normalised first: the product's truncation is then relative to the difference (left to
+            // the flux's own scale it doubled the 32^3 pulse's error against 64-bit references)
+            const XVal f = xquick(d[a], ed[a]);
+            d[a] = xmul(f.m, xb->h2[a].m);  // [60]
+            ed[a] = f.e + xb->h2[a].e + 3;
+          }
+        }
+        const int E = xmax(ed[0], xmax(ed[1], ed[2])) + (CURVI ? 2 : 0);
+        const long long t = xshr(d[0], E - ed[0]) + xshr(d[1], E - ed[1]) + xshr(d[2], E - ed[2]);
+        if constexpr (CURVI) {
+          const XVal r = xquick(t, E);
+          R[q] = xenc(xmul(r.m, iv.m), r.e + iv.e + 3);
+        } else {
+          R[q] = xenc(t, E);
+        }
+      }
+      if constexpr (STAGE == 0) {
+        const long long oc = ((long long)k * g.ny + cj) * g.nx + ci;
+        const long long n = (long long)g.nx * g.ny * g.nz;
+#pragma unroll
+        for (int m = 0; m < 5; ++m) P.rout[m * n + oc] = R[m];
+      } else {
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+          const double adv = qs_[m] - dtc * R[m];
+          if constexpr (STAGE == 1) out[m] = adv;
+          else if constexpr (STAGE == 2) out[m] = fma(0.75, qn_[m], 0.25 * adv);
+          else out[m] = fma(2.0 / 3.0, adv, (1.0 / 3.0) * qn_[m]);  // an FP64 division costs ~7 FMAs here
+          qout[m * g.field + o] = out[m];
+        }
+        if constexpr (PUSH && (STAGE == 1 || STAGE == 2))
+          if (ci < HALO || cj < HALO || k < HALO || ci >= g.nx - HALO || cj >= g.ny - HALO || k >= g.nz - HALO)
+            push_halo<double>(pushdst, g.nx, g.ny, g.nz, ci, cj, k, out[0], out[1], out[2], out[3], out[4]);
+        if constexpr (STAGE == 1) {
+#pragma unroll
+          for (int m = 0; m < 5; ++m) nacc[m] = fma(R[m], R[m], nacc[m]);
+        }
+        if constexpr (STAGE == 3) {
+          XPrim W;
+          const bool phys = xprim(out, XK, W);
+          if (!phys) bad = true;
+          const XVal c = xsound(W, XK.gam);
+          XVal rate;
+          if constexpr (!CURVI) {
+            rate = xrate<VISC>(W, c, xb->h2, xb->hsum, xb->vs);
+          } else {  // sum over directions of |u . S| + c |S|, over V
+            const double* mu[3] = {mc + 1, mc + BX, mring + mk1 * MSD + (row + HALO) * BX + lane + HALO};
+            XVal r[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              const double lo[3] = {mc[3 * a * MS], mc[(3 * a + 1) * MS], mc[(3 * a + 2) * MS]};
+              const double up[3] = {mu[a][3 * a * MS], mu[a][(3 * a + 1) * MS], mu[a][(3 * a + 2) * MS]};
+              r[a] = xradius<false>(W, c, lo, up, iv);
+            }
+            const XVal v = xsum3(r[0], r[1], r[2]);
+            rate = xnormed(xmul(v.m, iv.m), v.e + iv.e + 3);
+          }
+          // the largest rate, as the bits of a non-negative double
+          const long long rb = __double_as_longlong(xenc(rate.m, rate.e));
+          if (phys && rb > __double_as_longlong(rate_max)) rate_max = __longlong_as_double(rb);
+          if constexpr (!VISC)
+            if (ph.local_dt) {
+              const XVal ir = xrcp(rate);
+              static_cast<double*>(D->dtl)[o] = ph.cfl * xenc(ir.m, ir.e);
+            }
+        }
+      }
+    };
+
+    // plane k0 - 1 only gives the lower z-faces of plane k0; PIPE: turn k1 is the last plane's update only
+    for (int k = k0 - 1; k < k1 + (PIPE ? 1 : 0); ++k) {
+      if (k < k1 && !consume(k + 2)) { ok = false; break; }
       if (tid == 0) mrequest_upto(k + 1);  // its slot held plane k - 1, last read before consume's barrier
       mwait_upto(k < k0 ? k0 : k + 1);
       const int sm = ((k - 1) & 3) * SL, sk = (k & 3) * SL, sp = ((k + 1) & 3) * SL, s2 = ((k + 2) & 3) * SL;
-      const int nitem = k < k0 ? TY : NITEM;
+      const int nitem = k == k1 ? 0 : (k < k0 ? TY : NITEM);
+      if constexpr (PIPE)
+        if (k > k0 && (k == k1 || warp >= W1))
+#pragma unroll 1
+          for (int row = k == k1 ? warp : warp - W1; row < TY; row += k == k1 ? NW : WU) update(k - 1, row);
 #pragma unroll 1
       for (int it = warp; it < nitem; it += NW) {
         const int d = it < TY ? 2 : (it < 2 * TY + 1 ? 1 : 0);
@@ -391,8 +511,9 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
         }
         XFlux F;
         xface<VISC, CURVI, MS>(rm, re, I, d, xb, S, XK, ph.limiter, F);
-        const int f = d == 2 ? PL::NFX + PL::NFY + (k & 1) * PL::NFZ + row * TX + col
-                             : (d == 1 ? PL::NFX + row * TX + col : row * (TX + 1) + col);
+        const int f = d == 2 ? zslot(k) + row * TX + col
+                             : (d == 1 ? PL::FY0 + xslot(k) * PL::NFY + row * TX + col
+                                       : xslot(k) * PL::NFX + row * (TX + 1) + col);
         const int fs = d == 2 ? TY * TX : (d == 1 ? (TY + 1) * TX : TY * (TX + 1));
         const int to[5] = {f, f + (CURVI ? 1 : 1 + d) * fs, f + (CURVI ? 2 : (d == 2 ? 1 : 2 + d)) * fs,
                            f + (CURVI ? 3 : (d == 0 ? 3 : d)) * fs, f + 4 * fs};
@@ -403,107 +524,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
         }
       }
       __syncthreads();
-      if (k < k0) continue;
-      const int row = warp, ci = x0 + lane, cj = y0 + row;  // warp `row` owns row `row` of the tile
-      if (row < TY && ci < g.nx && cj < g.ny) {
-        const long long o = gidx(g, ci, cj, k);
-        double dtc = dt;
-        if constexpr (STAGE >= 1 && !VISC)  // local time steps: inviscid blocks only
-          if (ph.local_dt) dtc = __ldg(static_cast<const double*>(D->dtl) + o);
-        double qs_[5], qn_[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          if constexpr (STAGE >= 1) qs_[v] = __ldg(qs + v * g.field + o);
-          if constexpr (STAGE >= 2) qn_[v] = __ldg(qn + v * g.field + o);
-        }
-        const int mk = k & 1, mk1 = (k + 1) & 1;
-        constexpr int MSD = PL::MSLOT / sizeof(double);
-        const double* mc = mring + mk * MSD + (row + HALO) * BX + lane + HALO;  // the cell's metrics
-        XVal iv = {0, 0};
-        if constexpr (CURVI) iv = xrcp(xdec_pos<62>(mc[9 * MS]));
-        double R[5], out[5];
-        // R = sum over directions of (upper - lower face flux) / h (CURVI: / V)
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const int x = q * TY * (TX + 1) + row * (TX + 1) + lane, y = PL::NFX + q * (TY + 1) * TX + row * TX + lane,
-                    z = PL::NFX + PL::NFY + q * TY * TX + row * TX + lane;
-          const int up[3] = {x + 1, y + TX, z + (k & 1) * PL::NFZ}, lo[3] = {x, y, z + ((k - 1) & 1) * PL::NFZ};
-          long long d[3];
-          int ed[3];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            const int e1 = fe[up[a]], e0 = fe[lo[a]];
-            ed[a] = xmax(e1, e0) + 1;
-            d[a] = xshr(fm[up[a]], ed[a] - e1) - xshr(fm[lo[a]], ed[a] - e0);  // [62]
-            if constexpr (!CURVI) {
-              // normalised first: the product's truncation is then relative to the difference (left to
-              // the flux's own scale it doubled the 32^3 pulse's error against 64-bit references)
-              const XVal f = xquick(d[a], ed[a]);
-              d[a] = xmul(f.m, xb->h2[a].m);  // [60]
-              ed[a] = f.e + xb->h2[a].e + 3;
-            }
-          }
-          const int E = xmax(ed[0], xmax(ed[1], ed[2])) + (CURVI ? 2 : 0);
-          const long long t = xshr(d[0], E - ed[0]) + xshr(d[1], E - ed[1]) + xshr(d[2], E - ed[2]);
-          if constexpr (CURVI) {
-            const XVal r = xquick(t, E);
-            R[q] = xenc(xmul(r.m, iv.m), r.e + iv.e + 3);
-          } else {
-            R[q] = xenc(t, E);
-          }
-        }
-        if constexpr (STAGE == 0) {
-          const long long oc = ((long long)k * g.ny + cj) * g.nx + ci;
-          const long long n = (long long)g.nx * g.ny * g.nz;
-#pragma unroll
-          for (int m = 0; m < 5; ++m) P.rout[m * n + oc] = R[m];
-        } else {
-#pragma unroll
-          for (int m = 0; m < 5; ++m) {
-            const double adv = qs_[m] - dtc * R[m];
-            if constexpr (STAGE == 1) out[m] = adv;
-            else if constexpr (STAGE == 2) out[m] = fma(0.75, qn_[m], 0.25 * adv);
-            else out[m] = fma(2.0 / 3.0, adv, (1.0 / 3.0) * qn_[m]);  // an FP64 division costs ~7 FMAs here
-            qout[m * g.field + o] = out[m];
-          }
-          if constexpr (PUSH && (STAGE == 1 || STAGE == 2))
-            if (ci < HALO || cj < HALO || k < HALO || ci >= g.nx - HALO || cj >= g.ny - HALO || k >= g.nz - HALO)
-              push_halo<double>(pushdst, g.nx, g.ny, g.nz, ci, cj, k, out[0], out[1], out[2], out[3], out[4]);
-          if constexpr (STAGE == 1) {
-#pragma unroll
-            for (int m = 0; m < 5; ++m) nacc[m] = fma(R[m], R[m], nacc[m]);
-          }
-          if constexpr (STAGE == 3) {
-            XPrim W;
-            const bool phys = xprim(out, XK, W);
-            if (!phys) bad = true;
-            const XVal c = xsound(W, XK.gam);
-            XVal rate;
-            if constexpr (!CURVI) {
-              rate = xrate<VISC>(W, c, xb->h2, xb->hsum, xb->vs);
-            } else {  // sum over directions of |u . S| + c |S|, over V
-              const double* mu[3] = {mc + 1, mc + BX, mring + mk1 * MSD + (row + HALO) * BX + lane + HALO};
-              XVal r[3];
-#pragma unroll
-              for (int a = 0; a < 3; ++a) {
-                const double lo[3] = {mc[3 * a * MS], mc[(3 * a + 1) * MS], mc[(3 * a + 2) * MS]};
-                const double up[3] = {mu[a][3 * a * MS], mu[a][(3 * a + 1) * MS], mu[a][(3 * a + 2) * MS]};
-                r[a] = xradius<false>(W, c, lo, up, iv);
-              }
-              const XVal v = xsum3(r[0], r[1], r[2]);
-              rate = xnormed(xmul(v.m, iv.m), v.e + iv.e + 3);
-            }
-            // the largest rate, as the bits of a non-negative double
-            const long long rb = __double_as_longlong(xenc(rate.m, rate.e));
-            if (phys && rb > __double_as_longlong(rate_max)) rate_max = __longlong_as_double(rb);
-            if constexpr (!VISC)
-              if (ph.local_dt) {
-                const XVal ir = xrcp(rate);
-                static_cast<double*>(D->dtl)[o] = ph.cfl * xenc(ir.m, ir.e);
-              }
-          }
-        }
-      }
+      if (!PIPE && k >= k0 && warp < TY) update(k, warp);  // warp `row` owns row `row` of the tile
     }
     if (!ok) break;
   }

@@ -71,6 +71,19 @@ def test_residual_mixed(gb, viscous):
 
 # ---- time stepping -------------------------------------------------------------------------
 
+@pytest.mark.parametrize("viscous", [False, True])
+@pytest.mark.parametrize("n", [(32, 8, 4), (33, 9, 5), (31, 7, 37), (95, 25, 70)])
+def test_fp64_tile_edges(gb, n, viscous):
+    """A full tile, one cell over and one short, several ragged tiles; shares of one plane a CTA (4 x 8) and
+    of many (70 planes of 12 tiles): three steps, with the bars of this file."""
+    c = ragged_case(viscous, 11, *n)
+    ref, dts, norms = run_oracle(c, 3)
+    blk = gb.block_for_case(c, precision=gb.FP64)
+    gb.step([blk], 3)
+    assert max(per_var(blk.get_state().cpu().numpy(), ref)) <= 1e-12
+    assert np.allclose(blk.residual_norm(), norms[-1], rtol=1e-11, atol=1e-13 * np.max(norms[-1]))
+
+
 def test_gaussian_pulse_32_fp64_10_steps(gb):
     """32^3 Euler Gaussian pulse, CFL 0.5, MUSCL/minmod + Roe, 10 SSP-RK3 steps, FP64."""
     c = cases.gaussian_pulse(32, seed=0)
