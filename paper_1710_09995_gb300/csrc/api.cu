@@ -820,8 +820,8 @@ static bool group_can_push(const std::vector<gbcfd_block>& bl) {
   return true;
 }
 
-// split SMs x ctas_per_sm CTAs between the blocks in proportion to their tile-planes (each gets
-// at least one) and write the descriptor table for the stage kernel of tile height ty
+// split SMs x ctas_per_sm CTAs between the blocks so that the longest share of tile-planes is the shortest
+// (each block gets at least one) and write the descriptor table for the stage kernel of tile height ty
 static int group_split(gbcfd_group g, int ctas_per_sm, cudaStream_t s, int ty = -1) {
   const int nsm = g->blocks[0]->nsm;
   if (ty < 0) ty = g->ty;
@@ -833,16 +833,31 @@ static int group_split(gbcfd_group g, int ctas_per_sm, cudaStream_t s, int ty = 
   }
   set_group_nbrs(g);
   const long long target = (long long)nsm * ctas_per_sm;
-  long long W = 0;
-  for (auto& d : g->table_host) W += d.units;
+  // one CTA a block, then each further one to the block with the most tile-planes per CTA: the longest share
+  // is the smallest that whole CTAs allow (rounding each block's part gave a block of 1.49 parts one CTA: on
+  // 36 blocks with sides 16 .. 96 the longest share was 590 tile-planes, now 499, of 441 on average)
+  const int nb = (int)g->table_host.size();
+  std::vector<long long> share(nb, 1);
+  auto less = [&](int i, int j) {  // by tile-planes per CTA, the earlier block first among equals
+    const long long a = g->table_host[i].units * share[j], b = g->table_host[j].units * share[i];
+    return a != b ? a < b : i > j;
+  };
+  std::vector<int> heap(nb);
+  for (int i = 0; i < nb; ++i) heap[i] = i;
+  std::make_heap(heap.begin(), heap.end(), less);
+  for (long long left = target - nb; left > 0; --left) {
+    std::pop_heap(heap.begin(), heap.end(), less);
+    const int i = heap.back();
+    if (share[i] >= g->table_host[i].units) break;  // one tile-plane a CTA everywhere
+    ++share[i];
+    std::push_heap(heap.begin(), heap.end(), less);
+  }
   int c0 = 0;
-  for (size_t i = 0; i < g->table_host.size(); ++i) {
+  for (int i = 0; i < nb; ++i) {
     BlockDesc& d = g->table_host[i];
-    long long c = (target * d.units + W / 2) / W;
-    c = std::max(1LL, std::min(c, d.units));
     d.cta0 = c0;
-    d.ctas = (int)c;
-    c0 += (int)c;
+    d.ctas = (int)share[i];
+    c0 += d.ctas;
   }
   if ((size_t)c0 > g->partial_n) return fail(GBCFD_ERR_ARG, "too many CTAs for the group's partial sums");
   g->grid = c0;
@@ -1077,8 +1092,7 @@ extern "C" int gbcfd_group_tune_tile(gbcfd_group g, void* stream, int* ctas_per_
   gbcfd_block b0 = g->blocks[0];
   // candidates: every tile height compiled for the path, each with one resident wave (occ CTAs
   // per SM) and finer splits of 2x .. 16x that, up to 16 CTAs per SM: uneven blocks share the
-  // grid in proportion to their tile-planes with rounding, and several waves of smaller CTAs
-  // even that out (on the 96-block lattice 8 per SM beat 1 by 30% on the FP64 path)
+  // grid in whole CTAs, and several waves of smaller ones even out what that leaves
   int tys[4];
   const int ntile = stage_tiles(b0->p.precision, b0->p.viscous, b0->curvi, tys);
   cudaEvent_t e0, e1;
