@@ -182,7 +182,8 @@ def hbm_peak():
 def kernel_source_hash(curvi=False):
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1710_09995_gb300", "csrc")
-    for name in ("stage.cuh", "physics.cuh", "internal.cuh", "vmath.cuh", "stage_inst.cuh") + (("curvi.cuh",) if curvi else ()):
+    for name in ("stage.cuh", "stage_x.cuh", "xfix.cuh", "physics.cuh", "internal.cuh", "vmath.cuh", "stage_inst.cuh") + (
+            ("curvi.cuh", "stage_c.cuh") if curvi else ()):
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -463,7 +464,9 @@ def fp64_alu_roofline(res, cells, steps, hbm, workload="vortex256"):
     """FP64-pipe roofline of the FP64 stage kernel: its FP64 flops per cell (2 DFMA + DADD + DMUL,
     counted by ncu per stage) over the launch time, against the part's FP64 peak; and the share of
     the pipe's lane slots its FP64 instructions fill (DADD + DMUL + DFMA per cell against 152 SMs x
-    2 lanes x the clock)"""
+    2 lanes x the clock).  The kernel's faces and residuals run on the integer pipes (xfix.cuh), so only the
+    update and the norms are FP64 instructions and the share is small: the instruction counts are in the
+    committed ncu summary"""
     flops = profiled_numbers("fp64", "fp64 flops per cell and stage", workload)
     out = {"bound": "alu", "kernel": "stage_kernel", "unit": "TFLOP/s", "peak": FP64_PEAK_TFLOPS,
            "peak_kind": "FP64 FMA lanes x clock (152 SMs x 2 x 2 flops x 2.07 GHz; 1.2524 measured by gbcfd_op_rate)",
