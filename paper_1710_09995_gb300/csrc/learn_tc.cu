@@ -15,13 +15,15 @@
 // and the B matrix at weight group t CIP/8 (SBO 128 B, LBO = N x 16 B).
 //
 // Warps: four per 16 output channels read the accumulators back (thread = TMEM lane = cell) and
-// apply the epilogue, four load rows by cp.async (two groups of two warps, alternate rows), one
-// thread of the last issues the MMAs, its descriptors a constant away from the three rows'
-// (unrolled: formed per tap they were 1100 instructions of a single thread a tile).  They meet only at mbarriers: a row landed, a tile's MMAs done (tcgen05.commit), an
+// apply the epilogue, four load rows by cp.async (two groups of two warps, alternate rows), the last
+// issues the MMAs: it walks and waits as a warp, so that the descriptors (a constant away from the three
+// rows') stay in uniform registers, and one elected lane executes the MMA.  In a one-thread branch each
+// descriptor was moved there anew, about 100 cycles an MMA (two tiles' MMAs in turn were no faster): layer 2
+// 197 -> 121 us.  The warps meet only at mbarriers: a row landed, a tile's MMAs done (tcgen05.commit), an
 // accumulator read back.  The first version copied a tile's nine rows anew by TMA, with the
 // channel groups as 16-byte inner boxes: 36 copies of 130 such pieces a tile held it at 12 us
 // (every unit below 30% busy); now a tile loads three rows, in pieces the threads copy whole cells
-// at a time.  192 x 96 x 64 cells, three layers: 1.86 -> 0.53 ms.
+// at a time.  192 x 96 x 64 cells, three layers: 1.86 -> 0.38 ms.
 #include <atomic>
 
 #include "internal.cuh"
@@ -98,6 +100,12 @@ struct TcWalk {
     return true;
   }
 };
+
+__device__ __forceinline__ bool elect_one() {
+  unsigned p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
 
 // the 27 x CIP/16 MMAs of one tile into the accumulator at tmem (one thread), then a commit;
 // row[dy] = the descriptor of cell 0, plane 0 of the slot of row y + dy - 1, wdesc the weights'
@@ -176,7 +184,7 @@ __global__ void __launch_bounds__(TcWarps<N>::threads, CIP == 16 ? 2 : 1) conv_t
   float* bias = reinterpret_cast<float*>(wsm + NTAP * CIP * N);      // COP (FWD)
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(bias + 32);  // full[5], done[4], epi[2]
   unsigned* tslot = reinterpret_cast<unsigned*>(bar + 11);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform: the issuer's branch and values
   constexpr unsigned COLW = N < 32 ? 32 : N, COLS = 2 * COLW;
 
   if (warp == EPI + 4) {
@@ -245,21 +253,24 @@ __global__ void __launch_bounds__(TcWarps<N>::threads, CIP == 16 ? 2 : 1) conv_t
       g0 += walk.n + 2;
       s0 += walk.n;
     }
-  } else if (tid == 32 * (EPI + 4)) {
-    // ---- MMA issue ----
+  } else if (warp == EPI + 4) {
+    // ---- MMA issue: the warp walks and waits as one, one elected lane issues ----
+    const unsigned tm = __shfl_sync(0xffffffffu, tmem0, 0);
+    const bool lead = elect_one();
     const unsigned long long rdesc = smem_desc(rows0, RP * 16u, 128u), wdesc = smem_desc(w0, N * 16u, 128u);
     int g0 = 0, s = 0;
     while (ok && walk.next(A)) {
       for (int r = 0; r < walk.n + 2 && ok; ++r) {
         const int g = g0 + r;
-        ok = mbar_wait_limited(full0 + 8u * (g % TC_NR), (g / TC_NR) & 1);
+        ok = __all_sync(0xffffffffu, mbar_wait_limited(full0 + 8u * (g % TC_NR), (g / TC_NR) & 1));
         if (!ok || r < 2) continue;
-        if (s >= 2 && !(ok = mbar_wait_limited(epi0 + 8u * (s & 1), ((s >> 1) - 1) & 1))) break;
+        if (s >= 2 && !(ok = __all_sync(0xffffffffu, mbar_wait_limited(epi0 + 8u * (s & 1), ((s >> 1) - 1) & 1)))) break;
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const unsigned long long row[3] = {rdesc + (unsigned)((g - 2) % TC_NR) * (SLOTB / 16u),
                                            rdesc + (unsigned)((g - 1) % TC_NR) * (SLOTB / 16u),
                                            rdesc + (unsigned)(g % TC_NR) * (SLOTB / 16u)};
-        tc_issue<CIP, N>(row, wdesc, tmem0 + (s & 1) * COLW, done0 + 8u * (s & 3));
+        if (lead) tc_issue<CIP, N>(row, wdesc, tm + (s & 1) * COLW, done0 + 8u * (s & 3));
+        __syncwarp();
         ++s;
       }
       g0 += walk.n + 2;
