@@ -23,7 +23,7 @@
 // accumulator read back.  The first version copied a tile's nine rows anew by TMA, with the
 // channel groups as 16-byte inner boxes: 36 copies of 130 such pieces a tile held it at 12 us
 // (every unit below 30% busy); now a tile loads three rows, in pieces the threads copy whole cells
-// at a time.  192 x 96 x 64 cells, three layers: 1.86 -> 0.38 ms.
+// at a time.  192 x 96 x 64 cells, three layers: 1.86 -> 0.34 ms.
 #include <atomic>
 
 #include "internal.cuh"
@@ -324,13 +324,14 @@ static cudaError_t conv_tc_go(const ConvArgs& a, const bf16* wtc, int* flag, cud
     if (dev < 64) done.fetch_or(1ull << dev, std::memory_order_acq_rel);
   }
   if (((uintptr_t)a.in & 15u) != 0) return cudaErrorMisalignedAddress;
-  int nsm = 0, occ = 0;
+  int nsm = 0;
   e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, conv_tc_kernel<CIP, N, COP, MODE>, TcWarps<N>::threads, bytes);
   if (e != cudaSuccess) return e;
+  // resident CTAs by the kernel's launch bounds and shared memory (228 KB an SM, 1 KB of it a CTA's own; the
+  // occupancy query answered 1 for the two that ncu counts: layer 1 119 -> 82 us)
+  constexpr int occ = CIP == 16 ? 2 : 1;
   const long long tiles = (long long)((a.X + TC_M - 1) / TC_M) * a.Y * a.Z * a.B;
-  long long grid = (long long)nsm * (occ > 0 ? occ : 1);
+  long long grid = (long long)nsm * occ;
   if (grid > tiles) grid = tiles;
   conv_tc_kernel<CIP, N, COP, MODE><<<(unsigned)grid, TcWarps<N>::threads, bytes, s>>>(a, wtc, flag, tiles);
   return cudaGetLastError();
