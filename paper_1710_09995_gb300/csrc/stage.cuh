@@ -1,4 +1,7 @@
-// stage.cuh -- the fused Runge-Kutta stage kernel (residual of Eq. 3 + update of Eqs. 4-6).
+// stage.cuh -- the fused Runge-Kutta stage kernel (residual of Eq. 3 + update of Eqs. 4-6): mixed path on
+// Cartesian blocks, and viscous curvilinear blocks in FP64.  FP64 on Cartesian and inviscid curvilinear
+// blocks runs on the integer pipes (stage_x.cuh), the mixed path on curvilinear ones in stage_c.cuh; both share
+// this file's tiles, copies and reductions.
 //
 // Work decomposition: the block's (x, y) cross-section is cut into TX x TY tiles; a tile-plane
 // (tile, k) is one work unit.  The grid is persistent (a multiple of the SM count) and CTA c
