@@ -371,7 +371,7 @@ __device__ __forceinline__ void tma_abort(uint64_t* bar, unsigned pending, unsig
   atomicOr(&ctrl->flag, FLAG_TIMEOUT);
 }
 
-__global__ void __launch_bounds__(NTW) viscres_kernel(const __grid_constant__ Args a) {
+__global__ void __launch_bounds__(NTW, 2) viscres_kernel(const __grid_constant__ Args a) {
   using T = float;  // (FP64: xviscres_kernel, wcns_x.cuh)
   extern __shared__ __align__(128) unsigned char rsm[];
   T* wr = reinterpret_cast<T*>(rsm + RSmem::w);
@@ -426,46 +426,57 @@ __global__ void __launch_bounds__(NTW) viscres_kernel(const __grid_constant__ Ar
     // each thread owns tile cell (lane, warp): its x- and y-parts of Rv for planes p-2, p-1, p stay
     // in registers until the z-part of plane p-2 is known
     T rv2[4] = {0, 0, 0, 0}, rv1[4] = {0, 0, 0, 0};
+    // the union box: a warp per 32-cell row (rows 0..7, then 8..11), and warps 4, 5 of the second
+    // pass take the 4 extra columns of all 12 rows (a row stride of 44 spreads them over distinct
+    // banks); walking the 36-wide box row-major would split warps over two rows and conflict.  A thread's
+    // two cells are the same on every plane: their columns of five planes stay in registers, and a plane costs
+    // 40 shared loads a cell instead of 55 (128^3: 75 -> 68 us)
+    int gys[2] = {warp, RY + warp}, gxs[2] = {lane, lane};
+    bool have[2] = {true, true};
+    if (warp >= GY - RY) {
+      const int sidx = (warp - (GY - RY)) * 32 + lane;  // 0 .. 63; 48 side cells
+      have[1] = sidx < GY * (GX - RX);
+      gys[1] = sidx / (GX - RX);
+      gxs[1] = RX + sidx % (GX - RX);
+    }
+    T col[2][4][5];  // u, v, w, theta of the cell in planes p - 2 .. p + 2
     __syncthreads();  // the previous segment is done with the rings
     if (threadIdx.x == 0)
       for (int kp = k0 - 4; kp <= k0; ++kp) issue(kp);
     for (int kp = k0 - 4; kp <= k0 - 1; ++kp) wait(kp);
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass)
+      if (have[pass]) {
+        const int c = (gys[pass] + 2) * WX + gxs[pass] + 3;
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+#pragma unroll
+          for (int m = 0; m < 4; ++m) col[pass][f][m] = wr[ws(k0 - 4 + m) * RSmem::WP + f * RSmem::WF + c];
+      }
     for (int p = k0 - 2; p <= k1 + 1; ++p) {  // lead plane p, output plane p - 2
       if (threadIdx.x == 0 && p <= k1 && !*sabort) issue(p + 3);  // into the slot of plane p - 3
       wait(p + 2);
       __syncthreads();
       if (*sabort) break;
-      const T* pl[5];
-#pragma unroll
-      for (int m = 0; m < 5; ++m) pl[m] = wr + ws(p - 2 + m) * RSmem::WP;
+      const T *pc = wr + ws(p) * RSmem::WP, *pn = wr + ws(p + 2) * RSmem::WP;
       T* hzp = hzr + zs(p) * RSmem::HZP;
-      // the union box: a warp per 32-cell row (rows 0..7, then 8..11), and warps 4, 5 of the second
-      // pass take the 4 extra columns of all 12 rows (a row stride of 44 spreads them over distinct
-      // banks); walking the 36-wide box row-major would split warps over two rows and conflict
+#pragma unroll
       for (int pass = 0; pass < 2; ++pass) {
-        int gx, gy;
-        if (pass == 0) {
-          gy = warp;
-          gx = lane;
-        } else if (warp < GY - RY) {
-          gy = RY + warp;
-          gx = lane;
-        } else {
-          const int sidx = (warp - (GY - RY)) * 32 + lane;  // 0 .. 63; 48 side cells
-          if (sidx >= GY * (GX - RX)) continue;
-          gy = sidx / (GX - RX);
-          gx = RX + sidx % (GX - RX);
-        }
+        if (!have[pass]) continue;
+        const int gy = gys[pass], gx = gxs[pass];
         const int c = (gy + 2) * WX + gx + 3;  // the cell in the primitive box
         T gr[4][3], vel[3];
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
-          const T* p0 = pl[2] + f * RSmem::WF;
-          if (f < 3) vel[f] = p0[c];
+          const T* p0 = pc + f * RSmem::WF;
+          T(&z)[5] = col[pass][f];
+          z[4] = pn[f * RSmem::WF + c];
+          if (f < 3) vel[f] = z[2];
           gr[f][0] = ((p0[c - 2] - p0[c + 2]) + T(8) * (p0[c + 1] - p0[c - 1])) * ih0;
           gr[f][1] = ((p0[c - 2 * WX] - p0[c + 2 * WX]) + T(8) * (p0[c + WX] - p0[c - WX])) * ih1;
-          const int o = f * RSmem::WF + c;
-          gr[f][2] = ((pl[0][o] - pl[4][o]) + T(8) * (pl[3][o] - pl[1][o])) * ih2;
+          gr[f][2] = ((z[0] - z[4]) + T(8) * (z[3] - z[1])) * ih2;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) z[m] = z[m + 1];
         }
         const T div = gr[0][0] + gr[1][1] + gr[2][2];
         const bool rows = gy >= 2 && gy < RY + 2, cols = gx >= 2 && gx < RX + 2;
