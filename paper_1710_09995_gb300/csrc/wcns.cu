@@ -305,6 +305,10 @@ __global__ void __launch_bounds__(NTW) prim_multi_kernel(Args a, int with_rate, 
   prim_body<T, true>(a, with_rate, &tab);
 }
 
+// CTAs per SM of the primitive pass: mixed, the 6 that are resident (with 8 a third of them ran as a second wave:
+// 128^3, 31.4 -> 29.0 us on average); FP64, 8 (4 are resident, and 4 or 8 take the same time)
+template <typename T> constexpr int PRIM_CTAS = sizeof(T) == 8 ? 8 : 6;
+
 // the common time step of blocks advanced together: cfl / the largest of their rates, written
 // to every member (after each member's stage-1 primitive pass has reduced its own rate)
 __global__ void wcns_group_dt_kernel(const __grid_constant__ WTab tab, double cfl) {
@@ -1120,7 +1124,7 @@ cudaError_t launch_rest(gbcfd_wcns w, const Args& a, const cudaEvent_t* ev, cuda
 template <typename T>
 cudaError_t launch_pass(gbcfd_wcns w, Args a, int with_rate, const cudaEvent_t* ev, cudaStream_t s) {
   if (ev) cudaEventRecord(ev[0], s);
-  const int pgrid = std::min(w->rows, w->nsm * 8);
+  const int pgrid = std::min(w->rows, w->nsm * PRIM_CTAS<T>);
   prim_kernel<T><<<pgrid, NTW, 0, s>>>(a, with_rate);
   if (ev) cudaEventRecord(ev[1], s);
   return launch_rest<T>(w, a, ev, s);
@@ -1216,7 +1220,7 @@ cudaError_t run_stage_many(const gbcfd_wcns* blocks, int n, WTab& tab, int stage
   for (int i = 0; i < n && e == cudaSuccess; ++i) {
     const gbcfd_wcns w = blocks[i];
     tab.self = i;
-    const int pgrid = std::min(w->rows, w->nsm * 8);
+    const int pgrid = std::min(w->rows, w->nsm * PRIM_CTAS<T>);
     prim_multi_kernel<T><<<pgrid, NTW, 0, pool->st[i % NSIDE]>>>(stage_args(w, stage, nullptr), stage == 1, tab);
     e = cudaGetLastError();
   }
