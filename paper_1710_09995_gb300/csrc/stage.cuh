@@ -513,6 +513,8 @@ __global__ void __launch_bounds__(tile_threads(TYV), sizeof(T) == 4 ? (TYV <= 4 
     const int tix = (int)(tile % D->ntx), tiy = (int)(tile / D->ntx);
     const int x0 = tix * TX, y0 = tiy * TY;  // storage coordinates of the box origin
     const int last_plane = k1 + 1;
+    // the last plane's update reads the metric slots that this tile's first copies land in, with no barrier behind it
+    if constexpr (CURVI) __syncthreads();
     // arrays of this stage
     const CUtensorMap* tmq;
     const CUtensorMap* tmd = &D->td[0];

@@ -278,6 +278,8 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
     const int tix = (int)(tile % D->ntx), tiy = (int)(tile / D->ntx);
     const int x0 = tix * TX, y0 = tiy * TY;  // storage coordinates of the box origin
     const int last_plane = k1 + 1;
+    // the last plane's update reads the metric slots that this tile's first copy lands in, with no barrier behind it
+    if constexpr (CURVI) __syncthreads();
 
     auto request = [&](int kp) {  // thread 0 only
       const int s = (kp + 2) & (NST - 1);

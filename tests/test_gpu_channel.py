@@ -84,6 +84,34 @@ def test_channel_local_steps_mixed(gb):
     assert err[0] <= 1e-6 and err[4] <= 1e-6 and max(emom) <= 1e-5, (err, emom)
 
 
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-5)])
+def test_channel_local_steps_on_shares_of_many_planes(gb, precision, tol):
+    """96 x 48 x 33: about four planes a CTA, several tiles, shares that cross tiles; eight local-time-step
+    steps, each variable against the oracle in the larger of its own norm and a thousandth of the density's
+    (FP32: momentum components against the momentum vector's norm), the steps with the state's bars, and the
+    same bits in a second run"""
+    c = channel(96, 48, 33, seed=9)
+    bcs, M, p = oracle_setup(c)
+    ref, dts, norms = oracle.step_ex(p, oracle.pad(c.state), M, 8, bcs, local_dt=True)
+    want = oracle.interior(ref)
+    dt = oracle.dt_local(p, oracle.fill_halo_bc(ref, M, bcs), M).min()
+    mom = np.linalg.norm(want[1:4].ravel())
+    first = None
+    for _ in range(2):
+        blk = gb.block_for_case(c, precision=precision)
+        gb.step([blk], 8)
+        got = blk.get_state().cpu().numpy()
+        err = per_var(got, want)
+        if precision:
+            err[1:4] = [np.linalg.norm((got[m] - want[m]).ravel()) / mom for m in (1, 2, 3)]
+        assert max(err) <= tol, err
+        nt = (1e-10, 0.0) if precision == 0 else (1e-3, 1e-4 * np.max(norms[-1]))
+        assert np.allclose(blk.residual_norm(), norms[-1], rtol=nt[0], atol=nt[1])
+        assert abs(blk.get_dt() - dt) <= tol * dts[0]
+        assert first is None or np.array_equal(got, first)
+        first = got
+
+
 def test_channel_global_step_fp64(gb):
     """boundary conditions with the global time step too"""
     c = channel(seed=7)

@@ -85,6 +85,31 @@ def test_mixed_tile_edges(gb, n, viscous):
     assert abs(blk.get_dt() - oracle.dt(oparams(c), ref, M)) <= 1e-5 * dts[0]
 
 
+@pytest.mark.parametrize("viscous", [False, True])
+@pytest.mark.parametrize("precision,rtol,stol,ntol,dtol", [(0, 1e-12, 1e-12, 1e-11, 1e-13), (1, 3e-4, 1e-5, 3e-4, 1e-5)])
+@pytest.mark.parametrize("n", [(95, 25, 70), (95, 25, 71), (161, 65, 5)])
+def test_shares_of_many_planes_and_tiles(gb, n, precision, rtol, stol, ntol, dtol, viscous):
+    """CTAs that march many planes of a tile (the rings of state, metric and flux planes wrap) and go on to
+    another tile in the same launch, even and odd numbers of planes: residual, state, norm and time step,
+    with the bars of the smaller cases (FP32 residuals: their differences are divided by cells of 1/161, not of
+    1/70, so 1e-4 becomes 3e-4), and the same bits in a second run."""
+    c = warped_case(*n, viscous, seed=13)
+    M = oracle.metrics(c.nodes)
+    want = oracle.residual(oparams(c), oracle.pad(c.state), M)
+    ref, dts, norms = oracle.step(oparams(c), oracle.pad(c.state), M, 3)
+    first = None
+    for _ in range(2):
+        blk = gb.block_for_case(c, precision=precision)
+        assert max(per_var(blk.compute_residual().cpu().numpy(), want)) <= rtol
+        gb.step([blk], 3)
+        got, dt = blk.get_state().cpu().numpy(), blk.get_dt()
+        assert max(per_var(got, oracle.interior(ref))) <= stol
+        assert np.allclose(blk.residual_norm(), norms[-1], rtol=ntol, atol=1e-3 * ntol * np.max(norms[-1]))
+        assert abs(dt - oracle.dt(oparams(c), ref, M)) <= dtol * dts[0]
+        assert first is None or (np.array_equal(got, first[0]) and dt == first[1])
+        first = got, dt
+
+
 @pytest.mark.parametrize("precision", [0, 1])
 def test_freestream_preserved_warped(gb, precision):
     c = warped_case(36, 17, 10, True, amp=0.0)
