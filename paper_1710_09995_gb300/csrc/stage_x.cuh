@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
         const bool fill = !valid || !phys;  // rho = p = 1, no velocity
         auto put = [&](int v, long long a, int ea, bool one) {
           m[v * MS + c] = fill ? (one ? 1ll << 60 : 0ll) : a;
-          e[v * MS + c] = (short)(fill ? XRING_BIAS + 1 : XRING_BIAS + ea);
+          e[v * MS + c] = (short)(fill ? (one ? XRING_BIAS + 1 : XZERO) : XRING_BIAS + ea);
         };
         put(0, W.r.m >> 1, W.r.e + 1, true);
 #pragma unroll
@@ -397,13 +397,12 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
           const int e1 = fe[up[a]], e0 = fe[lo[a]];
           ed[a] = xmax(e1, e0) + 1;
           d[a] = xshr(fm[up[a]], ed[a] - e1) - xshr(fm[lo[a]], ed[a] - e0);  // [62]
-          if constexpr (!CURVI) {
-            // normalised first: the product's truncation is then relative to the difference (left to
-            // the flux's own scale it doubled the 32^3 pulse's error against 64-bit references)
-            const XVal f = xquick(d[a], ed[a]);
-            d[a] = xmul(f.m, xb->h2[a].m);  // [60]
-            ed[a] = f.e + xb->h2[a].e + 3;
-          }
+          // normalised first: the product's truncation is then relative to the difference (left to the
+          // flux's own scale it doubled the 32^3 pulse's error against 64-bit references), and a direction in
+          // which a component does not change does not take the others' bits
+          const XVal f = xquick0(d[a], ed[a]);
+          d[a] = CURVI ? f.m : xmul(f.m, xb->h2[a].m);  // [60]; CURVI [62]
+          ed[a] = f.e + (CURVI ? 0 : xb->h2[a].e + 3);
         }
         const int E = xmax(ed[0], xmax(ed[1], ed[2])) + (CURVI ? 2 : 0);
         const long long t = xshr(d[0], E - ed[0]) + xshr(d[1], E - ed[1]) + xshr(d[2], E - ed[2]);

@@ -111,6 +111,15 @@ __host__ __device__ __forceinline__ XVal xdec_pos(double a) {  // a > 0
   const unsigned long long mag = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b;
   return {(long long)(mag << (B - 53)), (int)((hi >> 20) & 0x7ffu) - 1023 + (62 - B)};
 }
+// the exponent of an exact zero: below that of any product of doubles, so that a zero takes no part in the
+// class of a sum
+constexpr int XZERO = -8000;
+// the same, a zero or subnormal as zero
+__host__ __device__ __forceinline__ XVal xdec_zero(double a) {
+  XVal v = xdec<62>(a);
+  if (v.e == -1023) v = {0, XZERO};
+  return v;
+}
 // the double nearest to m 2^(e - 61), |m| < 2^63; below the normal range 0, above it infinity, and
 // NaN for the exponents from XBAD up (a flux that has no value)
 constexpr int XBAD = 8192;
@@ -169,6 +178,12 @@ __host__ __device__ __forceinline__ XVal xquick(long long m, int e) {
   const int hi = (int)(m >> 32);
   const int n = xclz32(hi ^ (hi >> 31)) - 1;  // 0 .. 31
   return {(long long)((unsigned long long)m << n) >> 1, e + 1 - n};
+}
+
+// the same, an exact zero with its own exponent (a difference that vanishes)
+__host__ __device__ __forceinline__ XVal xquick0(long long m, int e) {
+  const XVal r = xquick(m, e);
+  return {r.m, m ? r.e : XZERO};
 }
 
 // float seeds of the reciprocal (root) of x, 1 <= x < 4
@@ -242,6 +257,13 @@ struct XPair {
   long long l, r;
   int e;
 };
+// a face's sides normalised together: the products of xroe are then rounded relative to the larger (edge
+// values have up to four spare bits: their squares lost eight, three times the FP64 form's error in
+// the energy residual)
+__host__ __device__ __forceinline__ XPair xpair_norm(long long l, long long r, int e) {
+  const int n = xclz32((int)((l ^ (l >> 63)) >> 32) | (int)((r ^ (r >> 63)) >> 32)) - 2;  // 0 .. 30
+  return {l << n, r << n, e - n};
+}
 // twice a face flux, each component in its own class, [62]; where a density or c^2 is not
 // positive the exponents are XBAD or more (NaN)
 struct XFlux {
@@ -255,13 +277,14 @@ struct XFlux {
 // the velocities, EH of the enthalpies and q^2/2, El of the wave speeds, EM of the mass fluxes.
 // Where a value may be much smaller than its class (jumps, products of several factors) it is
 // normalised, so that later roundings are relative to it.
-// CURVI: (u, v, w) are the x, y, z velocities, un the velocity along the face normal n (class 0,
-// [61]); the shear jumps are du - dun n, so the momentum flux is a x, y, z vector and needs no
+// CURVI: (u, v, w) are the x, y, z velocities, un the velocity along the face normal n, whose components have their
+// own classes (a component that is zero or small on the face keeps the pressure's class out of that momentum);
+// the shear jumps are du - dun n, so the momentum flux is a x, y, z vector and needs no
 // tangents.
 template <bool CURVI>
 __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, const XPair& v, const XPair& w,
                                               const XPair& p, const XConsts& K, XFlux& F, const XPair& un,
-                                              const long long* n) {
+                                              const XVal* n) {
   const int Eu = u.e, Ev = v.e, Ew = w.e, Ep = p.e, En = CURVI ? un.e : Eu;
   const long long ul = u.l, ur = u.r, vl = v.l, vr = v.r, wl = w.l, wr = w.r;
   // densities and pressures by themselves; reciprocal roots; the Roe weights a_l = isr iw,
@@ -364,13 +387,13 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
     const int Eg0 = lrt.e + jx.e + 3, Egn = lrt.e + ju.e + 3;
     const int EP = xmax(xmax(Edq, Egn), Ep + 2);
     const XVal P = xquick(xshr(p.l + p.r, EP - Ep) - xshr(dq, EP - Edq) + xshr(gn, EP - Egn), EP);  // along n, [62]
-    const int fp = P.e + 3;                                                                         // P n_x [59]
-    F.e[1] = xmax(xmax(f1, fp), Eg0);
-    F.e[2] = xmax(xmax(f2, fp), Eg1);
-    F.e[3] = xmax(xmax(f3, fp), Eg2);
-    F.m[1] = xshr(a1m, F.e[1] - f1) + xshr(xmul(P.m, n[0]), F.e[1] - fp) - xshr(g0, F.e[1] - Eg0);
-    F.m[2] = xshr(a2m, F.e[2] - f2) + xshr(xmul(P.m, n[1]), F.e[2] - fp) - xshr(g1, F.e[2] - Eg1);
-    F.m[3] = xshr(a3m, F.e[3] - f3) + xshr(xmul(P.m, n[2]), F.e[3] - fp) - xshr(g2, F.e[3] - Eg2);
+    const int p0 = P.e + n[0].e + 3, p1 = P.e + n[1].e + 3, p2 = P.e + n[2].e + 3;                   // P n_x [60]
+    F.e[1] = xmax(xmax(f1, p0), Eg0);
+    F.e[2] = xmax(xmax(f2, p1), Eg1);
+    F.e[3] = xmax(xmax(f3, p2), Eg2);
+    F.m[1] = xshr(a1m, F.e[1] - f1) + xshr(xmul(P.m, n[0].m), F.e[1] - p0) - xshr(g0, F.e[1] - Eg0);
+    F.m[2] = xshr(a2m, F.e[2] - f2) + xshr(xmul(P.m, n[1].m), F.e[2] - p1) - xshr(g1, F.e[2] - Eg1);
+    F.m[3] = xshr(a3m, F.e[3] - f3) + xshr(xmul(P.m, n[2].m), F.e[3] - p2) - xshr(g2, F.e[3] - Eg2);
     // shear work ut . (du - dun n); class E4 may be below these terms' own: they are aligned both ways
     const int e0 = Eg0 + Eu + 3, en = Egn + En + 3, E5 = xmax(E4, xmax(e0, en));
     d4 = xshr(d4, E5 - E4) + xshr(xmul(g0, ut), E5 - e0) - xshr(xmul(gn, nt), E5 - en);
@@ -390,30 +413,22 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   xroe<false>(r, u, v, w, p, K, F, u, nullptr);
 }
 
-// the unit normal (class 0, [61]) and half the length of a face's area vector
+// the unit normal, each component in its own class [62], and half the length of a face's area vector
 struct XNormal {
-  long long n[3];
+  XVal n[3];
   XVal half;
 };
 __host__ __device__ __forceinline__ XNormal xnormal(double sx, double sy, double sz) {
-  const XVal a = xdec<62>(sx), b = xdec<62>(sy), c = xdec<62>(sz);
+  const XVal a = xdec_zero(sx), b = xdec_zero(sy), c = xdec_zero(sz);
   const int E = xmax(a.e, xmax(b.e, c.e));
-  const XVal x = {xshr(a.m, E - a.e), E}, y = {xshr(b.m, E - b.e), E}, z = {xshr(c.m, E - c.e), E};
-  const XVal s2 = xnormed(xsq(x.m) + xsq(y.m) + xsq(z.m), 2 * E + 3);
+  const XVal s2 = xnormed(xsq(xshr(a.m, E - a.e)) + xsq(xshr(b.m, E - b.e)) + xsq(xshr(c.m, E - c.e)), 2 * E + 3);
   const XVal ia = xrsqrt(s2);
   XNormal N;
-  // S ia [60] << 2; |S| ia = 1 bounds the exponent: E + ia.e is 0 or -1 when the largest is near |S|
-  const int sh = -(E + ia.e);
-  N.n[0] = xshr(xmul(x.m, ia.m) << 3, sh);
-  N.n[1] = xshr(xmul(y.m, ia.m) << 3, sh);
-  N.n[2] = xshr(xmul(z.m, ia.m) << 3, sh);
+  N.n[0] = {xmul(a.m, ia.m) << 2, a.e + ia.e + 1};
+  N.n[1] = {xmul(b.m, ia.m) << 2, b.e + ia.e + 1};
+  N.n[2] = {xmul(c.m, ia.m) << 2, c.e + ia.e + 1};
   N.half = {xmul(s2.m, ia.m) << 2, s2.e + ia.e};
   return N;
-}
-// the velocity along n of one side, from (u, v, w) in their classes: class Emax + 1, [62]
-__host__ __device__ __forceinline__ long long xdot(const long long* n, long long u, int Eu, long long v, int Ev,
-                                                   long long w, int Ew, int E) {
-  return (xshr(xmul(u, n[0]), E - Eu) + xshr(xmul(v, n[1]), E - Ev) + xshr(xmul(w, n[2]), E - Ew)) << 2;
 }
 
 // twice the flux through a face of area vector (sx, sy, sz) from the sides' (rho, u, v, w, p), x, y, z
@@ -422,8 +437,12 @@ __host__ __device__ __forceinline__ void xroe_area(const XPair& r, const XPair& 
                                                    const XPair& p, double sx, double sy, double sz, const XConsts& K,
                                                    XFlux& F) {
   const XNormal N = xnormal(sx, sy, sz);
-  const int E = xmax(xmax(u.e, v.e), w.e);
-  const XPair un = {xdot(N.n, u.l, u.e, v.l, v.e, w.l, w.e, E), xdot(N.n, u.r, u.e, v.r, v.e, w.r, w.e, E), E + 1};
+  // the velocities along n, in the class of the largest product ([60] each)
+  const int e0 = u.e + N.n[0].e + 3, e1 = v.e + N.n[1].e + 3, e2 = w.e + N.n[2].e + 3, E = xmax(xmax(e0, e1), e2);
+  auto dot = [&](long long a, long long b, long long c) {
+    return xshr(xmul(a, N.n[0].m), E - e0) + xshr(xmul(b, N.n[1].m), E - e1) + xshr(xmul(c, N.n[2].m), E - e2);
+  };
+  const XPair un = xpair_norm(dot(u.l, v.l, w.l), dot(u.r, v.r, w.r), E);
   xroe<true>(r, u, v, w, p, K, F, un, N.n);
 #ifdef __CUDA_ARCH__
 #pragma unroll
@@ -451,11 +470,6 @@ __host__ __device__ __forceinline__ XPair xpair(double l, double r) {
 struct XPrim {
   XVal r, ir, u[3], p;
 };
-__host__ __device__ __forceinline__ XVal xdec_zero(double a) {  // zero and subnormals as zero
-  XVal v = xdec<62>(a);
-  if (v.e == -1023) v.m = 0;
-  return v;
-}
 __host__ __device__ __forceinline__ bool xprim(const double* q, const XConsts& K, XPrim& W) {
   W.r = xdec_pos<62>(q[0]);
   W.ir = xrcp(W.r);
@@ -568,13 +582,6 @@ __host__ __device__ __forceinline__ void xline_value(double v, long long* m, sho
   const long long sg = hi >> 31;
   *m = ex ? ((long long)(mag << 4) ^ sg) - sg : 0ll;
   *e = (short)(ex == 0x7ff ? XW_BAD : ex);
-}
-// a face's sides normalised together: the products of xroe are then rounded relative to the larger (edge
-// values have up to four spare bits: their squares lost eight, three times the FP64 form's error in
-// the energy residual)
-__host__ __device__ __forceinline__ XPair xpair_norm(long long l, long long r, int e) {
-  const int n = xclz32((int)((l ^ (l >> 63)) >> 32) | (int)((r ^ (r >> 63)) >> 32)) - 2;  // 0 .. 30
-  return {l << n, r << n, e - n};
 }
 // both edge values of a cell: u_{i+1/2} from the left, u_{i-1/2} from the right, class e, [62]
 struct XEdge {

@@ -1,0 +1,146 @@
+"""The block-floating arithmetic of the FP64 path (csrc/xfix.cuh) where values of very different size meet,
+compiled for the host.  The bar is the FP64 form's own error: the same formulas evaluated in doubles here, against
+long double, on the same inputs.  A component's root mean square error may be no larger than that
+form's and one rounding of the result to a double."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1710_09995_gb300", "csrc")
+ULP = 2.0 ** -53
+F64, LD = np.float64, np.longdouble
+_D = ctypes.POINTER(ctypes.c_double)
+_d = ctypes.c_double
+
+HARNESS = r"""
+#include <algorithm>
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#include "xfix.cuh"
+using namespace gbcfd;
+"""
+
+
+def _p(a):
+    return a.ctypes.data_as(_D)
+
+
+def compiled(tmp_path_factory, name, code):
+    d = tmp_path_factory.mktemp(name)
+    src, so = d / "x.cpp", d / "x.so"
+    src.write_text(HARNESS + code)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(so)], check=True)
+    return ctypes.CDLL(str(so))
+
+
+def rng(seed):
+    return np.random.Generator(np.random.PCG64(seed))
+
+
+def held(got, form, want):
+    """per component: the root mean square error against that of the FP64 form"""
+    got, form, want = (np.atleast_2d(x.T).T for x in (got, form, want))
+    for q in range(want.shape[1]):
+        rms = lambda x: float(np.sqrt(np.mean((x[:, q] / np.max(np.abs(want[:, q]) + LD(1e-300))) ** 2)))
+        a, b = rms(got.astype(LD) - want), rms(form.astype(LD) - want)
+        assert a <= b + ULP * rms(want), (q, a, b)
+
+
+def roe(L, R, gamma, eps, t):
+    """twice the Roe flux with Harten's fix in the face frame, columns (rho, un, ut1, ut2, p), evaluated in type t"""
+    l, r = L.astype(t).T, R.astype(t).T
+    gm1, ggm1 = t(float(gamma - 1.0)), t(float(gamma / (gamma - 1.0)))
+    h = lambda w: ggm1 * w[4] / w[0] + t(0.5) * (w[1] ** 2 + w[2] ** 2 + w[3] ** 2)
+    hl, hr, sl, sr = h(l), h(r), np.sqrt(l[0]), np.sqrt(r[0])
+    al, ar, rt = sl / (sl + sr), sr / (sl + sr), sl * sr
+    u, v, w, ht = (al * a + ar * b for a, b in ((l[1], r[1]), (l[2], r[2]), (l[3], r[3]), (hl, hr)))
+    q2 = u * u + v * v + w * w
+    c2 = gm1 * (ht - t(0.5) * q2)
+    c = np.sqrt(c2)
+    d = r - l
+    a1, a5 = (d[4] - rt * c * d[1]) / (2 * c2), (d[4] + rt * c * d[1]) / (2 * c2)
+    a2 = d[0] - d[4] / c2
+    delta = t(eps) * (abs(u) + c)
+    fix = lambda x: np.where(abs(x) < delta, (x * x + delta * delta) / (2 * np.where(delta > 0, delta, 1)), abs(x))
+    w1, w2, w5, l2 = fix(u - c) * a1, fix(u) * a2, fix(u + c) * a5, fix(u)
+    ml, mr, ws = l[0] * l[1], r[0] * r[1], w1 + w2 + w5
+    return np.stack([ml + mr - ws,
+                     (ml * l[1] + l[4]) + (mr * r[1] + r[4]) - (w1 * (u - c) + w2 * u + w5 * (u + c)),
+                     ml * l[2] + mr * r[2] - (ws * v + l2 * rt * d[2]),
+                     ml * l[3] + mr * r[3] - (ws * w + l2 * rt * d[3]),
+                     ml * hl + mr * hr - (w1 * (ht - c * u) + w5 * (ht + c * u) + w2 * t(0.5) * q2
+                                          + l2 * rt * (v * d[2] + w * d[3]))]).T
+
+
+def smooth(n, g, size=(1.0, 1.0, 1.0), jump=1e-2):
+    """both sides' (rho, u, v, w, p), velocities about `size`"""
+    u = lambda a=-1.0, b=1.0: g.uniform(a, b, n)
+    L = np.stack([1 + 0.1 * u(), size[0] * (0.5 + 0.1 * u()), size[1] * u(0.2, 0.4), size[2] * u(0.1, 0.3),
+                  (1 + 0.1 * u()) / 1.4], 1)
+    return np.ascontiguousarray(L), np.ascontiguousarray(L * (1 + jump * g.uniform(-1, 1, (n, 5))))
+
+
+# ---- faces with an area vector --------------------------------------------------------------------
+
+def roe_area(L, R, S, gamma, eps, t):
+    """the flux through S, x, y, z momentum: rotated into the face frame and back, as the FP64 form"""
+    s = S.astype(t)
+    area = np.sqrt((s * s).sum(1))
+    n = s / area[:, None]
+    a = np.abs(n).argmin(1)
+    e = np.eye(3)[a].astype(t)
+    na = np.take_along_axis(n, a[:, None], 1)
+    t1 = (e - na * n) / np.sqrt(1 - na * na)
+    t2 = np.cross(n, t1)
+    frame = lambda w: np.concatenate([w[:, :1].astype(t)] + [(w[:, 1:4].astype(t) * v).sum(1)[:, None] for v in (n, t1, t2)]
+                                     + [w[:, 4:].astype(t)], 1)
+    f = roe(frame(L), frame(R), gamma, eps, t)
+    m = f[:, 1:2] * n + f[:, 2:3] * t1 + f[:, 3:4] * t2
+    return np.concatenate([f[:, :1], m, f[:, 4:]], 1) * (t(0.5) * area)[:, None]
+
+
+@pytest.fixture(scope="module")
+def area_lib(tmp_path_factory):
+    return compiled(tmp_path_factory, "area", r"""
+extern "C" void flux(int n, const double* L, const double* R, const double* S, double gamma, double eps, double* F) {
+  const XConsts K = xconsts(gamma, eps);
+  for (int i = 0; i < n; ++i) {
+    const double *l = L + 5 * i, *r = R + 5 * i, *s = S + 3 * i;
+    XFlux f;
+    xroe_area(xpair(l[0], r[0]), xpair(l[1], r[1]), xpair(l[2], r[2]), xpair(l[3], r[3]), xpair(l[4], r[4]), s[0], s[1],
+              s[2], K, f);
+    for (int q = 0; q < 5; ++q) F[5 * i + q] = xflux(f, q, 0);
+  }
+}
+""")
+
+
+@pytest.mark.parametrize("size", [1.0, 1e-3, 1e-6, 1e-9])
+@pytest.mark.parametrize("faces", ["extruded", "aligned", "nearly aligned", "any"])
+def test_area_flux_of_small_components(area_lib, faces, size):
+    """one velocity component `size` times the others, on faces to which it is tangential (a grid extruded
+    in z, axis-aligned ones), nearly so, and on any"""
+    n, g = 6000, rng(3)
+    L, R = smooth(n, g, (1.0, 1.0, size))
+    S = g.uniform(0.2, 1.0, (n, 3)) * g.choice([-1.0, 1.0], (n, 3)) * 1e-3
+    if faces == "extruded":
+        S[:, 2] = 0.0
+    elif faces != "any":
+        off = ~np.eye(3, dtype=bool)[g.integers(0, 2, n)]
+        S[off] *= 0.0 if faces == "aligned" else 1e-9
+    F = np.empty((n, 5))
+    area_lib.flux(n, _p(L), _p(R), _p(np.ascontiguousarray(S)), _d(1.4), _d(0.1), _p(F))
+    held(F, roe_area(L, R, S, 1.4, 0.1, F64), roe_area(L, R, S, 1.4, 0.1, LD))
+
+
+def test_area_flux_of_no_velocity_along_z_is_zero_there(area_lib):
+    n, g = 500, rng(4)
+    L, R = smooth(n, g, (1.0, 1.0, 0.0))
+    S = np.stack([g.uniform(0.2, 1.0, n), g.uniform(0.2, 1.0, n), np.zeros(n)], 1)
+    F = np.empty((n, 5))
+    area_lib.flux(n, _p(L), _p(R), _p(S), _d(1.4), _d(0.1), _p(F))
+    assert np.all(F[:, 3] == 0.0)
