@@ -310,14 +310,15 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
                        xshr(xsq(wl), EHl - 2 * Ew - 2);  // [62]
   const long long hr = xshr(gr.m, EHr - gr.e) + xshr(xsq(ur), EHr - 2 * Eu - 2) + xshr(xsq(vr), EHr - 2 * Ev - 2) +
                        xshr(xsq(wr), EHr - 2 * Ew - 2);
-  // Roe averages: velocities in the classes of the sides [62]; enthalpy and q^2 / 2 in class EH [60]
+  // Roe averages: velocities in the classes of the sides [62]; enthalpy in class EH [60], q^2 / 2 in
+  // its own, Ek (in the enthalpies' the entropy wave's energy at a contact of 1 to 100 had 5e-15 of itself in error)
   const long long ut = (xmul(al, ul) + xmul(ar, ur)) << 2;
   const long long vt = (xmul(al, vl) + xmul(ar, vr)) << 2;
   const long long wt = (xmul(al, wl) + xmul(ar, wr)) << 2;
   const long long nt = CURVI ? (xmul(al, nl) + xmul(ar, nr)) << 2 : ut;
   const long long ht = xshr(xmul(al, hl), EH - EHl - 2) + xshr(xmul(ar, hr), EH - EHr - 2);
-  const long long q2 = xshr(xsq(ut), EH - 2 * Eu - 2) + xshr(xsq(vt), EH - 2 * Ev - 2) + xshr(xsq(wt), EH - 2 * Ew - 2);
-  const long long c2m = xmul(K.gm1.m, ht - q2);
+  const long long q2 = xshr(xsq(ut), Ek - 2 * Eu - 2) + xshr(xsq(vt), Ek - 2 * Ev - 2) + xshr(xsq(wt), Ek - 2 * Ew - 2);
+  const long long c2m = xmul(K.gm1.m, ht - xshr(q2, EH - Ek));
   const bool bad = r.l <= 0 || r.r <= 0 || c2m <= 0;
   // c^2 normalised, its reciprocal root, c
   const XVal c2 = xnormed(c2m, K.gm1.e + EH + 3);
@@ -325,24 +326,26 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const long long ic2 = xsq(ic.m) << 2;       // [62], class 2 ic.e + 1
   const long long cc = xmul(c2.m, ic.m) << 2;  // [62]
   const int Ec = c2.e + ic.e + 1;
-  // wave speeds; room for delta = eps (|u| + c) where eps >= 1
+  // wave speeds, |u_n| in its own class unless Harten's fix replaces it; room for delta = eps (|u| + c) where eps >= 1
   const int hx = K.eps.e >= 0 ? K.eps.e + 1 : 0;
   const int El = xmax(En, Ec) + 1 + hx;
   const long long ue = xshr(nt, El - En), ce = xshr(cc, El - Ec);  // [61]
-  long long l1 = xabs(ue - ce), l5 = xabs(ue + ce), l2 = xabs(ue);  // [62]
+  long long l1 = xabs(ue - ce), l5 = xabs(ue + ce);  // [62]
+  const long long ua = xabs(ue);
+  XVal l2 = {xabs(nt), En};
   {
-    long long d = xmul(K.eps.m, l2 + ce);  // class El + eps.e + 3
+    long long d = xmul(K.eps.m, ua + ce);  // class El + eps.e + 3
     d = K.eps.e >= -3 ? d << (K.eps.e + 3) : xshr(d, -3 - K.eps.e);  // [62]
-    if (l1 < d || l2 < d || l5 < d) {
+    if (l1 < d || ua < d || l5 < d) {
       const XHid hid = xhid(d);
       l1 = xharten(l1, d, hid);
-      l2 = xharten(l2, d, hid);
+      if (ua < d) l2 = {xharten(ua, d, hid), El};
       l5 = xharten(l5, d, hid);
     }
   }
   // jumps, normalised [62], and wave strengths: a1, a5 = (dp -+ rho c du) / (2 c^2), a2 = drho - dp / c^2
-  const XVal jr = xquick(r.r - r.l, r.e), ju = xquick(nr - nl, En), jv = xquick(vr - vl, Ev), jw = xquick(wr - wl, Ew),
-             jp = xquick(p.r - p.l, Ep);
+  const XVal jr = xquick0(r.r - r.l, r.e), ju = xquick(nr - nl, En), jv = xquick(vr - vl, Ev), jw = xquick(wr - wl, Ew),
+             jp = xquick0(p.r - p.l, Ep);
   const XVal rcd = xquick(xmul(xmul(rt.m, cc) << 2, ju.m), rt.e + Ec + ju.e + 4);
   const int Eq = xmax(rcd.e, jp.e) + 1;
   const long long dp = xshr(jp.m, Eq - jp.e), rq = xshr(rcd.m, Eq - rcd.e);               // [61]
@@ -353,13 +356,13 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const XVal s = xquick(w1 + w5, Ew15), dw = xquick(w5 - w1, Ew15);                       // [62]
   const int Ed = jp.e + 2 * ic.e + 4, EA = xmax(Ed, jr.e + 2);
   const XVal a2 = xquick(xshr(jr.m, EA - jr.e) - xshr(xmul(jp.m, ic2), EA - Ed), EA);
-  const XVal w2 = xquick(xmul(l2, a2.m), El + a2.e + 3);                                  // [62]
+  const XVal w2 = xquick(xmul(l2.m, a2.m), l2.e + a2.e + 3);                              // [62]
   // in the class of the mass fluxes [60]
   const int EM = xmax(xmax(Eml, Emr), xmax(s.e, w2.e) + 3);
   const long long fl = xshr(ml, EM - Eml), fr = xshr(mr, EM - Emr);
   const long long ws = xshr(s.m, EM - s.e) + xshr(w2.m, EM - w2.e);
   const long long dq = xmul(dw.m, cc);                                  // [60]
-  const XVal lrt = xquick(xmul(l2, rt.m), El + rt.e + 3);               // [62]
+  const XVal lrt = xquick(xmul(l2.m, rt.m), l2.e + rt.e + 3);           // [62]
   const long long g1 = xmul(lrt.m, jv.m), g2 = xmul(lrt.m, jw.m);       // [60]
   const int Edq = dw.e + Ec + 3, Eg1 = lrt.e + jv.e + 3, Eg2 = lrt.e + jw.e + 3;
   const long long a1m = xmul(fl, ul) + xmul(fr, ur) - xmul(ws, ut);  // [60]
@@ -367,7 +370,7 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const long long a3m = xmul(fl, wl) + xmul(fr, wr) - xmul(ws, wt);
   const int f1 = EM + Eu + 3, f2 = EM + Ev + 3, f3 = EM + Ew + 3;
   const int el = Eml + EHl + 3, er = Emr + EHr + 3, e1 = s.e + EH + 3, e2 = Edq + En + 3, e3 = Eg1 + Ev + 3, e4 = Eg2 + Ew + 3,
-            e5 = w2.e + EH + 3;
+            e5 = w2.e + Ek + 3;
   const int E4 = xmax(xmax(xmax(el, er), xmax(e1, e2)), xmax(xmax(e3, e4), e5));
   const long long a4 = xshr(xmul(ml, hl), E4 - el) + xshr(xmul(mr, hr), E4 - er);  // terms [58]
   const long long b4 = xshr(xmul(s.m, ht), E4 - e1) + xshr(xmul(w2.m, q2), E4 - e5);

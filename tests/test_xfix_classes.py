@@ -144,3 +144,35 @@ def test_area_flux_of_no_velocity_along_z_is_zero_there(area_lib):
     F = np.empty((n, 5))
     area_lib.flux(n, _p(L), _p(R), _p(S), _d(1.4), _d(0.1), _p(F))
     assert np.all(F[:, 3] == 0.0)
+
+
+# ---- the flux in the face frame -------------------------------------------------------------------
+
+@pytest.fixture(scope="module")
+def roe_lib(tmp_path_factory):
+    return compiled(tmp_path_factory, "roe", r"""
+extern "C" void flux(int n, const double* L, const double* R, double gamma, double eps, double* F) {
+  const XConsts K = xconsts(gamma, eps);
+  for (int i = 0; i < n; ++i) {
+    const double *l = L + 5 * i, *r = R + 5 * i;
+    XFlux f;
+    xroe(xpair(l[0], r[0]), xpair(l[1], r[1]), xpair(l[2], r[2]), xpair(l[3], r[3]), xpair(l[4], r[4]), K, f);
+    for (int q = 0; q < 5; ++q) F[5 * i + q] = xflux(f, q, 0);
+  }
+}
+""")
+
+
+@pytest.mark.parametrize("eps", [0.1, 0.0])
+@pytest.mark.parametrize("mach", [1.0, 1e-3, 1e-6])
+@pytest.mark.parametrize("ratio", [1.01, 2.0, 10.0, 30.0])
+def test_contact(roe_lib, ratio, mach, eps):
+    """a jump of the density alone: the entropy wave's kinetic energy is far below the enthalpies, its speed
+    below the sound speed"""
+    n, g = 6000, rng(5)
+    L, _ = smooth(n, g, (mach, mach, mach))
+    R = L.copy()
+    R[:, 0] *= np.where(g.random(n) < 0.5, ratio, 1 / ratio)
+    F = np.empty((n, 5))
+    roe_lib.flux(n, _p(L), _p(R), _d(1.4), _d(eps), _p(F))
+    held(F, roe(L, R, 1.4, eps, F64), roe(L, R, 1.4, eps, LD))
