@@ -22,20 +22,10 @@ struct MetIdx {
   int vl, vr;
 };
 
-template <typename T, bool VISC, int BY>
-__device__ __forceinline__ void face_flux_curvi(const T* __restrict__ ring, const T* __restrict__ mring,
-                                                int nv_ms, const int (&b)[4], const int (&tg)[8],
-                                                const MetIdx& mi, const Consts<T>& K, T* F) {
+// the Roe flux through the area vector S from the sides' (rho, u, v, w, p), x, y, z momentum
+template <typename T>
+__device__ __forceinline__ void roe_area(const T* L, const T* R, const T (&S)[3], const Consts<T>& K, T* F) {
   using O = VM<T>;
-  constexpr int MS = BY * BX;
-  (void)nv_ms;
-  T L[5], R[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    const int m = q * MS;
-    muscl(ring[b[0] + m], ring[b[1] + m], ring[b[2] + m], ring[b[3] + m], K.lim, L[q], R[q]);
-  }
-  const T S[3] = {mring[mi.sf], mring[mi.sf + MS], mring[mi.sf + 2 * MS]};
   const T s2 = O::fma(S[0], S[0], O::fma(S[1], S[1], S[2] * S[2]));
   const T ia = O::rsqrt(s2);
   const T area = s2 * ia;
@@ -67,6 +57,23 @@ __device__ __forceinline__ void face_flux_curvi(const T* __restrict__ ring, cons
 #pragma unroll
   for (int x = 0; x < 3; ++x) F[1 + x] = ha * O::fma(Fr[1], n[x], O::fma(Fr[2], t1[x], Fr[3] * t2[x]));
   F[4] = ha * Fr[4];
+}
+
+template <typename T, bool VISC, int BY>
+__device__ __forceinline__ void face_flux_curvi(const T* __restrict__ ring, const T* __restrict__ mring,
+                                                int nv_ms, const int (&b)[4], const int (&tg)[8],
+                                                const MetIdx& mi, const Consts<T>& K, T* F) {
+  using O = VM<T>;
+  constexpr int MS = BY * BX;
+  (void)nv_ms;
+  T L[5], R[5];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    const int m = q * MS;
+    muscl(ring[b[0] + m], ring[b[1] + m], ring[b[2] + m], ring[b[3] + m], K.lim, L[q], R[q]);
+  }
+  const T S[3] = {mring[mi.sf], mring[mi.sf + MS], mring[mi.sf + 2 * MS]};
+  roe_area<T>(L, R, S, K, F);
 
   if constexpr (VISC) {
     constexpr int TH = 5 * MS;

@@ -70,12 +70,6 @@ static_assert(sizeof(XBlk) == 20 * sizeof(XVal), "XPlan::blk");
 // ring values are 61-bit integers with a biased exponent: value = m 2^(e - 1022 - 61)
 constexpr int XRING_BIAS = 1022;
 
-// half the minmod slope's double: 0 when a and b differ in sign, else the one of smaller magnitude
-__device__ __forceinline__ long long xminmod(long long a, long long b) {
-  const long long r = ((a < b) != (a < 0)) ? a : b;
-  return (a ^ b) < 0 ? 0ll : r;
-}
-
 // one warp item's index data: cells c[0..3] along the normal (c[1] = L, c[2] = R) as indices into
 // variable 0 of the ring; variable offsets of the normal and tangential velocities; tangential
 // neighbours (added to c[1], c[2])
@@ -85,41 +79,70 @@ struct XItem {
   int t1p, t1m, t2p, t2m;
 };
 
+// a face whose sides are far apart (xfar) in FP64, from the stencil's values rounded to doubles: twice the flux
+// (CURVI: the flux).  Out of line: only faces with a jump of 2^5 or more in the density or the pressure call it.
+template <bool CURVI, int MS>
+__device__ __noinline__ XFlux xface_f64(const long long* rm, const short* re, int c0, int c1, int c2, int c3, int vn, int v1,
+                                        int v2, const double* S, double gm1, double ggm1, double eps, int lim) {
+  const int at[4] = {c0, c1, c2, c3}, var[5] = {0, vn, v1, v2, 4 * MS};
+  Consts<double> K;
+  K.gm1 = gm1;
+  K.ggm1 = ggm1;
+  K.eps = eps;
+  double L[5], R[5], F[5];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    double x[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) x[c] = xenc(rm[at[c] + var[q]], re[at[c] + var[q]] - XRING_BIAS);
+    muscl(x[0], x[1], x[2], x[3], lim, L[q], R[q]);
+  }
+  if constexpr (CURVI) {
+    const double a[3] = {S[0], S[MS], S[2 * MS]};
+    roe_area<double>(L, R, a, K, F);
+  } else {
+    roe_frame<double, true>(L, R, K, F);
+  }
+  return xflux_of(F);
+}
+
 // twice the flux (F - Fv) through the lane's face; CURVI: the flux, S its area vector (strides MS)
 template <bool VISC, bool CURVI, int MS>
 __device__ __forceinline__ void xface(const long long* __restrict__ rm, const short* __restrict__ re, const XItem& I,
                                       int d, const XBlk* __restrict__ X, const double* __restrict__ S,
-                                      const XConsts& K, int lim, XFlux& F) {
+                                      const XConsts& K, const PathK<double>& PK, int lim, XFlux& F) {
   long long dn[3];  // R - L of the velocities (viscous)
   long long us[3];
   int eu[3];
-  // MUSCL in the class of the stencil's largest exponent; states doubled (class e - 1) with minmod
-  auto states = [&](int off, int q) -> XPair {
-    int e[4];
-    long long m[4];
+  auto load = [&](const int (&ix)[4], int off, long long (&m)[4], int (&e)[4]) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      m[c] = rm[I.c[c] + off];
-      e[c] = re[I.c[c] + off];
+      m[c] = rm[ix[c] + off];
+      e[c] = re[ix[c] + off];
     }
-    const int E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3]));
-#pragma unroll
-    for (int c = 0; c < 4; ++c) m[c] = xshr(m[c], E - e[c]);  // [61]
-    const long long d01 = m[1] - m[0], d12 = m[2] - m[1], d23 = m[3] - m[2];
-    if (VISC && q >= 0) {
-      dn[q] = d12;
-      us[q] = m[1] + m[2];
-      eu[q] = E - XRING_BIAS;
-    }
-    if (lim) return {m[1] + ((d01 + d12) >> 2), m[2] - ((d12 + d23) >> 2), E - XRING_BIAS};
-    return {2 * m[1] + xminmod(d01, d12), 2 * m[2] - xminmod(d12, d23), E - XRING_BIAS - 1};
   };
-  const XPair r = states(0, -1), u = states(I.vn, 0), v = states(I.v1, 1), w = states(I.v2, 2), p = states(4 * MS, -1);
-  if constexpr (CURVI) {
+  auto states = [&](int off, int q) -> XPair {
+    long long m[4];
+    int e[4];
+    load(I.c, off, m, e);
+    XSten s = xmuscl(m, e, lim);
+    if (VISC && q >= 0) {
+      dn[q] = s.d;
+      us[q] = s.sum;
+      eu[q] = s.ed - XRING_BIAS;
+    }
+    s.s.e -= XRING_BIAS;
+    return s.s;
+  };
+  const XPos r = states(0, -1), p = states(4 * MS, -1);
+  const XPair u = states(I.vn, 0), v = states(I.v1, 1), w = states(I.v2, 2);
+  if (xfar(r, p)) {
+    F = xface_f64<CURVI, MS>(rm, re, I.c[0], I.c[1], I.c[2], I.c[3], I.vn, I.v1, I.v2, S, PK.gm1, PK.ggm1, PK.eps, lim);
+  } else if constexpr (CURVI) {
     xroe_area(r, u, v, w, p, S[0], S[MS], S[2 * MS], K, F);
-    return;
+  } else {
+    xroe(r, u, v, w, p, K, F);
   }
-  xroe(r, u, v, w, p, K, F);
   if constexpr (VISC) {
     // sum over the two cells of the central differences of a variable along a tangent, [62]
     auto tang = [&](int off, int tp, int tm, int& E) -> long long {
@@ -511,7 +534,7 @@ __global__ void __launch_bounds__(32 * NWV, 1) xstage_kernel(const GroupParams P
           S = mring + ((d == 2 ? k + 1 : k) & 1) * (PL::MSLOT / sizeof(double)) + 3 * d * MS + (row + HALO) * BX + col + HALO;
         }
         XFlux F;
-        xface<VISC, CURVI, MS>(rm, re, I, d, xb, S, XK, ph.limiter, F);
+        xface<VISC, CURVI, MS>(rm, re, I, d, xb, S, XK, P.pk.d, ph.limiter, F);
         const int f = d == 2 ? zslot(k) + row * TX + col
                              : (d == 1 ? PL::FY0 + xslot(k) * PL::NFY + row * TX + col
                                        : xslot(k) * PL::NFX + row * (TX + 1) + col);

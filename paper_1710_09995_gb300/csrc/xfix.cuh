@@ -264,6 +264,18 @@ __host__ __device__ __forceinline__ XPair xpair_norm(long long l, long long r, i
   const int n = xclz32((int)((l ^ (l >> 63)) >> 32) | (int)((r ^ (r >> 63)) >> 32)) - 2;  // 0 .. 30
   return {l << n, r << n, e - n};
 }
+// a positive variable's sides: the pair, and either side by itself, normalised to [62]
+struct XPos {
+  XPair c;
+  XVal l, r;
+  __host__ __device__ __forceinline__ XPos(const XPair& p) : c(p), l(xquick(p.l, p.e)), r(xquick(p.r, p.e)) {}
+};
+// sides so far apart (more than 2^5) that the smaller one's bits in the pair's class, or its products in the
+// classes of the larger one's, may be fewer than a double's: such a face is left to FP64
+__host__ __device__ __forceinline__ bool xfar(const XPos& r, const XPos& p) {
+  const int a = r.l.e - r.r.e, b = p.l.e - p.r.e;
+  return a > 5 || a < -5 || b > 5 || b < -5;
+}
 // twice a face flux, each component in its own class, [62]; where a density or c^2 is not
 // positive the exponents are XBAD or more (NaN)
 struct XFlux {
@@ -282,14 +294,14 @@ struct XFlux {
 // the shear jumps are du - dun n, so the momentum flux is a x, y, z vector and needs no
 // tangents.
 template <bool CURVI>
-__host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, const XPair& v, const XPair& w,
-                                              const XPair& p, const XConsts& K, XFlux& F, const XPair& un,
+__host__ __device__ __forceinline__ void xroe(const XPos& r, const XPair& u, const XPair& v, const XPair& w,
+                                              const XPos& p, const XConsts& K, XFlux& F, const XPair& un,
                                               const XVal* n) {
-  const int Eu = u.e, Ev = v.e, Ew = w.e, Ep = p.e, En = CURVI ? un.e : Eu;
+  const int Eu = u.e, Ev = v.e, Ew = w.e, Ep = p.c.e, En = CURVI ? un.e : Eu;
   const long long ul = u.l, ur = u.r, vl = v.l, vr = v.r, wl = w.l, wr = w.r;
   // densities and pressures by themselves; reciprocal roots; the Roe weights a_l = isr iw,
   // a_r = isl iw with iw = 1 / (isl + isr), class -1 (below 1, so [62])
-  const XVal rl = xnormed(r.l, r.e), rr = xnormed(r.r, r.e), pl = xnormed(p.l, p.e), pr = xnormed(p.r, p.e);  // [62]
+  const XVal rl = r.l, rr = r.r, pl = p.l, pr = p.r;  // [62]
   const XVal isl = xrsqrt(rl), isr = xrsqrt(rr);
   const int Ei = xmax(isl.e, isr.e) + 1;
   const XVal iw = xrcp(xnormed(xshr(isl.m, Ei - isl.e) + xshr(isr.m, Ei - isr.e), Ei));
@@ -299,8 +311,7 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const XVal rt = xquick(xmul(xmul(rl.m, isl.m) << 2, xmul(rr.m, isr.m) << 2), rl.e + isl.e + rr.e + isr.e + 5);  // [62]
   // mass fluxes
   const long long nl = CURVI ? un.l : ul, nr = CURVI ? un.r : ur;
-  const long long ml = xmul(rl.m, nl), mr = xmul(rr.m, nr);  // [60]
-  const int Eml = rl.e + En + 3, Emr = rr.e + En + 3;
+  const XVal ml = xquick(xmul(rl.m, nl), rl.e + En + 3), mr = xquick(xmul(rr.m, nr), rr.e + En + 3);  // [62]
   // enthalpies gamma/(gamma-1) p / rho + |u|^2 / 2, each side in its own class
   const XVal gl = xquick(xmul(K.ggm1.m, xmul(pl.m, xsq(isl.m) << 2) << 2), K.ggm1.e + pl.e + 2 * isl.e + 5);  // [62]
   const XVal gr = xquick(xmul(K.ggm1.m, xmul(pr.m, xsq(isr.m) << 2) << 2), K.ggm1.e + pr.e + 2 * isr.e + 5);
@@ -319,7 +330,7 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const long long ht = xshr(xmul(al, hl), EH - EHl - 2) + xshr(xmul(ar, hr), EH - EHr - 2);
   const long long q2 = xshr(xsq(ut), Ek - 2 * Eu - 2) + xshr(xsq(vt), Ek - 2 * Ev - 2) + xshr(xsq(wt), Ek - 2 * Ew - 2);
   const long long c2m = xmul(K.gm1.m, ht - xshr(q2, EH - Ek));
-  const bool bad = r.l <= 0 || r.r <= 0 || c2m <= 0;
+  const bool bad = r.c.l <= 0 || r.c.r <= 0 || c2m <= 0;
   // c^2 normalised, its reciprocal root, c
   const XVal c2 = xnormed(c2m, K.gm1.e + EH + 3);
   const XVal ic = xrsqrt(c2);
@@ -344,8 +355,8 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
     }
   }
   // jumps, normalised [62], and wave strengths: a1, a5 = (dp -+ rho c du) / (2 c^2), a2 = drho - dp / c^2
-  const XVal jr = xquick0(r.r - r.l, r.e), ju = xquick(nr - nl, En), jv = xquick(vr - vl, Ev), jw = xquick(wr - wl, Ew),
-             jp = xquick0(p.r - p.l, Ep);
+  const XVal jr = xquick0(r.c.r - r.c.l, r.c.e), ju = xquick(nr - nl, En), jv = xquick(vr - vl, Ev),
+             jw = xquick(wr - wl, Ew), jp = xquick0(p.c.r - p.c.l, Ep);
   const XVal rcd = xquick(xmul(xmul(rt.m, cc) << 2, ju.m), rt.e + Ec + ju.e + 4);
   const int Eq = xmax(rcd.e, jp.e) + 1;
   const long long dp = xshr(jp.m, Eq - jp.e), rq = xshr(rcd.m, Eq - rcd.e);               // [61]
@@ -358,8 +369,8 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const XVal a2 = xquick(xshr(jr.m, EA - jr.e) - xshr(xmul(jp.m, ic2), EA - Ed), EA);
   const XVal w2 = xquick(xmul(l2.m, a2.m), l2.e + a2.e + 3);                              // [62]
   // in the class of the mass fluxes [60]
-  const int EM = xmax(xmax(Eml, Emr), xmax(s.e, w2.e) + 3);
-  const long long fl = xshr(ml, EM - Eml), fr = xshr(mr, EM - Emr);
+  const int EM = xmax(xmax(ml.e, mr.e), xmax(s.e, w2.e)) + 2;
+  const long long fl = xshr(ml.m, EM - ml.e), fr = xshr(mr.m, EM - mr.e);
   const long long ws = xshr(s.m, EM - s.e) + xshr(w2.m, EM - w2.e);
   const long long dq = xmul(dw.m, cc);                                  // [60]
   const XVal lrt = xquick(xmul(l2.m, rt.m), l2.e + rt.e + 3);           // [62]
@@ -369,10 +380,10 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
   const long long a2m = xmul(fl, vl) + xmul(fr, vr) - xmul(ws, vt);
   const long long a3m = xmul(fl, wl) + xmul(fr, wr) - xmul(ws, wt);
   const int f1 = EM + Eu + 3, f2 = EM + Ev + 3, f3 = EM + Ew + 3;
-  const int el = Eml + EHl + 3, er = Emr + EHr + 3, e1 = s.e + EH + 3, e2 = Edq + En + 3, e3 = Eg1 + Ev + 3, e4 = Eg2 + Ew + 3,
+  const int el = ml.e + EHl + 3, er = mr.e + EHr + 3, e1 = s.e + EH + 3, e2 = Edq + En + 3, e3 = Eg1 + Ev + 3, e4 = Eg2 + Ew + 3,
             e5 = w2.e + Ek + 3;
   const int E4 = xmax(xmax(xmax(el, er), xmax(e1, e2)), xmax(xmax(e3, e4), e5));
-  const long long a4 = xshr(xmul(ml, hl), E4 - el) + xshr(xmul(mr, hr), E4 - er);  // terms [58]
+  const long long a4 = xshr(xmul(ml.m, hl), E4 - el) + xshr(xmul(mr.m, hr), E4 - er);  // terms [60]
   const long long b4 = xshr(xmul(s.m, ht), E4 - e1) + xshr(xmul(w2.m, q2), E4 - e5);
   long long d4 = xshr(xmul(dq, nt), E4 - e2) + xshr(xmul(g1, vt), E4 - e3) + xshr(xmul(g2, wt), E4 - e4);
   F.m[0] = fl + fr - ws;
@@ -381,7 +392,7 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
     F.e[1] = xmax(xmax(f1, Edq), Ep + 2);
     F.e[2] = xmax(f2, Eg1);
     F.e[3] = xmax(f3, Eg2);
-    F.m[1] = xshr(a1m, F.e[1] - f1) + xshr(p.l + p.r, F.e[1] - Ep) - xshr(dq, F.e[1] - Edq);
+    F.m[1] = xshr(a1m, F.e[1] - f1) + xshr(p.c.l + p.c.r, F.e[1] - Ep) - xshr(dq, F.e[1] - Edq);
     F.m[2] = xshr(a2m, F.e[2] - f2) - xshr(g1, F.e[2] - Eg1);
     F.m[3] = xshr(a3m, F.e[3] - f3) - xshr(g2, F.e[3] - Eg2);
   } else {
@@ -389,7 +400,7 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
     const long long g0 = xmul(lrt.m, jx.m), gn = xmul(lrt.m, ju.m);  // [60]
     const int Eg0 = lrt.e + jx.e + 3, Egn = lrt.e + ju.e + 3;
     const int EP = xmax(xmax(Edq, Egn), Ep + 2);
-    const XVal P = xquick(xshr(p.l + p.r, EP - Ep) - xshr(dq, EP - Edq) + xshr(gn, EP - Egn), EP);  // along n, [62]
+    const XVal P = xquick(xshr(p.c.l + p.c.r, EP - Ep) - xshr(dq, EP - Edq) + xshr(gn, EP - Egn), EP);  // along n, [62]
     const int p0 = P.e + n[0].e + 3, p1 = P.e + n[1].e + 3, p2 = P.e + n[2].e + 3;                   // P n_x [60]
     F.e[1] = xmax(xmax(f1, p0), Eg0);
     F.e[2] = xmax(xmax(f2, p1), Eg1);
@@ -411,8 +422,8 @@ __host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, co
     F.e[0] = F.e[1] = F.e[2] = F.e[3] = F.e[4] = 2 * XBAD;
   }
 }
-__host__ __device__ __forceinline__ void xroe(const XPair& r, const XPair& u, const XPair& v, const XPair& w,
-                                              const XPair& p, const XConsts& K, XFlux& F) {
+__host__ __device__ __forceinline__ void xroe(const XPos& r, const XPair& u, const XPair& v, const XPair& w,
+                                              const XPos& p, const XConsts& K, XFlux& F) {
   xroe<false>(r, u, v, w, p, K, F, u, nullptr);
 }
 
@@ -436,8 +447,8 @@ __host__ __device__ __forceinline__ XNormal xnormal(double sx, double sy, double
 
 // twice the flux through a face of area vector (sx, sy, sz) from the sides' (rho, u, v, w, p), x, y, z
 // momentum, times half the area: the face flux itself
-__host__ __device__ __forceinline__ void xroe_area(const XPair& r, const XPair& u, const XPair& v, const XPair& w,
-                                                   const XPair& p, double sx, double sy, double sz, const XConsts& K,
+__host__ __device__ __forceinline__ void xroe_area(const XPos& r, const XPair& u, const XPair& v, const XPair& w,
+                                                   const XPos& p, double sx, double sy, double sz, const XConsts& K,
                                                    XFlux& F) {
   const XNormal N = xnormal(sx, sy, sz);
   // the velocities along n, in the class of the largest product ([60] each)
@@ -457,10 +468,55 @@ __host__ __device__ __forceinline__ void xroe_area(const XPair& r, const XPair& 
   }
 }
 
+// a flux given in doubles
+__host__ __device__ __forceinline__ XFlux xflux_of(const double* f) {
+  XFlux F;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int q = 0; q < 5; ++q) {
+    const XVal v = xdec_zero(f[q]);
+    F.m[q] = v.m;
+    F.e[q] = v.e < 1024 ? v.e : 2 * XBAD;
+  }
+  return F;
+}
 // a flux component as a double, times 2^-h
 __host__ __device__ __forceinline__ double xflux(const XFlux& F, int q, int h) {
   return xenc(F.m[q], F.e[q] - h);
 }
+// ---- MUSCL ---------------------------------------------------------------------------------------
+// half the minmod slope's double: 0 when a and b differ in sign, else the one of smaller magnitude
+__host__ __device__ __forceinline__ long long xminmod(long long a, long long b) {
+  const long long r = ((a < b) != (a < 0)) ? a : b;
+  return (a ^ b) < 0 ? 0ll : r;
+}
+// the sides of the face between cells 1 and 2 of a stencil of four [61] (normalised but for zeros and the
+// smallest doubles) and for the viscous flux the difference and the sum of these two, class ed
+struct XSten {
+  XPair s;
+  long long d, sum;
+  int ed;
+};
+// With minmod the states lie between cells 1 and 2 and keep their class: a cell 0 or 3 that is larger by
+// more than 2^4 only has to give a slope larger than theirs, which it also does shifted into 2^4 times
+// that class (|m| >= 2^59 against a difference below 2^58).  In the class of all four a state beside a jump
+// had lost as many bits as the jump is high, less 8.  Doubled (class e - 1); with the central slope, where
+// the larger cell is a term of the state, the class of all four, not doubled.
+__host__ __device__ __forceinline__ XSten xmuscl(const long long (&m)[4], const int (&e)[4], int lim) {
+  const int Ei = xmax(e[1], e[2]), Eo = xmax(e[0], e[3]), Ec = Ei + 4, E = xmax(Ei, lim || Eo < Ec ? Eo : Ec);
+  const long long m0 = xshr(m[0], xmax(E - e[0], 0)), m1 = xshr(m[1], E - e[1]), m2 = xshr(m[2], E - e[2]),
+                  m3 = xshr(m[3], xmax(E - e[3], 0));
+  const long long d01 = m1 - m0, d12 = m2 - m1, d23 = m3 - m2;
+  XSten S;
+  S.d = d12;
+  S.sum = m1 + m2;
+  S.ed = E;
+  if (lim) S.s = xpair_norm(m1 + ((d01 + d12) >> 2), m2 - ((d12 + d23) >> 2), E);
+  else S.s = {(2 * m1 + xminmod(d01, d12)) << (E - Ei), (2 * m2 - xminmod(d12, d23)) << (E - Ei), Ei - 1};
+  return S;
+}
+
 // both sides of one variable from doubles
 __host__ __device__ __forceinline__ XPair xpair(double l, double r) {
   const XVal a = xdec<62>(l), b = xdec<62>(r);
@@ -491,7 +547,7 @@ __host__ __device__ __forceinline__ bool xprim(const double* q, const XConsts& K
   }
   const int Ek = xmax(xmax(ek[0], ek[1]), xmax(ek[2], E.e + 2));
   const long long d = xshr(E.m, Ek - E.e) - xshr(k[0], Ek - ek[0]) - xshr(k[1], Ek - ek[1]) - xshr(k[2], Ek - ek[2]);
-  W.p = xquick(xmul(K.gm1.m, d), K.gm1.e + Ek + 3);
+  W.p = xnormed(xmul(K.gm1.m, d), K.gm1.e + Ek + 3);
   const long long br = (long long)xbits(q[0]);
   // a non-finite momentum or energy has the exponent 1024
   return br > 0 && br < 0x7ff0000000000000ll && W.p.m > 0 && E.e < 1024 && W.u[0].e - W.ir.e < 1025 &&

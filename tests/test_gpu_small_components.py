@@ -168,3 +168,33 @@ def test_spanwise_momentum_on_an_extruded_grid(gb, size):
     c.nodes = curved_in_the_plane(c.nx, c.ny, c.nz)
     err = by_component(gpu_residual(gb.block_for_case(c, precision=gb.FP64)), fv_residual(c, *plane_metrics(c.nodes)))
     assert max(err) <= COMPONENT, err
+
+
+# ---- a strong jump --------------------------------------------------------------------------------
+
+def halves(n=(48, 8, 8), seed=9):
+    """a smooth slow state with density and pressure 1 for x < 1/2, 1e-4 and 1e-7 beyond (and the jump back at the
+    periodic boundary); the size of a residual's components in each cell, from the cell's own state"""
+    nx, ny, nz = n
+    c = cases.smooth_random(nx, ny, nz, seed=seed, amp=0.1)
+    w = np.stack([c.state[0], *(c.state[1:4] / c.state[0]), 0.4 * (c.state[4] - 0.5 * (c.state[1:4] ** 2).sum(0) / c.state[0])])
+    w[1:4] *= 1e-2
+    w[0, :, :, nx // 2:] *= 1e-4
+    w[4, :, :, nx // 2:] *= 1e-7
+    c.state = cases.conserved(*w)
+    s = np.abs(w[1:4]).sum(0) + np.sqrt(1.4 * w[4] / w[0])
+    return c, np.stack([w[0] * s, w[0] * s * s, w[0] * s * s, w[0] * s * s, w[0] * s ** 3]) / min(c.spacing)
+
+
+@pytest.mark.parametrize("curved", [False, True])
+def test_cells_beside_a_jump(gb, curved):
+    """every face at the jump, and those whose stencil it enters from beyond; in cells of the low side that have no face at
+    it errors stay relative to that side (some 100 roundings of 1.1e-16)"""
+    c, size = halves()
+    if curved:
+        c.nodes = curved_in_the_plane(c.nx, c.ny, c.nz)
+    ref = fv_residual(c, *(plane_metrics(c.nodes) if curved else cartesian(c)))
+    R = gpu_residual(gb.block_for_case(c, precision=gb.FP64))
+    assert max(by_component(R, ref)) <= COMPONENT
+    low = slice(c.nx // 2 + 1, c.nx - 1)
+    assert np.all(np.abs(R - ref)[..., low] <= COMPONENT * size[..., low])

@@ -176,3 +176,113 @@ def test_contact(roe_lib, ratio, mach, eps):
     F = np.empty((n, 5))
     roe_lib.flux(n, _p(L), _p(R), _d(1.4), _d(eps), _p(F))
     held(F, roe(L, R, 1.4, eps, F64), roe(L, R, 1.4, eps, LD))
+
+
+# ---- states beside jumps --------------------------------------------------------------------------
+
+@pytest.fixture(scope="module")
+def muscl_lib(tmp_path_factory):
+    return compiled(tmp_path_factory, "muscl", r"""
+static XPair states(const double* w, int lim) {
+  long long m[4];
+  int e[4];
+  for (int c = 0; c < 4; ++c) {
+    const XVal v = xdec_zero(w[c]);
+    m[c] = v.m >> 1;
+    e[c] = v.e + 1;
+  }
+  return xmuscl(m, e, lim).s;
+}
+extern "C" void muscl(int n, const double* w, int lim, double* LR) {
+  for (int i = 0; i < n; ++i) {
+    const XPair s = states(w + 4 * i, lim);
+    LR[2 * i] = xenc(s.l, s.e);
+    LR[2 * i + 1] = xenc(s.r, s.e);
+  }
+}
+extern "C" void flux(int n, const double* w, int lim, double* F, int* far) {  // w[i][variable][cell]
+  const XConsts K = xconsts(1.4, 0.1);
+  for (int i = 0; i < n; ++i) {
+    const double* a = w + 20 * i;
+    const XPos r = states(a, lim), p = states(a + 16, lim);
+    far[i] = xfar(r, p);
+    XFlux f;
+    xroe(r, states(a + 4, lim), states(a + 8, lim), states(a + 12, lim), p, K, f);
+    for (int q = 0; q < 5; ++q) F[5 * i + q] = xflux(f, q, 0);
+  }
+}
+""")
+
+
+def muscl(w, lim, t):
+    w = w.astype(t)
+    d01, d12, d23 = (w[..., i + 1] - w[..., i] for i in range(3))
+    if lim:
+        return w[..., 1] + t(0.25) * (d01 + d12), w[..., 2] - t(0.25) * (d12 + d23)
+    mm = lambda a, b: np.where((a > 0) == (b > 0), np.where(abs(a) < abs(b), a, b), t(0)) * ((a != 0) & (b != 0))
+    return w[..., 1] + t(0.5) * mm(d01, d12), w[..., 2] - t(0.5) * mm(d12, d23)
+
+
+@pytest.mark.parametrize("lim", [0, 1])
+@pytest.mark.parametrize("outer", [1.0, 3.0, 1e2, 1e6, 1e12, 0.0])
+def test_states_beside_a_jump(muscl_lib, outer, lim):
+    """cells 1 and 2 about 1, cell 0 or 3 (or both) `outer` times that, of either sign; with the central slope a state
+    takes the jump in, and only then may its error be relative to that"""
+    n, g = 8000, rng(7)
+    w = 1.0 + 0.1 * g.uniform(-1, 1, (n, 4))
+    for c in (0, 3):
+        w[g.random(n) < 0.7, c] *= outer * g.choice([-1.0, 1.0])
+    w = np.ascontiguousarray(w)
+    out = np.empty((n, 2))
+    muscl_lib.muscl(n, _p(w), lim, _p(out))
+    L, R = muscl(w, lim, LD)
+    want = np.stack([L, R], 1)
+    size = np.abs(w[:, 1:3]).max(1, keepdims=True) if not lim else np.abs(w).max(1, keepdims=True)
+    # the value and half a slope are rounded once each (FP64 form); the pair shares a class
+    assert np.all(np.abs(out - want) <= 2 * ULP * (np.abs(want) + size))
+
+
+@pytest.mark.parametrize("where", [0, 3])
+@pytest.mark.parametrize("jump", [10.0, 1e3, 1e6])
+def test_flux_beside_a_jump(muscl_lib, jump, where):
+    """the face's own cells are smooth, the cell beyond is `jump` times them in every variable"""
+    n, g = 6000, rng(8)
+    L, _ = smooth(n, g)
+    w = np.stack([L * (1 + 1e-2 * g.uniform(-1, 1, (n, 5))) for _ in range(4)], 2)
+    w[:, :, where] *= jump
+    w = np.ascontiguousarray(w)
+    F, far = np.empty((n, 5)), np.zeros(n, dtype=np.int32)
+    muscl_lib.flux(n, _p(w), 0, _p(F), far.ctypes.data_as(ctypes.c_void_p))
+    assert not far.any()
+    sides = lambda t: muscl(w, 0, t)
+    held(F, roe(*sides(F64), 1.4, 0.1, F64), roe(*sides(LD), 1.4, 0.1, LD))
+
+
+@pytest.mark.parametrize("v", [0, 4])
+def test_faces_far_apart_are_told(muscl_lib, v):
+    """a density or pressure jump of 2^7 and more at the face itself is left to FP64, one below 2^4 is not"""
+    n, g = 2000, rng(9)
+    for ratio, far_wanted in ((8.0, False), (128.0, True), (1e6, True)):
+        L, _ = smooth(n, g)
+        w = np.repeat(L[:, :, None], 4, 2)
+        w[:, v, 2:] *= np.where(g.random(n) < 0.5, ratio, 1 / ratio)[:, None]
+        F, far = np.empty((n, 5)), np.zeros(n, dtype=np.int32)
+        muscl_lib.flux(n, _p(np.ascontiguousarray(w)), 0, _p(F), far.ctypes.data_as(ctypes.c_void_p))
+        assert np.all(far == far_wanted), ratio
+
+
+@pytest.mark.parametrize("ratio", [2.0, 16.0])
+@pytest.mark.parametrize("vel", [1.0, 1e2])
+def test_flux_across_a_jump(muscl_lib, vel, ratio):
+    """jumps at the face that are not left to FP64: densities and pressures by `ratio`, velocities by `vel`, either way"""
+    n, g = 6000, rng(10)
+    L, _ = smooth(n, g)
+    w = np.repeat(L[:, :, None], 4, 2) * (1 + 1e-2 * g.uniform(-1, 1, (n, 5, 4)))
+    for v, k in ((0, ratio), (4, ratio)):
+        w[:, v, 2:] *= np.where(g.random(n) < 0.5, k, 1 / k)[:, None]
+    w[:, 1:4, 2:] *= np.where(g.random(n) < 0.5, vel, 1 / vel)[:, None, None]
+    w = np.ascontiguousarray(w)
+    F, far = np.empty((n, 5)), np.zeros(n, dtype=np.int32)
+    muscl_lib.flux(n, _p(w), 0, _p(F), far.ctypes.data_as(ctypes.c_void_p))
+    sides = lambda t: muscl(w, 0, t)
+    held(F, roe(*sides(F64), 1.4, 0.1, F64), roe(*sides(LD), 1.4, 0.1, LD))
