@@ -58,13 +58,6 @@ struct XPlan {
   static_assert(bytes <= 232448, "227 KB of shared memory per CTA");
 };
 
-// a block's coefficients: half the inverse cell sizes (of the doubled face fluxes); the viscous
-// ones, 2 mu / h and the tangential 2 mu / (4 h) with the factors 4/3 and 2/3 of the normal
-// stress, and 4 kappa / h; for the time step the sum of the inverse sizes and (viscous)
-// 4 max(4/3, gamma/Pr) mu (sum of their squares)
-struct XBlk {
-  XVal h2[3], a[3], a43[3], b[3], b23[3], k[3], hsum, vs;
-};
 static_assert(sizeof(XBlk) == 20 * sizeof(XVal), "XPlan::blk");
 
 // ring values are 61-bit integers with a biased exponent: value = m 2^(e - 1022 - 61)
@@ -111,7 +104,7 @@ template <bool VISC, bool CURVI, int MS>
 __device__ __forceinline__ void xface(const long long* __restrict__ rm, const short* __restrict__ re, const XItem& I,
                                       int d, const XBlk* __restrict__ X, const double* __restrict__ S,
                                       const XConsts& K, const PathK<double>& PK, int lim, XFlux& F) {
-  long long dn[3];  // R - L of the velocities (viscous)
+  XVal dn[4];  // R - L of the velocities and theta (viscous)
   long long us[3];
   int eu[3];
   auto load = [&](const int (&ix)[4], int off, long long (&m)[4], int (&e)[4]) {
@@ -127,7 +120,7 @@ __device__ __forceinline__ void xface(const long long* __restrict__ rm, const sh
     load(I.c, off, m, e);
     XSten s = xmuscl(m, e, lim);
     if (VISC && q >= 0) {
-      dn[q] = s.d;
+      dn[q] = xquick0(s.d, s.ed - XRING_BIAS);
       us[q] = s.sum;
       eu[q] = s.ed - XRING_BIAS;
     }
@@ -144,65 +137,18 @@ __device__ __forceinline__ void xface(const long long* __restrict__ rm, const sh
     xroe(r, u, v, w, p, K, F);
   }
   if constexpr (VISC) {
-    // sum over the two cells of the central differences of a variable along a tangent, [62]
-    auto tang = [&](int off, int tp, int tm, int& E) -> long long {
-      int e[4];
-      long long m[4];
+    auto tang = [&](int off, int tp, int tm) -> XVal {
       const int ix[4] = {I.c[1] + tp, I.c[1] + tm, I.c[2] + tp, I.c[2] + tm};
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        m[c] = rm[ix[c] + off];
-        e[c] = re[ix[c] + off];
-      }
-      E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3])) + 1;  // [60] each
-#pragma unroll
-      for (int c = 0; c < 4; ++c) m[c] = xshr(m[c], E - e[c]);
-      E -= XRING_BIAS;
-      return (m[0] - m[1]) + (m[2] - m[3]);
+      long long m[4];
+      int e[4];
+      load(ix, off, m, e);
+      return xtang(m, e, XRING_BIAS);
     };
     const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
-    // tau_nn = (4/3) 2 mu dun/dn - (2/3) 2 mu (dut1/dt1 + dut2/dt2), tau_nt = 2 mu (dut/dn + dun/dt)
-    XVal tn, t1, t2, th;
-    {  // products [60]
-      int e1, e2;
-      const long long g1 = tang(I.v1, I.t1p, I.t1m, e1), g2 = tang(I.v2, I.t2p, I.t2m, e2);
-      const int f0 = X->a43[d].e + eu[0] + 3, f1 = X->b23[d1].e + e1 + 3, f2 = X->b23[d2].e + e2 + 3;
-      tn.e = xmax(f0, xmax(f1, f2));
-      tn.m = xshr(xmul(X->a43[d].m, dn[0]), tn.e - f0) - xshr(xmul(X->b23[d1].m, g1), tn.e - f1) -
-             xshr(xmul(X->b23[d2].m, g2), tn.e - f2);
-    }
-    {
-      int e1;
-      const long long g1 = tang(I.vn, I.t1p, I.t1m, e1);
-      const int f0 = X->a[d].e + eu[1] + 3, f1 = X->b[d1].e + e1 + 3;
-      t1.e = xmax(f0, f1);
-      t1.m = xshr(xmul(X->a[d].m, dn[1]), t1.e - f0) + xshr(xmul(X->b[d1].m, g1), t1.e - f1);
-    }
-    {
-      int e2;
-      const long long g2 = tang(I.vn, I.t2p, I.t2m, e2);
-      const int f0 = X->a[d].e + eu[2] + 3, f2 = X->b[d2].e + e2 + 3;
-      t2.e = xmax(f0, f2);
-      t2.m = xshr(xmul(X->a[d].m, dn[2]), t2.e - f0) + xshr(xmul(X->b[d2].m, g2), t2.e - f2);
-    }
-    {
-      const int el = re[I.c[1] + 5 * MS], er = re[I.c[2] + 5 * MS], E = xmax(el, er);
-      th.m = xmul(X->k[d].m, xshr(rm[I.c[2] + 5 * MS], E - er) - xshr(rm[I.c[1] + 5 * MS], E - el));
-      th.e = X->k[d].e + E - XRING_BIAS + 3;
-    }
-    auto sub = [&](int q, const XVal& t) {
-      const int E = xmax(F.e[q], t.e) + 1;
-      F.m[q] = xshr(F.m[q], E - F.e[q]) - xshr(t.m, E - t.e);
-      F.e[q] = E;
-    };
-    sub(1, tn);
-    sub(2, t1);
-    sub(3, t2);
-    const int f0 = eu[0] + tn.e + 3, f1 = eu[1] + t1.e + 3, f2 = eu[2] + t2.e + 3;
-    const int E = xmax(xmax(f0, f1), xmax(f2, th.e));
-    const long long g = xshr(xmul(us[0], tn.m), E - f0) + xshr(xmul(us[1], t1.m), E - f1) +
-                        xshr(xmul(us[2], t2.m), E - f2) + xshr(th.m, E - th.e);
-    sub(4, {g, E - 1});
+    const int el = re[I.c[1] + 5 * MS], er = re[I.c[2] + 5 * MS], E = xmax(el, er);
+    dn[3] = xquick0(xshr(rm[I.c[2] + 5 * MS], E - er) - xshr(rm[I.c[1] + 5 * MS], E - el), E - XRING_BIAS);
+    xviscous(d, d1, d2, *X, dn, us, eu, tang(I.vn, I.t1p, I.t1m), tang(I.vn, I.t2p, I.t2m), tang(I.v1, I.t1p, I.t1m),
+             tang(I.v2, I.t2p, I.t2m), F);
   }
 }
 

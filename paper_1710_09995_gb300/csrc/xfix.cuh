@@ -624,6 +624,63 @@ __host__ __device__ __forceinline__ XVal xsum3(const XVal& a, const XVal& b, con
   return xnormed(xshr(a.m, E - a.e) + xshr(b.m, E - b.e) + xshr(c.m, E - c.e), E);
 }
 
+// ---- the viscous flux on uniform grids -------------------------------------------------------------
+// a block's coefficients: half the inverse cell sizes (of the doubled face fluxes); the viscous
+// ones, 2 mu / h and the tangential 2 mu / (4 h) with the factors 4/3 and 2/3 of the normal
+// stress, and 4 kappa / h; for the time step the sum of the inverse sizes and (viscous)
+// 4 max(4/3, gamma/Pr) mu (sum of their squares)
+struct XBlk {
+  XVal h2[3], a[3], a43[3], b[3], b23[3], k[3], hsum, vs;
+};
+// the sum over a face's two cells of the central differences along a tangent, from the neighbours
+// (+, -) of either; ring values [61] with biased exponents
+__host__ __device__ __forceinline__ XVal xtang(const long long (&m)[4], const int (&e)[4], int bias) {
+  const int E = xmax(xmax(e[0], e[1]), xmax(e[2], e[3])) + 1;  // [60] each
+  return xquick0((xshr(m[0], E - e[0]) - xshr(m[1], E - e[1])) + (xshr(m[2], E - e[2]) - xshr(m[3], E - e[3])), E - bias);
+}
+// Twice the viscous flux of a face normal to direction d, taken from twice the inviscid one: dn the
+// differences R - L of the velocities (n, t1, t2) and of theta, us (class eu) the sums of the two
+// cells' velocities, gnn1 and gnn2 the tangential sums of u_n along t1 and t2, gt1, gt2 those of u_t1 along t1
+// and of u_t2 along t2.  The differences come normalised, exact zeros with XZERO, so that every term of a stress has the
+// class of its own size: in the velocities' class a stress of a component 10^6 times smaller than u_n, or
+// next to a u_n that does not vary, had lost 20 bits.
+__host__ __device__ __forceinline__ void xviscous(int d, int d1, int d2, const XBlk& X, const XVal (&dn)[4],
+                                                  const long long (&us)[3], const int (&eu)[3], const XVal& gnn1,
+                                                  const XVal& gnn2, const XVal& gt1, const XVal& gt2, XFlux& F) {
+  // tau_nn = (4/3) 2 mu dun/dn - (2/3) 2 mu (dut1/dt1 + dut2/dt2), tau_nt = 2 mu (dut/dn + dun/dt); products [60]
+  XVal tn, t1, t2;
+  {
+    const int f0 = X.a43[d].e + dn[0].e + 3, f1 = X.b23[d1].e + gt1.e + 3, f2 = X.b23[d2].e + gt2.e + 3;
+    tn.e = xmax(f0, xmax(f1, f2));
+    tn.m = xshr(xmul(X.a43[d].m, dn[0].m), tn.e - f0) - xshr(xmul(X.b23[d1].m, gt1.m), tn.e - f1) -
+           xshr(xmul(X.b23[d2].m, gt2.m), tn.e - f2);
+  }
+  {
+    const int f0 = X.a[d].e + dn[1].e + 3, f1 = X.b[d1].e + gnn1.e + 3;
+    t1.e = xmax(f0, f1);
+    t1.m = xshr(xmul(X.a[d].m, dn[1].m), t1.e - f0) + xshr(xmul(X.b[d1].m, gnn1.m), t1.e - f1);
+  }
+  {
+    const int f0 = X.a[d].e + dn[2].e + 3, f2 = X.b[d2].e + gnn2.e + 3;
+    t2.e = xmax(f0, f2);
+    t2.m = xshr(xmul(X.a[d].m, dn[2].m), t2.e - f0) + xshr(xmul(X.b[d2].m, gnn2.m), t2.e - f2);
+  }
+  const XVal th = {xmul(X.k[d].m, dn[3].m), X.k[d].e + dn[3].e + 3};
+  auto sub = [&](int q, const XVal& t) {
+    const int E = xmax(F.e[q], t.e) + 1;
+    F.m[q] = xshr(F.m[q], E - F.e[q]) - xshr(t.m, E - t.e);
+    F.e[q] = E;
+  };
+  sub(1, tn);
+  sub(2, t1);
+  sub(3, t2);
+  const int f0 = eu[0] + tn.e + 3, f1 = eu[1] + t1.e + 3, f2 = eu[2] + t2.e + 3;
+  const int E = xmax(xmax(f0, f1), xmax(f2, th.e));
+  const long long g = xshr(xmul(us[0], tn.m), E - f0) + xshr(xmul(us[1], t1.m), E - f1) +
+                      xshr(xmul(us[2], t2.m), E - f2) + xshr(th.m, E - th.e);
+  sub(4, {g, E - 1});
+}
+
 // ---- WCNS-E-5 lines ----------------------------------------------------------------------------
 #ifdef __CUDACC__
 #define XNOINLINE __noinline__  // called per variable: inlined five times it was half the kernel's code

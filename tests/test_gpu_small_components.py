@@ -198,3 +198,11 @@ def test_cells_beside_a_jump(gb, curved):
     assert max(by_component(R, ref)) <= COMPONENT
     low = slice(c.nx // 2 + 1, c.nx - 1)
     assert np.all(np.abs(R - ref)[..., low] <= COMPONENT * size[..., low])
+
+
+@pytest.mark.parametrize("viscous", [False, True])
+@pytest.mark.parametrize("size", [1.0, 1e-3, 1e-6, 1e-9])
+def test_spanwise_momentum_on_a_uniform_grid(gb, size, viscous):
+    c = extruded(size, viscous)
+    err = by_component(gpu_residual(gb.block_for_case(c, precision=gb.FP64)), fv_residual(c, *cartesian(c)))
+    assert max(err) <= COMPONENT, err

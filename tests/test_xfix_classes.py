@@ -286,3 +286,94 @@ def test_flux_across_a_jump(muscl_lib, vel, ratio):
     muscl_lib.flux(n, _p(w), 0, _p(F), far.ctypes.data_as(ctypes.c_void_p))
     sides = lambda t: muscl(w, 0, t)
     held(F, roe(*sides(F64), 1.4, 0.1, F64), roe(*sides(LD), 1.4, 0.1, LD))
+
+
+# ---- the viscous flux on uniform grids ------------------------------------------------------------
+
+@pytest.fixture(scope="module")
+def visc_lib(tmp_path_factory):
+    return compiled(tmp_path_factory, "visc", r"""
+// w[i][variable u_n, u_t1, u_t2, theta][cell]: cells L, R and the neighbours + and - of L, then of R, along t1, then t2
+extern "C" void viscous(int n, const double* w, const double* h, double mu, double kappa, double* F) {
+  XBlk X;
+  for (int t = 0; t < 3; ++t) {
+    const double ih = 1.0 / h[t], m2 = mu + mu;
+    X.a[t] = xdec_pos<62>(m2 * ih);
+    X.a43[t] = xdec_pos<62>((4.0 / 3.0) * m2 * ih);
+    X.b[t] = xdec_pos<62>(m2 * (0.25 * ih));
+    X.b23[t] = xdec_pos<62>((2.0 / 3.0) * m2 * (0.25 * ih));
+    X.k[t] = xdec_pos<62>(4.0 * kappa * ih);
+  }
+  for (int i = 0; i < n; ++i) {
+    long long m[4][10];
+    int e[4][10];
+    for (int v = 0; v < 4; ++v)
+      for (int c = 0; c < 10; ++c) {
+        const XVal a = xdec_zero(w[(i * 4 + v) * 10 + c]);
+        m[v][c] = a.m >> 1;
+        e[v][c] = a.e + 1;
+      }
+    XVal dn[4];
+    long long us[3];
+    int eu[3];
+    for (int v = 0; v < 4; ++v) {
+      const int E = xmax(e[v][0], e[v][1]);
+      const long long l = xshr(m[v][0], E - e[v][0]), r = xshr(m[v][1], E - e[v][1]);
+      dn[v] = xquick0(r - l, E);
+      if (v < 3) {
+        us[v] = l + r;
+        eu[v] = E;
+      }
+    }
+    auto tang = [&](int v, int at) {
+      long long a[4];
+      int b[4];
+      for (int c = 0; c < 4; ++c) {
+        a[c] = m[v][at + c];
+        b[c] = e[v][at + c];
+      }
+      return xtang(a, b, 0);
+    };
+    XFlux f;
+    for (int q = 0; q < 5; ++q) {
+      f.m[q] = 0;
+      f.e[q] = XZERO;
+    }
+    xviscous(0, 1, 2, X, dn, us, eu, tang(0, 2), tang(0, 6), tang(1, 2), tang(2, 6), f);
+    for (int q = 0; q < 4; ++q) F[4 * i + q] = xflux(f, 1 + q, 0);
+  }
+}
+""")
+
+
+def viscous(w, h, mu, kappa, t):
+    w = w.astype(t)
+    ih = [t(1.0 / x) for x in h]
+    tang = lambda v, at, d: ((w[:, v, at] - w[:, v, at + 1]) + (w[:, v, at + 2] - w[:, v, at + 3])) * (t(0.25) * ih[d])
+    gn = [(w[:, v, 1] - w[:, v, 0]) * ih[0] for v in range(4)]
+    div = gn[0] + tang(1, 2, 1) + tang(2, 6, 2)
+    tau = [t(2 * mu) * (2 * gn[0] - t(2.0 / 3.0) * div), t(2 * mu) * (gn[1] + tang(0, 2, 1)), t(2 * mu) * (gn[2] + tang(0, 6, 2))]
+    e = sum((w[:, v, 0] + w[:, v, 1]) * tau[v] for v in range(3)) + t(4 * kappa) * gn[3]
+    return np.stack([-tau[0], -tau[1], -tau[2], t(-0.5) * e], 1)
+
+
+@pytest.mark.parametrize("size", [1.0, 1e-3, 1e-6, 1e-9])
+@pytest.mark.parametrize("small", [0, 1, 2])
+@pytest.mark.parametrize("still", ["none", "u_n along t1", "u_t1", "all but the small one"])
+def test_viscous_flux_of_small_components(visc_lib, still, small, size):
+    """one velocity component `size` times the others, which vary everywhere, or not along a tangent, or not
+    at all: no stress takes bits from another, nor a term from one that is zero"""
+    n, g = 3000, rng(11)
+    w = 1.0 + 0.05 * g.uniform(-1, 1, (n, 4, 10))
+    if still == "u_n along t1":
+        w[:, 0, 2:6] = w[:, 0, :1]
+    elif still == "u_t1":
+        w[:, 1] = w[:, 1, :1]
+    elif still != "none":
+        for v in {0, 1, 2} - {small}:
+            w[:, v] = w[:, v, :1]
+    w[:, small] *= size
+    w = np.ascontiguousarray(w)
+    h, F = np.array([1 / 64, 1 / 48, 1e-3]), np.empty((n, 4))
+    visc_lib.viscous(n, _p(w), _p(h), _d(1e-4), _d(4.9e-4), _p(F))
+    held(F, viscous(w, h, 1e-4, 4.9e-4, F64), viscous(w, h, 1e-4, 4.9e-4, LD))
