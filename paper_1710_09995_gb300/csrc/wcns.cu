@@ -87,7 +87,7 @@ struct Coef {
 struct Args {
   Coef<float> cf;
   Coef<double> cd;
-  CUtensorMap mwv;          // W: 6 padded fields, box 44 x 16 x 1 x 1 (one field's plane box)
+  CUtensorMap mwv;          // W: 6 padded fields, box 44 (FP64: 42) x 16 x 1 x 1 (one field's plane box)
   Box b;
   long long n;              // interior cells
   double gamma, mu, Pr, cfl, eps;
@@ -1311,7 +1311,7 @@ extern "C" int gbcfd_wcns_create(int nx, int ny, int nz, const gbcfd_params* par
   w->rows = L.rows;
   {
     const int elem = mixed ? 4 : 8;
-    const int rc = encode_box_map(&w->mwv, w->W, w->box, elem, NPW, WX, WY, 1);
+    const int rc = encode_box_map(&w->mwv, w->W, w->box, elem, NPW, mixed ? WX : XWX, WY, 1);
     if (rc != GBCFD_OK) {
       delete w;
       return rc;

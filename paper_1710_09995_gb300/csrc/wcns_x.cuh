@@ -225,37 +225,49 @@ __global__ void __launch_bounds__(NTW, 2) xdir_kernel(Args a) {
 
 // ---- the viscous residual, FP64 ------------------------------------------------------------------
 // Same tiles, planes and passes as viscres_kernel, on integers: that form's 204 FP64 operations a cell
-// held the FP64 pipe 78% of the time.  A plane that has landed is converted once, in place: the
-// velocities of a cell with one exponent, theta with its own.  A gradient cell brings the 12 cells of its
-// stencils to one exponent (velocities; theta) with four bits of room, so that D4 is exact in them;
-// gradients, stresses and the energy flux are then 62-bit products and sums in classes that differ from
-// that exponent by constants of the mesh and the viscosity.  The fluxes are kept as integers with an
-// exponent per cell for the stresses and one for the energy, and differenced in the same way; the sum of
-// the three directions is rounded once.  16 warps (the FP64 form had 8): a cell's four equations are
+// held the FP64 pipe 78% of the time.  A plane that has landed is converted once, in place: velocities to
+// integers with an exponent each, theta (positive) to a word of mantissa and exponent.  A difference D4 is
+// formed in the class of its four values with four bits of room, so that it is exact in them, and normalised; gradients,
+// stresses and the energy flux are then 62-bit products, and sums in the class of their largest term.
+// The fluxes are kept as integers with an exponent each, and differenced in the same way; the sum of
+// the three directions is rounded once.  (With one exponent for a cell's velocities, one for a gradient cell's
+// neighbours and one for its stresses, a component 10^6 times smaller than the others had 2^-38 of itself left.)
+// 16 warps (the FP64 form had 8): a cell's four equations are
 // shared by two threads.  Two barriers a plane: the conversion of the next plane runs beside the
 // differences.  Measured (96^3): 434 -> 134 us a stage, with the primitives' 117 -> 70 a 128^3 step
 // 9.75 -> 7.85 ms (7.43 with the loads of the passes' ends brought forward and a warp per row of primitives).
-constexpr int XVT = 512;
+constexpr int XVT = 512, XWX = 42;  // threads; columns of the primitive box (41 are read; 16-byte rows)
 struct XRSmem {
-  static constexpr int WF = WY * WX, WP = 4 * WF;
+  static constexpr int WF = WY * XWX, WP = 4 * WF;
   static constexpr int FX = RY * GX, GY_ = GY * RX, HZ = RY * RX;  // cells of one flux buffer
+  static constexpr int ERING = 5;                                  // exponents: of planes p - 2 .. p + 2
   static constexpr size_t w = 0;                                   // staged doubles, then their integers
   static constexpr size_t fx = w + 8 * WRING * WP;
   static constexpr size_t gy = fx + 8 * 4 * FX;
   static constexpr size_t hz = gy + 8 * 4 * GY_;
-  static constexpr size_t we = hz + 8 * ZRING * 4 * HZ;            // exponents: velocity, theta
-  static constexpr size_t fxe = we + 2 * WRING * 2 * WF;           // stresses, energy
-  static constexpr size_t gye = fxe + 2 * 2 * FX;
-  static constexpr size_t hze = gye + 2 * 2 * GY_;
-  static constexpr size_t bar = (hze + 2 * ZRING * 2 * HZ + 15) / 16 * 16;
+  static constexpr size_t we = hz + 8 * ZRING * 4 * HZ;            // exponents: u, v, w
+  static constexpr size_t fxe = we + 2 * ERING * 3 * WF;           // of the fluxes: three stresses, energy
+  static constexpr size_t gye = fxe + 2 * 4 * FX;
+  static constexpr size_t hze = gye + 2 * 4 * GY_;
+  static constexpr size_t bar = (hze + 2 * ZRING * 4 * HZ + 15) / 16 * 16;
   static constexpr size_t bytes = bar + 8 * WRING + 16;
-  static_assert(bytes <= 232448, "227 KB of shared memory per CTA");
+  static_assert(bytes <= 232448 - 256, "227 KB of shared memory per CTA");
 };
-// a velocity or theta: as xdec_zero, its exponent XBAD and more if it is not finite
+// a velocity: as xdec_zero, its exponent XBAD and more if it is not finite
 __device__ __forceinline__ XVal xvalue(double d) {
   XVal v = xdec_zero(d);
   if (v.e >= 1024) v.e = 2 * XBAD;
   return v;
+}
+// theta > 0 as a word: its 53-bit mantissa above its biased exponent
+__device__ __forceinline__ long long xword(long long bits) {
+  const int ex = (int)(bits >> 52) & 0x7ff;
+  const long long m = bits & 0xfffffffffffffll;
+  return (ex ? (m | (1ll << 52)) << 11 | ex : m << 11 | 1);
+}
+__device__ __forceinline__ int xword_e(long long w) { return (int)w & 0x7ff; }
+__device__ __forceinline__ long long xword_m(long long w) {  // [62]
+  return (long long)(((unsigned long long)w & ~0x7ffull) >> 2);
 }
 // (a - d) + 8 (b - c) of four values brought to a class by right shifts s; [58] in, below 2^62.2
 __device__ __forceinline__ long long xd4(long long a, int sa, long long b, int sb, long long c, int sc, long long d, int sd) {
@@ -290,12 +302,10 @@ __global__ void __launch_bounds__(XVT, 1) xviscres_kernel(const __grid_constant_
   if (threadIdx.x == 64) cst[4] = xdec_pos<62>(2.0 / 3.0 * a.cd.mu);
   if (threadIdx.x == 96) cst[5] = xdec_pos<62>(a.cd.kappa);
   __syncthreads();
-  const int he[3] = {cst[0].e, cst[1].e, cst[2].e}, hE = xmax(he[0], xmax(he[1], he[2]));
-  // exponent of the stress in component q, direction d, above that of the cell's velocity stencil
-  auto tau_e = [&](int d, int q) { return 6 + (q == d ? hE + cst[4].e : xmax(he[d], he[q]) + cst[3].e); };
   unsigned parity = 0, pending = 0;  // per W slot (parity uniform; pending in thread 0)
   bool fail = false;                 // a copy did not arrive (uniform)
   auto ws = [](int kp) { return (kp + 4 * WRING) % WRING; };
+  auto es = [](int kp) { return (kp + 4 * SM::ERING) % SM::ERING; };
   auto zs = [](int kp) { return (kp + 4 * ZRING) % ZRING; };
   for (long long u = u0; u < u1 && !fail;) {
     const long long tile = u / b.nz;
@@ -316,17 +326,18 @@ __global__ void __launch_bounds__(XVT, 1) xviscres_kernel(const __grid_constant_
       const int q = ws(kp);
       const bool ok = mbar_wait_bounded(&bar[q], (parity >> q) & 1u);
       long long* m = wr + q * SM::WP;
-      short* e = wer + q * 2 * SM::WF;
+      short* e = wer + es(kp) * 3 * SM::WF;
       for (int c = threadIdx.x; c < SM::WF; c += XVT) {
-        const XVal vu = xvalue(__longlong_as_double(m[c])), vv = xvalue(__longlong_as_double(m[SM::WF + c])),
-                   vw = xvalue(__longlong_as_double(m[2 * SM::WF + c])), th = xvalue(__longlong_as_double(m[3 * SM::WF + c]));
-        const int E = xmax(vu.e, xmax(vv.e, vw.e));
-        m[c] = xshr(vu.m, E - vu.e);
-        m[SM::WF + c] = xshr(vv.m, E - vv.e);
-        m[2 * SM::WF + c] = xshr(vw.m, E - vw.e);
-        m[3 * SM::WF + c] = th.m;
-        e[c] = (short)E;
-        e[SM::WF + c] = (short)th.e;
+        long long x[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) x[f] = m[f * SM::WF + c];
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          const XVal v = xvalue(__longlong_as_double(x[f]));
+          m[f * SM::WF + c] = v.m;
+          e[f * SM::WF + c] = (short)v.e;
+        }
+        m[3 * SM::WF + c] = xword(x[3]);
       }
       return ok;
     };
@@ -337,7 +348,7 @@ __global__ void __launch_bounds__(XVT, 1) xviscres_kernel(const __grid_constant_
     // a thread owns tile cell (lane, warp % 8), equations 2 (warp / 8) and the next: its x- and y-parts of
     // Rv for planes p - 2, p - 1, p stay in registers until the z-part of plane p - 2 is known
     const int crow = warp & 7, q0 = (warp >> 3) * 2;
-    XVal rv2[2] = {{0, -2000}, {0, -2000}}, rv1[2] = {{0, -2000}, {0, -2000}};
+    XVal rv2[2] = {{0, XZERO}, {0, XZERO}}, rv1[2] = {{0, XZERO}, {0, XZERO}};
     if (threadIdx.x == 0) {
       fence_proxy_async();
       for (int kp = k0 - 4; kp <= k0 + 1; ++kp) issue(kp);
@@ -358,62 +369,64 @@ __global__ void __launch_bounds__(XVT, 1) xviscres_kernel(const __grid_constant_
         gx = RX + sidx % (GX - RX);
       }
       if (gy < GY) {
-        const int c = (gy + 2) * WX + gx + 3;  // the cell in the primitive box
-        // neighbours along d at distances -2, -1, +1, +2: offset from the ring's start, slot included
+        const int c = (gy + 2) * XWX + gx + 3;  // the cell in the primitive box
+        // neighbours along d at distances -2, -1, +1, +2: slots of the planes and offsets in them
         const int s0 = ws(p), nb[3][4] = {{s0, s0, s0, s0}, {s0, s0, s0, s0}, {ws(p - 2), ws(p - 1), ws(p + 1), ws(p + 2)}};
-        const int of[3][4] = {{c - 2, c - 1, c + 1, c + 2}, {c - 2 * WX, c - WX, c + WX, c + 2 * WX}, {c, c, c, c}};
-        int sv[3][4], st[3][4], EV = -32768, ET = -32768;
-#pragma unroll
-        for (int d = 0; d < 3; ++d)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            sv[d][i] = wer[nb[d][i] * 2 * SM::WF + of[d][i]];
-            st[d][i] = wer[nb[d][i] * 2 * SM::WF + SM::WF + of[d][i]];
-            EV = xmax(EV, sv[d][i]);
-            ET = xmax(ET, st[d][i]);
-          }
-        EV += 4;
-        ET += 4;
-        long long gr[4][3];  // classes EV (theta ET) + 3 + he[d]; below 2^60.2
+        const int t0 = es(p), ne[3][4] = {{t0, t0, t0, t0}, {t0, t0, t0, t0}, {es(p - 2), es(p - 1), es(p + 1), es(p + 2)}};
+        const int of[3][4] = {{c - 2, c - 1, c + 1, c + 2}, {c - 2 * XWX, c - XWX, c + XWX, c + 2 * XWX}, {c, c, c, c}};
+        XVal gr[4][3];  // [60]
 #pragma unroll
         for (int d = 0; d < 3; ++d)
 #pragma unroll
           for (int f = 0; f < 4; ++f) {
-            const long long v0 = wr[nb[d][0] * SM::WP + f * SM::WF + of[d][0]], v1 = wr[nb[d][1] * SM::WP + f * SM::WF + of[d][1]],
-                            v2 = wr[nb[d][2] * SM::WP + f * SM::WF + of[d][2]], v3 = wr[nb[d][3] * SM::WP + f * SM::WF + of[d][3]];
-            gr[f][d] = f < 3 ? xmul(xd4(v0, EV - sv[d][0], v2, EV - sv[d][2], v1, EV - sv[d][1], v3, EV - sv[d][3]), cst[d].m)
-                             : xmul(xd4(v0, ET - st[d][0], v2, ET - st[d][2], v1, ET - st[d][1], v3, ET - st[d][3]), cst[d].m);
-          }
-        long long dg[3];  // diagonal, class EV + 3 + hE
+            long long v[4];
+            int sv[4];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) dg[d] = xshr(gr[d][d], hE - he[d]);
-        const long long div = dg[0] + dg[1] + dg[2];  // below 2^61.8
-        long long off[3];  // stresses xy, yz, zx
+            for (int i = 0; i < 4; ++i) {
+              v[i] = wr[nb[d][i] * SM::WP + f * SM::WF + of[d][i]];
+              if (f < 3) {
+                sv[i] = wer[(ne[d][i] * 3 + f) * SM::WF + of[d][i]];
+              } else {
+                sv[i] = xword_e(v[i]);
+                v[i] = xword_m(v[i]);
+              }
+            }
+            int E = xmax(xmax(sv[0], sv[1]), xmax(sv[2], sv[3]));
+            const XVal D = xquick0(xd4(v[0], E + 4 - sv[0], v[2], E + 4 - sv[2], v[1], E + 4 - sv[1], v[3], E + 4 - sv[3]),
+                                   f < 3 ? E + 4 : (E == 0x7ff ? 2 * XBAD : E - 1023 + 4));
+            gr[f][d] = {xmul(D.m, cst[d].m), D.e + cst[d].e + 3};
+          }
+        const int Ed = xmax(gr[0][0].e, xmax(gr[1][1].e, gr[2][2].e));
+        long long dg[3];  // the diagonal in one class
+#pragma unroll
+        for (int d = 0; d < 3; ++d) dg[d] = xshr(gr[d][d].m, Ed - gr[d][d].e);
+        const long long div = dg[0] + dg[1] + dg[2];  // below 2^61.6
+        XVal off[3];  // stresses xy, yz, zx
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const int q = (d + 1) % 3, E = xmax(he[d], he[q]);
-          off[d] = xmul(xshr(gr[q][d], E - he[d]) + xshr(gr[d][q], E - he[q]), cst[3].m);  // [59.2]
+          const int q = (d + 1) % 3, E = xmax(gr[q][d].e, gr[d][q].e);
+          off[d] = {xmul(xshr(gr[q][d].m, E - gr[q][d].e) + xshr(gr[d][q].m, E - gr[d][q].e), cst[3].m), E + cst[3].e + 3};  // [59]
         }
-        const int ev = wer[s0 * 2 * SM::WF + c];
+        const short* ve = wer + t0 * 3 * SM::WF + c;
         const long long* vel = wr + s0 * SM::WP + c;
         const bool rows = gy >= 2 && gy < RY + 2, cols = gx >= 2 && gx < RX + 2;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           if ((d == 0 && !rows) || (d == 1 && !cols) || (d == 2 && !(rows && cols))) continue;
-          long long tau[3];
-          // 2 g - 2/3 div = 2/3 (3 g - div); 3 g - div is below 2^62.2, the stress below 2^60.2
-          tau[d] = xmul(3 * dg[d] - div, cst[4].m);
+          XVal tau[3];
+          // 2 g - 2/3 div = 2/3 (3 g - div); 3 g - div is 2 of g less the others: below 2^62
+          tau[d] = {xmul(3 * dg[d] - div, cst[4].m), Ed + cst[4].e + 3};
           tau[(d + 1) % 3] = off[d];
           tau[(d + 2) % 3] = off[(d + 2) % 3];
-          long long w[4];  // u . tau + kappa dtheta, each below 2^58.2
+          long long w[4];  // u . tau + kappa dtheta, [58]
           int we[4], E = -32768;
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
-            w[q] = xmul(vel[q * SM::WF], tau[q]);
-            we[q] = ev + EV + tau_e(d, q) + 3;
+            w[q] = xmul(vel[q * SM::WF], tau[q].m);
+            we[q] = ve[q * SM::WF] + tau[q].e + 3;
           }
-          w[3] = xmul(gr[3][d], cst[5].m);
-          we[3] = ET + he[d] + cst[5].e + 6;
+          w[3] = xmul(gr[3][d].m, cst[5].m);
+          we[3] = gr[3][d].e + cst[5].e + 3;
 #pragma unroll
           for (int q = 0; q < 4; ++q) E = xmax(E, we[q]);
           const long long e = xshr(w[0], E - we[0]) + xshr(w[1], E - we[1]) + xshr(w[2], E - we[2]) + xshr(w[3], E - we[3]);
@@ -423,15 +436,16 @@ __global__ void __launch_bounds__(XVT, 1) xviscres_kernel(const __grid_constant_
           if (d == 0) { dst = fxr; de = fxe; stride = SM::FX; dst += (gy - 2) * GX + gx; de += (gy - 2) * GX + gx; }
           else if (d == 1) { dst = gyr; de = gye; stride = SM::GY_; dst += gy * RX + gx - 2; de += gy * RX + gx - 2; }
           else {
-            const int o = (gy - 2) * RX + gx - 2;
-            dst = hzr + zs(p) * 4 * SM::HZ + o; de = hze + zs(p) * 2 * SM::HZ + o; stride = SM::HZ;
+            const int o = zs(p) * 4 * SM::HZ + (gy - 2) * RX + gx - 2;
+            dst = hzr + o; de = hze + o; stride = SM::HZ;
           }
-          dst[0] = tau[0];
-          dst[stride] = tau[1];
-          dst[2 * stride] = tau[2];
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            dst[q * stride] = tau[q].m;
+            de[q * stride] = (short)min(tau[q].e, 3 * XBAD);
+          }
           dst[3 * stride] = e;
-          de[0] = (short)EV;
-          de[stride] = (short)min(E, 3 * XBAD);
+          de[3 * stride] = (short)min(E, 3 * XBAD);
         }
       }
       __syncthreads();
@@ -441,32 +455,32 @@ __global__ void __launch_bounds__(XVT, 1) xviscres_kernel(const __grid_constant_
       }
       bool ok = true;
       if (p <= k1) ok = convert(p + 3);
-      // D4 of a flux along one direction, class E + 2 + its own + he + 3; flux values [60.2]
-      auto diff = [&](const long long* f, const short* e, int st, int d, int q) -> XVal {
+      // D4 of a flux along one direction, [60]; flux values [60]
+      auto diff = [&](const long long* f, const short* e, int st, int d) -> XVal {
         const int e0 = e[-2 * st], e1 = e[-st], e2 = e[st], e3 = e[2 * st];
         const int E = xmax(xmax(e0, e1), xmax(e2, e3)) + 2;
-        return {xmul(xd4(f[-2 * st], E - e0, f[st], E - e2, f[-st], E - e1, f[2 * st], E - e3), cst[d].m),
-                E + (q < 3 ? tau_e(d, q) : 0) + he[d] + 3};  // below 2^60.4
+        const XVal D = xquick0(xd4(f[-2 * st], E - e0, f[st], E - e2, f[-st], E - e1, f[2 * st], E - e3), E);
+        return {xmul(D.m, cst[d].m), D.e + cst[d].e + 3};
       };
       const int k = p - 2, i = x0 + lane, j = y0 + crow;
       const bool out = k >= k0 && i < b.nx && j < b.ny;
       const long long cc = ((long long)k * b.ny + j) * b.nx + i;
 #pragma unroll
       for (int n = 0; n < 2; ++n) {
-        const int q = q0 + n, ee = q < 3 ? 0 : 1;
-        const int ox = crow * GX + lane + 2, oy = (crow + 2) * RX + lane;
-        const XVal dx = diff(fxr + q * SM::FX + ox, fxe + ee * SM::FX + ox, 1, 0, q);
-        const XVal dy = diff(gyr + q * SM::GY_ + oy, gye + ee * SM::GY_ + oy, RX, 1, q);
+        const int q = q0 + n;
+        const int ox = q * SM::FX + crow * GX + lane + 2, oy = q * SM::GY_ + (crow + 2) * RX + lane;
+        const XVal dx = diff(fxr + ox, fxe + ox, 1, 0);
+        const XVal dy = diff(gyr + oy, gye + oy, RX, 1);
         const int E = xmax(dx.e, dy.e);
-        const XVal rv0 = {xshr(dx.m, E - dx.e) + xshr(dy.m, E - dy.e), E};  // below 2^61.4
+        const XVal rv0 = {xshr(dx.m, E - dx.e) + xshr(dy.m, E - dy.e), E};  // [61]
         if (out) {
-          const int o = crow * RX + lane;
-          auto zf = [&](int kp) { return hzr[(zs(kp) * 4 + q) * SM::HZ + o]; };
-          auto ze = [&](int kp) { return (int)hze[(zs(kp) * 2 + ee) * SM::HZ + o]; };
+          const int o = q * SM::HZ + crow * RX + lane;
+          auto zf = [&](int kp) { return hzr[zs(kp) * 4 * SM::HZ + o]; };
+          auto ze = [&](int kp) { return (int)hze[zs(kp) * 4 * SM::HZ + o]; };
           const int e0 = ze(k - 2), e1 = ze(k - 1), e2 = ze(k + 1), e3 = ze(k + 2);
           const int Ez = xmax(xmax(e0, e1), xmax(e2, e3)) + 2;
-          const XVal dz = {xmul(xd4(zf(k - 2), Ez - e0, zf(k + 1), Ez - e2, zf(k - 1), Ez - e1, zf(k + 2), Ez - e3), cst[2].m),
-                           Ez + (q < 3 ? tau_e(2, q) : 0) + he[2] + 3};
+          const XVal D = xquick0(xd4(zf(k - 2), Ez - e0, zf(k + 1), Ez - e2, zf(k - 1), Ez - e1, zf(k + 2), Ez - e3), Ez);
+          const XVal dz = {xmul(D.m, cst[2].m), D.e + cst[2].e + 3};
           const int Es = xmax(rv2[n].e, dz.e);
           Rv[q * a.n + cc] = xenc(-(xshr(rv2[n].m, Es - rv2[n].e) + xshr(dz.m, Es - dz.e)), Es);
         }

@@ -206,3 +206,20 @@ def test_spanwise_momentum_on_a_uniform_grid(gb, size, viscous):
     c = extruded(size, viscous)
     err = by_component(gpu_residual(gb.block_for_case(c, precision=gb.FP64)), fv_residual(c, *cartesian(c)))
     assert max(err) <= COMPONENT, err
+
+
+@pytest.mark.parametrize("viscous", [False, True])
+@pytest.mark.parametrize("size", [1.0, 1e-3, 1e-6, 1e-9])
+def test_spanwise_momentum_wcns(gb, size, viscous):
+    """the viscous part alone too, as the difference of the residuals with and without viscosity (the inviscid
+    parts subtracted are some 10 times as large)"""
+    c = extruded(size, viscous)
+    R, ref = gpu_residual(gb.wcns_block_for_case(c, precision=gb.FP64)), wcns_residual(c)
+    err = by_component(R, ref)
+    assert max(err) <= COMPONENT, err
+    if viscous:
+        c.viscous = False
+        R = R - gpu_residual(gb.wcns_block_for_case(c, precision=gb.FP64))
+        ref = ref - wcns_residual(c)
+        err = [float(np.linalg.norm(R[m] - ref[m]) / np.linalg.norm(ref[m])) for m in (1, 2, 3)]
+        assert max(err) <= 10 * COMPONENT, err
