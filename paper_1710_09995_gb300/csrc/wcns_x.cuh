@@ -26,6 +26,26 @@ struct XSmem {
   static constexpr size_t cst = red + sizeof(double) * (NTW / 32) * 5;        // Eq. 2's coefficients, the weights' 1e-6
   static constexpr size_t bytes = (cst + 4 * sizeof(XVal) + 127) / 128 * 128;
 };
+// an edge whose sides are far apart (xfar) in FP64: twice the flux.  Out of line: only edges at a jump of 2^5 or more in
+// the density or the pressure call it
+template <int D>
+__device__ __noinline__ void xedge_f64(const double (&L)[5], const double (&R)[5], double gm1, double ggm1, double eps,
+                                       long long* Fm, short* Fe, int o, bool bad) {
+  Consts<double> K;
+  K.gm1 = gm1;
+  K.ggm1 = ggm1;
+  K.eps = eps;
+  constexpr int idx[5] = {0, Fr<D>::N, Fr<D>::T1, Fr<D>::T2, 4};
+  double f[5];
+  roe_frame<double, true>(L, R, K, f);
+  const XFlux F = xflux_of(f);
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    Fm[idx[q] * (LMAX + 5) * NLP + o] = F.m[q];
+    Fe[idx[q] * (LMAX + 5) * NLP + o] = (short)(bad ? XW_BAD : F.e[q]);
+  }
+}
+
 template <int D, int MODE>
 __global__ void __launch_bounds__(NTW, 2) xdir_kernel(Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -125,26 +145,48 @@ __global__ void __launch_bounds__(NTW, 2) xdir_kernel(Args a) {
       const int f = FCH * ch + lane;
       if (a0 + l >= na || FCH * ch >= nfc) continue;  // warp-uniform
       const int m = min(f + 2, nfc + 2);              // centres 2 .. nfc + 2 (stencil <= nst - 1)
+      // one variable's value on either side of the lane's edge
+      auto sides = [&](int q, XVal& left, XVal& right) {
+        const int o = (idx[q] * (LMAX + 10) + m - 2) * NLP + l;
+        const XEdge g = xedge_values<NLP>(Wm + o, We + o, linear, cst[3]);
+        left = {g.up, g.e};
+        right = {__shfl_down_sync(0xffffffffu, g.um, 1), __shfl_down_sync(0xffffffffu, g.e, 1)};
+      };
       XPair S[5];
       int worst = 0;
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        const int o = (idx[q] * (LMAX + 10) + m - 2) * NLP + l;
-        const XEdge g = xedges<NLP>(Wm + o, We + o, linear, cst[3]);
-        const long long r = __shfl_down_sync(0xffffffffu, g.um, 1);
-        const int er = __shfl_down_sync(0xffffffffu, g.e, 1), E = xmax(g.e, er);
-        S[q] = xpair_norm(xshr(g.up, E - g.e), xshr(r, E - er), E);
+        XVal left, right;
+        sides(q, left, right);
+        const int E = xmax(left.e, right.e);
+        S[q] = xpair_norm(xshr(left.m, E - left.e), xshr(right.m, E - right.e), E);
         worst = xmax(worst, E);
       }
+      bool far = false;
       if (lane < FCH && f < nfc) {
-        XFlux F;
-        xroe(S[0], S[1], S[2], S[3], S[4], a.cd.x, F);
+        const XPos r = S[0], p = S[4];
+        far = xfar(r, p);
+        if (!far) {
+          XFlux F;
+          xroe(r, S[1], S[2], S[3], p, a.cd.x, F);
+#pragma unroll
+          for (int q = 0; q < 5; ++q) {
+            const int o = (idx[q] * (LMAX + 5) + f) * NLP + l;
+            Fm[o] = F.m[q];
+            Fe[o] = (short)(worst >= XBAD ? XW_BAD : F.e[q]);
+          }
+        }
+      }
+      if (__any_sync(0xffffffffu, far)) {  // edges between densities or pressures far apart, in FP64
+        double Ld[5], Rd[5];
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
-          const int o = (idx[q] * (LMAX + 5) + f) * NLP + l;
-          Fm[o] = F.m[q];
-          Fe[o] = (short)(worst >= XBAD ? XW_BAD : F.e[q]);
+          XVal left, right;
+          sides(q, left, right);
+          Ld[q] = xenc(left.m, left.e);
+          Rd[q] = xenc(right.m, right.e);
         }
+        if (far) xedge_f64<D>(Ld, Rd, a.cd.K.gm1, a.cd.K.ggm1, a.cd.K.eps, Fm, Fe, f * NLP + l, worst >= XBAD);
       }
     }
     __syncthreads();
@@ -187,7 +229,7 @@ __global__ void __launch_bounds__(NTW, 2) xdir_kernel(Args a) {
         for (int x = 0; x < 3; ++x) {  // edges 3 - 2, 4 - 1, 5 - 0 around the cell
           const int h = o + (3 + x) * NLP, w = o + (2 - x) * NLP, e1 = Fe[h], e0 = Fe[w], E = xmax(e1, e0) + 1;
           // normalised, so that the product's truncation is relative to the difference
-          const XVal g = xquick(xshr(Fm[h], E - e1) - xshr(Fm[w], E - e0), E);
+          const XVal g = xquick0(xshr(Fm[h], E - e1) - xshr(Fm[w], E - e0), E);
           d[x] = xmul(g.m, cst[x].m);  // [60]
           ed[x] = g.e + cst[x].e + 3;
         }

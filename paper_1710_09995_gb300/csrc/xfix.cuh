@@ -685,7 +685,7 @@ __host__ __device__ __forceinline__ void xviscous(int d, int d1, int d2, const X
 #ifdef __CUDACC__
 #define XNOINLINE __noinline__  // called per variable: inlined five times it was half the kernel's code
 #else
-#define XNOINLINE inline
+#define XNOINLINE
 #endif
 constexpr int XW_BIAS = 1018;       // staged value = m 2^(e - 1018 - 61), |m| < 2^57
 constexpr int XW_BAD = 2 * XBAD;    // exponent of a staged value that is not finite
@@ -699,11 +699,32 @@ __host__ __device__ __forceinline__ void xline_value(double v, long long* m, sho
   *m = ex ? ((long long)(mag << 4) ^ sg) - sg : 0ll;
   *e = (short)(ex == 0x7ff ? XW_BAD : ex);
 }
-// both edge values of a cell: u_{i+1/2} from the left, u_{i-1/2} from the right, class e, [62]
+// both edge values of a cell: u_{i+1/2} from the left, u_{i-1/2} from the right, class e, [62]; weak: both the cell's
+// value and an edge value's distance from it are small beside the stencil's largest value, whose class leaves them
+// fewer bits than a double has (a jump that the weights keep out of the value)
 struct XEdge {
   long long up, um;
   int e;
+  bool weak;
 };
+// the interpolation in doubles, as edges() in wcns.cu, for weak edges; staged values are doubles, so nothing is
+// lost on the way in
+inline __host__ __device__ XNOINLINE XEdge xedges_f64(double u0, double u1, double u2, double u3, double u4, bool linear) {
+  const double gA = 0.5 * (u0 - 4.0 * u1 + 3.0 * u2), gB = 0.5 * (u3 - u1), gC = 0.5 * (4.0 * u3 - 3.0 * u2 - u4);
+  const double sA = u0 - 2.0 * u1 + u2, sB = u1 - 2.0 * u2 + u3, sC = u2 - 2.0 * u3 + u4;
+  double wA = 1.0, wB = 1.0, wC = 1.0;  // products of the other stencils' (1e-6 + g^2 + s^2)^2
+  if (!linear) {
+    const double a = 1e-6 + (gA * gA + sA * sA), b = 1e-6 + (gB * gB + sB * sB), c = 1e-6 + (gC * gC + sC * sC);
+    wA = b * b * (c * c);
+    wB = a * a * (c * c);
+    wC = a * a * (b * b);
+  }
+  const double nB = 10.0 * wB, n = wA + nB + 5.0 * wC, k = 5.0 * wA + nB + wC;
+  const double up = wA * (0.5 * gA + 0.125 * sA) + nB * (0.5 * gB + 0.125 * sB) + 5.0 * wC * (0.5 * gC + 0.125 * sC);
+  const double um = 5.0 * wA * (0.125 * sA - 0.5 * gA) + nB * (0.125 * sB - 0.5 * gB) + wC * (0.125 * sC - 0.5 * gC);
+  const XPair e = xpair(u2 + up / n, u2 + um / k);
+  return {e.l, e.r, e.e, false};
+}
 // the weighted interpolation of WCNS-E-5 (edges() in wcns.cu) from the five staged values at wm, we.
 // With d_j the first differences of u_{i-2} .. u_{i+2}: eight times the candidates' distances from u_i
 // are small integer combinations of them, twice the first derivatives too.  Each stencil's
@@ -731,42 +752,58 @@ __host__ __device__ XNOINLINE XEdge xedges(const long long* __restrict__ wm, con
   // 8 (candidate - u_i) at i + 1/2 and i - 1/2 [62]
   long long pA = x7(d1) - x3(d0), pB = x3(d2) + d1, pC = x5(d2) - d3;
   long long qA = d0 - x5(d1), qB = -(x3(d1) + d2), qC = x3(d3) - x7(d2);
-  XEdge o;
-  o.e = E - 3;
-  if (linear) {
-    o.up = (u[2] << 3) + ((pA >> 4) + x10(pB >> 4) + x5(pC >> 4));
-    o.um = (u[2] << 3) + (x5(qA >> 4) + x10(qB >> 4) + (qC >> 4));
-    return o;
-  }
-  // (1e-6 + g^2 + s^2)^2 of a stencil from 2 g and 2 s [60], normalised [62]
-  auto weight = [&](long long g, long long s) -> XVal {
+  auto edge = [&](long long tp, long long tm) -> XEdge {  // u_i and the distances in class E - 3; |u| is 2^60 at most
+    const long long uc = u[2] << 3;
+    const int hu = (int)(uc >> 32), hp = (int)(tp >> 32), hm = (int)(tm >> 32), ap = hp ^ (hp >> 31), am = hm ^ (hm >> 31);
+    return {uc + tp, uc + tm, E - 3, (hu ^ (hu >> 31)) + (ap < am ? ap : am) < (1 << 24)};  // 2^56
+  };
+  if (linear)
+    return edge(((pA >> 2) + x10(pB >> 2) + x5(pC >> 2)) >> 2, (x5(qA >> 2) + x10(qB >> 2) + (qC >> 2)) >> 2);
+  // 1e-6 + g^2 + s^2 of a stencil from 2 g and 2 s [60], normalised [62]
+  auto smooth = [&](long long g, long long s) -> XVal {
     const int n = xclz32((int)((g ^ (g >> 63)) >> 32) | (int)((s ^ (s >> 63)) >> 32)) - 2;  // 2 .. 30
     const long long q = xsq(g << n) + xsq(s << n);                                          // 4 (g^2 + s^2) [61]
     const int eb = 2 * (E - n) + 1, ed = xmax(eb, eps.e + 1);
-    const XVal d = xquick(xshr(q, ed - eb) + xshr(eps.m, ed - eps.e), ed);
-    return {xsq(d.m) << 2, 2 * d.e + 1};
+    return xquick(xshr(q, ed - eb) + xshr(eps.m, ed - eps.e), ed);
   };
-  const XVal A = weight(x3(d1) - d0, (d1 - d0) << 1), B = weight(d1 + d2, (d2 - d1) << 1),
-             C = weight(x3(d2) - d3, (d3 - d2) << 1);
-  const int ea = B.e + C.e, eb = A.e + C.e, ec = A.e + B.e, Em = xmax(ea, xmax(eb, ec)) + 2;
-  const long long a = xshr(xmul(B.m, C.m), Em - ea), b = x10(xshr(xmul(A.m, C.m), Em - eb)), c = xshr(xmul(A.m, B.m), Em - ec);
-  const int En = Em + 3;
-  const long long a5 = x5(a), c5 = x5(c);  // a, c [58]; b, a5, c5 [62]
-  const XVal rp = xrcp(xnormed(a + b + c5, En)), rm = xrcp(xnormed(a5 + b + c, En));
-  // the candidates' distances, normalised together
+  const XVal A = smooth(x3(d1) - d0, (d1 - d0) << 1), B = smooth(d1 + d2, (d2 - d1) << 1),
+             C = smooth(x3(d2) - d3, (d3 - d2) << 1);
+  // a stencil's weight: the square of the product of the others' smoothness, in [2^58, 2^60)
+  auto weight = [](const XVal& x, const XVal& y) -> XVal {
+    const long long m = xmul(x.m, y.m);  // [2^58, 2^60)
+    const int n = 3 - (int)(m >> 59);
+    return {xsq(m << n), 2 * (x.e + y.e + 3 - n) + 3};
+  };
+  const XVal wa = weight(B, C), wb = weight(A, C), wc = weight(A, B);
+  const int Em = xmax(wa.e, xmax(wb.e, wc.e)) + 2;
+  const long long a = xshr(wa.m, Em - wa.e), b = x10(xshr(wb.m, Em - wb.e)), c = xshr(wc.m, Em - wc.e);
+  const XVal rp = xrcp(xquick(a + b + x5(c), Em)), rm = xrcp(xquick(x5(a) + b + c, Em));  // sums [62]
+  // the weights' shares first (2^62 = 1, to 2^-59), then the distances of the candidates, normalised together: the error is
+  // some 2^-60 of the largest distance.  (Products of weights and distances summed first and divided last left 2^-50 of
+  // it beside a jump, where one weight outgrows the others.)
   const long long any = (pA ^ (pA >> 63)) | (pB ^ (pB >> 63)) | (pC ^ (pC >> 63)) | (qA ^ (qA >> 63)) | (qB ^ (qB >> 63)) |
                         (qC ^ (qC >> 63));
   const int n = xclz32((int)(any >> 32)) - 2;
-  const int et = En + E - 3 - n + 3;
-  auto value = [&](long long t, const XVal& r) -> long long {  // u_i + t r in class E - 3
-    const XVal f = xquick(t, et);
-    const long long v = xmul(f.m, r.m);
-    const int sh = E - 3 - (f.e + r.e + 3);  // at least -4: the distance is at most 10/8 of the values' span
-    return (u[2] << 3) + (sh >= 0 ? xshr(v, sh) : v << -sh);
+  auto part = [&](long long m, int e, const XVal& r, long long p) {
+    return xmul(xshr(xmul(m, r.m) << 2, 1 - (e + r.e)) << 3, p << n);
   };
-  o.up = value(xmul(a, pA << n) + xmul(b, pB << n) + xmul(c5, pC << n), rp);
-  o.um = value(xmul(a5, qA << n) + xmul(b, qB << n) + xmul(c, qC << n), rm);
-  return o;
+  const long long tp = xshr((part(wa.m << 2, wa.e - 2, rp, pA) + part(x5(wb.m), wb.e + 1, rp, pB) + part(x5(wc.m), wc.e, rp, pC)) << 2, n);
+  const long long tm = xshr((part(x5(wa.m), wa.e, rm, qA) + part(x5(wb.m), wb.e + 1, rm, qB) + part(wc.m << 2, wc.e - 2, rm, qC)) << 2, n);
+  return edge(tp, tm);
+}
+// the edge values of a cell: on integers, weak ones in FP64
+template <int STRIDE>
+__host__ __device__ __forceinline__ XEdge xedge_values(const long long* __restrict__ wm, const short* __restrict__ we,
+                                                       bool linear, XVal eps) {
+  const XEdge g = xedges<STRIDE>(wm, we, linear, eps);
+  if (g.weak && g.e < XBAD && (g.up | g.um) != 0) {
+    double u[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) u[c] = xenc(wm[c * STRIDE], we[c * STRIDE] - XW_BIAS);
+    const XEdge h = xedges_f64(u[0], u[1], u[2], u[3], u[4], linear);
+    if (h.e < 1024) return h;  // (fourth powers of values past 1e38 overflow)
+  }
+  return g;
 }
 
 }  // namespace gbcfd

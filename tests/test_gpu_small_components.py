@@ -223,3 +223,14 @@ def test_spanwise_momentum_wcns(gb, size, viscous):
         ref = ref - wcns_residual(c)
         err = [float(np.linalg.norm(R[m] - ref[m]) / np.linalg.norm(ref[m])) for m in (1, 2, 3)]
         assert max(err) <= 10 * COMPONENT, err
+
+
+def test_cells_beside_a_jump_wcns(gb):
+    """the same for WCNS-E-5, in cells of the low side with no edge of Eq. 2 at the jump; the weights there are some
+    10^12 apart and carry 20 roundings to what they let in"""
+    c, size = halves()
+    ref = wcns_residual(c)
+    R = gpu_residual(gb.wcns_block_for_case(c, precision=gb.FP64))
+    assert max(by_component(R, ref)) <= COMPONENT
+    low = slice(c.nx // 2 + 4, c.nx - 4)
+    assert np.all(np.abs(R - ref)[..., low] <= COMPONENT * size[..., low])

@@ -377,3 +377,68 @@ def test_viscous_flux_of_small_components(visc_lib, still, small, size):
     h, F = np.array([1 / 64, 1 / 48, 1e-3]), np.empty((n, 4))
     visc_lib.viscous(n, _p(w), _p(h), _d(1e-4), _d(4.9e-4), _p(F))
     held(F, viscous(w, h, 1e-4, 4.9e-4, F64), viscous(w, h, 1e-4, 4.9e-4, LD))
+
+
+# ---- WCNS-E-5 edges beside jumps ------------------------------------------------------------------
+
+@pytest.fixture(scope="module")
+def edge_lib(tmp_path_factory):
+    return compiled(tmp_path_factory, "edges", r"""
+extern "C" void edges(int n, const double* u, int linear, double* out) {
+  const XVal eps = xdec_pos<62>(1e-6);
+  for (int i = 0; i < n; ++i) {
+    long long m[5];
+    short e[5];
+    for (int c = 0; c < 5; ++c) xline_value(u[5 * i + c], m + c, e + c);
+    const XEdge g = xedge_values<1>(m, e, linear != 0, eps);
+    out[2 * i] = xenc(g.up, g.e);
+    out[2 * i + 1] = xenc(g.um, g.e);
+  }
+}
+""")
+
+
+def edges(u, linear, t):
+    w = u.astype(t).T
+
+    def edge(a):
+        g = [t(0.5) * (a[0] - 4 * a[1] + 3 * a[2]), t(0.5) * (a[3] - a[1]), t(0.5) * (4 * a[3] - 3 * a[2] - a[4])]
+        s = [a[0] - 2 * a[1] + a[2], a[1] - 2 * a[2] + a[3], a[2] - 2 * a[3] + a[4]]
+        al = [t(c) if linear else t(c) / (t(1e-6) + (gk * gk + sk * sk)) ** 2 for c, gk, sk in zip((1, 10, 5), g, s)]
+        return a[2] + sum(k * (t(0.5) * gk + t(0.125) * sk) for k, gk, sk in zip(al, g, s)) / sum(al)
+
+    return np.stack([edge(w), edge(w[::-1])], 1)
+
+
+@pytest.mark.parametrize("linear", [0, 1])
+@pytest.mark.parametrize("low", [0.5, 0.1, 1e-2, 1e-4, 1e-8])
+@pytest.mark.parametrize("side,at", [(0, 1), (0, 2), (0, 3), (1, 2), (1, 3), (1, 4)])
+def test_edges_beside_a_jump(edge_lib, side, at, low, linear):
+    """cells on one side of the jump are 1, on the other `low`: the weights keep the jump out of the values on either
+    side.  Errors relative to the cell's value and its distance from the edge's (what the FP64 form rounds)."""
+    n, g = 3000, rng(13)
+    hi = (np.arange(5) >= at) if side else (np.arange(5) < at)
+    u = np.ascontiguousarray(np.where(hi, 1.0, low) * (1 + 0.05 * g.uniform(-1, 1, (n, 5))))
+    out = np.empty((n, 2))
+    edge_lib.edges(n, _p(u), linear, _p(out))
+    want, form = edges(u, linear, LD), edges(u, linear, F64)
+    size = np.maximum(np.abs(u[:, 2:3]), np.abs(want - u[:, 2:3]))
+    rms = lambda x: float(np.sqrt(np.mean((x / size) ** 2)))
+    assert rms(out - want) <= rms(form - want) + ULP
+
+
+@pytest.mark.parametrize("u", [(0.0,) * 5, (1.0,) * 5, (1e-30,) * 5])
+def test_edges_of_a_constant_are_that_constant(edge_lib, u):
+    a, out = np.array(u), np.empty(2)
+    for linear in (0, 1):
+        edge_lib.edges(1, _p(a), linear, _p(out))
+        assert np.all(out == u[2])
+
+
+def test_edges_that_are_not_finite_stay_so(edge_lib):
+    for c in range(5):
+        for bad in (np.nan, np.inf, -np.inf):
+            a, out = np.array([1e-9] * 5), np.empty(2)
+            a[c] = bad
+            edge_lib.edges(1, _p(a), 0, _p(out))
+            assert not np.isfinite(out).any()
