@@ -114,13 +114,16 @@ __host__ __device__ __forceinline__ XVal xdec_pos(double a) {  // a > 0
 // the exponent of an exact zero: below that of any product of doubles, so that a zero takes no part in the
 // class of a sum
 constexpr int XZERO = -8000;
-// the same, a zero or subnormal as zero
+// any finite double: a zero as zero, a subnormal with its own (fewer) bits
 __host__ __device__ __forceinline__ XVal xdec_zero(double a) {
   XVal v = xdec<62>(a);
-  if (v.e == -1023) v = {0, XZERO};
+  if (v.e == -1023) {
+    const long long m = (long long)(xbits(a) & 0xfffffffffffffull) << 9;
+    v = {v.m < 0 ? -m : m, m ? -1022 : XZERO};
+  }
   return v;
 }
-// the double nearest to m 2^(e - 61), |m| < 2^63; below the normal range 0, above it infinity, and
+// the double nearest to m 2^(e - 61), |m| < 2^63; below the normal range subnormal, above it infinity, and
 // NaN for the exponents from XBAD up (a flux that has no value)
 constexpr int XBAD = 8192;
 __host__ __device__ __forceinline__ int xclz32(int a) {
@@ -137,7 +140,8 @@ __host__ __device__ inline double xenc_rare(long long m, int e) {
   a <<= (n & 63);
   const int f = e + 2 - n + 1022;  // biased exponent - 1
   unsigned long long b = ((unsigned long long)(unsigned)f << 52) + (a >> 11) + ((a >> 10) & 1ull);
-  if ((unsigned)f >= 2046u) b = f < 0 ? 0ull : 0x7ff0000000000000ull;
+  if ((unsigned)f >= 2046u) b = 0x7ff0000000000000ull;
+  if (f < 0) b = f < -53 ? 0ull : ((a >> (10 - f)) + 1ull) >> 1;
   if (a == 0ull) b = 0ull;
   if (e >= XBAD) b = 0x7ff8000000000000ull;
   return xdouble(b | ((unsigned long long)s & 0x8000000000000000ull));
@@ -481,9 +485,10 @@ __host__ __device__ __forceinline__ XFlux xflux_of(const double* f) {
   }
   return F;
 }
-// a flux component as a double, times 2^-h
+// a flux component as a double, times 2^-h; below the normal range zero
 __host__ __device__ __forceinline__ double xflux(const XFlux& F, int q, int h) {
-  return xenc(F.m[q], F.e[q] - h);
+  const double f = xenc(F.m[q], F.e[q] - h);
+  return (xbits(f) & 0x7ff0000000000000ull) == 0ull ? 0.0 : f;
 }
 // ---- MUSCL ---------------------------------------------------------------------------------------
 // half the minmod slope's double: 0 when a and b differ in sign, else the one of smaller magnitude
@@ -690,14 +695,14 @@ __host__ __device__ __forceinline__ void xviscous(int d, int d1, int d2, const X
 constexpr int XW_BIAS = 1018;       // staged value = m 2^(e - 1018 - 61), |m| < 2^57
 constexpr int XW_BAD = 2 * XBAD;    // exponent of a staged value that is not finite
 
-// a double as a staged value (zero and subnormals as zero, a value that is not finite by its exponent)
+// a double as a staged value (subnormals with their own bits, a value that is not finite by its exponent)
 __host__ __device__ __forceinline__ void xline_value(double v, long long* m, short* e) {
   const unsigned long long bits = xbits(v);
   const int hi = (int)(bits >> 32), ex = (int)(((unsigned)hi >> 20) & 0x7ffu);
-  const unsigned long long mag = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)bits;
+  const unsigned long long mag = ((unsigned long long)(((unsigned)hi & 0xfffffu) | (ex ? 0x100000u : 0u)) << 32) | (unsigned)bits;
   const long long sg = hi >> 31;
-  *m = ex ? ((long long)(mag << 4) ^ sg) - sg : 0ll;
-  *e = (short)(ex == 0x7ff ? XW_BAD : ex);
+  *m = ((long long)(mag << 4) ^ sg) - sg;
+  *e = (short)(ex == 0x7ff ? XW_BAD : xmax(ex, 1));
 }
 // both edge values of a cell: u_{i+1/2} from the left, u_{i-1/2} from the right, class e, [62]; weak: both the cell's
 // value and an edge value's distance from it are small beside the stencil's largest value, whose class leaves them

@@ -442,3 +442,52 @@ def test_edges_that_are_not_finite_stay_so(edge_lib):
             a[c] = bad
             edge_lib.edges(1, _p(a), 0, _p(out))
             assert not np.isfinite(out).any()
+
+
+# ---- below the normal range -----------------------------------------------------------------------
+
+@pytest.fixture(scope="module")
+def tiny_lib(tmp_path_factory):
+    return compiled(tmp_path_factory, "tiny", r"""
+extern "C" void again(int n, const double* a, double* b, double* c, double* d) {  // through a value, a line's, and scaled
+  for (int i = 0; i < n; ++i) {
+    const XVal v = xdec_zero(a[i]);
+    b[i] = xenc(v.m, v.e);
+    long long m;
+    short e;
+    xline_value(a[i], &m, &e);
+    c[i] = xenc(m, e - XW_BIAS);
+    d[i] = xenc(v.m, v.e - 30);
+  }
+}
+extern "C" void velocity(int n, const double* q, double* u) {
+  const XConsts K = xconsts(1.4, 0.1);
+  for (int i = 0; i < n; ++i) {
+    XPrim W;
+    xprim(q + 5 * i, K, W);
+    for (int x = 0; x < 3; ++x) u[3 * i + x] = xenc(W.u[x].m, W.u[x].e);
+  }
+}
+""")
+
+
+def test_doubles_below_the_normal_range(tiny_lib):
+    """every double survives; scaled down it is rounded to the nearest multiple of 2^-1074"""
+    g = rng(17)
+    a = np.concatenate([g.uniform(-1, 1, 4000) * 2.0 ** -1021, g.integers(-2 ** 20, 2 ** 20, 4000) * 2.0 ** -1074,
+                        [0.0, 2.0 ** -1074, -2.0 ** -1074, 2.0 ** -1022, np.nextafter(2.0 ** -1022, 0)]])
+    b, c, d = (np.empty_like(a) for _ in range(3))
+    tiny_lib.again(len(a), _p(a), _p(b), _p(c), _p(d))
+    assert np.array_equal(a, b) and np.array_equal(a, c)
+    assert np.all(np.abs(d.astype(LD) - a.astype(LD) * LD(2) ** -30) <= LD(2) ** -1075)
+
+
+def test_velocities_below_the_normal_range(tiny_lib):
+    n, g = 2000, rng(18)
+    q = np.ones((n, 5))
+    q[:, 0] = g.uniform(0.5, 2, n)
+    q[:, 1:4] = g.uniform(-1, 1, (n, 3)) * 10.0 ** g.uniform(-315, -306, (n, 3))
+    u = np.empty((n, 3))
+    tiny_lib.velocity(n, _p(q), _p(u))
+    want = q[:, 1:4].astype(LD) / q[:, :1].astype(LD)
+    assert np.all(np.abs(u - want) <= LD(2) ** -1074 + ULP * np.abs(want))
