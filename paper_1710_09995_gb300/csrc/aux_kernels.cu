@@ -157,10 +157,14 @@ cudaError_t launch_gather(const Geometry& g, const double* src, double* dst, cud
 // rate = sum over directions of (|u_d| + c) / h_d (+ 4 max(4/3, gamma/Pr) mu / rho / h_d^2 when
 // viscous); the CFL step is cfl / max(rate).  From the padded f64 state, in the path's flux
 // precision T (the mixed path's time step is an f32 evaluation, like its fluxes).
-// A warp per row of cells.  FP64 blocks evaluate it on the integer pipes (xfix.cuh).  The maxima are
+// A warp takes a row of cells, or 2, 4 or 8 rows of at most 16, 8 or 4 (with a warp a row 28 lanes idled on blocks 4
+// cells wide: setting the state of 4 x 512 x 512 cells took 750 us, now 574, against 663 with a thread a cell).  FP64 blocks
+// evaluate it on the integer pipes (xfix.cuh).  The maxima are
 // compared as bit patterns and the CTAs' folded by a warp of the last CTA: one thread walking all
 // partial rows took most of the 60 us this pass cost a 32^3 block.
 constexpr int RATE_THREADS = 256;
+// log2 of the threads a row takes
+__device__ __forceinline__ int row_shift(int nx) { return nx > 16 ? 5 : (nx > 8 ? 4 : (nx > 4 ? 3 : 2)); }
 __device__ __forceinline__ void rate_fold(long long best, DevCtrl* ctrl, double* partial, double cfl) {
   __shared__ long long wmax[RATE_THREADS / 32];
   __shared__ int last;
@@ -209,10 +213,10 @@ __global__ void __launch_bounds__(RATE_THREADS) init_rate_kernel(Geometry g, int
                                                                   double* partial, float* dtl) {
   float best = 0.f;
   bool bad = false;
-  const int rows = g.ny * g.nz, lane = threadIdx.x & 31;
-  for (int row = blockIdx.x * (RATE_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += gridDim.x * (RATE_THREADS / 32)) {
+  const int rows = g.ny * g.nz, sh = row_shift(g.nx), per = RATE_THREADS >> sh;
+  for (int row = blockIdx.x * per + (threadIdx.x >> sh); row < rows; row += gridDim.x * per) {
     const int j = row % g.ny, k = row / g.ny;
-    for (int i = lane; i < g.nx; i += 32) {
+    for (int i = threadIdx.x & ((1 << sh) - 1); i < g.nx; i += 1 << sh) {
       const long long o = gidx(g, i, j, k);
       const float rho = float(q[o]), ir = 1.f / rho;
       const float u = float(q[g.field + o]) * ir, v = float(q[2 * g.field + o]) * ir, w = float(q[3 * g.field + o]) * ir;
@@ -245,10 +249,10 @@ __global__ void __launch_bounds__(RATE_THREADS) init_rate_x_kernel(Geometry g, P
   __syncthreads();
   long long best = 0;
   bool bad = false;
-  const int rows = g.ny * g.nz, lane = threadIdx.x & 31;
-  for (int row = blockIdx.x * (RATE_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += gridDim.x * (RATE_THREADS / 32)) {
+  const int rows = g.ny * g.nz, sh = row_shift(g.nx), per = RATE_THREADS >> sh;
+  for (int row = blockIdx.x * per + (threadIdx.x >> sh); row < rows; row += gridDim.x * per) {
     const int j = row % g.ny, k = row / g.ny;
-    for (int i = lane; i < g.nx; i += 32) {
+    for (int i = threadIdx.x & ((1 << sh) - 1); i < g.nx; i += 1 << sh) {
       const long long o = gidx(g, i, j, k);
       const double Q[5] = {q[o], q[g.field + o], q[2 * g.field + o], q[3 * g.field + o], q[4 * g.field + o]};
       XPrim W;
@@ -426,10 +430,10 @@ __global__ void __launch_bounds__(RATE_THREADS) init_rate_curvi_kernel(Geometry 
   const long long fm = g.fieldf;
   float best = 0.f;
   bool bad = false;
-  const int rows = g.ny * g.nz, lane = threadIdx.x & 31;
-  for (int row = blockIdx.x * (RATE_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += gridDim.x * (RATE_THREADS / 32)) {
+  const int rows = g.ny * g.nz, sh = row_shift(g.nx), per = RATE_THREADS >> sh;
+  for (int row = blockIdx.x * per + (threadIdx.x >> sh); row < rows; row += gridDim.x * per) {
     const int j = row % g.ny, k = row / g.ny;
-    for (int i = lane; i < g.nx; i += 32) {
+    for (int i = threadIdx.x & ((1 << sh) - 1); i < g.nx; i += 1 << sh) {
       const long long o = gidx(g, i, j, k), om = gidxf(g, i, j, k);
       const long long up[3] = {1, g.pxf, g.planef};
       const float rho = float(q[o]), ir = 1.f / rho;

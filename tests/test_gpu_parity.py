@@ -84,6 +84,22 @@ def test_fp64_tile_edges(gb, n, viscous):
     assert np.allclose(blk.residual_norm(), norms[-1], rtol=1e-11, atol=1e-13 * np.max(norms[-1]))
 
 
+@pytest.mark.parametrize("curved", [False, True])
+@pytest.mark.parametrize("precision,tol", [(0, 1e-13), (1, 3e-6)])
+@pytest.mark.parametrize("nx", [4, 5, 8, 9, 16, 17, 40])
+def test_time_step_of_narrow_blocks(gb, nx, precision, tol, curved):
+    """the time step of a state just set, which a warp takes in 8, 4, 2 or one row: rows of every kind, the fastest
+    cell once in the first column and once in the last (FP32: some 20 roundings of 6e-8)"""
+    for i in (0, nx - 1):
+        c = ragged_case(True, seed=nx, nx=nx, ny=37, nz=29)
+        c.state[4, 17, 30, i] *= 4.0
+        if curved:
+            c.nodes = cases.warped_nodes(nx, 37, 29, 0.05)
+        blk = gb.block_for_case(c, precision=precision)
+        want = oracle.dt(oparams(c), oracle.pad(c.state), oracle.metrics(c.grid_nodes()))
+        assert abs(blk.get_dt() - want) <= tol * want
+
+
 def test_gaussian_pulse_32_fp64_10_steps(gb):
     """32^3 Euler Gaussian pulse, CFL 0.5, MUSCL/minmod + Roe, 10 SSP-RK3 steps, FP64."""
     c = cases.gaussian_pulse(32, seed=0)
