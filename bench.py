@@ -424,6 +424,7 @@ def e2e_path(gbcfd, torch, case, precision, steps, world, device):
 # GB300 FP64 peak from unit counts and clock: 152 SMs x 2 FP64 FMA lanes per clock x 2 flops x
 # 2.07 GHz (the recipe's nominal 1.25 TFLOP/s; gbcfd_op_rate's DFMA chains measure 1.2524)
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
+STAGE_KERNEL = {"fp64": "xstage_kernel", "mixed": "stage_kernel", "curvilinear": "cstage_kernel"}  # FP64 is Cartesian here
 ISSUE_PER_CLK = 152 * 4 * 32  # SMs x schedulers x lanes: thread instructions issued per clock
 
 
@@ -457,18 +458,18 @@ def roofline(precision, res, cells, steps, peak, peak_kind, workload="vortex256"
             "traffic": traffic, "algorithmic_bytes_per_launch": nbytes / (3 * steps),
             "design_bytes_per_launch": dbytes / (3 * steps),
             "design_frac": round(dbytes / sec / 1e9 / peak, 4),
-            "kernel": "stage_kernel", "avg_launch_ms": round(sec * 1e3 / (3 * steps), 4)}
+            "kernel": STAGE_KERNEL["curvilinear" if workload == "warped512" else precision], "avg_launch_ms": round(sec * 1e3 / (3 * steps), 4)}
 
 
 def fp64_alu_roofline(res, cells, steps, hbm, workload="vortex256"):
-    """FP64-pipe roofline of the FP64 stage kernel: its FP64 flops per cell (2 DFMA + DADD + DMUL,
-    counted by ncu per stage) over the launch time, against the part's FP64 peak; and the share of
-    the pipe's lane slots its FP64 instructions fill (DADD + DMUL + DFMA per cell against 152 SMs x
-    2 lanes x the clock).  The kernel's faces and residuals run on the integer pipes (xfix.cuh), so only the
-    update and the norms are FP64 instructions and the share is small: the instruction counts are in the
-    committed ncu summary"""
+    """The FP64 stage kernel against the part's FP64 peak: its FP64 flops per cell (2 DFMA + DADD + DMUL, counted by ncu per
+    stage) over the launch time, and the share of the pipe's lane slots its FP64 instructions fill (DADD + DMUL +
+    DFMA per cell against 152 SMs x 2 lanes x the clock).  The kernel's faces, residuals and conversions run on the
+    integer pipes (xfix.cuh): what bounds it is those and instruction issue (the line's `issue`), only the update and the
+    norms are FP64 instructions, and both shares are small"""
     flops = profiled_numbers("fp64", "fp64 flops per cell and stage", workload)
-    out = {"bound": "alu", "kernel": "stage_kernel", "unit": "TFLOP/s", "peak": FP64_PEAK_TFLOPS,
+    out = {"bound": "alu", "kernel": hbm.get("kernel", "xstage_kernel"), "unit": "TFLOP/s", "peak": FP64_PEAK_TFLOPS,
+           "limiter": "integer pipes and instruction issue; the FP64 pipe holds the update and the norms",
            "peak_kind": "FP64 FMA lanes x clock (152 SMs x 2 x 2 flops x 2.07 GHz; 1.2524 measured by gbcfd_op_rate)",
            "avg_launch_ms": hbm["avg_launch_ms"],
            "traffic": hbm["traffic"], "hbm_frac": hbm["frac"]}

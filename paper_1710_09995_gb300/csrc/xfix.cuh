@@ -114,14 +114,13 @@ __host__ __device__ __forceinline__ XVal xdec_pos(double a) {  // a > 0
 // the exponent of an exact zero: below that of any product of doubles, so that a zero takes no part in the
 // class of a sum
 constexpr int XZERO = -8000;
-// any finite double: a zero as zero, a subnormal with its own (fewer) bits
+// any finite double [62]: a zero as zero, a subnormal with its own (fewer) bits
 __host__ __device__ __forceinline__ XVal xdec_zero(double a) {
-  XVal v = xdec<62>(a);
-  if (v.e == -1023) {
-    const long long m = (long long)(xbits(a) & 0xfffffffffffffull) << 9;
-    v = {v.m < 0 ? -m : m, m ? -1022 : XZERO};
-  }
-  return v;
+  const unsigned long long b = xbits(a);
+  const int hi = (int)(b >> 32), ex = (int)(((unsigned)hi >> 20) & 0x7ffu);
+  const unsigned long long mag = ((unsigned long long)(((unsigned)hi & 0xfffffu) | (ex ? 0x100000u : 0u)) << 32) | (unsigned)b;
+  const long long s = hi >> 31;
+  return {((long long)(mag << 9) ^ s) - s, ex ? ex - 1023 : (mag ? -1022 : XZERO)};
 }
 // the double nearest to m 2^(e - 61), |m| < 2^63; below the normal range subnormal, above it infinity, and
 // NaN for the exponents from XBAD up (a flux that has no value)
