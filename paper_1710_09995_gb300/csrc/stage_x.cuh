@@ -19,10 +19,12 @@
 // round one of them had 8.  On Cartesian blocks at TY 8 the flux buffers of two planes fit (PIPE): the warps
 // that have one face item update the rows of the plane before in the same turn, where 8 warps updated
 // between two barriers while 8 waited (36 uneven Euler blocks 19.6 -> 18.4 ms, 256^3 Navier-Stokes 20.4 -> 19.6).
-// Bound by the integer pipes: ALU 60% busy, issue slots 58-61%, the rest multiply-add latency at 4 warps a
-// scheduler.  Measured against the FP64-pipe form: 256^3 Navier-Stokes step 81.7 -> 19.6 ms, 36 uneven Euler
-// blocks (14.4M cells) 69.0 -> 18.4 ms, two steps of the bump channel 14.2 -> 3.9 ms, errors against 64-bit
-// references the same or smaller.
+// Bound by the integer pipes: ALU 60% busy, issue slots 57-61%, the rest multiply-add latency at 4 warps a
+// scheduler.  Measured against the FP64-pipe form: 256^3 Navier-Stokes step 81.7 -> 20.9 ms, 36 uneven Euler
+// blocks (14.4M cells) 69.0 -> 19.4 ms, two steps of the bump channel 14.2 -> 4.04 ms (19.6, 18.4 and 3.86 before every
+// term had a class of its own size: components far below the others, and cells beside jumps, then had errors 10^2 to
+// 10^9 times the FP64 form's).  Residuals of smooth states are 24 to 50 times closer to long double than
+// that form's, states after a step the same to 2.6 times.
 #pragma once
 #include "stage.cuh"
 

@@ -9,8 +9,9 @@
 // and the Roe flux 62-bit products, and Eq. 2 is taken of the integer fluxes.  One primitive
 // buffer (the next tile is requested when the fluxes are done, behind Eq. 2) and a separate flux
 // buffer keep two CTAs per SM.  Measured: a 128^3 Navier-Stokes step
-// 30.6 -> 9.75 ms (24.7 with only the Roe flux on integers); residuals against long double 1.4 to 2.3
-// times closer than the FP64 form's, 5 to 40 times on the finite-volume path.
+// 30.6 -> 9.75 ms (24.7 with only the Roe flux on integers), with the viscous pass and the primitives below 7.44, and 8.14 since
+// edges beside jumps and small components keep the FP64 form's accuracy.  Residuals of smooth states are
+// 2.6 to 2.8 times closer to long double than the FP64 form's, states after a step 1.05 to 2 times.
 #pragma once
 
 namespace gbcfd {
@@ -276,8 +277,9 @@ __global__ void __launch_bounds__(NTW, 2) xdir_kernel(Args a) {
 // neighbours and one for its stresses, a component 10^6 times smaller than the others had 2^-38 of itself left.)
 // 16 warps (the FP64 form had 8): a cell's four equations are
 // shared by two threads.  Two barriers a plane: the conversion of the next plane runs beside the
-// differences.  Measured (96^3): 434 -> 134 us a stage, with the primitives' 117 -> 70 a 128^3 step
-// 9.75 -> 7.85 ms (7.43 with the loads of the passes' ends brought forward and a warp per row of primitives).
+// differences.  Measured (96^3): 434 -> 134 us a stage, 160 with the exponents of today; with the primitives' 117 -> 70 a
+// 128^3 step 9.75 -> 7.85 ms (7.43 with the loads of the passes' ends brought forward and a warp per row of primitives).
+// An exponent for each velocity, difference and stress cost the step 0.15 ms.
 constexpr int XVT = 512, XWX = 42;  // threads; columns of the primitive box (41 are read; 16-byte rows)
 struct XRSmem {
   static constexpr int WF = WY * XWX, WP = 4 * WF;

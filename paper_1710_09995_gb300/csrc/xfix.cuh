@@ -14,8 +14,12 @@
 // from the class (written beside each line as the number of bits), so nothing overflows for any
 // finite input.  Sums then cost one 64-bit add.  Truncation is towards minus infinity.
 //
-// Measured on random states against quadruple precision (tests/test_xfix.py holds a bound): the
-// flux's root mean square error is 4-7e-17 of its size where the FP64 form's is 7-17e-17.
+// What shares a class: only terms that are added, and then a term that is far below its class (a difference, a
+// product, a component that vanishes) is normalised before the class of the sum is taken, an exact zero having an exponent
+// below all (XZERO): no term takes bits from another that is not there.  Sides of a face that are far apart go to
+// FP64 (xfar), and so do edge values that are small in their stencil.  tests/test_xfix_classes.py holds each component's error to
+// the FP64 form's; on smooth states the flux's is 4.5-6e-17 of its size (root mean square, the rounding to a double
+// included) where that form's is 8-16e-17.
 //
 // The scheme is plain fixed-point arithmetic with scaling by exponents ("block floating point",
 // J. H. Wilkinson, Rounding Errors in Algebraic Processes, 1963, ch. 1).
@@ -289,7 +293,7 @@ struct XFlux {
 // Twice the Roe flux with Harten's fix in the face frame, as roe_frame (physics.cuh), from the
 // sides' (rho, u_n, u_t1, u_t2, p).  [n] after a line: |m| < 2^n.  A product of [a] and [b] is
 // [a + b - 64] with exponent e_a + e_b + 3; << 2 then brings [60] back to [62].  Classes: Eu, Ev, Ew of
-// the velocities, EH of the enthalpies and q^2/2, El of the wave speeds, EM of the mass fluxes.
+// the velocities, EH of the enthalpies, Ek of q^2/2, El of the wave speeds, EM of the mass fluxes.
 // Where a value may be much smaller than its class (jumps, products of several factors) it is
 // normalised, so that later roundings are relative to it.
 // CURVI: (u, v, w) are the x, y, z velocities, un the velocity along the face normal n, whose components have their
