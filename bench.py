@@ -482,8 +482,9 @@ def fp64_alu_roofline(res, cells, steps, hbm, workload="vortex256"):
                     "flops_per_cell": flops})
         if ops:  # FP64 instructions per FMA issue slot (a DADD or DMUL counted as one; they issue at 84% of an FMA's rate)
             nops = sum(ops[s - 1] * cells * steps for s in (1, 2, 3))
-            out.update({"lane_slot_frac": round(nops / sec / (FP64_PEAK_TFLOPS / 2 * 1e12), 4),
-                        "ops_per_cell": ops})
+            lanes = round(nops / sec / (FP64_PEAK_TFLOPS / 2 * 1e12), 4)
+            if lanes > out["frac"]:  # (launches too short for four digits say nothing)
+                out.update({"lane_slot_frac": lanes, "ops_per_cell": ops})
     else:
         out.update({"achieved": None, "frac": None})
     return out
