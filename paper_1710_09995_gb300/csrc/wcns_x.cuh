@@ -11,7 +11,7 @@
 // buffer keep two CTAs per SM.  Measured: a 128^3 Navier-Stokes step
 // 30.6 -> 9.75 ms (24.7 with only the Roe flux on integers), with the viscous pass and the primitives below 7.44, and 8.14 since
 // edges beside jumps and small components keep the FP64 form's accuracy.  Residuals of smooth states are
-// 2.6 to 2.8 times closer to long double than the FP64 form's, states after a step 1.05 to 2 times.
+// 2.6 to 2.8 times closer to long double than the FP64 form's, states after a step 1.01 to 1.8 times.
 #pragma once
 
 namespace gbcfd {
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(NTW, 2) xdir_kernel(Args a) {
           const double adv = qs[q] - dt * tot;
           double out;
           if (a.stage == 1) out = adv;
-          else if (a.stage == 2) out = fma(0.75, qn[q], 0.25 * adv);
+          else if (a.stage == 2) out = fma(0.25, adv, 0.75 * qn[q]);  // rounded as the FP64 form was
           else {  // Q^n / 3 with one correction of the product (a division costs ~5 FMAs here)
             const double q3 = (1.0 / 3.0) * qn[q];
             out = fma(2.0 / 3.0, adv, fma(fma(-3.0, q3, qn[q]), 1.0 / 3.0, q3));
