@@ -186,11 +186,12 @@ def halves(n=(48, 8, 8), seed=9):
     return c, np.stack([w[0] * s, w[0] * s * s, w[0] * s * s, w[0] * s * s, w[0] * s ** 3]) / min(c.spacing)
 
 
-@pytest.mark.parametrize("curved", [False, True])
-def test_cells_beside_a_jump(gb, curved):
+@pytest.mark.parametrize("curved,viscous", [(False, False), (False, True), (True, False)])
+def test_cells_beside_a_jump(gb, curved, viscous):
     """every face at the jump, and those whose stencil it enters from beyond; in cells of the low side that have no face at
     it errors stay relative to that side (some 100 roundings of 1.1e-16)"""
     c, size = halves()
+    c.viscous, c.mu = viscous, 1e-7 if viscous else 0.0  # stresses about the size of the low side's fluxes
     if curved:
         c.nodes = curved_in_the_plane(c.nx, c.ny, c.nz)
     ref = fv_residual(c, *(plane_metrics(c.nodes) if curved else cartesian(c)))
